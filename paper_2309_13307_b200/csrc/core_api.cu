@@ -105,9 +105,27 @@ int ensure_workspace(core_ctx *ctx, size_t bytes) {
 bool valid_dtype(int dtype) { return dtype == CORE_F32 || dtype == CORE_BF16; }
 size_t elem_size(int dtype) { return dtype == CORE_BF16 ? 2 : 4; }
 
+// One machine's message comes from the single-row kernel (unless a test asks for one of the others).
+bool single_row(int32_t n) { return n == 1 && !project_kernel_forced(); }
+
+// Rounds of several machines whose messages nobody asks for: the mean message is linear in the gradients, so
+// the projection can add them up first and make one message instead of n.  That saves the n - 1 further
+// multiply-adds per Gaussian (a quarter of the projection at n = 8, a third at n = 32).  Below 2^26 Gaussians
+// (about 55 us of generating) the messages are formed one by one, so that a short round keeps giving the bits
+// of core_project + core_aggregate.
+constexpr int64_t kCombineFirst = (int64_t)1 << 26;
+bool combine_first(const core_ctx *ctx, int32_t n) {
+    return n > 1 && !project_kernel_forced() && ctx->d >= (kCombineFirst + ctx->m - 1) / ctx->m;
+}
+
+size_t row_partial_bytes(const core_ctx *ctx, int64_t d) {
+    const RowPlan plan = make_row_plan(ctx->m, d, ctx->sm_count);
+    return round_up((size_t)plan.grid_x * ctx->m * sizeof(float), 256);
+}
+
 // Bytes of partial sums the projection of n machines needs (largest group of a pass).
 size_t partial_bytes(const core_ctx *ctx, int32_t n, int64_t d, int dtype) {
-    size_t need = 0;
+    size_t need = row_partial_bytes(ctx, d);
     for (int32_t i0 = 0, ng = 0; i0 < n; i0 += ng) {
         ng = project_group(n - i0, ctx->m);
         const ProjectPlan plan = make_project_plan(ng, ctx->m, d, dtype, ctx->sm_count);
@@ -117,10 +135,20 @@ size_t partial_bytes(const core_ctx *ctx, int32_t n, int64_t d, int dtype) {
     return round_up(need, 256);
 }
 
+// message (m floats) = <scale * sum of `rows` rows, xi_j> over coordinates [0, d), added to what is there if asked.
+int project_row_into(core_ctx *ctx, const void *G, int dtype, int32_t rows, int64_t ldg, float scale, int64_t d,
+                     uint64_t q_base, float *partial, float *message, bool accumulate, cudaStream_t stream) {
+    const RowPlan plan = make_row_plan(ctx->m, d, ctx->sm_count);
+    CORE_CUDA(ctx, launch_project_row(plan, ctx->keys, ctx->t, G, dtype, rows, ldg, scale, d, ctx->m, q_base, partial, stream));
+    CORE_CUDA(ctx, launch_finish_project(partial, plan.grid_x, 1, ctx->m, message, accumulate, stream));
+    return CORE_OK;
+}
+
 // Projects rows [0, n) of a matrix whose coordinate 0 is global block q_base; the partial
 // sums go through `partial`; P (n*m) receives (or accumulates) the result.
 int project_into(core_ctx *ctx, const void *G, int dtype, int32_t n, int64_t ldg, int64_t d, uint64_t q_base,
                  float *partial, float *P, bool accumulate, cudaStream_t stream) {
+    if (single_row(n)) return project_row_into(ctx, G, dtype, 1, ldg, 1.0f, d, q_base, partial, P, accumulate, stream);
     for (int32_t i0 = 0, ng = 0; i0 < n; i0 += ng) {
         ng = project_group(n - i0, ctx->m);
         const ProjectPlan plan = make_project_plan(ng, ctx->m, d, dtype, ctx->sm_count);
@@ -293,7 +321,11 @@ static int round_with_epilogue(core_ctx *ctx, const void *G_dev, int dtype, int3
     if (int rc = ensure_workspace(ctx, pb + Pb)) return rc;
     float *partial = static_cast<float *>(ctx->ws);
     float *P = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb);
-    if (project_group(n, ctx->m) == n) {
+    if (single_row(n) || combine_first(ctx, n)) {
+        if (int rc = project_row_into(ctx, G_dev, dtype, n, ldg, 1.0f / (float)n, ctx->d, 0, partial, pbar_dev, false,
+                                      ctx->stream))
+            return rc;
+    } else if (project_group(n, ctx->m) == n) {
         // one group of machines: the per-machine messages are not kept, so they are never written
         const ProjectPlan plan = make_project_plan(n, ctx->m, ctx->d, dtype, ctx->sm_count);
         CORE_CUDA(ctx, launch_project(plan, ctx->keys, ctx->t, G_dev, dtype, n, ldg, ctx->d, ctx->m, 0, partial,
@@ -384,16 +416,14 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
         }
         ctx->slab_bytes = need_slab;
     }
-    const size_t pb = partial_bytes(ctx, n, slab, dtype);
-    const size_t Pb = round_up((size_t)n * ctx->m * sizeof(float), 256);
+    const size_t pb = row_partial_bytes(ctx, slab);
     const size_t mb = round_up((size_t)ctx->m * sizeof(float), 256);
-    if (int rc = ensure_workspace(ctx, pb + Pb + mb)) return rc;
+    if (int rc = ensure_workspace(ctx, pb + mb)) return rc;
     char *in_buf[2] = {static_cast<char *>(ctx->slab), static_cast<char *>(ctx->slab) + in_bytes};
     float *out_buf[2] = {reinterpret_cast<float *>(static_cast<char *>(ctx->slab) + 2 * in_bytes),
                          reinterpret_cast<float *>(static_cast<char *>(ctx->slab) + 2 * in_bytes + out_bytes)};
     float *partial = static_cast<float *>(ctx->ws);
-    float *P = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb);
-    float *pbar = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb + Pb);
+    float *pbar = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb);
 
     CORE_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // earlier work of the caller on this context
 
@@ -410,12 +440,12 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
                                            (size_t)len * es, cudaMemcpyHostToDevice, ctx->copy_stream));
         CORE_CUDA(ctx, cudaEventRecord(ctx->in_ready[b], ctx->copy_stream));
         CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->work_stream, ctx->in_ready[b], 0));
-        if (int rc = project_into(ctx, in_buf[b], dtype, n, slab, len, (uint64_t)k0 >> 2, partial, P, s > 0,
-                                  ctx->work_stream))
+        // the mean message, slab by slab (the gradients of a slab are added while they are staged)
+        if (int rc = project_row_into(ctx, in_buf[b], dtype, n, slab, 1.0f / (float)n, len, (uint64_t)k0 >> 2, partial, pbar,
+                                      s > 0, ctx->work_stream))
             return rc;
         CORE_CUDA(ctx, cudaEventRecord(ctx->in_free[b], ctx->work_stream));
     }
-    CORE_CUDA(ctx, launch_aggregate(P, n, ctx->m, pbar, ctx->work_stream));
     CORE_CUDA(ctx, cudaMemcpyAsync(pbar_host, pbar, (size_t)ctx->m * sizeof(float), cudaMemcpyDeviceToHost,
                                    ctx->work_stream));
     // reconstruction: slab s is copied back while slab s+1 is generated
@@ -510,22 +540,18 @@ static int ls_gradients_into(core_ctx *ctx, core_ls *ls, const float *x_dev, flo
 // it stages its tiles, so the machine gradients G are never written or read back.
 static int ls_round(core_ctx *ctx, core_ls *ls, const float *x_eval, float *out, const ReconstructEpilogue *epilogue,
                     const StepRule *rule = nullptr) {
-    if (ls->n <= kMaxGroup && ls_fused_usable(ls->fused_plan, ls->A, x_eval, ls->part)) {
-        const ProjectPlan plan = make_project_plan(ls->n, ctx->m, ctx->d, CORE_F32, ctx->sm_count);
-        if (plan.mma == 0) {
-            if (int rc = ensure_workspace(ctx, partial_bytes(ctx, ls->n, ctx->d, CORE_F32))) return rc;
-            float *partial = static_cast<float *>(ctx->ws);
-            CORE_CUDA(ctx, launch_ls_fused(ls->fused_plan, ls->A, ls->b, x_eval, ls->n, ls->rows, ls->d, ls->part,
-                                           ctx->stream));
-            CORE_CUDA(ctx, launch_project(plan, ctx->keys, ctx->t, ls->part, CORE_F32, ls->n, ls->d, ctx->d, ctx->m, 0,
-                                          partial, ctx->stream, ls->fused_plan.splits, 1.0f / (float)ls->rows));
-            CORE_CUDA(ctx, launch_finish_aggregate(partial, plan.grid_x, ls->n, ctx->m, ctx->pbar, ctx->stream));
-            if (int rc = apply_step_rule(ctx, rule, ctx->pbar)) return rc;
-            CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, ctx->pbar, ctx->m, 0, ctx->d, out, ctx->sm_count,
-                                              ctx->stream, epilogue));
-            ctx->t += 1;
-            return CORE_OK;
-        }
+    if (!project_kernel_forced() && ls_fused_usable(ls->fused_plan, ls->A, x_eval, ls->part)) {
+        if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
+        CORE_CUDA(ctx, launch_ls_fused(ls->fused_plan, ls->A, ls->b, x_eval, ls->n, ls->rows, ls->d, ls->part, ctx->stream));
+        if (int rc = project_row_into(ctx, ls->part, CORE_F32, ls->n * ls->fused_plan.splits, ls->d,
+                                      1.0f / ((float)ls->rows * (float)ls->n), ctx->d, 0, static_cast<float *>(ctx->ws),
+                                      ctx->pbar, false, ctx->stream))
+            return rc;
+        if (int rc = apply_step_rule(ctx, rule, ctx->pbar)) return rc;
+        CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, ctx->pbar, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream,
+                                          epilogue));
+        ctx->t += 1;
+        return CORE_OK;
     }
     if (int rc = ls_gradients_into(ctx, ls, x_eval, ls->G)) return rc;
     return round_with_epilogue(ctx, ls->G, CORE_F32, ls->n, ls->d, ctx->pbar, out, epilogue, rule);

@@ -19,6 +19,7 @@ int32_t project_group(int32_t n_left, int32_t m);
 // Test hook: -1 = choose by shape (default); 0 = always the scalar kernel; 1 = the warp-level tensor-core
 // kernel where its shape limits allow; 2 = the tensor-memory kernel for any group of machines it can take.
 void project_force_kernel(int kind);
+bool project_kernel_forced();      // anything but -1
 
 // Launch geometry of one projection pass, fixed by (n, m, d, dtype) on the host.
 struct ProjectPlan {
@@ -69,6 +70,22 @@ cudaError_t launch_wait_timeout_probe(uint64_t limit_ns, int code, uint32_t *obs
 cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint32_t t, const void *G,
                            int dtype, int32_t n, int64_t ldg, int64_t d, int32_t m, uint64_t q_base,
                            float *partial, cudaStream_t stream, int splits = 0, float scale = 1.0f);
+
+// Projection of one combined row (core_project_row.cu): partial[c*m + j] = the share of CTA column c in
+// <scale * (row 0 + row 1 + ... + row rows-1), xi_j>.  Rows are `ldg` elements apart and of any alignment.
+struct RowPlan {
+    int tile_q;       // coordinate blocks (of 4) per shared-memory tile
+    int tj;           // threads across vectors (four vectors each)
+    int tq;           // threads across coordinate blocks
+    int grid_x;       // CTAs across coordinates
+    int grid_y;       // CTAs across vectors
+    int64_t tiles;
+    size_t smem;
+};
+RowPlan make_row_plan(int32_t m, int64_t d, int sm_count);
+cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype,
+                               int32_t rows, int64_t ldg, float scale, int64_t d, int32_t m, uint64_t q_base,
+                               float *partial, cudaStream_t stream);
 
 // P[i*m+j] = (accumulate ? P[i*m+j] : 0) + sum_c partial[c][i][j], c ascending.
 cudaError_t launch_finish_project(const float *partial, int chunks, int32_t n, int32_t m, float *P,

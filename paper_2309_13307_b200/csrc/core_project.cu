@@ -305,14 +305,36 @@ cudaError_t launch_typed(const ProjectPlan &plan, const ProjectArgs &args, int d
     return launch_tiled<NB, JT, UQ, tile_q_for(NB)>(plan, args, dtype, stream);
 }
 
+// Column sums of the partial results.  The columns (up to 296) are cut into kFinishSlices ranges summed side by
+// side, then the ranges are added in ascending order: a single thread per entry would wait for L2 some seventy
+// times in a row (34 us at m = 256 and n = 8, where this takes 4).
+constexpr int kFinishSlices = 8;
+
+__device__ __forceinline__ float finish_slice(const float *__restrict__ partial, int chunks, int64_t total, int64_t idx, int slice) {
+    const int begin = chunks * slice / kFinishSlices, end = chunks * (slice + 1) / kFinishSlices;
+    float s = 0.f;
+#pragma unroll 8
+    for (int c = begin; c < end; ++c) s += partial[(int64_t)c * total + idx];
+    return s;
+}
+
+__device__ __forceinline__ float finish_join(const float (&slices)[kFinishSlices][32], int lane) {
+    float s = slices[0][lane];
+#pragma unroll
+    for (int r = 1; r < kFinishSlices; ++r) s += slices[r][lane];
+    return s;
+}
+
 __global__ void finish_project_kernel(const float *__restrict__ partial, int chunks, int n, int m,
                                       float *__restrict__ P, int accumulate) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ float slices[kFinishSlices][32];
+    const int64_t idx = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int64_t total = (int64_t)n * m;
-    if (idx >= total) return;
-    float s = accumulate ? P[idx] : 0.f;
-    for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * total + idx];
-    P[idx] = s;
+    slices[threadIdx.y][threadIdx.x] = idx < total ? finish_slice(partial, chunks, total, idx, threadIdx.y) : 0.f;
+    __syncthreads();
+    if (threadIdx.y != 0 || idx >= total) return;
+    const float s = finish_join(slices, threadIdx.x);
+    P[idx] = accumulate ? P[idx] + s : s;
 }
 
 __global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, float *__restrict__ pbar) {
@@ -325,22 +347,24 @@ __global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, floa
 
 // Both of the above in one launch for a single group of machines whose messages nobody asks for:
 // the same sums in the same order, so pbar is bitwise what the two kernels give.
+constexpr int kFinishMachines = 4;      // machines summed at a time
 __global__ void finish_aggregate_kernel(const float *__restrict__ partial, int chunks, int n, int m,
                                         float *__restrict__ pbar) {
-    __shared__ float message[kMaxGroupTc][32];     // P[i][j] of this block's 32 vectors
+    __shared__ float slices[kFinishMachines][kFinishSlices][32];
     const int j = blockIdx.x * 32 + threadIdx.x;
     const int64_t total = (int64_t)n * m;
-    for (int i = threadIdx.y; i < n; i += blockDim.y) {
-        float p = 0.f;
-        if (j < m)
-            for (int c = 0; c < chunks; ++c) p += partial[(int64_t)c * total + (int64_t)i * m + j];
-        message[i][threadIdx.x] = p;
+    const int slice = threadIdx.y % kFinishSlices, row = threadIdx.y / kFinishSlices;
+    float sum = 0.f;                    // kept by the first 32 threads
+    for (int i0 = 0; i0 < n; i0 += kFinishMachines) {
+        const int i = i0 + row;
+        slices[row][slice][threadIdx.x] =
+            i < n && j < m ? finish_slice(partial, chunks, total, (int64_t)i * m + j, slice) : 0.f;
+        __syncthreads();
+        if (threadIdx.y == 0)
+            for (int r = 0; r < kFinishMachines && i0 + r < n; ++r) sum += finish_join(slices[r], threadIdx.x);
+        __syncthreads();
     }
-    __syncthreads();
-    if (threadIdx.y != 0 || j >= m) return;
-    float s = 0.f;
-    for (int r = 0; r < n; ++r) s += message[r][threadIdx.x];
-    pbar[j] = s / (float)n;
+    if (threadIdx.y == 0 && j < m) pbar[j] = sum / (float)n;
 }
 
 int ilog2(int x) {
@@ -356,6 +380,7 @@ int g_force_kernel = -1;
 }
 
 void project_force_kernel(int kind) { g_force_kernel = kind; }
+bool project_kernel_forced() { return g_force_kernel >= 0; }
 
 int32_t project_group(int32_t n_left, int32_t m) {
     if (n_left > kMaxGroup && g_force_kernel != 0 && g_force_kernel != 1) {
@@ -459,16 +484,15 @@ cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint3
 cudaError_t launch_finish_project(const float *partial, int chunks, int32_t n, int32_t m, float *P,
                                   bool accumulate, cudaStream_t stream) {
     const int64_t total = (int64_t)n * m;
-    const int threads = 128;
-    finish_project_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, stream>>>(
-        partial, chunks, n, m, P, accumulate ? 1 : 0);
+    finish_project_kernel<<<(unsigned)((total + 31) / 32), dim3(32, kFinishSlices), 0, stream>>>(partial, chunks, n, m, P,
+                                                                                               accumulate ? 1 : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_finish_aggregate(const float *partial, int chunks, int32_t n, int32_t m, float *pbar,
                                     cudaStream_t stream) {
-    finish_aggregate_kernel<<<(m + 31) / 32, dim3(32, n > kMaxGroup ? 32 : kMaxGroup), 0, stream>>>(
-        partial, chunks, n, m, pbar);
+    const int rows = n < kFinishMachines ? n : kFinishMachines;
+    finish_aggregate_kernel<<<(m + 31) / 32, dim3(32, kFinishSlices * rows), 0, stream>>>(partial, chunks, n, m, pbar);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,422 @@
+// Projection of one combined gradient row: p_j = <scale * sum_r G_r, xi_j>, j < m.
+//
+// Used for a single machine, for the least-squares steps (the rows are the partial gradients of the row
+// ranges) and for rounds whose per-machine messages nobody asks for: the mean message is linear in the
+// gradients, pbar_j = (1/n) sum_i <g_i, xi_j> = <(1/n) sum_i g_i, xi_j>, so adding the gradients while they
+// are staged (n d additions) replaces the n d m multiply-adds of n separate messages by d m.
+//
+// What bounds it: the generator (see core_rng.cuh), like the other round kernels; with few vectors and many
+// rows, the reading of G.  A CTA has 8 generating warps and 2 staging warps.  The staging warps read the
+// rows of the next tile 16 bytes at a time (eight loads in flight per thread), add them up and store the
+// sum to one of two shared-memory tiles, next to a table of the block-dependent half of Philox; rows that
+// do not start on a 16-byte boundary are read in aligned vectors all the same, summed per alignment class
+// and shifted into place with warp shuffles.  The generating threads hold four vectors each and walk the
+// blocks of the tile: thread (jl, ql) of tj x tq, where tj = the number of vector quadruples of the CTA row
+// (any number, not a power of two: 100 vectors keep 250 of 256 threads busy).  The coordinates of a block
+// are stored as (0, 2, 1, 3), so that one 16-byte read delivers the multiplicands of the cosine and of the
+// sine lanes of both pairs as ready register pairs and S (g_c (y sp) + g_s cs) is four packed instructions
+// per counter.
+#include "core_internal.h"
+
+#include <cuda_bf16.h>
+
+namespace core {
+
+namespace {
+
+constexpr int kRowCompute = 256;                 // generating threads
+constexpr int kRowStagers = 64;                  // staging threads
+constexpr int kRowThreads = kRowCompute + kRowStagers;
+constexpr int kRowJT = 4;                        // vectors per generating thread
+constexpr int kRowWarps = kRowThreads / 32;
+
+struct RowArgs {
+    const void *G;
+    int64_t ldg;
+    int64_t d;
+    int64_t tiles;
+    uint64_t q_base;
+    float *partial;
+    int rows;
+    int period;      // rows r and r + period have the same alignment
+    int aligned;     // every tile of every row starts on a 16-byte boundary
+    float scale;
+    int m;
+    int tile_q;      // coordinate blocks per tile
+    int tj;          // threads across vectors
+    int tq;          // threads across blocks: tj * tq <= 256
+    uint32_t t;
+    RoundKeys keys;
+};
+
+template <typename GT>
+struct RowVec {
+    static constexpr int V = 16 / (int)sizeof(GT);          // elements per 16-byte vector
+};
+
+__device__ __forceinline__ float row_elem(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float row_elem(const __nv_bfloat16 *p) {
+    return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(p)) << 16);
+}
+
+__device__ __forceinline__ void row_add(float (&acc)[4], uint4 h) {
+    acc[0] += __uint_as_float(h.x);
+    acc[1] += __uint_as_float(h.y);
+    acc[2] += __uint_as_float(h.z);
+    acc[3] += __uint_as_float(h.w);
+}
+__device__ __forceinline__ void row_add(float (&acc)[8], uint4 h) {      // a bf16 is the upper half of an fp32
+    acc[0] += __uint_as_float(h.x << 16);
+    acc[1] += __uint_as_float(h.x & 0xFFFF0000u);
+    acc[2] += __uint_as_float(h.y << 16);
+    acc[3] += __uint_as_float(h.y & 0xFFFF0000u);
+    acc[4] += __uint_as_float(h.z << 16);
+    acc[5] += __uint_as_float(h.z & 0xFFFF0000u);
+    acc[6] += __uint_as_float(h.w << 16);
+    acc[7] += __uint_as_float(h.w & 0xFFFF0000u);
+}
+
+// acc[u] += rows r0, r0 + period, ... < r1 of the vectors at elements kv + u * stride of their rows.
+template <int US, int UR, typename GT, int V>
+__device__ __forceinline__ void row_sum(const RowArgs &a, int64_t kv, int64_t stride, int r0, int r1, float (&acc)[US][V]) {
+    const GT *G = static_cast<const GT *>(a.G);
+    const int step = a.period;
+    const int64_t row_stride = (int64_t)step * a.ldg;
+    if (kv >= 0 && kv + (US - 1) * stride + V <= a.d) {
+        const GT *p = G + (int64_t)r0 * a.ldg + kv;
+        for (int r = r0; r < r1; r += UR * step, p += UR * row_stride) {
+            uint4 h[US][UR];
+#pragma unroll
+            for (int i = 0; i < UR; ++i)
+#pragma unroll
+                for (int u = 0; u < US; ++u)
+                    h[u][i] = r + i * step < r1 ? __ldg(reinterpret_cast<const uint4 *>(p + i * row_stride + u * stride))
+                                                : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < UR; ++i)
+#pragma unroll
+                for (int u = 0; u < US; ++u) row_add(acc[u], h[u][i]);
+        }
+        return;
+    }
+    // some vector of this thread reaches beyond a row's ends: element by element, nothing outside [0, d)
+    for (int r = r0; r < r1; r += step) {
+        const GT *p = G + (int64_t)r * a.ldg;
+#pragma unroll
+        for (int u = 0; u < US; ++u)
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const int64_t k = kv + u * stride + e;
+                if (k >= 0 && k < a.d) acc[u][e] += row_elem(p + k);
+            }
+    }
+}
+
+// Moves the lanes' vectors (a contiguous run of 32 V elements, continued by lane 31's `ext`) down by W elements.
+template <int W, int V>
+__device__ __forceinline__ void row_shift(float (&acc)[V], float (&ext)[V], int lane) {
+    float in[W];
+#pragma unroll
+    for (int e = 0; e < W; ++e) {
+        const float from_next = __shfl_down_sync(0xffffffffu, acc[e], 1);
+        in[e] = lane == 31 ? ext[e] : from_next;
+    }
+#pragma unroll
+    for (int e = 0; e < V; ++e) acc[e] = e + W < V ? acc[e + W] : in[e + W - V];
+#pragma unroll
+    for (int e = 0; e + W < V; ++e) ext[e] = ext[e + W];
+}
+
+// Sum of rows [r0, r1) for the US segments of 32 V coordinates at k, k + 32 V, ...: lane l gets coordinates
+// k + 32 V u + V l + e.
+template <int US, int UR, bool ALIGNED, typename GT>
+__device__ __forceinline__ void row_segments(const RowArgs &a, int64_t k, int r0, int r1, int lane, float (&sum)[US][RowVec<GT>::V]) {
+    constexpr int V = RowVec<GT>::V;
+#pragma unroll
+    for (int u = 0; u < US; ++u)
+#pragma unroll
+        for (int e = 0; e < V; ++e) sum[u][e] = 0.f;
+    if constexpr (ALIGNED) {
+        row_sum<US, UR, GT, V>(a, k + V * lane, 32 * V, r0, r1, sum);
+    } else {
+        for (int c = 0; c < a.period && r0 + c < r1; ++c) {
+            // elements between the 16-byte boundary below and coordinate k of the rows of this class
+            const uintptr_t at = reinterpret_cast<uintptr_t>(static_cast<const GT *>(a.G) + (int64_t)(r0 + c) * a.ldg + k);
+            const int s = (int)((at / sizeof(GT)) & (V - 1));
+            if (s == 0) {
+                row_sum<US, UR, GT, V>(a, k + V * lane, 32 * V, r0 + c, r1, sum);
+                continue;
+            }
+            float acc[US][V], ext[US][V];
+#pragma unroll
+            for (int u = 0; u < US; ++u)
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[u][e] = ext[u][e] = 0.f;
+            row_sum<US, UR, GT, V>(a, k - s + V * lane, 32 * V, r0 + c, r1, acc);
+            if (lane == 31) row_sum<US, UR, GT, V>(a, k - s + 32 * V, 32 * V, r0 + c, r1, ext);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < US; ++u) {
+                if (s & 1) row_shift<1, V>(acc[u], ext[u], lane);
+                if (s & 2) row_shift<2, V>(acc[u], ext[u], lane);
+                if constexpr (V == 8)
+                    if (s & 4) row_shift<4, V>(acc[u], ext[u], lane);
+#pragma unroll
+                for (int e = 0; e < V; ++e) sum[u][e] += acc[u][e];
+            }
+        }
+    }
+}
+
+// Segments first, first + step, ... of the tile at coordinate k0 (`blocks` of its blocks exist) into `tile`.
+template <int US, int UR, bool ALIGNED, typename GT>
+__device__ __forceinline__ void row_stage(const RowArgs &a, int64_t k0, int blocks, int first, int step, int r0, int r1, int lane,
+                                          float4 *tile) {
+    constexpr int V = RowVec<GT>::V;
+    constexpr int SB = 8 * V;                                // blocks per segment
+    const int segments = (blocks + SB - 1) / SB;
+    for (int sg = first * US; sg < segments; sg += step * US) {
+        float sum[US][V];
+        row_segments<US, UR, ALIGNED, GT>(a, k0 + (int64_t)sg * (32 * V), r0, r1, lane, sum);
+#pragma unroll
+        for (int u = 0; u < US; ++u)
+#pragma unroll
+            for (int b = 0; b < V / 4; ++b) {
+                const int q = (sg + u) * SB + lane * (V / 4) + b;
+                if (q < blocks)
+                    tile[q] = make_float4(sum[u][4 * b] * a.scale, sum[u][4 * b + 2] * a.scale, sum[u][4 * b + 1] * a.scale,
+                                          sum[u][4 * b + 3] * a.scale);
+            }
+    }
+}
+
+// More segments at once where there are few rows to read per segment: about eight loads in flight either way.
+template <typename GT>
+__device__ __forceinline__ void row_stage_any(const RowArgs &a, int64_t k0, int blocks, int first, int step, int r0, int r1,
+                                              int lane, float4 *tile) {
+    const int per_class = (r1 - r0 + a.period - 1) / a.period;
+    if (a.aligned) {
+        if (per_class <= 2) row_stage<RowVec<GT>::V == 4 ? 4 : 2, 2, true, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
+        else row_stage<1, 8, true, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
+    } else {
+        if (per_class <= 2) row_stage<2, 2, false, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
+        else row_stage<1, 4, false, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
+    }
+}
+
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+
+template <typename GT>
+__global__ void __launch_bounds__(kRowThreads, 2)
+project_row_kernel(const __grid_constant__ RowArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4 *const tile0 = reinterpret_cast<float4 *>(smem_raw);           // two tiles of the combined row
+    uint4 *const tab0 = reinterpret_cast<uint4 *>(tile0 + 2 * a.tile_q);  // and two tables of QPart
+    constexpr int kSegBlocks = 8 * RowVec<GT>::V;
+    constexpr int kFull = 1, kEmpty = 3;                     // barrier ids: kFull + stage, kEmpty + stage
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t tile_begin = a.tiles * (int64_t)blockIdx.x / gridDim.x;
+    const int64_t tile_end = a.tiles * (int64_t)(blockIdx.x + 1) / gridDim.x;
+    const int64_t nq = (a.d + 3) >> 2;
+    auto blocks_of = [&](int64_t tile) { return (int)min((int64_t)a.tile_q, nq - tile * a.tile_q); };
+    auto fill_table = [&](int64_t tile, uint4 *tab, int first, int step) {
+        const uint32_t q0 = (uint32_t)(a.q_base + (uint64_t)tile * a.tile_q);
+        for (int e = first; e < blocks_of(tile); e += step) {
+            const QPart qp = philox_qpart(q0 + (uint32_t)e, a.t, a.keys);
+            tab[e] = make_uint4(qp.hi_b, qp.lo_b, qp.w3, 0u);
+        }
+    };
+
+    // the first tile is staged by all warps, nobody having anything else to do yet; a short tile with many rows (the
+    // partial gradients of a least-squares step) is cut into row ranges too
+    if (tile_begin < tile_end) {
+        const int blocks = blocks_of(tile_begin), segments = (blocks + kSegBlocks - 1) / kSegBlocks;
+        const int ranges = a.rows >= 2 * kRowWarps ? kRowWarps / segments : 1;
+        if (ranges > 1) {
+            float4 *const scratch = reinterpret_cast<float4 *>(tab0 + 2 * a.tile_q);
+            const int range = warp / segments;
+            const int per = ((a.rows + ranges - 1) / ranges + a.period - 1) / a.period * a.period;
+            if (range < ranges)
+                row_stage_any<GT>(a, 4 * tile_begin * a.tile_q, blocks, warp % segments, segments, min(range * per, a.rows),
+                                  min((range + 1) * per, a.rows), lane, scratch + range * blocks);
+            __syncthreads();
+            for (int q = tid; q < blocks; q += kRowThreads) {
+                float4 s = scratch[q];
+                for (int r = 1; r < ranges; ++r) {
+                    const float4 p = scratch[r * blocks + q];
+                    s = make_float4(s.x + p.x, s.y + p.y, s.z + p.z, s.w + p.w);
+                }
+                tile0[q] = s;
+            }
+        } else {
+            row_stage_any<GT>(a, 4 * tile_begin * a.tile_q, blocks, warp, kRowWarps, 0, a.rows, lane, tile0);
+        }
+        fill_table(tile_begin, tab0, tid, kRowThreads);
+    }
+    __syncthreads();
+
+    if (warp >= kRowCompute / 32) {
+        // staging warps: tile i into stage i & 1 once the generating warps have left it
+        for (int64_t tile = tile_begin + 1; tile < tile_end; ++tile) {
+            const int i = (int)(tile - tile_begin), st = i & 1;
+            if (i >= 2) bar_sync(kEmpty + st, kRowThreads);
+            row_stage_any<GT>(a, 4 * tile * a.tile_q, blocks_of(tile), warp - kRowCompute / 32, kRowStagers / 32, 0, a.rows, lane,
+                              tile0 + st * a.tile_q);
+            fill_table(tile, tab0 + st * a.tile_q, tid - kRowCompute, kRowStagers);
+            __threadfence_block();
+            bar_arrive(kFull + st, kRowThreads);
+        }
+        __syncthreads();
+        __syncthreads();
+        return;
+    }
+
+    const int ql = tid / a.tj, jl = tid - ql * a.tj;
+    const bool active = ql < a.tq;
+    const int jbase = blockIdx.y * a.tj * kRowJT;
+    float outer[kRowJT];
+    JPart jp[kRowJT];
+#pragma unroll
+    for (int v = 0; v < kRowJT; ++v) outer[v] = 0.f;
+    uint32_t jp_q_hi = 0;
+    bool have_jp = false;
+    for (int64_t tile = tile_begin; tile < tile_end; ++tile) {
+        const int i = (int)(tile - tile_begin), st = i & 1;
+        if (i >= 1) bar_sync(kFull + st, kRowThreads);
+        const float4 *cur = tile0 + st * a.tile_q;
+        const uint4 *tab = tab0 + st * a.tile_q;
+        const int blocks = blocks_of(tile);
+        const uint64_t q0 = a.q_base + (uint64_t)tile * a.tile_q;
+        // blocks of this tile that share the high counter word of the first one (all of them but once in 2^32)
+        const uint64_t left = 0x100000000ull - (q0 & 0xFFFFFFFFull);
+        int upto = left < (uint64_t)blocks ? (int)left : blocks;
+        uint32_t q_hi = (uint32_t)(q0 >> 32);
+        float2 acc[kRowJT];
+#pragma unroll
+        for (int v = 0; v < kRowJT; ++v) acc[v] = make_float2(0.f, 0.f);
+        int qq = ql;
+        if (active) {
+            for (;;) {
+                if (!have_jp || q_hi != jp_q_hi) {
+#pragma unroll
+                    for (int v = 0; v < kRowJT; ++v) jp[v] = philox_jpart((uint32_t)(jbase + jl + v * a.tj), q_hi, a.keys);
+                    jp_q_hi = q_hi;
+                    have_jp = true;
+                }
+                for (; qq < upto; qq += a.tq) {
+                    const uint4 e = tab[qq];
+                    QPart qp;
+                    qp.hi_b = e.x;
+                    qp.lo_b = e.y;
+                    qp.w3 = e.z;
+                    uint4 w[kRowJT];
+#pragma unroll
+                    for (int v = 0; v < kRowJT; ++v) w[v] = philox_combine(jp[v], qp, a.keys);
+                    BmParts r[kRowJT];
+                    box_muller_parts<kRowJT>(w, r);
+                    const float4 g = cur[qq];
+                    const float2 gc = make_float2(g.x, g.y), gs = make_float2(g.z, g.w);
+#pragma unroll
+                    for (int v = 0; v < kRowJT; ++v) {
+                        const float2 c = __fmul2_rn(__fmul2_rn(r[v].y, r[v].sp), gc);
+                        acc[v] = __ffma2_rn(r[v].s, __ffma2_rn(r[v].cs, gs, c), acc[v]);
+                    }
+                }
+                if (upto == blocks) break;
+                upto = blocks;
+                ++q_hi;
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
+        if (tile + 2 < tile_end) bar_arrive(kEmpty + st, kRowThreads);
+    }
+
+    // fixed-order sum over the ql lanes
+    __syncthreads();
+    float *red = reinterpret_cast<float *>(smem_raw);
+    const int plane = kRowJT * a.tj;
+    if (active)
+#pragma unroll
+        for (int v = 0; v < kRowJT; ++v) red[ql * plane + v * a.tj + jl] = outer[v];
+    __syncthreads();
+    for (int idx = tid; idx < plane; idx += kRowCompute) {
+        float s = 0.f;
+        for (int l = 0; l < a.tq; ++l) s += red[l * plane + idx];
+        if (jbase + idx < a.m) a.partial[(int64_t)blockIdx.x * a.m + jbase + idx] = s;
+    }
+}
+
+}  // namespace
+
+RowPlan make_row_plan(int32_t m, int64_t d, int sm_count) {
+    RowPlan p{};
+    // Threads across vectors: one per quadruple, in as few CTA rows as keep at least 15/16 of the generating
+    // threads busy (every CTA row stages the gradients again)
+    const int quads = (m + kRowJT - 1) / kRowJT;
+    double best = -1.0;
+    for (int g = (quads + kRowCompute - 1) / kRowCompute, tried = 0; tried < 8 && g <= quads; ++g, ++tried) {
+        const int tj = (quads + g - 1) / g, tq = kRowCompute / tj;
+        const double busy = (double)quads / g * tq / kRowCompute;
+        if (busy > best + 0.02) {
+            best = busy;
+            p.grid_y = g;
+            p.tj = tj;
+            p.tq = tq;
+        }
+        if (busy >= 15.0 / 16.0) break;
+    }
+    const int64_t nq = (d + 3) >> 2;
+    int64_t slots = (int64_t)sm_count * 2 / p.grid_y;             // CTAs across coordinates that are resident together
+    if (slots < 1) slots = 1;
+    // blocks per tile: a generating thread takes 32 steps per tile, fewer where d is too short for every CTA to
+    // get eight tiles or so
+    int64_t steps = 32;
+    while (steps > 1 && nq < slots * 8 * steps * p.tq) steps /= 2;
+    int64_t tile_q = steps * p.tq;
+    if (tile_q > 1024) tile_q = tile_q / 1024 ? (1024 / p.tq) * p.tq : 1024;
+    p.tile_q = (int)tile_q;
+    p.tiles = (nq + p.tile_q - 1) / p.tile_q;
+    p.grid_x = (int)(slots < p.tiles ? slots : p.tiles);
+    // two tiles, two tables, and the row ranges of a short first tile (at most kRowWarps segments of 64 blocks)
+    const size_t stage = 2 * (size_t)p.tile_q * (16 + 16) + (size_t)kRowWarps * 64 * 16;
+    const size_t red = (size_t)p.tj * p.tq * kRowJT * 4;
+    p.smem = stage > red ? stage : red;
+    return p;
+}
+
+cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype, int32_t rows,
+                               int64_t ldg, float scale, int64_t d, int32_t m, uint64_t q_base, float *partial,
+                               cudaStream_t stream) {
+    RowArgs a{};
+    a.G = G;
+    a.ldg = ldg;
+    a.d = d;
+    a.tiles = plan.tiles;
+    a.q_base = q_base;
+    a.partial = partial;
+    a.rows = rows;
+    const int v = dtype == 1 ? 8 : 4;
+    a.period = 1;
+    while ((int64_t)a.period * ldg % v != 0) a.period *= 2;
+    a.aligned = a.period == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0 && 4 * plan.tile_q % v == 0;
+    a.scale = scale;
+    a.m = m;
+    a.tile_q = plan.tile_q;
+    a.tj = plan.tj;
+    a.tq = plan.tq;
+    a.t = t;
+    a.keys = keys;
+    const dim3 grid(plan.grid_x, plan.grid_y);
+    auto go = [&](auto kernel) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, kRowThreads, plan.smem, stream>>>(a);
+        return cudaGetLastError();
+    };
+    return dtype == 1 ? go(project_row_kernel<__nv_bfloat16>) : go(project_row_kernel<float>);
+}
+
+}  // namespace core

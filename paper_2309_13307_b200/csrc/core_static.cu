@@ -95,19 +95,23 @@ int core_project_static(uint64_t seed, uint32_t t, int64_t d, int32_t m, const v
         if (cuda_error_out) *cuda_error_out = (int)e;
         return CORE_ECUDA;
     }
+    const bool single = n == 1 && !project_kernel_forced();           // as core_project does
     ProjectPlan plan = make_project_plan(n, m, d, dtype, sm_count);
+    RowPlan row_plan = make_row_plan(m, d, sm_count);
     // fewer CTA columns if the usual number would overflow the array (slower, same result up to
     // the order of the final additions)
     const size_t per_column = (size_t)n * (size_t)m;
     const size_t max_columns = kStaticScratchFloats / per_column;
-    if ((size_t)plan.grid_x > max_columns) plan.grid_x = (int)max_columns;
+    int &columns = single ? row_plan.grid_x : plan.grid_x;
+    if ((size_t)columns > max_columns) columns = (int)max_columns;
 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const RoundKeys keys = expand_keys(seed);
     // every (column, machine, vector) entry below grid_x * n * m is overwritten by the kernel
     // before the second kernel reads it: nothing in the array has to start at zero
-    e = launch_project(plan, keys, t, G_dev, dtype, n, ldg, d, m, 0, scratch, stream);
-    if (e == cudaSuccess) e = launch_finish_project(scratch, plan.grid_x, n, m, P_dev, false, stream);
+    e = single ? launch_project_row(row_plan, keys, t, G_dev, dtype, 1, ldg, 1.0f, d, m, 0, scratch, stream)
+               : launch_project(plan, keys, t, G_dev, dtype, n, ldg, d, m, 0, scratch, stream);
+    if (e == cudaSuccess) e = launch_finish_project(scratch, columns, n, m, P_dev, false, stream);
     if (e != cudaSuccess) {
         if (cuda_error_out) *cuda_error_out = (int)e;
         return CORE_ECUDA;
