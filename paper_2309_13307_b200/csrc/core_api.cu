@@ -110,10 +110,10 @@ bool single_row(int32_t n) { return n == 1 && !project_kernel_forced(); }
 
 // Rounds of several machines whose messages nobody asks for: the mean message is linear in the gradients, so
 // the projection can add them up first and make one message instead of n.  That saves the n - 1 further
-// multiply-adds per Gaussian (a quarter of the projection at n = 8, a third at n = 32).  Below 2^26 Gaussians
-// (about 55 us of generating) the messages are formed one by one, so that a short round keeps giving the bits
+// multiply-adds per Gaussian (a quarter of the projection at n = 8, a third at n = 32).  Below 2^25 Gaussians
+// (about 28 us of generating) the messages are formed one by one, so that a short round keeps giving the bits
 // of core_project + core_aggregate.
-constexpr int64_t kCombineFirst = (int64_t)1 << 26;
+constexpr int64_t kCombineFirst = (int64_t)1 << 25;
 bool combine_first(const core_ctx *ctx, int32_t n) {
     return n > 1 && !project_kernel_forced() && ctx->d >= (kCombineFirst + ctx->m - 1) / ctx->m;
 }

@@ -8,7 +8,7 @@
 // What bounds it: the generator (see core_rng.cuh), like the other round kernels; with few vectors and many
 // rows, the reading of G.  A CTA has 8 generating warps and 2 staging warps.  The staging warps read the
 // rows of the next tile 16 bytes at a time (eight loads in flight per thread), add them up and store the
-// sum to one of two shared-memory tiles, next to a table of the block-dependent half of Philox; rows that
+// sum to one of two shared-memory tiles, next to the block-dependent half of Philox; rows that
 // do not start on a 16-byte boundary are read in aligned vectors all the same, summed per alignment class
 // and shifted into place with warp shuffles.  The generating threads hold four vectors each and walk the
 // blocks of the tile: thread (jl, ql) of tj x tq, where tj = the number of vector quadruples of the CTA row
@@ -168,9 +168,10 @@ __device__ __forceinline__ void row_segments(const RowArgs &a, int64_t k, int r0
     }
 }
 
-// Segments first, first + step, ... of the tile at coordinate k0 (`blocks` of its blocks exist) into `tile`.
+// Segments first, first + step, ... of the tile at coordinate k0 (`blocks` of its blocks exist) into `tile`, `stride` float4
+// apart per block.
 template <int US, int UR, bool ALIGNED, typename GT>
-__device__ __forceinline__ void row_stage(const RowArgs &a, int64_t k0, int blocks, int first, int step, int r0, int r1, int lane,
+__device__ __forceinline__ void row_stage(int stride, const RowArgs &a, int64_t k0, int blocks, int first, int step, int r0, int r1, int lane,
                                           float4 *tile) {
     constexpr int V = RowVec<GT>::V;
     constexpr int SB = 8 * V;                                // blocks per segment
@@ -184,23 +185,25 @@ __device__ __forceinline__ void row_stage(const RowArgs &a, int64_t k0, int bloc
             for (int b = 0; b < V / 4; ++b) {
                 const int q = (sg + u) * SB + lane * (V / 4) + b;
                 if (q < blocks)
-                    tile[q] = make_float4(sum[u][4 * b] * a.scale, sum[u][4 * b + 2] * a.scale, sum[u][4 * b + 1] * a.scale,
+                    tile[q * stride] = make_float4(sum[u][4 * b] * a.scale, sum[u][4 * b + 2] * a.scale, sum[u][4 * b + 1] * a.scale,
                                           sum[u][4 * b + 3] * a.scale);
             }
     }
 }
 
-// More segments at once where there are few rows to read per segment: about eight loads in flight either way.
+// More segments at once where there are few rows to read per segment: about eight loads in flight either way, twelve
+// where there are many rows (n = 50, m = 21, d = 1.2e7: 1596 -> 951 us together with eight for unaligned rows).
 template <typename GT>
-__device__ __forceinline__ void row_stage_any(const RowArgs &a, int64_t k0, int blocks, int first, int step, int r0, int r1,
+__device__ __forceinline__ void row_stage_any(int stride, const RowArgs &a, int64_t k0, int blocks, int first, int step, int r0, int r1,
                                               int lane, float4 *tile) {
     const int per_class = (r1 - r0 + a.period - 1) / a.period;
     if (a.aligned) {
-        if (per_class <= 2) row_stage<RowVec<GT>::V == 4 ? 4 : 2, 2, true, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
-        else row_stage<1, 8, true, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
+        if (per_class <= 2) row_stage<RowVec<GT>::V == 4 ? 4 : 2, 2, true, GT>(stride, a, k0, blocks, first, step, r0, r1, lane, tile);
+        else if (per_class > 8) row_stage<1, 12, true, GT>(stride, a, k0, blocks, first, step, r0, r1, lane, tile);
+        else row_stage<1, 8, true, GT>(stride, a, k0, blocks, first, step, r0, r1, lane, tile);
     } else {
-        if (per_class <= 2) row_stage<2, 2, false, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
-        else row_stage<1, 4, false, GT>(a, k0, blocks, first, step, r0, r1, lane, tile);
+        if (per_class <= 2) row_stage<2, 2, false, GT>(stride, a, k0, blocks, first, step, r0, r1, lane, tile);
+        else row_stage<1, 8, false, GT>(stride, a, k0, blocks, first, step, r0, r1, lane, tile);
     }
 }
 
@@ -211,8 +214,9 @@ template <typename GT>
 __global__ void __launch_bounds__(kRowThreads, 2)
 project_row_kernel(const __grid_constant__ RowArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4 *const tile0 = reinterpret_cast<float4 *>(smem_raw);           // two tiles of the combined row
-    uint4 *const tab0 = reinterpret_cast<uint4 *>(tile0 + 2 * a.tile_q);  // and two tables of QPart
+    // two tiles of {coordinates of the combined row, QPart} per block, side by side so that a step addresses both
+    // with one pointer (two separate arrays: 5426 against 5276 us at d = 2.5e7, m = 256)
+    float4 *const tile0 = reinterpret_cast<float4 *>(smem_raw);
     constexpr int kSegBlocks = 8 * RowVec<GT>::V;
     constexpr int kFull = 1, kEmpty = 3;                     // barrier ids: kFull + stage, kEmpty + stage
 
@@ -221,11 +225,11 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     const int64_t tile_end = a.tiles * (int64_t)(blockIdx.x + 1) / gridDim.x;
     const int64_t nq = (a.d + 3) >> 2;
     auto blocks_of = [&](int64_t tile) { return (int)min((int64_t)a.tile_q, nq - tile * a.tile_q); };
-    auto fill_table = [&](int64_t tile, uint4 *tab, int first, int step) {
+    auto fill_table = [&](int64_t tile, float4 *dst, int first, int step) {
         const uint32_t q0 = (uint32_t)(a.q_base + (uint64_t)tile * a.tile_q);
         for (int e = first; e < blocks_of(tile); e += step) {
             const QPart qp = philox_qpart(q0 + (uint32_t)e, a.t, a.keys);
-            tab[e] = make_uint4(qp.hi_b, qp.lo_b, qp.w3, 0u);
+            reinterpret_cast<uint4 *>(dst)[2 * e + 1] = make_uint4(qp.hi_b, qp.lo_b, qp.w3, 0u);
         }
     };
 
@@ -235,11 +239,11 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         const int blocks = blocks_of(tile_begin), segments = (blocks + kSegBlocks - 1) / kSegBlocks;
         const int ranges = a.rows >= 2 * kRowWarps ? kRowWarps / segments : 1;
         if (ranges > 1) {
-            float4 *const scratch = reinterpret_cast<float4 *>(tab0 + 2 * a.tile_q);
+            float4 *const scratch = tile0 + 4 * a.tile_q;
             const int range = warp / segments;
             const int per = ((a.rows + ranges - 1) / ranges + a.period - 1) / a.period * a.period;
             if (range < ranges)
-                row_stage_any<GT>(a, 4 * tile_begin * a.tile_q, blocks, warp % segments, segments, min(range * per, a.rows),
+                row_stage_any<GT>(1, a, 4 * tile_begin * a.tile_q, blocks, warp % segments, segments, min(range * per, a.rows),
                                   min((range + 1) * per, a.rows), lane, scratch + range * blocks);
             __syncthreads();
             for (int q = tid; q < blocks; q += kRowThreads) {
@@ -248,12 +252,12 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                     const float4 p = scratch[r * blocks + q];
                     s = make_float4(s.x + p.x, s.y + p.y, s.z + p.z, s.w + p.w);
                 }
-                tile0[q] = s;
+                tile0[2 * q] = s;
             }
         } else {
-            row_stage_any<GT>(a, 4 * tile_begin * a.tile_q, blocks, warp, kRowWarps, 0, a.rows, lane, tile0);
+            row_stage_any<GT>(2, a, 4 * tile_begin * a.tile_q, blocks, warp, kRowWarps, 0, a.rows, lane, tile0);
         }
-        fill_table(tile_begin, tab0, tid, kRowThreads);
+        fill_table(tile_begin, tile0, tid, kRowThreads);
     }
     __syncthreads();
 
@@ -262,9 +266,9 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         for (int64_t tile = tile_begin + 1; tile < tile_end; ++tile) {
             const int i = (int)(tile - tile_begin), st = i & 1;
             if (i >= 2) bar_sync(kEmpty + st, kRowThreads);
-            row_stage_any<GT>(a, 4 * tile * a.tile_q, blocks_of(tile), warp - kRowCompute / 32, kRowStagers / 32, 0, a.rows, lane,
-                              tile0 + st * a.tile_q);
-            fill_table(tile, tab0 + st * a.tile_q, tid - kRowCompute, kRowStagers);
+            row_stage_any<GT>(2, a, 4 * tile * a.tile_q, blocks_of(tile), warp - kRowCompute / 32, kRowStagers / 32, 0, a.rows, lane,
+                              tile0 + 2 * st * a.tile_q);
+            fill_table(tile, tile0 + 2 * st * a.tile_q, tid - kRowCompute, kRowStagers);
             __threadfence_block();
             bar_arrive(kFull + st, kRowThreads);
         }
@@ -285,8 +289,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     for (int64_t tile = tile_begin; tile < tile_end; ++tile) {
         const int i = (int)(tile - tile_begin), st = i & 1;
         if (i >= 1) bar_sync(kFull + st, kRowThreads);
-        const float4 *cur = tile0 + st * a.tile_q;
-        const uint4 *tab = tab0 + st * a.tile_q;
+        const float4 *cur = tile0 + 2 * st * a.tile_q;
         const int blocks = blocks_of(tile);
         const uint64_t q0 = a.q_base + (uint64_t)tile * a.tile_q;
         // blocks of this tile that share the high counter word of the first one (all of them but once in 2^32)
@@ -305,18 +308,18 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                     jp_q_hi = q_hi;
                     have_jp = true;
                 }
-                for (; qq < upto; qq += a.tq) {
-                    const uint4 e = tab[qq];
+                const float4 *entry = cur + 2 * qq;
+                for (; qq < upto; qq += a.tq, entry += 2 * a.tq) {
+                    const float4 g = entry[0], e = entry[1];
                     QPart qp;
-                    qp.hi_b = e.x;
-                    qp.lo_b = e.y;
-                    qp.w3 = e.z;
+                    qp.hi_b = __float_as_uint(e.x);
+                    qp.lo_b = __float_as_uint(e.y);
+                    qp.w3 = __float_as_uint(e.z);
                     uint4 w[kRowJT];
 #pragma unroll
                     for (int v = 0; v < kRowJT; ++v) w[v] = philox_combine(jp[v], qp, a.keys);
                     BmParts r[kRowJT];
                     box_muller_parts<kRowJT>(w, r);
-                    const float4 g = cur[qq];
                     const float2 gc = make_float2(g.x, g.y), gs = make_float2(g.z, g.w);
 #pragma unroll
                     for (int v = 0; v < kRowJT; ++v) {
@@ -371,13 +374,19 @@ RowPlan make_row_plan(int32_t m, int64_t d, int sm_count) {
     const int64_t nq = (d + 3) >> 2;
     int64_t slots = (int64_t)sm_count * 2 / p.grid_y;             // CTAs across coordinates that are resident together
     if (slots < 1) slots = 1;
-    // blocks per tile: a generating thread takes 32 steps per tile, fewer where d is too short for every CTA to
-    // get eight tiles or so
-    int64_t steps = 32;
-    while (steps > 1 && nq < slots * 8 * steps * p.tq) steps /= 2;
-    int64_t tile_q = steps * p.tq;
-    if (tile_q > 1024) tile_q = tile_q / 1024 ? (1024 / p.tq) * p.tq : 1024;
-    p.tile_q = (int)tile_q;
+    // blocks per tile: as many steps per tile and generating thread as fit (32, or 1024 blocks: two tiles take 64 KB),
+    // and of the tile counts per CTA from there on the one that leaves the fewest steps to the CTA with most of them
+    // (d = 1e6, m = 100: 104 -> 98 us)
+    const int64_t most = 32 * p.tq < 1024 ? 32 * p.tq : 1024 / p.tq * p.tq;
+    const int64_t least_tiles = (nq + slots * most - 1) / (slots * most);
+    int64_t best_steps = -1;
+    for (int64_t k = least_tiles; k <= 2 * least_tiles && k < least_tiles + 16; ++k) {
+        const int64_t steps = ((nq + slots * k - 1) / (slots * k) + p.tq - 1) / p.tq;
+        if (best_steps < 0 || k * steps < best_steps) {
+            best_steps = k * steps;
+            p.tile_q = (int)(steps * p.tq);
+        }
+    }
     p.tiles = (nq + p.tile_q - 1) / p.tile_q;
     p.grid_x = (int)(slots < p.tiles ? slots : p.tiles);
     // two tiles, two tables, and the row ranges of a short first tile (at most kRowWarps segments of 64 blocks)
