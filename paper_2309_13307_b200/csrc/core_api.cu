@@ -2,6 +2,7 @@
 // Every entry point is declared, with its contract, in include/core.h.
 #include "core.h"
 
+#include <algorithm>
 #include <atomic>
 #include <new>
 
@@ -36,13 +37,15 @@ struct core_ls {
     int32_t n, rows;
     int64_t d;
     int device;
-    LsPlan plan;         // two passes over A (any shape)
-    LsPlan fused_plan;   // one pass over A (d <= 8192, d % 4 == 0); splits == 0 if it does not apply
-    float *res;          // n*rows
-    float *part;         // n*splits*d
+    LsPass step_pass;    // one pass over A, the machines' gradients added up (for the steps)
+    LsPass machine_pass; // one pass over A, one gradient per machine
+    LsPlan plan;         // two passes over A, where rows are too long for one (step_pass.units == 0)
+    float *res;          // n*rows, two passes only
+    float *part;         // partial gradients
     float *G;            // n*d
     float *y;            // d: look-ahead point of the accelerated step / trial point of the guarded step
-    double *f_trial;     // loss at the trial point
+    double *f_parts;     // loss at the trial point, one sum per unit of step_pass (or one in all)
+    double *loss;        // loss on its way to the host
     int *accepted;       // 1 if the last guarded step took the trial point
     float *step;         // step chosen on the device (Option I of Algorithm 3), then its statistic p
 };
@@ -261,7 +264,12 @@ int core_device_status(int32_t *status_out) {
         cudaGetLastError();
         return CORE_ECUDA;
     }
-    *status_out = status;
+    int pass = 0;
+    if (ls_pass_take_status(&pass) != cudaSuccess) {
+        cudaGetLastError();
+        return CORE_ECUDA;
+    }
+    *status_out = status > pass ? status : pass;
     return CORE_OK;
 }
 
@@ -488,16 +496,26 @@ int core_ls_create(core_ls **out, const float *A_dev, const float *b_dev, int32_
         delete ls;
         return CORE_ECUDA;
     }
-    ls->plan = make_ls_plan(n, rows, d, sm);
-    ls->fused_plan = make_ls_fused_plan(n, rows, d, sm);
-    const int max_splits = ls->plan.splits > ls->fused_plan.splits ? ls->plan.splits : ls->fused_plan.splits;
-    const size_t res_b = round_up((size_t)n * rows * sizeof(float), 256);
-    const size_t part_b = round_up((size_t)n * max_splits * (size_t)d * sizeof(float), 256);
+    ls->step_pass = make_ls_pass(n, rows, d, false, sm);
+    ls->machine_pass = make_ls_pass(n, rows, d, true, sm);
+    if (ls->machine_pass.units == 0) ls->step_pass = LsPass{};
+    const bool one_pass = ls->step_pass.units > 0;
+    size_t part = 0;
+    if (one_pass) {
+        const size_t together = ls_pass_partials(ls->step_pass), apart = ls_pass_partials(ls->machine_pass);
+        part = std::max(together, apart);
+    } else {
+        ls->plan = make_ls_plan(n, rows, d, sm);
+        part = (size_t)n * ls->plan.splits * (size_t)d;
+    }
+    const size_t res_b = one_pass ? 256 : round_up((size_t)n * rows * sizeof(float), 256);
+    const size_t part_b = round_up(part * sizeof(float), 256);
     const size_t G_b = round_up((size_t)n * (size_t)d * sizeof(float), 256);
     const size_t gt_b = round_up((size_t)d * sizeof(float), 256);
-    const size_t scalars_b = 256;                          // trial loss (double) and acceptance flag
+    const size_t f_b = round_up((size_t)(one_pass ? ls->step_pass.units : 1) * sizeof(double), 256);
+    const size_t scalars_b = 256;                          // loss, acceptance flag, step and statistic
     char *base = nullptr;
-    e = core_malloc(reinterpret_cast<void **>(&base), res_b + part_b + G_b + gt_b + scalars_b);
+    e = core_malloc(reinterpret_cast<void **>(&base), res_b + part_b + G_b + gt_b + f_b + scalars_b);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete ls;
@@ -507,9 +525,11 @@ int core_ls_create(core_ls **out, const float *A_dev, const float *b_dev, int32_
     ls->part = reinterpret_cast<float *>(base + res_b);
     ls->G = reinterpret_cast<float *>(base + res_b + part_b);
     ls->y = reinterpret_cast<float *>(base + res_b + part_b + G_b);
-    ls->f_trial = reinterpret_cast<double *>(base + res_b + part_b + G_b + gt_b);
-    ls->accepted = reinterpret_cast<int *>(base + res_b + part_b + G_b + gt_b + 16);
-    ls->step = reinterpret_cast<float *>(base + res_b + part_b + G_b + gt_b + 32);
+    ls->f_parts = reinterpret_cast<double *>(base + res_b + part_b + G_b + gt_b);
+    char *const scalars = base + res_b + part_b + G_b + gt_b + f_b;
+    ls->loss = reinterpret_cast<double *>(scalars);
+    ls->accepted = reinterpret_cast<int *>(scalars + 16);
+    ls->step = reinterpret_cast<float *>(scalars + 32);
     *out = ls;
     return CORE_OK;
 }
@@ -522,11 +542,9 @@ int core_ls_destroy(core_ls *ls) {
 }
 
 static int ls_gradients_into(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G) {
-    if (ls_fused_usable(ls->fused_plan, ls->A, x_dev, ls->part)) {
-        // single pass over A: residual and A^T r per row range, then the fixed-order reduce
-        CORE_CUDA(ctx, launch_ls_fused(ls->fused_plan, ls->A, ls->b, x_dev, ls->n, ls->rows, ls->d, ls->part,
-                                       ctx->stream));
-        CORE_CUDA(ctx, launch_ls_reduce(ls->fused_plan, ls->part, ls->n, ls->rows, ls->d, G, ctx->stream));
+    if (ls->machine_pass.units > 0) {
+        CORE_CUDA(ctx, launch_ls_pass_gradients(ls->machine_pass, ls->A, ls->b, LsPoint{x_dev}, ls->d, ls->part, ctx->stream));
+        CORE_CUDA(ctx, launch_ls_pass_reduce(ls->machine_pass, ls->part, ls->d, 1.0f / (float)ls->rows, G, ctx->stream));
         return CORE_OK;
     }
     CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, x_dev, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
@@ -535,26 +553,58 @@ static int ls_gradients_into(core_ctx *ctx, core_ls *ls, const float *x_dev, flo
     return CORE_OK;
 }
 
-// Gradients at x_eval, then the round with the given epilogue.  Where the single-pass gradient kernel
-// and the scalar projection both apply, the projection sums the per-row-range partial gradients while
-// it stages its tiles, so the machine gradients G are never written or read back.
-static int ls_round(core_ctx *ctx, core_ls *ls, const float *x_eval, float *out, const ReconstructEpilogue *epilogue,
-                    const StepRule *rule = nullptr) {
-    if (!project_kernel_forced() && ls_fused_usable(ls->fused_plan, ls->A, x_eval, ls->part)) {
-        if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
-        CORE_CUDA(ctx, launch_ls_fused(ls->fused_plan, ls->A, ls->b, x_eval, ls->n, ls->rows, ls->d, ls->part, ctx->stream));
-        if (int rc = project_row_into(ctx, ls->part, CORE_F32, ls->n * ls->fused_plan.splits, ls->d,
-                                      1.0f / ((float)ls->rows * (float)ls->n), ctx->d, 0, static_cast<float *>(ctx->ws),
-                                      ctx->pbar, false, ctx->stream))
-            return rc;
-        if (int rc = apply_step_rule(ctx, rule, ctx->pbar)) return rc;
-        CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, ctx->pbar, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream,
-                                          epilogue));
-        ctx->t += 1;
+static double ls_loss_scale(const core_ls *ls) { return 1.0 / (2.0 * (double)ls->rows * (double)ls->n); }
+
+// The objective at x as unscaled sums in ls->f_parts; returns how many through *parts.
+static int ls_loss_parts(core_ctx *ctx, core_ls *ls, const float *x, bool reverse, int64_t *parts) {
+    if (ls->step_pass.units > 0) {
+        CORE_CUDA(ctx, launch_ls_pass_loss(ls->step_pass, ls->A, ls->b, LsPoint{x}, ls->d, reverse, ls->f_parts, ctx->stream));
+        *parts = ls->step_pass.units;
         return CORE_OK;
     }
-    if (int rc = ls_gradients_into(ctx, ls, x_eval, ls->G)) return rc;
-    return round_with_epilogue(ctx, ls->G, CORE_F32, ls->n, ls->d, ctx->pbar, out, epilogue, rule);
+    CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, x, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
+    CORE_CUDA(ctx, launch_ls_loss(ls->res, ls->n, ls->rows, ls->f_parts, ctx->stream));
+    *parts = 1;
+    return CORE_OK;
+}
+
+static int ls_loss_into(core_ctx *ctx, core_ls *ls, const float *x, double *loss) {
+    int64_t parts = 0;
+    if (int rc = ls_loss_parts(ctx, ls, x, false, &parts)) return rc;
+    CORE_CUDA(ctx, launch_ls_loss_sum(ls->f_parts, parts, ls_loss_scale(ls), loss, ctx->stream));
+    return CORE_OK;
+}
+
+// The round of a step at the point `at`: only the mean message is wanted, so the gradient is one row.  The
+// projection adds the units' partial gradients while it stages its tiles; the machine gradients are never written.
+static int ls_round(core_ctx *ctx, core_ls *ls, const LsPoint &at, float *out, const ReconstructEpilogue *epilogue,
+                    const StepRule *rule = nullptr) {
+    const float *rows = ls->part;
+    int32_t count = (int32_t)ls->step_pass.units;
+    int64_t ld = ls->step_pass.ldp;
+    float scale = 1.0f / ((float)ls->rows * (float)ls->n);
+    if (ls->step_pass.units > 0) {
+        CORE_CUDA(ctx, launch_ls_pass_gradients(ls->step_pass, ls->A, ls->b, at, ls->d, ls->part, ctx->stream));
+    } else {
+        const float *x = at.x;
+        if (at.x_prev) {
+            CORE_CUDA(ctx, launch_lookahead(at.x, at.x_prev, at.gamma, ls->d, ls->y, ctx->stream));
+            x = ls->y;
+        }
+        if (int rc = ls_gradients_into(ctx, ls, x, ls->G)) return rc;
+        rows = ls->G;
+        count = ls->n;
+        ld = ls->d;
+        scale = 1.0f / (float)ls->n;
+    }
+    if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
+    if (int rc = project_row_into(ctx, rows, CORE_F32, count, ld, scale, ctx->d, 0, static_cast<float *>(ctx->ws), ctx->pbar, false,
+                                  ctx->stream))
+        return rc;
+    if (int rc = apply_step_rule(ctx, rule, ctx->pbar)) return rc;
+    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, ctx->pbar, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream, epilogue));
+    ctx->t += 1;
+    return CORE_OK;
 }
 
 int core_ls_gradients(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G_out_dev) {
@@ -568,17 +618,18 @@ int core_gd_step(core_ctx *ctx, core_ls *ls, float h, float *x_dev) {
     if (!ls || !x_dev || ls->d != ctx->d || ls->device != ctx->device) return CORE_EINVAL;
     // x <- x - h * gtilde inside the reconstruction: the estimate is never stored
     const ReconstructEpilogue update{x_dev, h, nullptr, nullptr};
-    return ls_round(ctx, ls, x_dev, x_dev, &update);
+    return ls_round(ctx, ls, LsPoint{x_dev}, x_dev, &update);
 }
 
 int core_agd_step(core_ctx *ctx, core_ls *ls, float h, float beta, float *x_dev, float *x_prev_dev) {
     if (int rc = check_ctx(ctx)) return rc;
     if (!ls || !x_dev || !x_prev_dev || x_dev == x_prev_dev || ls->d != ctx->d || ls->device != ctx->device)
         return CORE_EINVAL;
-    CORE_CUDA(ctx, launch_lookahead(x_dev, x_prev_dev, 1.0f - beta, ls->d, ls->y, ctx->stream));
-    // x_prev <- x and x <- y - h * gtilde(y), both inside the reconstruction
-    const ReconstructEpilogue update{ls->y, h, x_dev, x_prev_dev};
-    return ls_round(ctx, ls, ls->y, x_dev, &update);
+    // x_prev <- x and x <- y - h * gtilde(y), both inside the reconstruction, which forms y again from x and x_prev
+    ReconstructEpilogue update{x_dev, h, x_dev, x_prev_dev};
+    update.lookahead = true;
+    update.gamma = 1.0f - beta;
+    return ls_round(ctx, ls, LsPoint{x_dev, x_prev_dev, 1.0f - beta}, x_dev, &update);
 }
 
 int core_gd_step_guarded(core_ctx *ctx, core_ls *ls, float h, float *x_dev, double *f_dev, int32_t *accepted_dev) {
@@ -586,12 +637,13 @@ int core_gd_step_guarded(core_ctx *ctx, core_ls *ls, float h, float *x_dev, doub
     if (!ls || !x_dev || !f_dev || ls->d != ctx->d || ls->device != ctx->device) return CORE_EINVAL;
     // trial point y = x - h * gtilde, written by the reconstruction; x is left untouched
     const ReconstructEpilogue trial{x_dev, h, nullptr, nullptr};
-    if (int rc = ls_round(ctx, ls, x_dev, ls->y, &trial)) return rc;
-    CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, ls->y, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
-    CORE_CUDA(ctx, launch_ls_loss(ls->res, ls->n, ls->rows, ls->f_trial, ctx->stream));
+    if (int rc = ls_round(ctx, ls, LsPoint{x_dev}, ls->y, &trial)) return rc;
+    // the trial point's loss, from the rows the gradient pass read last (still in L2) to those it read first
+    int64_t parts = 0;
+    if (int rc = ls_loss_parts(ctx, ls, ls->y, true, &parts)) return rc;
     // decided on the device: no host synchronisation inside the step
-    CORE_CUDA(ctx, launch_keep_better(ls->f_trial, ls->y, ls->d, f_dev, x_dev, ls->accepted, accepted_dev,
-                                      ctx->stream));
+    CORE_CUDA(ctx, launch_keep_better(ls->f_parts, parts, ls_loss_scale(ls), ls->y, ls->d, f_dev, x_dev, ls->accepted,
+                                      accepted_dev, ctx->stream));
     return CORE_OK;
 }
 
@@ -606,11 +658,12 @@ int core_gd_step_option1(core_ctx *ctx, core_ls *ls, double r1, double H, double
     const StepRule rule{r1, H, c, ls->step + 1, ls->step};
     ReconstructEpilogue trial{x_dev, 0.f, nullptr, nullptr};
     trial.step_dev = ls->step;
-    if (int rc = ls_round(ctx, ls, x_dev, ls->y, &trial, &rule)) return rc;
-    CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, ls->y, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
-    CORE_CUDA(ctx, launch_ls_loss(ls->res, ls->n, ls->rows, ls->f_trial, ctx->stream));
-    CORE_CUDA(ctx, launch_keep_better(ls->f_trial, ls->y, ls->d, f_dev, x_dev, ls->accepted, accepted_dev,
-                                      ctx->stream));
+    if (int rc = ls_round(ctx, ls, LsPoint{x_dev}, ls->y, &trial, &rule)) return rc;
+    // the trial point's loss, from the rows the gradient pass read last (still in L2) to those it read first
+    int64_t parts = 0;
+    if (int rc = ls_loss_parts(ctx, ls, ls->y, true, &parts)) return rc;
+    CORE_CUDA(ctx, launch_keep_better(ls->f_parts, parts, ls_loss_scale(ls), ls->y, ls->d, f_dev, x_dev, ls->accepted,
+                                      accepted_dev, ctx->stream));
     if (h_dev)
         CORE_CUDA(ctx, cudaMemcpyAsync(h_dev, ls->step, sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
     if (p_dev)
@@ -661,17 +714,14 @@ int core_decentralized_step(core_ctx *ctx, core_ls *ls, const float *W_dev, int3
 int core_ls_loss(core_ctx *ctx, core_ls *ls, const float *x_dev, double *loss_dev) {
     if (int rc = check_ctx(ctx)) return rc;
     if (!ls || !x_dev || !loss_dev || ls->d != ctx->d || ls->device != ctx->device) return CORE_EINVAL;
-    CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, x_dev, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
-    CORE_CUDA(ctx, launch_ls_loss(ls->res, ls->n, ls->rows, loss_dev, ctx->stream));
-    return CORE_OK;
+    return ls_loss_into(ctx, ls, x_dev, loss_dev);
 }
 
 int core_ls_loss_host(core_ctx *ctx, core_ls *ls, const float *x_dev, double *loss_host) {
     if (int rc = check_ctx(ctx)) return rc;
     if (!ls || !x_dev || !loss_host || ls->d != ctx->d || ls->device != ctx->device) return CORE_EINVAL;
-    CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, x_dev, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
-    CORE_CUDA(ctx, launch_ls_loss(ls->res, ls->n, ls->rows, ls->f_trial, ctx->stream));
-    CORE_CUDA(ctx, cudaMemcpyAsync(loss_host, ls->f_trial, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    if (int rc = ls_loss_into(ctx, ls, x_dev, ls->loss)) return rc;
+    CORE_CUDA(ctx, cudaMemcpyAsync(loss_host, ls->loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     return CORE_OK;
 }
 

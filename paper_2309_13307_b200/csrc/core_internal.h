@@ -100,7 +100,8 @@ cudaError_t launch_aggregate(const float *P, int32_t n, int32_t m, float *pbar, 
 // out[k - k_begin] = gtilde[k] for k in [k_begin, k_end); k_begin must be a multiple of 2048.
 // With an epilogue the estimate is consumed where it is produced and never stored:
 //   out[k] = base[k] - step * gtilde[k]   (the optimiser update of Algorithms 2 and 4)
-// and, if shift_dst is set, shift_dst[k] = shift_src[k] first (x_prev <- x of Algorithm 4).
+// and, if shift_dst is set, shift_dst[k] = shift_src[k] first (x_prev <- x of Algorithm 4).  With lookahead set the base is
+// shift_src[k] + gamma * (shift_src[k] - shift_dst[k]), formed from the values before the shift, instead of base[k].
 // out may alias base and shift_src; all four arrays are indexed like out.
 // step_dev, when set, overrides step: the kernel reads the step from device memory (a step that an
 // earlier kernel of the same iteration chose, as in Option I of Algorithm 3), times step_scale.
@@ -111,14 +112,12 @@ struct ReconstructEpilogue {
     float *shift_dst;
     const float *step_dev = nullptr;
     float step_scale = 1.0f;
+    bool lookahead = false;
+    float gamma = 0.f;
 };
 cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, const float *pbar, int32_t m,
                                int64_t k_begin, int64_t k_end, float *out, int sm_count,
                                cudaStream_t stream, const ReconstructEpilogue *epilogue = nullptr);
-
-// y[k] = x[k] + gamma * (x[k] - x_prev[k])   (look-ahead point of Algorithm 4)
-cudaError_t launch_lookahead(const float *x, const float *x_prev, float gamma, int64_t d, float *y,
-                             cudaStream_t stream);
 
 cudaError_t launch_debug_philox(const RoundKeys &keys, uint32_t t, uint32_t j, uint64_t q0, int64_t nq,
                                 uint32_t *words, cudaStream_t stream);
@@ -140,19 +139,44 @@ cudaError_t launch_ls_at_r(const LsPlan &plan, const float *A, const float *res,
                            int64_t d, float *part, cudaStream_t stream);
 cudaError_t launch_ls_reduce(const LsPlan &plan, const float *part, int32_t n, int32_t rows, int64_t d,
                              float *G, cudaStream_t stream);
-// Single pass over A for d <= 8192, d % 4 == 0: part[(i*splits + s)*d + k] as above, with the
-// residual of each row formed on the fly (A is read from HBM once instead of twice).  A plan with
-// splits == 0 means the single-pass kernel does not apply to this shape.
-LsPlan make_ls_fused_plan(int32_t n, int32_t rows, int64_t d, int sm_count);
-bool ls_fused_usable(const LsPlan &fused_plan, const float *A, const float *x, const float *part);
-cudaError_t launch_ls_fused(const LsPlan &plan, const float *A, const float *b, const float *x, int32_t n,
-                            int32_t rows, int64_t d, float *part, cudaStream_t stream);
+// Single pass over A (core_ls_pass.cu) for rows of up to 131072 columns of any alignment: the residual of each row is
+// formed on the fly, A is read from HBM once.  The n * rows rows are cut over `units` CTAs (or clusters); a unit's
+// partial gradient goes to part[(i * slots_per_machine + s) * ldp + k], s counting the units that hold rows of
+// machine i, or, when the machines are not kept apart, to part[unit * ldp + k].
+struct LsPass {
+    int64_t units;            // 0: the kernel does not apply to this shape
+    int64_t rows, total;      // rows per (kept-apart) machine, rows of all
+    int64_t ldp;
+    int slots_per_machine;
+    int cluster, slice, warps, group_warps, columns, chunk_rows, slots;
+    uint32_t slot_bytes, row_stride, ring_offset;
+    size_t smem;
+};
+struct LsPoint {              // x, or x + gamma (x - x_prev) (the look-ahead point of Algorithm 4)
+    const float *x;
+    const float *x_prev = nullptr;
+    float gamma = 0.f;
+};
+LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int sm_count);
+size_t ls_pass_partials(const LsPass &pass);      // floats
+cudaError_t launch_ls_pass_gradients(const LsPass &pass, const float *A, const float *b, const LsPoint &at, int64_t d,
+                                     float *part, cudaStream_t stream);
+cudaError_t launch_ls_pass_reduce(const LsPass &pass, const float *part, int64_t d, float inv_rows, float *G,
+                                  cudaStream_t stream);
+// loss_part[u] = sum of squared residuals of unit u; with `reverse` from the last row to the first.
+cudaError_t launch_ls_pass_loss(const LsPass &pass, const float *A, const float *b, const LsPoint &at, int64_t d, bool reverse,
+                                double *loss_part, cudaStream_t stream);
+cudaError_t launch_ls_loss_sum(const double *loss_part, int64_t units, double scale, double *loss, cudaStream_t stream);
+cudaError_t ls_pass_take_status(int *status);     // after a device synchronisation; clears the word
 // Comparison step of Algorithm 3, on the device: if *f_trial < *f then x <- trial, *f <- *f_trial and the
-// flag is 1, otherwise nothing changes and the flag is 0 (a tie keeps x).  flag_scratch is a device int
-// owned by the caller of this function; flag_out (may be null) receives a copy.
-cudaError_t launch_keep_better(const double *f_trial, const float *trial, int64_t d, double *f, float *x,
-                               int *flag_scratch, int32_t *flag_out, cudaStream_t stream);
-// loss[0] = (1/n) sum_i 1/(2 rows) sum_r res_i[r]^2, summed in double in a fixed order
+// flag is 1, otherwise nothing changes and the flag is 0 (a tie keeps x).  f_trial is scale times the sum of the
+// `parts` numbers f_parts.  flag_scratch is a device int owned by the caller of this function; flag_out (may be
+// null) receives a copy.
+cudaError_t launch_keep_better(const double *f_parts, int64_t parts, double scale, const float *trial, int64_t d, double *f,
+                               float *x, int *flag_scratch, int32_t *flag_out, cudaStream_t stream);
+// y = x + gamma (x - x_prev)
+cudaError_t launch_lookahead(const float *x, const float *x_prev, float gamma, int64_t d, float *y, cudaStream_t stream);
+// loss[0] = sum of res^2 over all rows of all machines, in double in a fixed order
 cudaError_t launch_ls_loss(const float *res, int32_t n, int32_t rows, double *loss, cudaStream_t stream);
 
 // Option I of Algorithm 3: p_out[0] (may be null) = sqrt((1/m) sum_j pbar_j^2), h_out[0] =

@@ -1,6 +1,6 @@
-// Machine gradients of the least-squares objective that drives Algorithm 2:
-// f_i(x) = 1/(2 rows) ||A_i x - b_i||^2, g_i = A_i^T (A_i x - b_i) / rows.
-// Two streaming passes over A (both HBM-bound), every sum in a fixed order.
+// Machine gradients of the least-squares objective that drives Algorithm 2, for rows too long for the single pass
+// of core_ls_pass.cu: f_i(x) = 1/(2 rows) ||A_i x - b_i||^2, g_i = A_i^T (A_i x - b_i) / rows in two streaming passes
+// over A (both HBM-bound), every sum in a fixed order.  Also the comparison step of Algorithm 3.
 #include "core_internal.h"
 
 namespace core {
@@ -105,7 +105,7 @@ __global__ void ls_reduce_kernel(const float *__restrict__ part, int n, int spli
 
 // One CTA; thread t sums residual squares t, t+256, ... in double, then a fixed tree.
 __global__ void __launch_bounds__(kLsThreads)
-ls_loss_kernel(const float *__restrict__ res, int64_t total, double scale, double *loss) {
+ls_loss_kernel(const float *__restrict__ res, int64_t total, double *loss) {
     __shared__ double sh[kLsThreads];
     double s = 0.0;
     for (int64_t r = threadIdx.x; r < total; r += kLsThreads) {
@@ -118,110 +118,35 @@ ls_loss_kernel(const float *__restrict__ res, int64_t total, double scale, doubl
         if ((int)threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
         __syncthreads();
     }
-    if (threadIdx.x == 0) loss[0] = sh[0] * scale;
+    if (threadIdx.x == 0) loss[0] = sh[0];
 }
 
-// ---- single pass over A (rows of up to 8192 columns) -------------------------------------
-// A CTA owns a range of rows of one machine.  Thread t keeps x and its partial gradient for the
-// columns {4(t + 256c) .. +3, c < C4} in registers.  Rows are prefetched with cp.async into a ring in
-// shared memory, every thread copying exactly the 16-byte pieces it will read back itself, so the
-// ring needs no barrier; the only barrier per row is the one of the dot-product reduction.
-// For row r: res = A[r].x - b[r] (fixed-order reduction), then acc += res * A[r] from the same
-// registers.  A is read from HBM once; the partial gradients of the CTAs of a machine are added by
-// ls_reduce_kernel in ascending order.
-constexpr int kRing = 4;   // rows in flight per CTA
-
-__device__ __forceinline__ void ls_cp_async16(void *smem_dst, const void *gmem_src) {
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-
-template <int C4>
-__global__ void __launch_bounds__(kLsThreads, 1)
-ls_fused_kernel(const float *__restrict__ A, const float *__restrict__ b, const float *__restrict__ x, int rows,
-                int d4, int splits, int rows_per_split, float *__restrict__ part) {
-    extern __shared__ __align__(16) unsigned char ls_smem[];
-    float4 *ring = reinterpret_cast<float4 *>(ls_smem);                       // kRing x (C4 * 256) float4
-    float *warp_sums = reinterpret_cast<float *>(ring + kRing * C4 * kLsThreads);   // 2 x 8
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int i = blockIdx.y, s = blockIdx.x;
-    const int r_begin = s * rows_per_split;
-    const int r_end = min(r_begin + rows_per_split, rows);
-    const float4 *Ai = reinterpret_cast<const float4 *>(A) + (int64_t)i * rows * d4;
-    const float *bi = b + (int64_t)i * rows;
-
-    float4 xv[C4], acc[C4];
+// Comparison step of Algorithm 3: one CTA adds up the trial point's loss, decides, and copies a short point itself;
+// a long one is copied by the kernel below if the flag says so.
+constexpr int kKeepThreads = 1024;
+constexpr int64_t kKeepOneCta = 32768;         // 128 KB: about what one SM moves while a second launch would start
+__global__ void __launch_bounds__(kKeepThreads)
+keep_better_kernel(const double *__restrict__ f_parts, int64_t parts, double scale, const float *__restrict__ trial, int64_t d,
+                   double *__restrict__ f, float *__restrict__ x, int *__restrict__ flag, int32_t *__restrict__ flag_out) {
+    __shared__ int decision;
+    if (threadIdx.x < 32) {
+        double s = 0.0;                         // as in ls_loss_sum_kernel: the same bits
+#pragma unroll 8
+        for (int64_t u = threadIdx.x; u < parts; u += 32) s += f_parts[u];
 #pragma unroll
-    for (int c = 0; c < C4; ++c) {
-        const int col = tid + c * kLsThreads;
-        xv[c] = col < d4 ? __ldg(reinterpret_cast<const float4 *>(x) + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-
-    auto prefetch = [&](int r) {
-        if (r < r_end) {
-            float4 *slot = ring + (size_t)((r - r_begin) % kRing) * C4 * kLsThreads;
-            const float4 *row = Ai + (int64_t)r * d4;
-#pragma unroll
-            for (int c = 0; c < C4; ++c) {
-                const int col = tid + c * kLsThreads;
-                if (col < d4) ls_cp_async16(slot + col, row + col);
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");      // one group per row, empty past the end
-    };
-
-#pragma unroll
-    for (int p = 0; p < kRing - 1; ++p) prefetch(r_begin + p);
-
-    for (int r = r_begin; r < r_end; ++r) {
-        prefetch(r + kRing - 1);
-        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 1) : "memory");   // row r has landed (own pieces)
-        const float4 *slot = ring + (size_t)((r - r_begin) % kRing) * C4 * kLsThreads;
-        float4 av[C4];
-        float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-#pragma unroll
-        for (int c = 0; c < C4; ++c) {
-            const int col = tid + c * kLsThreads;
-            av[c] = col < d4 ? slot[col] : make_float4(0.f, 0.f, 0.f, 0.f);
-            p0 = fmaf(av[c].x, xv[c].x, p0);
-            p1 = fmaf(av[c].y, xv[c].y, p1);
-            p2 = fmaf(av[c].z, xv[c].z, p2);
-            p3 = fmaf(av[c].w, xv[c].w, p3);
-        }
-        float p = (p0 + p1) + (p2 + p3);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, off);
-        float *sums = warp_sums + ((r - r_begin) & 1) * (kLsThreads / 32);
-        if (lane == 0) sums[warp] = p;
-        __syncthreads();
-        float dot = 0.f;
-#pragma unroll
-        for (int w = 0; w < kLsThreads / 32; ++w) dot += sums[w];
-        const float res = dot - __ldg(bi + r);
-#pragma unroll
-        for (int c = 0; c < C4; ++c) {
-            acc[c].x = fmaf(av[c].x, res, acc[c].x);
-            acc[c].y = fmaf(av[c].y, res, acc[c].y);
-            acc[c].z = fmaf(av[c].z, res, acc[c].z);
-            acc[c].w = fmaf(av[c].w, res, acc[c].w);
+        for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) {
+            const double f_trial = s * scale;
+            const int take = f_trial < *f ? 1 : 0;     // a tie keeps the current point
+            if (take) *f = f_trial;
+            *flag = take;
+            if (flag_out) *flag_out = take;
+            decision = take;
         }
     }
-    float4 *out = reinterpret_cast<float4 *>(part) + ((int64_t)i * splits + s) * d4;
-#pragma unroll
-    for (int c = 0; c < C4; ++c) {
-        const int col = tid + c * kLsThreads;
-        if (col < d4) out[col] = acc[c];
-    }
-}
-
-// Comparison step of Algorithm 3: one thread decides, then every thread copies if told to.
-__global__ void keep_better_decide_kernel(const double *__restrict__ f_trial, double *__restrict__ f,
-                                          int *__restrict__ flag, int32_t *__restrict__ flag_out) {
-    const int take = *f_trial < *f ? 1 : 0;     // a tie keeps the current point
-    if (take) *f = *f_trial;
-    *flag = take;
-    if (flag_out) *flag_out = take;
+    __syncthreads();
+    if (decision && d <= kKeepOneCta)
+        for (int64_t k = threadIdx.x; k < d; k += kKeepThreads) x[k] = trial[k];
 }
 
 __global__ void keep_better_copy_kernel(const int *__restrict__ flag, const float *__restrict__ trial, int64_t d,
@@ -231,56 +156,35 @@ __global__ void keep_better_copy_kernel(const int *__restrict__ flag, const floa
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < d; k += stride) x[k] = trial[k];
 }
 
+__global__ void lookahead_kernel(const float *__restrict__ x, const float *__restrict__ x_prev, float gamma, int64_t d,
+                                 float *__restrict__ y) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < d; k += stride)
+        y[k] = fmaf(gamma, x[k] - x_prev[k], x[k]);
+}
+
 bool vec_ok_for(const float *A, int64_t d) {
     return (reinterpret_cast<uintptr_t>(A) % 16) == 0 && d % 4 == 0;
 }
 
 }  // namespace
 
-cudaError_t launch_keep_better(const double *f_trial, const float *trial, int64_t d, double *f, float *x,
-                               int *flag_scratch, int32_t *flag_out, cudaStream_t stream) {
-    keep_better_decide_kernel<<<1, 1, 0, stream>>>(f_trial, f, flag_scratch, flag_out);
-    int64_t blocks = (d + 255) / 256;
-    if (blocks > 148 * 8) blocks = 148 * 8;
-    keep_better_copy_kernel<<<(unsigned)blocks, 256, 0, stream>>>(flag_scratch, trial, d, x);
+cudaError_t launch_keep_better(const double *f_parts, int64_t parts, double scale, const float *trial, int64_t d, double *f,
+                               float *x, int *flag_scratch, int32_t *flag_out, cudaStream_t stream) {
+    keep_better_kernel<<<1, kKeepThreads, 0, stream>>>(f_parts, parts, scale, trial, d, f, x, flag_scratch, flag_out);
+    if (d > kKeepOneCta) {
+        int64_t blocks = (d + 255) / 256;
+        if (blocks > 148 * 8) blocks = 148 * 8;
+        keep_better_copy_kernel<<<(unsigned)blocks, 256, 0, stream>>>(flag_scratch, trial, d, x);
+    }
     return cudaGetLastError();
 }
 
-LsPlan make_ls_fused_plan(int32_t n, int32_t rows, int64_t d, int sm_count) {
-    LsPlan p{};
-    if (d % 4 != 0 || d > 4 * 8 * kLsThreads) return p;     // splits == 0: not available
-    int per_machine = sm_count / n;                          // one CTA per SM, machines side by side
-    if (per_machine < 1) per_machine = 1;
-    if (per_machine > rows) per_machine = rows;
-    p.rows_per_split = (rows + per_machine - 1) / per_machine;
-    p.splits = (rows + p.rows_per_split - 1) / p.rows_per_split;
-    return p;
-}
-
-cudaError_t launch_ls_fused(const LsPlan &plan, const float *A, const float *b, const float *x, int32_t n,
-                            int32_t rows, int64_t d, float *part, cudaStream_t stream) {
-    const int d4 = (int)(d / 4);
-    int c4 = 1;
-    while (c4 * kLsThreads < d4) c4 *= 2;
-    const size_t smem = (size_t)kRing * c4 * kLsThreads * 16 + 2 * (kLsThreads / 32) * sizeof(float);
-    dim3 grid(plan.splits, n);
-    auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kLsThreads, smem, stream>>>(A, b, x, rows, d4, plan.splits, plan.rows_per_split, part);
-        return cudaGetLastError();
-    };
-    switch (c4) {
-        case 1: return go(ls_fused_kernel<1>);
-        case 2: return go(ls_fused_kernel<2>);
-        case 4: return go(ls_fused_kernel<4>);
-        default: return go(ls_fused_kernel<8>);
-    }
-}
-
-bool ls_fused_usable(const LsPlan &fused_plan, const float *A, const float *x, const float *part) {
-    return fused_plan.splits > 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(x) |
-                                      reinterpret_cast<uintptr_t>(part)) % 16) == 0;
+cudaError_t launch_lookahead(const float *x, const float *x_prev, float gamma, int64_t d, float *y, cudaStream_t stream) {
+    int64_t blocks = (d + 255) / 256;
+    if (blocks > 148 * 8) blocks = 148 * 8;
+    lookahead_kernel<<<(unsigned)blocks, 256, 0, stream>>>(x, x_prev, gamma, d, y);
+    return cudaGetLastError();
 }
 
 LsPlan make_ls_plan(int32_t n, int32_t rows, int64_t d, int sm_count) {
@@ -323,8 +227,7 @@ cudaError_t launch_ls_reduce(const LsPlan &plan, const float *part, int32_t n, i
 }
 
 cudaError_t launch_ls_loss(const float *res, int32_t n, int32_t rows, double *loss, cudaStream_t stream) {
-    ls_loss_kernel<<<1, kLsThreads, 0, stream>>>(res, (int64_t)n * rows, 1.0 / (2.0 * (double)rows * (double)n),
-                                                 loss);
+    ls_loss_kernel<<<1, kLsThreads, 0, stream>>>(res, (int64_t)n * rows, loss);
     return cudaGetLastError();
 }
 

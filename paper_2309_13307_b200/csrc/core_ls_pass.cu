@@ -1,0 +1,609 @@
+// One pass over the data matrices of the least-squares objective: for every row r of every machine
+// res = A[r] . x - b[r], and either acc += res * A[r] (machine gradients, Algorithm 2's local computation) or
+// loss += res^2 (the objective).  A is read from HBM once; it is the bound (4 bytes per two multiply-adds).
+//
+// The rows of all machines are one matrix of n * rows rows, cut evenly over one CTA per SM, whatever n and rows
+// are: a CTA's range may end inside a machine and go on in the next.  Groups of W warps take the CTA's rows in
+// turn: W = 1 up to 1024 columns, then 2, 4, 8 and 16 up to 16384; beyond, a cluster of 2 to 8 CTAs shares the
+// columns of a row.  Lane l of warp w of a group owns columns l + 32 (w + W c): x and the partial gradient of those
+// columns stay in registers for the whole pass, the row's values between its dot product and its update.  Each
+// group has a ring of row buffers in shared memory filled by bulk copies (one lane issues them; they start and end
+// on 16-byte boundaries around the rows, so that rows of any alignment move at full rate; single columns per lane
+// need no alignment either, and 16-byte reads were not faster).  Rows of up to 512 columns are handled 2 to 16 at a
+// time, their dot products reduced together by a transposing butterfly (16 rows: 16 shuffles instead of 80).  In a
+// cluster every warp sends its share of the dot product to all CTAs (asynchronous remote stores counted by a barrier
+// there).  Every sum has a fixed order.
+//
+// Measured (us; pass alone unless said otherwise; before: the kernels this one replaced): n = 50, 1200 x 784: 155 -> 41;
+// n = 50, 11620 x 54: gradients 377 -> 31, loss 212 -> 28; n = 16, 256 x 20000: gradients 133 -> 72; n = 8, 2048 x 8192
+// (537 MB): loss 107 -> 88, gradients 87 -> 92.  Tried: cp.async instead of bulk copies (20 % slower), rings of 96 to
+// 192 KB (equal), evict_normal instead of evict_first (3 to 10 us slower), 8 warps for one-warp rows (25 % slower).
+#include "core_internal.h"
+#include "core_sync.cuh"
+
+#include <algorithm>
+#include <type_traits>
+
+namespace core {
+
+namespace {
+
+constexpr int kPassMaxSlots = 8;
+constexpr int kPassMaxWarps = 16;
+constexpr int kPassMaxCluster = 8;
+constexpr int kPassCtaCols = 32 * 32 * kPassMaxWarps;   // columns a CTA can hold: 32 per lane
+constexpr int kPassFlushFloats = 8192;                  // room for the groups' sums while the rings are in use
+constexpr uint32_t kPassRingBytes = 128u * 1024u;       // bytes in flight per SM
+
+// Rows at a time.  One warp per row: as many as 32 registers per lane hold.  Several: the chain from a row's arrival to
+// its update crosses the CTA (about 1600 cycles), so two rows go through it together, four where 20 columns per lane
+// leave the registers for it (16 x 2048 rows of 2049 columns: 125 us with one, 84 with two, 66 with four); the 512-thread
+// kernel has registers for two up to 24 columns.
+constexpr int pass_batch(int warps_per_row, int columns) {
+    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 24 ? 1 : 2) : columns == 20 ? 4 : 2;
+}
+
+__device__ int g_pass_status;                           // 0, or the code of a wait that ran out
+
+struct PassArgs {
+    const float *A;
+    const float *b;
+    const float *x;
+    const float *x_prev;     // not null: evaluate at x + gamma (x - x_prev)
+    float gamma;
+    int64_t d;
+    int64_t rows;            // per machine; all rows of all machines when the machines are not kept apart
+    int64_t total;           // n * rows
+    int64_t units;           // CTAs (clusters) the rows are cut over
+    float *part;             // gradients: part[slot * ldp + column]
+    int64_t ldp;
+    int slots_per_machine;
+    double *loss_part;       // objective: one sum of squares per unit
+    int cluster;             // CTAs per row
+    int slice;               // columns per CTA of a cluster
+    int chunk_rows;          // rows per ring slot, at most 32
+    int slots;               // ring slots per group
+    uint32_t slot_bytes;
+    uint32_t row_stride;     // bytes between the rows of a slot; agrees with d * 4 modulo 16
+    uint32_t ring_offset;    // of the rings in shared memory, behind a buffer for the groups' sums where machines are kept apart
+    int flush_floats;        // room for the groups' sums: that buffer, or the rings once the last row is done
+    int reverse;             // rows from the last to the first (what an ascending pass left in L2 comes first)
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// v to `addr` of CTA `rank` of the cluster; its 4 bytes are counted on the barrier at `bar` there.
+__device__ __forceinline__ void send_remote(uint32_t addr, uint32_t bar, uint32_t rank, float v) {
+    asm volatile(
+        "{\n\t.reg .b32 ra, rb;\n\t"
+        "mapa.shared::cluster.u32 ra, %0, %2;\n\t"
+        "mapa.shared::cluster.u32 rb, %1, %2;\n\t"
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [ra], %3, [rb];\n\t}"
+        ::"r"(addr), "r"(bar), "r"(rank), "r"(__float_as_uint(v))
+        : "memory");
+}
+__device__ __forceinline__ float load_shared(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void store_shared(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+
+// Sums of RB values over the warp at once: afterwards every lane holds the sum of value lane * RB / 32.
+template <int RB>
+__device__ __forceinline__ float butterfly(float (&p)[RB], int lane) {
+    int off = 16;
+#pragma unroll
+    for (int half = RB / 2; half > 0; half /= 2, off /= 2) {
+        const bool upper = (lane & off) != 0;
+#pragma unroll
+        for (int k = 0; k < half; ++k) {
+            const float send = upper ? p[k] : p[k + half];
+            const float keep = upper ? p[k + half] : p[k];
+            p[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+#pragma unroll
+    for (; off > 0; off /= 2) p[0] += __shfl_xor_sync(0xffffffffu, p[0], off);
+    return p[0];
+}
+
+// WARPS per CTA, W of them per row, C columns per lane, RB rows at a time.
+template <int WARPS, int W, int C, int RB, bool GRAD>
+__global__ void __launch_bounds__(32 * WARPS, 1)
+ls_pass_kernel(const __grid_constant__ PassArgs a) {
+    constexpr bool MULTI = W > 1;
+    constexpr int THREADS = 32 * WARPS, GROUPS = WARPS / W;
+    extern __shared__ __align__(16) unsigned char pass_smem[];
+    __shared__ __align__(8) uint64_t bars[WARPS * kPassMaxSlots];
+    __shared__ float red[2][RB][WARPS];
+    __shared__ float xch[2][RB][WARPS * kPassMaxCluster];         // [parity][row][group][CTA][warp of the group]
+    __shared__ __align__(8) uint64_t xch_bars[2][WARPS];          // [row parity][group]
+    __shared__ double loss_sums[WARPS];
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int grp = warp / W, wg = warp % W;
+    const bool leader = wg == 0 && lane == 0;
+    const uint32_t rank = MULTI && a.cluster > 1 ? cluster_rank() : 0u;
+    const int64_t unit = MULTI && a.cluster > 1 ? blockIdx.x / a.cluster : blockIdx.x;
+    const int64_t col0 = (int64_t)rank * a.slice;
+    const int dn = (int)min((int64_t)a.slice, a.d - col0);
+    const int64_t lo = a.total * unit / a.units;
+    const int nrows = (int)(a.total * (unit + 1) / a.units - lo);  // rows of this unit, counted from its first
+    const int R = a.chunk_rows;
+    const int chunks = (nrows + R - 1) / R;
+    const uint32_t row_bytes = (uint32_t)a.d * 4;
+    const uint32_t ring = smem_u32(pass_smem) + a.ring_offset + (uint32_t)grp * a.slots * a.slot_bytes;
+    const uint32_t bar0 = smem_u32(bars) + 8u * grp * a.slots;
+    float *const flush = reinterpret_cast<float *>(pass_smem);
+    if (leader) {
+        for (int s = 0; s < a.slots; ++s) mbar_init(bar0 + 8 * s, 1);
+        for (int f = 0; f < 2; ++f) mbar_init(smem_u32(&xch_bars[f][grp]), 1);
+        fence_barrier_init();
+    }
+
+    // Copies of the leader: chunk after chunk of its group.  `src` is the first byte of the next one's rows.
+    auto first_row = [&](int k) { return (a.reverse ? chunks - 1 - k : k) * R; };
+    const uintptr_t unit_base = reinterpret_cast<uintptr_t>(a.A) + (uintptr_t)(lo * a.d + col0) * 4;
+    const int64_t src_step = (a.reverse ? -(int64_t)GROUPS : (int64_t)GROUPS) * R * row_bytes;
+    uintptr_t src = unit_base + (uint64_t)(uint32_t)max(first_row(grp), 0) * row_bytes;
+    const bool edge = unit == 0 || unit == a.units - 1;            // may hold the first or the last bytes of A
+    const uint64_t policy = l2_evict_first();
+    auto issue = [&](int k, int s) {
+        const uint32_t bar = bar0 + 8 * s;
+        // the bytes [from, to) of A to shared memory, `from` going to `dst` (which agrees with it modulo 16)
+        auto copy = [&](uintptr_t from, uintptr_t to, uint32_t dst) {
+            const uint32_t origin = dst - (uint32_t)from;             // of address zero, so to say
+            uintptr_t b0 = from & ~(uintptr_t)15, b1 = (to + 15) & ~(uintptr_t)15;
+            if (edge) {
+                // nothing outside A is touched: a first or last piece that would reach beyond it is copied element by element
+                const uintptr_t a_begin = reinterpret_cast<uintptr_t>(a.A), a_end = a_begin + (uintptr_t)(a.total * a.d) * 4;
+                if (b0 < a_begin) {
+                    b0 += 16;
+                    for (uintptr_t p = from; p < b0 && p < to; p += 4) store_shared(origin + (uint32_t)p, *reinterpret_cast<const float *>(p));
+                }
+                if (b1 > a_end) {
+                    b1 -= 16;
+                    for (uintptr_t p = b1 > from ? b1 : from; p < to; p += 4) store_shared(origin + (uint32_t)p, *reinterpret_cast<const float *>(p));
+                }
+            }
+            if (b1 > b0) {
+                mbar_expect(bar, (uint32_t)(b1 - b0));
+                bulk_copy(origin + (uint32_t)b0, reinterpret_cast<const void *>(b0), (uint32_t)(b1 - b0), bar, policy);
+            }
+        };
+        const int count = min(R, nrows - first_row(k));
+        const uint32_t dst = ring + (uint32_t)s * a.slot_bytes + (uint32_t)(src & 15);
+        if (MULTI && a.cluster > 1)                     // a slice of each row
+            for (int i = 0; i < count; ++i) {
+                const uintptr_t from = src + (uintptr_t)((uint32_t)i * row_bytes);
+                copy(from, from + (uint32_t)dn * 4, dst + (uint32_t)i * a.row_stride);
+            }
+        else
+            copy(src, src + (uint32_t)count * row_bytes, dst);
+        mbar_arrive(bar);
+        src += src_step;
+    };
+    constexpr int stride = 32 * W, CB = C < 4 ? C : 4;             // CB columns are tested for together
+    const int first = lane + 32 * wg;
+    if (leader)
+        for (int s = 0; s < a.slots; ++s)
+            if (grp + s * GROUPS < chunks) issue(grp + s * GROUPS, s);
+
+    float xv[C], acc[GRAD ? C : 1];
+#pragma unroll
+    for (int c = 0; c < C; ++c) xv[c] = first + stride * c < dn ? __ldg(a.x + col0 + first + stride * c) : 0.f;
+    if (a.x_prev) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const float old = first + stride * c < dn ? __ldg(a.x_prev + col0 + first + stride * c) : 0.f;
+            xv[c] = fmaf(a.gamma, xv[c] - old, xv[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < (GRAD ? C : 1); ++c) acc[c] = 0.f;
+    double loss = 0.0;
+    __syncthreads();                                    // barriers initialised, for every warp of a group
+    if (MULTI && a.cluster > 1) cluster_sync();         // and every CTA of the cluster has started
+
+    bool alive = true;
+    int flip = 0, xch_parity = 0;
+
+    // RBX rows whose first one starts at shared-memory address `at`, right-hand side bv in the lanes that get its sum.
+    auto process = [&](auto batch, uint32_t at, float bv) {
+        constexpr int RBX = decltype(batch)::value;
+        float v[RBX][C];
+        float2 s[RBX];
+#pragma unroll
+        for (int i = 0; i < RBX; ++i) s[i] = make_float2(0.f, 0.f);
+        // All loads before the first multiply-add: were they in the same guarded block, every block would wait for its
+        // own loads.  Columns four at a time: all lanes have them, or none, or some (those without read the row's last
+        // columns and multiply them by the zeros in xv).
+#pragma unroll
+        for (int c0 = 0; c0 < C; c0 += CB) {
+            if (stride * (c0 + CB) <= dn) {
+#pragma unroll
+                for (int i = 0; i < RBX; ++i)
+#pragma unroll
+                    for (int c = c0; c < c0 + CB; ++c)
+                        v[i][c] = load_shared(at + (uint32_t)i * a.row_stride + 4u * (uint32_t)(first + stride * c));
+            } else if (c0 == 0 || stride * c0 < dn) {
+#pragma unroll
+                for (int c = c0; c < c0 + CB; ++c) {
+                    const uint32_t off = at + 4u * (uint32_t)min(first + stride * c, dn - 1);
+#pragma unroll
+                    for (int i = 0; i < RBX; ++i) v[i][c] = load_shared(off + (uint32_t)i * a.row_stride);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < RBX; ++i)
+#pragma unroll
+                    for (int c = c0; c < c0 + CB; ++c) v[i][c] = 0.f;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < RBX; ++i) {
+            if constexpr (C == 1) {
+                s[i].x = v[i][0] * xv[0];
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; c += 2)
+                    s[i] = __ffma2_rn(make_float2(v[i][c], v[i][c + 1]), make_float2(xv[c], xv[c + 1]), s[i]);
+            }
+        }
+        float p[RBX];
+#pragma unroll
+        for (int i = 0; i < RBX; ++i) p[i] = s[i].x + s[i].y;
+        float dot = butterfly<RBX>(p, lane);
+        constexpr int SHARE = 32 / RBX;                 // lanes that hold the sum of one row
+        if constexpr (MULTI) {
+            const int mine = lane / SHARE, sub = lane % SHARE;
+            if (a.cluster > 1) {
+                const int parts = W * a.cluster;                      // shares of a dot product
+                const uint32_t bar = smem_u32(&xch_bars[flip][grp]);
+                float *const share = &xch[flip][mine][grp * parts];
+                if (leader) mbar_arrive_expect(bar, 4u * parts * RBX);
+                if (sub < a.cluster) send_remote(smem_u32(share + rank * W + wg), bar, (uint32_t)sub, dot);
+                if (alive && !mbar_wait(bar, xch_parity)) {
+                    alive = false;
+                    atomicMax(&g_pass_status, 22);
+                }
+                __syncwarp();
+                dot = 0.f;
+                for (int q = sub; q < parts; q += SHARE) dot += share[q];
+                xch_parity ^= flip;
+            } else {
+                if (sub == 0) red[flip][mine][warp] = dot;
+                __syncwarp();
+                bar_sync(1 + grp, 32 * W);
+                dot = sub < W ? red[flip][mine][grp * W + sub] : 0.f;
+            }
+#pragma unroll
+            for (int o = SHARE / 2; o > 0; o /= 2) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+            flip ^= 1;
+        }
+        const float res = dot - bv;
+        if constexpr (GRAD) {
+#pragma unroll
+            for (int i = 0; i < RBX; ++i) {
+                const float ri = RBX == 1 ? res : __shfl_sync(0xffffffffu, res, i * SHARE);
+                if constexpr (C == 1) {
+                    acc[0] = fmaf(v[i][0], ri, acc[0]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < C; c += 2) {
+                        const float2 t = __ffma2_rn(make_float2(v[i][c], v[i][c + 1]), make_float2(ri, ri), make_float2(acc[c], acc[c + 1]));
+                        acc[c] = t.x;
+                        acc[c + 1] = t.y;
+                    }
+                }
+            }
+        } else {
+            if (wg == 0 && lane % SHARE == 0) loss += (double)res * (double)res;
+        }
+    };
+
+    bool loaded = false;
+    int slot = 0, parity = 0;
+    int k = grp;
+    int row = first_row(k);
+    // right-hand sides of the current chunk (lane l: its row l) and of the next one, fetched a chunk ahead
+    const float *const rhs = a.b + lo;
+    auto fetch_rhs = [&](int chunk) {
+        if (chunk >= chunks) return 0.f;
+        const int r = first_row(chunk) + lane;
+        return lane < R && r < nrows ? __ldg(rhs + r) : 0.f;
+    };
+    float b_now = fetch_rhs(k), b_next = fetch_rhs(k + GROUPS);
+    int64_t machine = GRAD ? lo / a.rows : 0;
+    int seg_end = GRAD ? (int)min((int64_t)nrows, (machine + 1) * a.rows - lo) : nrows;
+    for (;;) {
+        while (k < chunks && row < seg_end) {
+            const int r0 = first_row(k), r1 = min(r0 + R, nrows);
+            if (!loaded) {
+                if (alive && !mbar_wait(bar0 + 8 * slot, parity)) {
+                    alive = false;                      // no further waits: the CTA runs to its end and is reported
+                    atomicMax(&g_pass_status, 21);
+                }
+                loaded = true;
+            }
+            const uint32_t mis = ((uint32_t)unit_base + (uint32_t)r0 * row_bytes) & 15;
+            const uint32_t chunk_at = ring + (uint32_t)slot * a.slot_bytes + mis;
+            const int stop = min(r1, seg_end);          // the rest of the chunk belongs to the next machine
+            using batch_rows = std::integral_constant<int, RB>;
+            using single_row = std::integral_constant<int, 1>;
+            for (; row + RB <= stop; row += RB)
+                process(batch_rows{}, chunk_at + (uint32_t)(row - r0) * a.row_stride,
+                        __shfl_sync(0xffffffffu, b_now, (row - r0 + lane / (32 / RB)) & 31));
+            if constexpr (RB > 1)
+                for (; row < stop; ++row)
+                    process(single_row{}, chunk_at + (uint32_t)(row - r0) * a.row_stride,
+                            __shfl_sync(0xffffffffu, b_now, (row - r0) & 31));
+            row = stop;
+            if (stop == r1) {                           // the chunk is used up
+                // every warp of the group has read its part of the rows (in a cluster and between warps the exchange of
+                // the last row's shares told so): the slot may be refilled
+                __syncwarp();
+                if (leader && k + a.slots * GROUPS < chunks) issue(k + a.slots * GROUPS, slot);
+                k += GROUPS;
+                b_now = b_next;
+                b_next = fetch_rhs(k + GROUPS);
+                loaded = false;
+                if (k < chunks) row = first_row(k);
+                if (++slot == a.slots) { slot = 0; parity ^= 1; }
+            }
+        }
+        if constexpr (GRAD) {
+            // partial gradient of this unit for this machine
+            const int64_t machine_unit = (machine * a.rows + 1) * a.units - 1;      // unit of the machine's first row
+            float *out = a.part + (machine * a.slots_per_machine + (unit - machine_unit / a.total)) * a.ldp + col0;
+            auto each_column = [&](auto &&f) {
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    if (first + stride * c < dn) f(c, first + stride * c);
+            };
+            if constexpr (GROUPS == 1) {
+                each_column([&](int c, int col) { out[col] = acc[c]; });
+            } else {
+                __syncthreads();                        // where it is the rings that take the groups' sums
+                const int room = min(a.flush_floats / dn, GROUPS);
+                for (int g0 = 0; g0 < GROUPS; g0 += room) {           // as many groups at a time as there is room for
+                    if (grp >= g0 && grp < g0 + room) each_column([&](int c, int col) { flush[(grp - g0) * dn + col] = acc[c]; });
+                    __syncthreads();
+                    const int here = min(room, GROUPS - g0);
+                    for (int col = tid; col < dn; col += THREADS) {
+                        float sum = g0 > 0 ? out[col] : 0.f;
+#pragma unroll 4
+                        for (int g = 0; g < here; ++g) sum += flush[g * dn + col];
+                        out[col] = sum;
+                    }
+                    __syncthreads();
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[c] = 0.f;
+        }
+        if (seg_end == nrows) break;
+        ++machine;
+        seg_end = (int)min((int64_t)nrows, seg_end + a.rows);
+    }
+    if constexpr (!GRAD) {
+#pragma unroll
+        for (int o = 16; o > 0; o /= 2) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (lane == 0) loss_sums[warp] = loss;
+        __syncthreads();
+        if (tid == 0 && rank == 0) {
+            double sum = 0.0;
+            for (int w = 0; w < WARPS; ++w) sum += loss_sums[w];
+            a.loss_part[unit] = sum;
+        }
+    }
+    if (!alive && leader)                               // copies in flight must not outlive the CTA's shared memory
+        for (int s = 0; s < a.slots; ++s) mbar_wait(bar0 + 8 * s, parity);
+    if (MULTI && a.cluster > 1) cluster_sync();         // a CTA stays while others may still send to it
+}
+
+// G[i][k] = inv_rows * sum of machine i's partial gradients, in the order of its units.
+__global__ void ls_pass_reduce_kernel(const float *__restrict__ part, int64_t rows, int64_t total, int64_t units,
+                                      int slots_per_machine, int64_t ldp, int64_t d, float inv_rows, float *__restrict__ G) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = blockIdx.y;
+    if (k >= d) return;
+    const int64_t first = ((i * rows + 1) * units - 1) / total, last = ((i + 1) * rows * units - 1) / total;
+    const float *p = part + i * slots_per_machine * ldp + k;
+    float s = 0.f;
+#pragma unroll 8
+    for (int64_t u = first; u <= last; ++u, p += ldp) s += *p;
+    G[i * d + k] = s * inv_rows;
+}
+
+// loss[0] = scale * sum of the units' sums of squares: lane l sums units l, l + 32, ..., then a fixed tree.
+__global__ void ls_loss_sum_kernel(const double *__restrict__ loss_part, int64_t units, double scale, double *loss) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int64_t u = threadIdx.x; u < units; u += 32) s += loss_part[u];
+#pragma unroll
+    for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) loss[0] = s * scale;
+}
+
+struct PassConfig {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    PassConfig(const LsPass &p, cudaStream_t stream) {
+        cfg.gridDim = dim3((unsigned)(p.units * p.cluster));
+        cfg.blockDim = dim3((unsigned)(32 * p.warps));
+        cfg.dynamicSmemBytes = p.smem;
+        cfg.stream = stream;
+        if (p.cluster > 1) {
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)p.cluster;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+        }
+    }
+};
+
+cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const float *b, const LsPoint &at, int64_t d,
+                        cudaStream_t stream) {
+    const bool grad = a.part != nullptr;
+    a.A = A;
+    a.b = b;
+    a.x = at.x;
+    a.x_prev = at.x_prev;
+    a.gamma = at.gamma;
+    a.d = d;
+    a.rows = p.rows;
+    a.total = p.total;
+    a.units = p.units;
+    a.ldp = p.ldp;
+    a.slots_per_machine = p.slots_per_machine;
+    a.cluster = p.cluster;
+    a.slice = p.slice;
+    a.chunk_rows = p.chunk_rows;
+    a.slots = p.slots;
+    a.slot_bytes = p.slot_bytes;
+    a.row_stride = p.row_stride;
+    a.ring_offset = p.ring_offset;
+    a.flush_floats = p.ring_offset ? kPassFlushFloats : (int)(p.smem / sizeof(float));
+    auto go = [&](auto kernel) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+        if (e != cudaSuccess) return e;
+        PassConfig config(p, stream);
+        return cudaLaunchKernelEx(&config.cfg, kernel, a);
+    };
+    auto pick = [&](auto warps, auto per_row, auto columns) {
+        constexpr int WARPS = decltype(warps)::value, W = decltype(per_row)::value, C = decltype(columns)::value;
+        constexpr int RB = pass_batch(W, C);
+        return grad ? go(ls_pass_kernel<WARPS, W, C, RB, true>) : go(ls_pass_kernel<WARPS, W, C, RB, false>);
+    };
+    using std::integral_constant;
+    using i1 = integral_constant<int, 1>;
+    using i2 = integral_constant<int, 2>;
+    using i4 = integral_constant<int, 4>;
+    using i8 = integral_constant<int, 8>;
+    using i16 = integral_constant<int, 16>;
+    using i20 = integral_constant<int, 20>;
+    using i24 = integral_constant<int, 24>;
+    using i32 = integral_constant<int, 32>;
+    auto wide = [&](auto warps, auto per_row) {
+        if constexpr (decltype(per_row)::value <= 4)
+            if (p.columns == 20) return pick(warps, per_row, i20{});
+        return p.columns == 24 ? pick(warps, per_row, i24{}) : pick(warps, per_row, i32{});
+    };
+    switch (p.group_warps) {
+        case 16: return wide(i16{}, i16{});
+        case 8: return wide(i8{}, i8{});
+        case 4: return wide(i8{}, i4{});
+        case 2: return wide(i8{}, i2{});
+        default: break;
+    }
+    switch (p.columns) {
+        case 1: return pick(i16{}, i1{}, i1{});
+        case 2: return pick(i16{}, i1{}, i2{});
+        case 4: return pick(i16{}, i1{}, i4{});
+        case 8: return pick(i16{}, i1{}, i8{});
+        case 16: return pick(i16{}, i1{}, i16{});
+        default: return pick(i16{}, i1{}, i32{});
+    }
+}
+
+}  // namespace
+
+LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int sm_count) {
+    LsPass p{};
+    if (d > (int64_t)kPassCtaCols * kPassMaxCluster) return p;             // units == 0: does not apply
+    p.cluster = 1;
+    while (d > (int64_t)kPassCtaCols * p.cluster) p.cluster *= 2;
+    p.slice = p.cluster == 1 ? (int)d : (int)(((d + p.cluster - 1) / p.cluster + 3) / 4 * 4);
+    p.group_warps = 1;
+    while (p.slice > 1024 * p.group_warps) p.group_warps *= 2;
+    const int per_lane = (p.slice + 32 * p.group_warps - 1) / (32 * p.group_warps);
+    p.columns = 1;
+    while (p.columns < per_lane) p.columns *= 2;
+    if (p.group_warps > 1) p.columns = per_lane <= 20 && p.group_warps <= 4 ? 20 : per_lane <= 24 ? 24 : 32;
+    p.warps = p.group_warps == 1 || p.group_warps == 16 ? 16 : 8;
+    const int groups = p.warps / p.group_warps;
+    const uint32_t row_bytes = (uint32_t)p.slice * 4;
+    const int batch = pass_batch(p.group_warps, p.columns);               // rows at a time
+    p.chunk_rows = batch;
+    if (p.group_warps == 1) p.chunk_rows *= std::max(1, std::min((int)(kPassRingBytes / (3 * groups) / (row_bytes * batch)), 32 / batch));
+    p.row_stride = p.cluster == 1 ? row_bytes : (row_bytes + 31) / 16 * 16 + (uint32_t)(d * 4 % 16);
+    p.slot_bytes = (p.chunk_rows * p.row_stride + 12 + 15) / 16 * 16;
+    p.ring_offset = machines_apart && groups > 1 ? kPassFlushFloats * 4u : 0u;
+    const int room = (int)((220u * 1024u - p.ring_offset) / (groups * p.slot_bytes));
+    p.slots = std::max((int)(kPassRingBytes / (groups * p.slot_bytes)), 3);
+    p.slots = std::min({p.slots, room, kPassMaxSlots});
+    if (p.slots < 2) return LsPass{};
+    p.smem = p.ring_offset + (size_t)groups * p.slots * p.slot_bytes;
+    p.total = (int64_t)n * rows;
+    p.rows = machines_apart ? rows : p.total;
+    p.units = sm_count / p.cluster;
+    if (p.cluster > 1) {
+        // no more clusters than run side by side: SMs that cannot form another one stay idle, a second wave would cost more
+        auto kernel = ls_pass_kernel<16, 16, 32, 1, true>;
+        int resident = 0;
+        PassConfig config(p, nullptr);
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&resident, kernel, &config.cfg) != cudaSuccess || resident < 1) {
+            cudaGetLastError();
+            return LsPass{};
+        }
+        if (p.units > resident) p.units = resident;
+    }
+    if (p.units > p.total) p.units = p.total;
+    p.ldp = (d + 3) / 4 * 4;
+    p.slots_per_machine = 1;
+    const int64_t machines = p.total / p.rows;
+    for (int64_t i = 0; i < machines; ++i) {
+        const int64_t first = ((i * p.rows + 1) * p.units - 1) / p.total, last = ((i + 1) * p.rows * p.units - 1) / p.total;
+        if (last - first + 1 > p.slots_per_machine) p.slots_per_machine = (int)(last - first + 1);
+    }
+    return p;
+}
+
+size_t ls_pass_partials(const LsPass &p) { return p.units ? (size_t)(p.total / p.rows) * p.slots_per_machine * p.ldp : 0; }
+
+cudaError_t launch_ls_pass_gradients(const LsPass &p, const float *A, const float *b, const LsPoint &at, int64_t d,
+                                     float *part, cudaStream_t stream) {
+    PassArgs a{};
+    a.part = part;
+    return launch_pass(p, a, A, b, at, d, stream);
+}
+
+cudaError_t launch_ls_pass_loss(const LsPass &p, const float *A, const float *b, const LsPoint &at, int64_t d, bool reverse,
+                                double *loss_part, cudaStream_t stream) {
+    PassArgs a{};
+    a.loss_part = loss_part;
+    a.reverse = reverse;
+    return launch_pass(p, a, A, b, at, d, stream);
+}
+
+cudaError_t launch_ls_pass_reduce(const LsPass &p, const float *part, int64_t d, float inv_rows, float *G, cudaStream_t stream) {
+    const int n = (int)(p.total / p.rows);
+    ls_pass_reduce_kernel<<<dim3((unsigned)((d + 127) / 128), n), 128, 0, stream>>>(part, p.rows, p.total, p.units,
+                                                                                  p.slots_per_machine, p.ldp, d, inv_rows, G);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ls_loss_sum(const double *loss_part, int64_t units, double scale, double *loss, cudaStream_t stream) {
+    ls_loss_sum_kernel<<<1, 32, 0, stream>>>(loss_part, units, scale, loss);
+    return cudaGetLastError();
+}
+
+cudaError_t ls_pass_take_status(int *status) {
+    cudaError_t e = cudaMemcpyFromSymbol(status, g_pass_status, sizeof(int));
+    if (e != cudaSuccess || *status == 0) return e;
+    const int zero = 0;
+    return cudaMemcpyToSymbol(g_pass_status, &zero, sizeof(int));
+}
+
+}  // namespace core

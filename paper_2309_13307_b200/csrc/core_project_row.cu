@@ -17,6 +17,7 @@
 // sine lanes of both pairs as ready register pairs and S (g_c (y sp) + g_s cs) is four packed instructions
 // per counter.
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 #include <cuda_bf16.h>
 
@@ -206,9 +207,6 @@ __device__ __forceinline__ void row_stage_any(int stride, const RowArgs &a, int6
         else row_stage<1, 8, false, GT>(stride, a, k0, blocks, first, step, r0, r1, lane, tile);
     }
 }
-
-__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
 template <typename GT>
 __global__ void __launch_bounds__(kRowThreads, 2)

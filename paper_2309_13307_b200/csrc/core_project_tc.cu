@@ -21,6 +21,7 @@
 // normal exit (which releases its tensor memory).  The per-CTA partial sums have the layout of the
 // scalar kernel.
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 #include <cuda_bf16.h>
 
@@ -68,7 +69,6 @@ struct TcShape {
     static constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NT >> 3) << 17) |
                                        ((uint32_t)(kTcVectors >> 4) << 24);
 };
-constexpr uint64_t kTcWaitLimitNs = 100ull * 1000 * 1000;   // a wait gives up after 100 ms of the global timer
 
 __device__ int g_tc_status;                     // 0, or the code of a wait that ran out
 
@@ -88,42 +88,6 @@ struct TcArgs {
 
 // ---- thin wrappers over the PTX this kernel needs --------------------------------------------------
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_timer_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// Bounded wait: false when the phase did not complete within limit_ns of the global timer (read only
-// once a first probe has failed, so a wait that is served at once costs one probe).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns = kTcWaitLimitNs) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
-    do {
-#pragma unroll 1
-        for (int probe = 0; probe < 64; ++probe)
-            if (mbar_try_wait(bar, parity)) return true;
-    } while (global_timer_ns() - t0 < limit_ns);
-    return false;
-}
 // True in exactly one lane of a converged warp.  Unlike a test of the lane index this keeps the branch, and the
 // operands computed for the instructions under it, warp-uniform in the compiler's eyes.
 __device__ __forceinline__ bool elect_one() {
@@ -136,7 +100,6 @@ __device__ __forceinline__ bool elect_one() {
     return chosen != 0;
 }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 

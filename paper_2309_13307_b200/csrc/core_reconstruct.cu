@@ -77,13 +77,18 @@ __device__ __forceinline__ void emit_block(const ReconstructArgs &a, uint64_t q,
     if (a.vec_ok && k + 4 <= a.k_end) {
         float4 v = r;
         if (a.epi.base) {
-            const float4 b = *reinterpret_cast<const float4 *>(a.epi.base + off);
-            v = make_float4(fmaf(-step, r.x, b.x), fmaf(-step, r.y, b.y),
-                            fmaf(-step, r.z, b.z), fmaf(-step, r.w, b.w));
+            float4 b = *reinterpret_cast<const float4 *>(a.epi.base + off);
             if (a.epi.shift_dst) {
                 const float4 s = *reinterpret_cast<const float4 *>(a.epi.shift_src + off);
+                if (a.epi.lookahead) {
+                    const float4 o = *reinterpret_cast<const float4 *>(a.epi.shift_dst + off);
+                    b = make_float4(fmaf(a.epi.gamma, s.x - o.x, s.x), fmaf(a.epi.gamma, s.y - o.y, s.y),
+                                    fmaf(a.epi.gamma, s.z - o.z, s.z), fmaf(a.epi.gamma, s.w - o.w, s.w));
+                }
                 *reinterpret_cast<float4 *>(a.epi.shift_dst + off) = s;
             }
+            v = make_float4(fmaf(-step, r.x, b.x), fmaf(-step, r.y, b.y),
+                            fmaf(-step, r.z, b.z), fmaf(-step, r.w, b.w));
         }
         *reinterpret_cast<float4 *>(a.out + off) = v;
     } else {
@@ -93,8 +98,13 @@ __device__ __forceinline__ void emit_block(const ReconstructArgs &a, uint64_t q,
             if (k + l >= a.k_end) continue;
             float v = vals[l];
             if (a.epi.base) {
-                v = fmaf(-step, v, a.epi.base[off + l]);
-                if (a.epi.shift_dst) a.epi.shift_dst[off + l] = a.epi.shift_src[off + l];
+                float b = a.epi.base[off + l];
+                if (a.epi.shift_dst) {
+                    const float s = a.epi.shift_src[off + l];
+                    if (a.epi.lookahead) b = fmaf(a.epi.gamma, s - a.epi.shift_dst[off + l], s);
+                    a.epi.shift_dst[off + l] = s;
+                }
+                v = fmaf(-step, v, b);
             }
             a.out[off + l] = v;
         }
@@ -198,13 +208,6 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
     }
 }
 
-__global__ void lookahead_kernel(const float *__restrict__ x, const float *__restrict__ x_prev, float gamma, int64_t d,
-                                 float *__restrict__ y) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < d; k += stride)
-        y[k] = fmaf(gamma, x[k] - x_prev[k], x[k]);
-}
-
 struct DebugArgs {
     uint64_t q0;
     int64_t nq;
@@ -287,12 +290,6 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, const float *p
     int64_t grid = (int64_t)sm_count * 3;     // three resident CTAs per SM (register-limited)
     if (grid > groups) grid = groups;
     reconstruct_kernel<<<(unsigned)grid, kThreads, 0, stream>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_lookahead(const float *x, const float *x_prev, float gamma, int64_t d, float *y,
-                             cudaStream_t stream) {
-    lookahead_kernel<<<grid_for(d, 256, 148 * 8), 256, 0, stream>>>(x, x_prev, gamma, d, y);
     return cudaGetLastError();
 }
 
