@@ -695,12 +695,7 @@ int core_decentralized_step(core_ctx *ctx, core_ls *ls, const float *W_dev, int3
     if (int rc = ls_gradients_into(ctx, ls, x_dev, ls->G)) return rc;
     if (int rc = project_into(ctx, ls->G, CORE_F32, n, ls->d, ctx->d, 0, partial, P, false, ctx->stream)) return rc;
     // the m-dimensional averaging problem, by gossip with the neighbours: row i is machine i's estimate
-    for (int32_t r = 0; r < rounds; ++r) {
-        CORE_CUDA(ctx, launch_gossip_round(W_dev, P, n, ctx->m, P_next, ctx->stream));
-        float *swap = P;
-        P = P_next;
-        P_next = swap;
-    }
+    CORE_CUDA(ctx, launch_gossip_rounds(W_dev, P, n, ctx->m, rounds, P_next, &P, ctx->stream));
     if (spread_dev) CORE_CUDA(ctx, launch_consensus_spread(P, n, ctx->m, reader, spread_dev, ctx->stream));
     // reconstruction from the reader's estimate, update inside the kernel; the printed prefactor n/m is
     // the mean convention's 1/m with an n times longer step

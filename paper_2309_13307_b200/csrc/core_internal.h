@@ -185,6 +185,9 @@ cudaError_t launch_option1_step(const float *pbar, int32_t m, int64_t d, double 
                                 float *h_out, cudaStream_t stream);
 // Algorithm 5's averaging by gossip: out[i*m + j] = sum_l W[i*n + l] in[l*m + j], l ascending (in != out).
 cudaError_t launch_gossip_round(const float *W, const float *in, int32_t n, int32_t m, float *out, cudaStream_t stream);
+// `rounds` of them: P and scratch (n x m each) are both written, *result tells which holds the outcome.
+cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m, int32_t rounds, float *scratch, float **result,
+                                 cudaStream_t stream);
 // spread[0] = max_ij |P[i*m + j] - P[reader*m + j]|
 cudaError_t launch_consensus_spread(const float *P, int32_t n, int32_t m, int32_t reader, float *spread,
                                     cudaStream_t stream);
