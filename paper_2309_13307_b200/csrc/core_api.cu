@@ -377,6 +377,15 @@ int core_round_host(core_ctx *ctx, const void *G_host, int dtype, int32_t n, int
     return rc;
 }
 
+// Length of the slab that starts at coordinate k0 of d: growing from `least` with what is behind it, shrinking to
+// `least` with what is ahead, multiples of 4096 but for the end of the vector.
+static int64_t next_slab(int64_t k0, int64_t d, int64_t least, int64_t most) {
+    const int64_t left = d - k0;
+    int64_t len = std::min(most, std::min(k0 + least, std::max(left / 2, least)));
+    len = std::max<int64_t>(len / 4096 * 4096, 4096);
+    return left - len < least / 2 ? (left <= most ? left : len) : len;
+}
+
 static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t n, int64_t ldg, float *pbar_host,
                            float *gtilde_host) {
     if (!ctx->host_ready) {
@@ -402,13 +411,20 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
     }
     const size_t es = elem_size(dtype);
     const int64_t d = ctx->d;
-    // slab: a multiple of 4096 coordinates, about 64 MiB of input per slab over all machines
-    int64_t slab = ((int64_t)64 << 20) / (int64_t)(es * (size_t)n);
-    slab = slab / 4096 * 4096;
-    if (slab < 4096) slab = 4096;
-    if (slab > (d + 4095) / 4096 * 4096) slab = (d + 4095) / 4096 * 4096;
-    const size_t in_bytes = round_up((size_t)n * (size_t)slab * es, 256);
-    const size_t out_bytes = round_up((size_t)slab * sizeof(float), 256);
+    // Slabs of at most 64 MiB of input over all machines and 16 MiB of output, all multiples of 4096 coordinates.  The
+    // first and the last ones are shorter (next_slab): what is not overlapped is the projection of the last slab and the
+    // reconstruction of the first one (and, where the kernels are the slower side, the first copy in and the last out).
+    const int64_t whole = (d + 4095) / 4096 * 4096;
+    auto limit = [&](int64_t bytes, size_t per_coordinate) {
+        int64_t slab = bytes / (int64_t)per_coordinate / 4096 * 4096;
+        return slab < 4096 ? 4096 : slab > whole ? whole : slab;
+    };
+    const int64_t in_most = limit((int64_t)64 << 20, es * (size_t)n), out_most = limit((int64_t)16 << 20, sizeof(float));
+    // at least 256 KB per machine and copy
+    const int64_t in_least = std::min(in_most, limit(std::max((int64_t)4 << 20, (int64_t)n << 18), es * (size_t)n));
+    const int64_t out_least = std::min(out_most, limit((int64_t)1 << 20, sizeof(float)));
+    const size_t in_bytes = round_up((size_t)n * (size_t)in_most * es, 256);
+    const size_t out_bytes = round_up((size_t)out_most * sizeof(float), 256);
     const size_t need_slab = 2 * in_bytes + 2 * out_bytes;
     if (need_slab > ctx->slab_bytes) {
         if (ctx->slab) {
@@ -424,7 +440,9 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
         }
         ctx->slab_bytes = need_slab;
     }
-    const size_t pb = row_partial_bytes(ctx, slab);
+    size_t pb = row_partial_bytes(ctx, in_most);       // of the longest slab, and of every shorter one
+    for (int64_t k0 = 0; k0 < d; k0 += next_slab(k0, d, in_least, in_most))
+        pb = std::max(pb, row_partial_bytes(ctx, next_slab(k0, d, in_least, in_most)));
     const size_t mb = round_up((size_t)ctx->m * sizeof(float), 256);
     if (int rc = ensure_workspace(ctx, pb + mb)) return rc;
     char *in_buf[2] = {static_cast<char *>(ctx->slab), static_cast<char *>(ctx->slab) + in_bytes};
@@ -435,32 +453,37 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
 
     CORE_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // earlier work of the caller on this context
 
-    // projection: slab s is copied while slab s-1 is projected
-    const int64_t slabs = (d + slab - 1) / slab;
-    for (int64_t s = 0; s < slabs; ++s) {
-        const int b = (int)(s & 1);
-        const int64_t k0 = s * slab;
-        const int64_t len = d - k0 < slab ? d - k0 : slab;
+    // projection: slab s is copied while slab s-1 is projected; the mean message grows slab by slab (the gradients of a
+    // slab are added while they are staged)
+    int64_t len = 0;
+    int s = 0;
+    for (int64_t k0 = 0; k0 < d; k0 += len, ++s) {
+        const int b = s & 1;
+        len = next_slab(k0, d, in_least, in_most);
         if (s >= 2) CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->in_free[b], 0));
-        for (int32_t i = 0; i < n; ++i)   // one copy per row: row strides may exceed the 2-D copy pitch limit
-            CORE_CUDA(ctx, cudaMemcpyAsync(in_buf[b] + (size_t)i * (size_t)slab * es,
-                                           static_cast<const char *>(G_host) + ((size_t)i * (size_t)ldg + (size_t)k0) * es,
-                                           (size_t)len * es, cudaMemcpyHostToDevice, ctx->copy_stream));
+        const char *const from = static_cast<const char *>(G_host) + (size_t)k0 * es;
+        if ((size_t)ldg * es <= (size_t)INT32_MAX)          // one copy for all rows, where the stride is a legal pitch
+            CORE_CUDA(ctx, cudaMemcpy2DAsync(in_buf[b], (size_t)in_most * es, from, (size_t)ldg * es, (size_t)len * es, (size_t)n,
+                                             cudaMemcpyHostToDevice, ctx->copy_stream));
+        else
+            for (int32_t i = 0; i < n; ++i)
+                CORE_CUDA(ctx, cudaMemcpyAsync(in_buf[b] + (size_t)i * (size_t)in_most * es, from + (size_t)i * (size_t)ldg * es,
+                                               (size_t)len * es, cudaMemcpyHostToDevice, ctx->copy_stream));
         CORE_CUDA(ctx, cudaEventRecord(ctx->in_ready[b], ctx->copy_stream));
         CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->work_stream, ctx->in_ready[b], 0));
-        // the mean message, slab by slab (the gradients of a slab are added while they are staged)
-        if (int rc = project_row_into(ctx, in_buf[b], dtype, n, slab, 1.0f / (float)n, len, (uint64_t)k0 >> 2, partial, pbar,
+        if (int rc = project_row_into(ctx, in_buf[b], dtype, n, in_most, 1.0f / (float)n, len, (uint64_t)k0 >> 2, partial, pbar,
                                       s > 0, ctx->work_stream))
             return rc;
         CORE_CUDA(ctx, cudaEventRecord(ctx->in_free[b], ctx->work_stream));
     }
-    CORE_CUDA(ctx, cudaMemcpyAsync(pbar_host, pbar, (size_t)ctx->m * sizeof(float), cudaMemcpyDeviceToHost,
-                                   ctx->work_stream));
+    // the last slab's event also tells that the message is complete
+    CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->in_free[(s - 1) & 1], 0));
+    CORE_CUDA(ctx, cudaMemcpyAsync(pbar_host, pbar, (size_t)ctx->m * sizeof(float), cudaMemcpyDeviceToHost, ctx->copy_stream));
     // reconstruction: slab s is copied back while slab s+1 is generated
-    for (int64_t s = 0; s < slabs; ++s) {
-        const int b = (int)(s & 1);
-        const int64_t k0 = s * slab;
-        const int64_t len = d - k0 < slab ? d - k0 : slab;
+    s = 0;
+    for (int64_t k0 = 0; k0 < d; k0 += len, ++s) {
+        const int b = s & 1;
+        len = next_slab(k0, d, out_least, out_most);
         if (s >= 2) CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->work_stream, ctx->out_free[b], 0));
         CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar, ctx->m, k0, k0 + len, out_buf[b], ctx->sm_count,
                                           ctx->work_stream));
