@@ -4,11 +4,32 @@
 
 #include <algorithm>
 #include <atomic>
+#include <map>
+#include <mutex>
 #include <new>
+#include <utility>
 
 #include "core_internal.h"
 
 using namespace core;
+
+namespace core {
+
+cudaError_t allow_shared(const void *kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    int device = 0;
+    if (cudaError_t e = cudaGetDevice(&device)) return e;
+    static std::mutex mutex;
+    static std::map<std::pair<int, const void *>, size_t> granted;        // one entry per kernel and device
+    std::lock_guard<std::mutex> lock(mutex);
+    size_t &most = granted[{device, kernel}];
+    if (bytes <= most) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) most = bytes;
+    return e;
+}
+
+}  // namespace core
 
 struct core_ctx {
     uint64_t seed;
@@ -300,7 +321,7 @@ int core_aggregate(core_ctx *ctx, const float *P_dev, int32_t n, float *pbar_dev
 int core_reconstruct(core_ctx *ctx, const float *pbar_dev, float *gtilde_dev) {
     if (int rc = check_ctx(ctx)) return rc;
     if (!pbar_dev || !gtilde_dev) return CORE_EINVAL;
-    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar_dev, ctx->m, 0, ctx->d, gtilde_dev, ctx->sm_count,
+    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, const_cast<float *>(pbar_dev), ctx->m, 0, ctx->d, gtilde_dev, ctx->sm_count,
                                       ctx->stream));
     return CORE_OK;
 }
@@ -320,6 +341,24 @@ static int apply_step_rule(core_ctx *ctx, const StepRule *rule, const float *pba
     return CORE_OK;
 }
 
+// The round of one combined row (see launch_project_row): message, step rule, reconstruction, then t <- t + 1.  A short
+// round leaves it to the reconstruction to finish the message.
+static int finish_round(core_ctx *ctx, const void *G, int dtype, int32_t rows, int64_t ldg, float scale, float *partial,
+                        float *pbar_dev, float *out, const ReconstructEpilogue *epilogue, const StepRule *rule) {
+    const RowPlan plan = make_row_plan(ctx->m, ctx->d, ctx->sm_count);
+    CORE_CUDA(ctx, launch_project_row(plan, ctx->keys, ctx->t, G, dtype, rows, ldg, scale, ctx->d, ctx->m, 0, partial, ctx->stream));
+    const MessageParts parts{partial, plan.grid_x, 1};
+    const bool join = !rule && reconstruct_joins(plan.grid_x, 1, ctx->m, ctx->d, ctx->sm_count);
+    if (!join) {
+        CORE_CUDA(ctx, launch_finish_project(partial, plan.grid_x, 1, ctx->m, pbar_dev, false, ctx->stream));
+        if (int rc = apply_step_rule(ctx, rule, pbar_dev)) return rc;
+    }
+    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar_dev, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream, epilogue,
+                                      join ? &parts : nullptr));
+    ctx->t += 1;
+    return CORE_OK;
+}
+
 // project -> aggregate -> reconstruct with the current t, then t <- t + 1.  With an epilogue the
 // reconstruction writes the optimiser update into `out` instead of the estimate.
 static int round_with_epilogue(core_ctx *ctx, const void *G_dev, int dtype, int32_t n, int64_t ldg, float *pbar_dev,
@@ -329,15 +368,20 @@ static int round_with_epilogue(core_ctx *ctx, const void *G_dev, int dtype, int3
     if (int rc = ensure_workspace(ctx, pb + Pb)) return rc;
     float *partial = static_cast<float *>(ctx->ws);
     float *P = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb);
-    if (single_row(n) || combine_first(ctx, n)) {
-        if (int rc = project_row_into(ctx, G_dev, dtype, n, ldg, 1.0f / (float)n, ctx->d, 0, partial, pbar_dev, false,
-                                      ctx->stream))
-            return rc;
-    } else if (project_group(n, ctx->m) == n) {
+    if (single_row(n) || combine_first(ctx, n))
+        return finish_round(ctx, G_dev, dtype, n, ldg, 1.0f / (float)n, partial, pbar_dev, out, epilogue, rule);
+    if (project_group(n, ctx->m) == n) {
         // one group of machines: the per-machine messages are not kept, so they are never written
         const ProjectPlan plan = make_project_plan(n, ctx->m, ctx->d, dtype, ctx->sm_count);
         CORE_CUDA(ctx, launch_project(plan, ctx->keys, ctx->t, G_dev, dtype, n, ldg, ctx->d, ctx->m, 0, partial,
                                       ctx->stream));
+        if (!rule && reconstruct_joins(plan.grid_x, n, ctx->m, ctx->d, ctx->sm_count)) {
+            const MessageParts parts{partial, plan.grid_x, n};
+            CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar_dev, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream,
+                                              epilogue, &parts));
+            ctx->t += 1;
+            return CORE_OK;
+        }
         CORE_CUDA(ctx, launch_finish_aggregate(partial, plan.grid_x, n, ctx->m, pbar_dev, ctx->stream));
     } else {
         if (int rc = project_into(ctx, G_dev, dtype, n, ldg, ctx->d, 0, partial, P, false, ctx->stream)) return rc;
@@ -621,13 +665,7 @@ static int ls_round(core_ctx *ctx, core_ls *ls, const LsPoint &at, float *out, c
         scale = 1.0f / (float)ls->n;
     }
     if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
-    if (int rc = project_row_into(ctx, rows, CORE_F32, count, ld, scale, ctx->d, 0, static_cast<float *>(ctx->ws), ctx->pbar, false,
-                                  ctx->stream))
-        return rc;
-    if (int rc = apply_step_rule(ctx, rule, ctx->pbar)) return rc;
-    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, ctx->pbar, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream, epilogue));
-    ctx->t += 1;
-    return CORE_OK;
+    return finish_round(ctx, rows, CORE_F32, count, ld, scale, static_cast<float *>(ctx->ws), ctx->pbar, out, epilogue, rule);
 }
 
 int core_ls_gradients(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G_out_dev) {

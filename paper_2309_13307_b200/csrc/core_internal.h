@@ -9,6 +9,42 @@
 
 namespace core {
 
+// Grants `kernel` that much dynamic shared memory on the current device (once; later calls only look it up).
+cudaError_t allow_shared(const void *kernel, size_t bytes);
+
+// Launches a kernel of a chain: it may be scheduled while its predecessor in the stream drains (programmatic stream
+// serialisation), which hides its launch latency (1 to 1.5 us a kernel).  Such a kernel calls grid_wait() before it touches
+// global memory and reads what an earlier kernel wrote past the L1 cache (__ldcg).
+struct ChainedLaunch {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attrs[2];
+    ChainedLaunch(bool chain, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster = 1) {
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attrs[0].val.programmaticStreamSerializationAllowed = chain ? 1 : 0;
+        attrs[1].id = cudaLaunchAttributeClusterDimension;
+        attrs[1].val.clusterDim.x = (unsigned)cluster;
+        attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
+        cfg.attrs = attrs;
+        cfg.numAttrs = cluster > 1 ? 2 : 1;
+    }
+};
+template <typename... P, typename... A>
+cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    if (cudaError_t e = allow_shared(reinterpret_cast<const void *>(kernel), smem)) return e;
+    const ChainedLaunch launch(chain, grid, block, smem, stream);
+    return cudaLaunchKernelEx(&launch.cfg, kernel, static_cast<P>(args)...);
+}
+// CTAs of a chained kernel go wherever there is room first.  If they do not fill the chip, that packs them on few SMs (n = 7,
+// d = 3210, m = 940: 45 -> 64 us), so kernels that generate are chained only where they do fill it (`capacity` CTAs are
+// resident together), or where the whole work, d * m Gaussians, takes less than the 2 us or so that are at stake.
+inline bool chain_pays(int64_t ctas, int64_t capacity, int64_t d, int64_t m) {
+    return ctas * 10 >= capacity * 9 || d <= ((int64_t)1 << 21) / m;
+}
+
 constexpr int kThreads = 256;        // threads per CTA in the round kernels
 constexpr int kMaxGroup = 16;        // machines handled by one pass of the scalar projection
 constexpr int kMaxGroupTc = 64;      // most machines one pass of the tensor-memory projection can take
@@ -34,6 +70,7 @@ struct ProjectPlan {
     int64_t tiles;    // ceil(d / (4 * tile_q))
     size_t smem;      // dynamic shared memory per CTA
     int mma;          // 0: scalar kernel; 1: warp-level tensor-core kernel; 2: tcgen05 kernel
+    bool chain;       // see chain_pays
 };
 
 ProjectPlan make_project_plan(int32_t n_group, int32_t m, int64_t d, int dtype, int sm_count);
@@ -64,12 +101,9 @@ cudaError_t launch_wait_timeout_probe(uint64_t limit_ns, int code, uint32_t *obs
 // One projection pass over coordinates [0, d) of rows G + i*ldg, i < n <= 16.
 // q_base is the global index of the block holding coordinate 0 of G (non-zero when G
 // is a slab of a longer vector).  Writes partial[(c * n + i) * m + j], c < plan.grid_x.
-// With splits > 0 (fp32, scalar kernel only: plan.mma == 0) row i is not stored anywhere: it is
-// scale * (G[(i*splits + 0)*ldg + k] + ... + G[(i*splits + splits-1)*ldg + k]), summed in that order
-// while the tile is staged (the per-row-range partial gradients of the least-squares kernels).
 cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint32_t t, const void *G,
                            int dtype, int32_t n, int64_t ldg, int64_t d, int32_t m, uint64_t q_base,
-                           float *partial, cudaStream_t stream, int splits = 0, float scale = 1.0f);
+                           float *partial, cudaStream_t stream);
 
 // Projection of one combined row (core_project_row.cu): partial[c*m + j] = the share of CTA column c in
 // <scale * (row 0 + row 1 + ... + row rows-1), xi_j>.  Rows are `ldg` elements apart and of any alignment.
@@ -81,6 +115,7 @@ struct RowPlan {
     int grid_y;       // CTAs across vectors
     int64_t tiles;
     size_t smem;
+    bool chain;       // see chain_pays
 };
 RowPlan make_row_plan(int32_t m, int64_t d, int sm_count);
 cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype,
@@ -115,9 +150,18 @@ struct ReconstructEpilogue {
     bool lookahead = false;
     float gamma = 0.f;
 };
-cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, const float *pbar, int32_t m,
+// With parts the message is not in pbar yet: the kernel forms it from the projection's partial sums (partial[c][i][j],
+// c < chunks, i < n; the same bits as launch_finish_aggregate) and writes it there.  reconstruct_joins tells where it can.
+struct MessageParts {
+    const float *partial;
+    int chunks;
+    int n;
+};
+bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count);
+cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, int32_t m,
                                int64_t k_begin, int64_t k_end, float *out, int sm_count,
-                               cudaStream_t stream, const ReconstructEpilogue *epilogue = nullptr);
+                               cudaStream_t stream, const ReconstructEpilogue *epilogue = nullptr,
+                               const MessageParts *parts = nullptr);
 
 cudaError_t launch_debug_philox(const RoundKeys &keys, uint32_t t, uint32_t j, uint64_t q0, int64_t nq,
                                 uint32_t *words, cudaStream_t stream);

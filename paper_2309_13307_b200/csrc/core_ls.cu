@@ -2,6 +2,7 @@
 // of core_ls_pass.cu: f_i(x) = 1/(2 rows) ||A_i x - b_i||^2, g_i = A_i^T (A_i x - b_i) / rows in two streaming passes
 // over A (both HBM-bound), every sum in a fixed order.  Also the comparison step of Algorithm 3.
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 namespace core {
 
@@ -128,11 +129,13 @@ constexpr int64_t kKeepOneCta = 32768;         // 128 KB: about what one SM move
 __global__ void __launch_bounds__(kKeepThreads)
 keep_better_kernel(const double *__restrict__ f_parts, int64_t parts, double scale, const float *__restrict__ trial, int64_t d,
                    double *__restrict__ f, float *__restrict__ x, int *__restrict__ flag, int32_t *__restrict__ flag_out) {
+    grid_trigger();
+    grid_wait();
     __shared__ int decision;
     if (threadIdx.x < 32) {
         double s = 0.0;                         // as in ls_loss_sum_kernel: the same bits
 #pragma unroll 8
-        for (int64_t u = threadIdx.x; u < parts; u += 32) s += f_parts[u];
+        for (int64_t u = threadIdx.x; u < parts; u += 32) s += __ldcg(f_parts + u);
 #pragma unroll
         for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (threadIdx.x == 0) {
@@ -146,7 +149,7 @@ keep_better_kernel(const double *__restrict__ f_parts, int64_t parts, double sca
     }
     __syncthreads();
     if (decision && d <= kKeepOneCta)
-        for (int64_t k = threadIdx.x; k < d; k += kKeepThreads) x[k] = trial[k];
+        for (int64_t k = threadIdx.x; k < d; k += kKeepThreads) x[k] = __ldcg(trial + k);
 }
 
 __global__ void keep_better_copy_kernel(const int *__restrict__ flag, const float *__restrict__ trial, int64_t d,
@@ -171,7 +174,9 @@ bool vec_ok_for(const float *A, int64_t d) {
 
 cudaError_t launch_keep_better(const double *f_parts, int64_t parts, double scale, const float *trial, int64_t d, double *f,
                                float *x, int *flag_scratch, int32_t *flag_out, cudaStream_t stream) {
-    keep_better_kernel<<<1, kKeepThreads, 0, stream>>>(f_parts, parts, scale, trial, d, f, x, flag_scratch, flag_out);
+    if (cudaError_t e = launch_chained(true, keep_better_kernel, dim3(1), dim3(kKeepThreads), 0, stream, f_parts, parts, scale, trial, d, f, x,
+                                       flag_scratch, flag_out))
+        return e;
     if (d > kKeepOneCta) {
         int64_t blocks = (d + 255) / 256;
         if (blocks > 148 * 8) blocks = 148 * 8;

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1)
 ls_pass_kernel(const __grid_constant__ PassArgs a) {
     constexpr bool MULTI = W > 1;
     constexpr int THREADS = 32 * WARPS, GROUPS = WARPS / W;
+    grid_trigger();
     extern __shared__ __align__(16) unsigned char pass_smem[];
     __shared__ __align__(8) uint64_t bars[WARPS * kPassMaxSlots];
     __shared__ float red[2][RB][WARPS];
@@ -193,17 +194,18 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     };
     constexpr int stride = 32 * W, CB = C < 4 ? C : 4;             // CB columns are tested for together
     const int first = lane + 32 * wg;
+    grid_wait();
     if (leader)
         for (int s = 0; s < a.slots; ++s)
             if (grp + s * GROUPS < chunks) issue(grp + s * GROUPS, s);
 
     float xv[C], acc[GRAD ? C : 1];
 #pragma unroll
-    for (int c = 0; c < C; ++c) xv[c] = first + stride * c < dn ? __ldg(a.x + col0 + first + stride * c) : 0.f;
+    for (int c = 0; c < C; ++c) xv[c] = first + stride * c < dn ? __ldcg(a.x + col0 + first + stride * c) : 0.f;
     if (a.x_prev) {
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            const float old = first + stride * c < dn ? __ldg(a.x_prev + col0 + first + stride * c) : 0.f;
+            const float old = first + stride * c < dn ? __ldcg(a.x_prev + col0 + first + stride * c) : 0.f;
             xv[c] = fmaf(a.gamma, xv[c] - old, xv[c]);
         }
     }
@@ -319,7 +321,7 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     auto fetch_rhs = [&](int chunk) {
         if (chunk >= chunks) return 0.f;
         const int r = first_row(chunk) + lane;
-        return lane < R && r < nrows ? __ldg(rhs + r) : 0.f;
+        return lane < R && r < nrows ? __ldcg(rhs + r) : 0.f;
     };
     float b_now = fetch_rhs(k), b_next = fetch_rhs(k + GROUPS);
     int64_t machine = GRAD ? lo / a.rows : 0;
@@ -413,6 +415,8 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
 // G[i][k] = inv_rows * sum of machine i's partial gradients, in the order of its units.
 __global__ void ls_pass_reduce_kernel(const float *__restrict__ part, int64_t rows, int64_t total, int64_t units,
                                       int slots_per_machine, int64_t ldp, int64_t d, float inv_rows, float *__restrict__ G) {
+    grid_trigger();
+    grid_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = blockIdx.y;
     if (k >= d) return;
@@ -420,37 +424,21 @@ __global__ void ls_pass_reduce_kernel(const float *__restrict__ part, int64_t ro
     const float *p = part + i * slots_per_machine * ldp + k;
     float s = 0.f;
 #pragma unroll 8
-    for (int64_t u = first; u <= last; ++u, p += ldp) s += *p;
+    for (int64_t u = first; u <= last; ++u, p += ldp) s += __ldcg(p);
     G[i * d + k] = s * inv_rows;
 }
 
 // loss[0] = scale * sum of the units' sums of squares: lane l sums units l, l + 32, ..., then a fixed tree.
 __global__ void ls_loss_sum_kernel(const double *__restrict__ loss_part, int64_t units, double scale, double *loss) {
+    grid_trigger();
+    grid_wait();
     double s = 0.0;
 #pragma unroll 8
-    for (int64_t u = threadIdx.x; u < units; u += 32) s += loss_part[u];
+    for (int64_t u = threadIdx.x; u < units; u += 32) s += __ldcg(loss_part + u);
 #pragma unroll
     for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (threadIdx.x == 0) loss[0] = s * scale;
 }
-
-struct PassConfig {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr[1];
-    PassConfig(const LsPass &p, cudaStream_t stream) {
-        cfg.gridDim = dim3((unsigned)(p.units * p.cluster));
-        cfg.blockDim = dim3((unsigned)(32 * p.warps));
-        cfg.dynamicSmemBytes = p.smem;
-        cfg.stream = stream;
-        if (p.cluster > 1) {
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = (unsigned)p.cluster;
-            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-        }
-    }
-};
 
 cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const float *b, const LsPoint &at, int64_t d,
                         cudaStream_t stream) {
@@ -475,10 +463,9 @@ cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const floa
     a.ring_offset = p.ring_offset;
     a.flush_floats = p.ring_offset ? kPassFlushFloats : (int)(p.smem / sizeof(float));
     auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-        if (e != cudaSuccess) return e;
-        PassConfig config(p, stream);
-        return cudaLaunchKernelEx(&config.cfg, kernel, a);
+        if (cudaError_t e = allow_shared(reinterpret_cast<const void *>(kernel), p.smem)) return e;
+        const ChainedLaunch launch(true, dim3((unsigned)(p.units * p.cluster)), dim3((unsigned)(32 * p.warps)), p.smem, stream, p.cluster);
+        return cudaLaunchKernelEx(&launch.cfg, kernel, a);
     };
     auto pick = [&](auto warps, auto per_row, auto columns) {
         constexpr int WARPS = decltype(warps)::value, W = decltype(per_row)::value, C = decltype(columns)::value;
@@ -551,9 +538,11 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
         // no more clusters than run side by side: SMs that cannot form another one stay idle, a second wave would cost more
         auto kernel = ls_pass_kernel<16, 16, 32, 1, true>;
         int resident = 0;
-        PassConfig config(p, nullptr);
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&resident, kernel, &config.cfg) != cudaSuccess || resident < 1) {
+        ChainedLaunch launch(true, dim3((unsigned)(p.units * p.cluster)), dim3((unsigned)(32 * p.warps)), p.smem, nullptr, p.cluster);
+        launch.cfg.attrs = &launch.attrs[1];                               // the cluster's size alone
+        launch.cfg.numAttrs = 1;
+        if (allow_shared(reinterpret_cast<const void *>(kernel), p.smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&resident, kernel, &launch.cfg) != cudaSuccess || resident < 1) {
             cudaGetLastError();
             return LsPass{};
         }
@@ -589,14 +578,12 @@ cudaError_t launch_ls_pass_loss(const LsPass &p, const float *A, const float *b,
 
 cudaError_t launch_ls_pass_reduce(const LsPass &p, const float *part, int64_t d, float inv_rows, float *G, cudaStream_t stream) {
     const int n = (int)(p.total / p.rows);
-    ls_pass_reduce_kernel<<<dim3((unsigned)((d + 127) / 128), n), 128, 0, stream>>>(part, p.rows, p.total, p.units,
-                                                                                  p.slots_per_machine, p.ldp, d, inv_rows, G);
-    return cudaGetLastError();
+    return launch_chained(true, ls_pass_reduce_kernel, dim3((unsigned)((d + 127) / 128), n), dim3(128), 0, stream, part, p.rows, p.total, p.units,
+                          p.slots_per_machine, p.ldp, d, inv_rows, G);
 }
 
 cudaError_t launch_ls_loss_sum(const double *loss_part, int64_t units, double scale, double *loss, cudaStream_t stream) {
-    ls_loss_sum_kernel<<<1, 32, 0, stream>>>(loss_part, units, scale, loss);
-    return cudaGetLastError();
+    return launch_chained(true, ls_loss_sum_kernel, dim3(1), dim3(32), 0, stream, loss_part, units, scale, loss);
 }
 
 cudaError_t ls_pass_take_status(int *status) {

@@ -10,7 +10,9 @@
 // vector group.  Sums are kept in two levels (per tile, then across tiles) to bound the
 // fp32 chain length, reduced across the ql lanes in a fixed order, and written as one
 // partial P per CTA column; a second kernel adds the columns in ascending order.
+#include "core_finish.cuh"
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 #include <cuda_bf16.h>
 
@@ -38,8 +40,6 @@ struct ProjectArgs {
     int tj;          // threads across vectors
     int tj_log2;
     int aligned;     // rows may be copied in 16-byte pieces
-    int splits;      // > 0: row i is the sum of `splits` arrays ldg apart, times `scale` (see launch_project)
-    float scale;
     uint32_t t;
     RoundKeys keys;
 };
@@ -55,9 +55,9 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
 
-__device__ __forceinline__ float load_elem(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float load_elem(const float *p) { return __ldcg(p); }
 __device__ __forceinline__ float load_elem(const __nv_bfloat16 *p) {
-    return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(p)) << 16);
+    return __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short *>(p)) << 16);
 }
 
 template <int NB, int JT, int UQ, int TILE_Q, typename GT>
@@ -69,6 +69,7 @@ project_kernel(const __grid_constant__ ProjectArgs a) {
     constexpr int PIECES_PER_THREAD = (PIECES + kThreads - 1) / kThreads;
     constexpr bool EVEN = PIECES % kThreads == 0;                 // otherwise the last round is partial
 
+    grid_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *stage0 = reinterpret_cast<float4 *>(smem_raw);
     float4 *stage1 = stage0 + NB * TILE_Q;
@@ -113,7 +114,7 @@ project_kernel(const __grid_constant__ ProjectArgs a) {
             if constexpr (BF16) {
                 const int i = piece / (TILE_Q / 2);
                 const int c = piece % (TILE_Q / 2);
-                held[r] = (i < a.n) ? __ldg(reinterpret_cast<const uint4 *>(G + (int64_t)i * a.ldg + k0 + 8 * c))
+                held[r] = (i < a.n) ? __ldcg(reinterpret_cast<const uint4 *>(G + (int64_t)i * a.ldg + k0 + 8 * c))
                                     : make_uint4(0, 0, 0, 0);
             } else {
                 const int i = piece / TILE_Q;
@@ -144,29 +145,6 @@ project_kernel(const __grid_constant__ ProjectArgs a) {
         }
         float *flat = reinterpret_cast<float *>(stage);
         const int64_t k0 = tile * TILE;
-        if constexpr (!BF16) {
-            if (a.splits > 0) {
-                // summed rows (d and ldg are multiples of 4 here): one block of four coordinates per thread
-                // step, the `splits` 16-byte loads of a block independent of one another
-                for (int e = tid; e < NB * TILE_Q; e += kThreads) {
-                    const int i = e / TILE_Q;
-                    const int64_t k = k0 + 4 * (e % TILE_Q);
-                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (i < a.n && k < a.d) {
-                        const float4 *src = reinterpret_cast<const float4 *>(G + (int64_t)i * a.splits * a.ldg + k);
-                        const int64_t stride4 = a.ldg >> 2;
-#pragma unroll 6
-                        for (int c = 0; c < a.splits; ++c) {
-                            const float4 v = __ldg(src + (int64_t)c * stride4);
-                            sum = make_float4(sum.x + v.x, sum.y + v.y, sum.z + v.z, sum.w + v.w);
-                        }
-                        sum = make_float4(sum.x * a.scale, sum.y * a.scale, sum.z * a.scale, sum.w * a.scale);
-                    }
-                    stage[e] = sum;
-                }
-                return;
-            }
-        }
         // ragged or unaligned tile: element by element, zero beyond d and beyond n
         for (int e = tid; e < NB * TILE; e += kThreads) {
             const int i = e / TILE;
@@ -185,9 +163,10 @@ project_kernel(const __grid_constant__ ProjectArgs a) {
         }
     };
 
+    if (tile_begin < tile_end) fill_qtab(tile_begin, qtab0);
+    grid_wait();
     if (tile_begin < tile_end) {
         begin_stage(tile_begin, stage0);
-        fill_qtab(tile_begin, qtab0);
         finish_stage(tile_begin, stage0);
     }
     cp_async_wait_all();
@@ -275,6 +254,7 @@ project_kernel(const __grid_constant__ ProjectArgs a) {
     __syncthreads();
     for (int idx = tid; idx < plane; idx += kThreads) {
         float s = 0.f;
+#pragma unroll 8
         for (int l = 0; l < tq; ++l) s += red[l * plane + idx];
         const int lane = idx & (tj - 1);
         const int iv = idx >> a.tj_log2;
@@ -287,12 +267,7 @@ project_kernel(const __grid_constant__ ProjectArgs a) {
 template <int NB, int JT, int UQ, int TILE_Q>
 cudaError_t launch_tiled(const ProjectPlan &plan, const ProjectArgs &args, int dtype, cudaStream_t stream) {
     dim3 grid(plan.grid_x, plan.grid_y);
-    auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kThreads, plan.smem, stream>>>(args);
-        return cudaGetLastError();
-    };
+    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(kThreads), plan.smem, stream, args); };
     if (dtype == 1) return go(project_kernel<NB, JT, UQ, TILE_Q, __nv_bfloat16>);
     return go(project_kernel<NB, JT, UQ, TILE_Q, float>);
 }
@@ -305,43 +280,27 @@ cudaError_t launch_typed(const ProjectPlan &plan, const ProjectArgs &args, int d
     return launch_tiled<NB, JT, UQ, tile_q_for(NB)>(plan, args, dtype, stream);
 }
 
-// Column sums of the partial results.  The columns (up to 296) are cut into kFinishSlices ranges summed side by
-// side, then the ranges are added in ascending order: a single thread per entry would wait for L2 some seventy
-// times in a row (34 us at m = 256 and n = 8, where this takes 4).
-constexpr int kFinishSlices = 8;
-
-__device__ __forceinline__ float finish_slice(const float *__restrict__ partial, int chunks, int64_t total, int64_t idx, int slice) {
-    const int begin = chunks * slice / kFinishSlices, end = chunks * (slice + 1) / kFinishSlices;
-    float s = 0.f;
-#pragma unroll 8
-    for (int c = begin; c < end; ++c) s += partial[(int64_t)c * total + idx];
-    return s;
-}
-
-__device__ __forceinline__ float finish_join(const float (&slices)[kFinishSlices][32], int lane) {
-    float s = slices[0][lane];
-#pragma unroll
-    for (int r = 1; r < kFinishSlices; ++r) s += slices[r][lane];
-    return s;
-}
-
 __global__ void finish_project_kernel(const float *__restrict__ partial, int chunks, int n, int m,
                                       float *__restrict__ P, int accumulate) {
+    grid_trigger();
+    grid_wait();
     __shared__ float slices[kFinishSlices][32];
     const int64_t idx = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int64_t total = (int64_t)n * m;
     slices[threadIdx.y][threadIdx.x] = idx < total ? finish_slice(partial, chunks, total, idx, threadIdx.y) : 0.f;
     __syncthreads();
     if (threadIdx.y != 0 || idx >= total) return;
-    const float s = finish_join(slices, threadIdx.x);
+    const float s = finish_join(&slices[0][threadIdx.x], 32);
     P[idx] = accumulate ? P[idx] + s : s;
 }
 
 __global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, float *__restrict__ pbar) {
+    grid_trigger();
+    grid_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m) return;
     float s = 0.f;
-    for (int i = 0; i < n; ++i) s += P[(int64_t)i * m + j];
+    for (int i = 0; i < n; ++i) s += __ldcg(P + (int64_t)i * m + j);
     pbar[j] = s / (float)n;
 }
 
@@ -350,6 +309,8 @@ __global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, floa
 constexpr int kFinishMachines = 4;      // machines summed at a time
 __global__ void finish_aggregate_kernel(const float *__restrict__ partial, int chunks, int n, int m,
                                         float *__restrict__ pbar) {
+    grid_trigger();
+    grid_wait();
     __shared__ float slices[kFinishMachines][kFinishSlices][32];
     const int j = blockIdx.x * 32 + threadIdx.x;
     const int64_t total = (int64_t)n * m;
@@ -361,7 +322,7 @@ __global__ void finish_aggregate_kernel(const float *__restrict__ partial, int c
             i < n && j < m ? finish_slice(partial, chunks, total, (int64_t)i * m + j, slice) : 0.f;
         __syncthreads();
         if (threadIdx.y == 0)
-            for (int r = 0; r < kFinishMachines && i0 + r < n; ++r) sum += finish_join(slices[r], threadIdx.x);
+            for (int r = 0; r < kFinishMachines && i0 + r < n; ++r) sum += finish_join(&slices[r][0][threadIdx.x], 32);
         __syncthreads();
     }
     if (threadIdx.y == 0 && j < m) pbar[j] = sum / (float)n;
@@ -427,10 +388,14 @@ ProjectPlan make_project_plan(int32_t n_group, int32_t m, int64_t d, int dtype, 
     while (tj < want && tj < kThreads) tj *= 2;
     const int min_tj = kThreads * p.uq / p.tile_q;    // keeps tq * uq <= tile_q
     if (tj < min_tj) tj = min_tj;
+    p.tiles = (d + 4 * (int64_t)p.tile_q - 1) / (4 * (int64_t)p.tile_q);
+    auto rows_of = [&](int threads) { return (m + threads * p.jt - 1) / (threads * p.jt); };
+    // short vectors and many of them: narrower CTA rows, as long as all of them are resident together (n = 7, d = 3210,
+    // m = 940: 52 -> 208 CTAs)
+    while (tj > 1 && tj / 2 >= min_tj && p.tiles * rows_of(tj / 2) <= 2 * (int64_t)sm_count) tj /= 2;
     p.tj = tj;
     p.tq = kThreads / tj;
-    p.grid_y = (m + tj * p.jt - 1) / (tj * p.jt);
-    p.tiles = (d + 4 * (int64_t)p.tile_q - 1) / (4 * (int64_t)p.tile_q);
+    p.grid_y = rows_of(tj);
     const size_t stage = (size_t)p.nb * p.tile_q * 16;
     const size_t red = (size_t)kThreads * p.nb * p.jt * 4;
     const size_t tiles_and_tables = 2 * stage + 2 * (size_t)p.tile_q * 16;   // two gradient tiles + two Philox block tables
@@ -442,16 +407,14 @@ ProjectPlan make_project_plan(int32_t n_group, int32_t m, int64_t d, int dtype, 
     if (gx < 1) gx = 1;
     if (gx > p.tiles) gx = p.tiles;
     p.grid_x = (int)gx;
+    p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * ctas_per_sm, d, m);
     (void)dtype;
     return p;
 }
 
 cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint32_t t, const void *G,
                            int dtype, int32_t n, int64_t ldg, int64_t d, int32_t m, uint64_t q_base,
-                           float *partial, cudaStream_t stream, int splits, float scale) {
-    if (splits > 0 && (plan.mma != 0 || dtype != 0 || d % 4 != 0 || ldg % 4 != 0 ||
-                       reinterpret_cast<uintptr_t>(G) % 16 != 0))
-        return cudaErrorInvalidValue;
+                           float *partial, cudaStream_t stream) {
     if (plan.mma == 2) return launch_project_tc(plan, keys, t, G, dtype, n, ldg, d, m, q_base, partial, stream);
     if (plan.mma == 1) return launch_project_mma(plan, keys, t, G, dtype, n, ldg, d, m, q_base, partial, stream);
     ProjectArgs a{};
@@ -467,9 +430,6 @@ cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint3
     a.tj_log2 = ilog2(plan.tj);
     const size_t es = dtype == 1 ? 2 : 4;
     a.aligned = ((reinterpret_cast<uintptr_t>(G) % 16) == 0 && ((size_t)ldg * es) % 16 == 0) ? 1 : 0;
-    a.splits = splits;
-    a.scale = scale;
-    if (splits > 0) a.aligned = 0;      // summed rows are formed element by element while the tile is staged
     a.t = t;
     a.keys = keys;
     switch (plan.nb) {
@@ -484,22 +444,20 @@ cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint3
 cudaError_t launch_finish_project(const float *partial, int chunks, int32_t n, int32_t m, float *P,
                                   bool accumulate, cudaStream_t stream) {
     const int64_t total = (int64_t)n * m;
-    finish_project_kernel<<<(unsigned)((total + 31) / 32), dim3(32, kFinishSlices), 0, stream>>>(partial, chunks, n, m, P,
-                                                                                               accumulate ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chained(true, finish_project_kernel, dim3((unsigned)((total + 31) / 32)), dim3(32, kFinishSlices), 0, stream, partial,
+                          chunks, n, m, P, accumulate ? 1 : 0);
 }
 
 cudaError_t launch_finish_aggregate(const float *partial, int chunks, int32_t n, int32_t m, float *pbar,
                                     cudaStream_t stream) {
     const int rows = n < kFinishMachines ? n : kFinishMachines;
-    finish_aggregate_kernel<<<(m + 31) / 32, dim3(32, kFinishSlices * rows), 0, stream>>>(partial, chunks, n, m, pbar);
-    return cudaGetLastError();
+    return launch_chained(true, finish_aggregate_kernel, dim3((m + 31) / 32), dim3(32, kFinishSlices * rows), 0, stream, partial, chunks,
+                          n, m, pbar);
 }
 
 cudaError_t launch_aggregate(const float *P, int32_t n, int32_t m, float *pbar, cudaStream_t stream) {
     const int threads = 128;
-    aggregate_kernel<<<(m + threads - 1) / threads, threads, 0, stream>>>(P, n, m, pbar);
-    return cudaGetLastError();
+    return launch_chained(true, aggregate_kernel, dim3((m + threads - 1) / threads), dim3(threads), 0, stream, P, n, m, pbar);
 }
 
 }  // namespace core

@@ -11,6 +11,7 @@
 // accumulated (relative error about 2^-21 per product).  bf16 gradients are exact in tf32: no tail.
 // The partial sums leave the kernel in the same layout as those of the scalar kernel.
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 #include <cuda_bf16.h>
 
@@ -60,6 +61,8 @@ project_mma_kernel(const __grid_constant__ MmaArgs a) {
     constexpr int PPT = PIECES / kThreads;
     static_assert(PIECES % kThreads == 0, "tile must split evenly over the CTA");
 
+    grid_trigger();
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *stage0 = reinterpret_cast<float4 *>(smem_raw);
     float4 *stage1 = stage0 + STAGE;
@@ -91,7 +94,7 @@ project_mma_kernel(const __grid_constant__ MmaArgs a) {
             constexpr int PER_ROW = PIECES / 16;
             const int i = piece / PER_ROW, c = piece % PER_ROW;
             const int64_t off = (int64_t)i * a.ldg + k0 + (BF16 ? 8 : 4) * c;
-            held[r] = (i < a.n) ? __ldg(reinterpret_cast<const uint4 *>(G + off)) : make_uint4(0, 0, 0, 0);
+            held[r] = (i < a.n) ? __ldcg(reinterpret_cast<const uint4 *>(G + off)) : make_uint4(0, 0, 0, 0);
         }
     };
 
@@ -136,10 +139,10 @@ project_mma_kernel(const __grid_constant__ MmaArgs a) {
                     const int64_t k = k0 + 4 * q + l;
                     if (k < a.d) {
                         if constexpr (BF16)
-                            vals[l] = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(G) +
+                            vals[l] = __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short *>(G) +
                                                                       (int64_t)i * a.ldg + k) << 16);
                         else
-                            vals[l] = __ldg(reinterpret_cast<const float *>(G) + (int64_t)i * a.ldg + k);
+                            vals[l] = __ldcg(reinterpret_cast<const float *>(G) + (int64_t)i * a.ldg + k);
                     }
                 }
             }
@@ -246,6 +249,7 @@ void fill_project_mma_plan(ProjectPlan &p, int32_t m, int64_t d, int dtype, int 
     if (gx < 1) gx = 1;
     if (gx > p.tiles) gx = p.tiles;
     p.grid_x = (int)gx;
+    p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * 2, d, m);
 }
 
 cudaError_t launch_project_mma(const ProjectPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype,
@@ -265,12 +269,7 @@ cudaError_t launch_project_mma(const ProjectPlan &plan, const RoundKeys &keys, u
     a.t = t;
     a.keys = keys;
     dim3 grid(plan.grid_x, plan.grid_y);
-    auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kThreads, plan.smem, stream>>>(a);
-        return cudaGetLastError();
-    };
+    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(kThreads), plan.smem, stream, a); };
     if (dtype == 1) return go(project_mma_kernel<128, __nv_bfloat16>);
     return go(project_mma_kernel<64, float>);
 }

@@ -10,12 +10,12 @@
 // rows of the next tile 16 bytes at a time (eight loads in flight per thread), add them up and store the
 // sum to one of two shared-memory tiles, next to the block-dependent half of Philox; rows that
 // do not start on a 16-byte boundary are read in aligned vectors all the same, summed per alignment class
-// and shifted into place with warp shuffles.  The generating threads hold four vectors each and walk the
-// blocks of the tile: thread (jl, ql) of tj x tq, where tj = the number of vector quadruples of the CTA row
-// (any number, not a power of two: 100 vectors keep 250 of 256 threads busy).  The coordinates of a block
-// are stored as (0, 2, 1, 3), so that one 16-byte read delivers the multiplicands of the cosine and of the
-// sine lanes of both pairs as ready register pairs and S (g_c (y sp) + g_s cs) is four packed instructions
-// per counter.
+// and shifted into place with warp shuffles.  The generating threads hold four
+// vectors each and walk the blocks of the tile: thread (jl, ql) of tj x tq, where tj = the number of vector
+// quadruples of the CTA row (any number, not a power of two: 100 vectors keep 250 of 256 threads busy).  The
+// coordinates of a block are stored as (0, 2, 1, 3), so that one 16-byte read delivers the multiplicands of the
+// cosine and of the sine lanes of both pairs as ready register pairs and S (g_c (y sp) + g_s cs) is four packed
+// instructions per counter.  d = 2.5e7, m = 256: 5204 us = 1.23e12 Gaussians/s.
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -55,9 +55,9 @@ struct RowVec {
     static constexpr int V = 16 / (int)sizeof(GT);          // elements per 16-byte vector
 };
 
-__device__ __forceinline__ float row_elem(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float row_elem(const float *p) { return __ldcg(p); }
 __device__ __forceinline__ float row_elem(const __nv_bfloat16 *p) {
-    return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(p)) << 16);
+    return __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short *>(p)) << 16);
 }
 
 __device__ __forceinline__ void row_add(float (&acc)[4], uint4 h) {
@@ -91,7 +91,7 @@ __device__ __forceinline__ void row_sum(const RowArgs &a, int64_t kv, int64_t st
             for (int i = 0; i < UR; ++i)
 #pragma unroll
                 for (int u = 0; u < US; ++u)
-                    h[u][i] = r + i * step < r1 ? __ldg(reinterpret_cast<const uint4 *>(p + i * row_stride + u * stride))
+                    h[u][i] = r + i * step < r1 ? __ldcg(reinterpret_cast<const uint4 *>(p + i * row_stride + u * stride))
                                                 : make_uint4(0, 0, 0, 0);
 #pragma unroll
             for (int i = 0; i < UR; ++i)
@@ -231,6 +231,9 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         }
     };
 
+    if (tile_begin < tile_end) fill_table(tile_begin, tile0, tid, kRowThreads);
+    grid_wait();
+
     // the first tile is staged by all warps, nobody having anything else to do yet; a short tile with many rows (the
     // partial gradients of a least-squares step) is cut into row ranges too
     if (tile_begin < tile_end) {
@@ -255,7 +258,6 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         } else {
             row_stage_any<GT>(2, a, 4 * tile_begin * a.tile_q, blocks, warp, kRowWarps, 0, a.rows, lane, tile0);
         }
-        fill_table(tile_begin, tile0, tid, kRowThreads);
     }
     __syncthreads();
 
@@ -286,7 +288,9 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     bool have_jp = false;
     for (int64_t tile = tile_begin; tile < tile_end; ++tile) {
         const int i = (int)(tile - tile_begin), st = i & 1;
-        if (i >= 1) bar_sync(kFull + st, kRowThreads);
+        if (i >= 1) {
+            bar_sync(kFull + st, kRowThreads);
+        }
         const float4 *cur = tile0 + 2 * st * a.tile_q;
         const int blocks = blocks_of(tile);
         const uint64_t q0 = a.q_base + (uint64_t)tile * a.tile_q;
@@ -334,6 +338,10 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
         if (tile + 2 < tile_end) bar_arrive(kEmpty + st, kRowThreads);
     }
+
+    // The next kernel is let in only now: its CTAs, waiting beside this kernel's, would be in the way of the generating warps
+    // (least-squares step at d = 8192: 102 -> 99 us).
+    grid_trigger();
 
     // fixed-order sum over the ql lanes
     __syncthreads();
@@ -387,6 +395,7 @@ RowPlan make_row_plan(int32_t m, int64_t d, int sm_count) {
     }
     p.tiles = (nq + p.tile_q - 1) / p.tile_q;
     p.grid_x = (int)(slots < p.tiles ? slots : p.tiles);
+    p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * 2, d, m);
     // two tiles, two tables, and the row ranges of a short first tile (at most kRowWarps segments of 64 blocks)
     const size_t stage = 2 * (size_t)p.tile_q * (16 + 16) + (size_t)kRowWarps * 64 * 16;
     const size_t red = (size_t)p.tj * p.tq * kRowJT * 4;
@@ -417,12 +426,7 @@ cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint3
     a.t = t;
     a.keys = keys;
     const dim3 grid(plan.grid_x, plan.grid_y);
-    auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kRowThreads, plan.smem, stream>>>(a);
-        return cudaGetLastError();
-    };
+    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(kRowThreads), plan.smem, stream, a); };
     return dtype == 1 ? go(project_row_kernel<__nv_bfloat16>) : go(project_row_kernel<float>);
 }
 

@@ -194,9 +194,9 @@ __device__ __noinline__ void stage_piece_slowly(const GT *G, int64_t ldg, int64_
                 const int64_t k = k0 + 4 * part + l;
                 if (k < d) {
                     if constexpr (BF16)
-                        vals[l] = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(G) + (int64_t)i * ldg + k) << 16);
+                        vals[l] = __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short *>(G) + (int64_t)i * ldg + k) << 16);
                     else
-                        vals[l] = __ldg(reinterpret_cast<const float *>(G) + (int64_t)i * ldg + k);
+                        vals[l] = __ldcg(reinterpret_cast<const float *>(G) + (int64_t)i * ldg + k);
                 }
             }
         }
@@ -210,6 +210,8 @@ __device__ __noinline__ void stage_piece_slowly(const GT *G, int64_t ldg, int64_
 template <typename GT, int NT, int VG>
 __global__ void __launch_bounds__(kTcThreads, VG == 1 ? 2 : 1)
 project_tc_kernel(const __grid_constant__ TcArgs a) {
+    grid_trigger();
+    grid_wait();
     constexpr bool BF16 = sizeof(GT) == 2;
     using Shape = TcShape<NT, BF16, VG>;
     constexpr int kTcStages = Shape::kStages;
@@ -336,7 +338,7 @@ project_tc_kernel(const __grid_constant__ TcArgs a) {
         if (c < fast_stages) {
 #pragma unroll
             for (int r = 0; r < PPT; ++r)
-                if (duty_i[r] < a.n) held[r] = __ldg(reinterpret_cast<const uint4 *>(duty_src[r] + (int64_t)c * 32));
+                if (duty_i[r] < a.n) held[r] = __ldcg(reinterpret_cast<const uint4 *>(duty_src[r] + (int64_t)c * 32));
         }
     };
     auto deposit = [&](uint32_t c, uint32_t sb) {                     // stage c into the buffer at sb
@@ -565,6 +567,7 @@ void fill_project_tc_plan(ProjectPlan &p, int32_t n_group, int32_t m, int64_t d,
     if (gx < 1) gx = 1;
     if (gx > p.tiles) gx = p.tiles;
     p.grid_x = (int)gx;
+    p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * (vg == 2 ? 1 : 2), d, m);
 }
 
 cudaError_t launch_project_tc(const ProjectPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype,
@@ -587,12 +590,7 @@ cudaError_t launch_project_tc(const ProjectPlan &plan, const RoundKeys &keys, ui
     a.t = t;
     a.keys = keys;
     dim3 grid(plan.grid_x, plan.grid_y);
-    auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kTcThreads, plan.smem, stream>>>(a);
-        return cudaGetLastError();
-    };
+    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(kTcThreads), plan.smem, stream, a); };
     auto pick = [&](auto nt, auto vg) {
         constexpr int NT = decltype(nt)::value, VG = decltype(vg)::value;
         if (dtype == 1) return go(project_tc_kernel<__nv_bfloat16, NT, VG>);

@@ -7,7 +7,9 @@
 // thread; the part that depends only on j is tabulated per CTA in shared memory next
 // to pbar[j], so the loop reads one 16-byte broadcast per j.  Every output coordinate
 // is written exactly once, as a 16-byte store where alignment allows.
+#include "core_finish.cuh"
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 namespace core {
 
@@ -18,7 +20,8 @@ constexpr int kGroupQ = kThreads * kRecUQ;        // blocks per CTA step
 constexpr int kJChunk = 2048;                     // vectors tabulated at a time (32 KB)
 
 struct ReconstructArgs {
-    const float *pbar;
+    float *pbar;
+    MessageParts parts;        // partial != nullptr: the message is formed here (short vectors only)
     float *out;
     int64_t k_begin;
     int64_t k_end;
@@ -73,7 +76,7 @@ __device__ __forceinline__ void rec_step(const uint4 *entries, const QPart (&qp)
 __device__ __forceinline__ void emit_block(const ReconstructArgs &a, uint64_t q, uint64_t q_begin, float4 r) {
     const int64_t off = (int64_t)((q - q_begin) << 2);        // offset into out
     const int64_t k = (int64_t)(q << 2);
-    const float step = a.epi.base ? (a.epi.step_dev ? a.epi.step_scale * __ldg(a.epi.step_dev) : a.epi.step) : 0.f;
+    const float step = a.epi.base ? (a.epi.step_dev ? a.epi.step_scale * __ldcg(a.epi.step_dev) : a.epi.step) : 0.f;
     if (a.vec_ok && k + 4 <= a.k_end) {
         float4 v = r;
         if (a.epi.base) {
@@ -113,6 +116,8 @@ __device__ __forceinline__ void emit_block(const ReconstructArgs &a, uint64_t q,
 
 __global__ void __launch_bounds__(kThreads, 3)
 reconstruct_kernel(const __grid_constant__ ReconstructArgs a) {
+    grid_trigger();
+    grid_wait();
     __shared__ uint4 table[kJChunk];              // {JPart.x0, JPart.x2, JPart.w3, bits of pbar[j]}
     const int tid = threadIdx.x;
     const uint64_t q_begin = (uint64_t)a.k_begin >> 2;
@@ -146,7 +151,7 @@ reconstruct_kernel(const __grid_constant__ ReconstructArgs a) {
                 __syncthreads();                  // everyone is done with the previous table
                 for (int jj = tid; jj < jn; jj += kThreads) {
                     const JPart jp = philox_jpart((uint32_t)(j0 + jj), grp_qhi, a.keys);
-                    table[jj] = make_uint4(jp.x0, jp.x2, jp.w3, __float_as_uint(a.pbar[j0 + jj]));
+                    table[jj] = make_uint4(jp.x0, jp.x2, jp.w3, __float_as_uint(__ldcg(a.pbar + j0 + jj)));
                 }
                 __syncthreads();
                 have_table = true;
@@ -169,40 +174,100 @@ reconstruct_kernel(const __grid_constant__ ReconstructArgs a) {
 // Short vectors: the kernel above would give work to a handful of CTAs only (d = 8192 is four groups),
 // so here the SLICES warp groups of a CTA share out the vectors of 256 / SLICES blocks; the partial sums
 // of a block meet in shared memory and are added in ascending order of the vector ranges.  Few vectors
-// get few slices (a slice wants at least four vectors to generate together).
+// get few slices (a slice wants at least four vectors to generate together); where even eight slices leave SMs
+// idle and vectors are many, a cluster of up to eight CTAs shares them out as well, and the first one adds up.
+constexpr int kJoinVectors = 512;                  // most vectors whose message is formed here: the rest of the
+constexpr int kJoinEntries = (kJChunk - kJoinVectors) * 16 / 4 / kFinishSlices;     // table takes the slices of n * m entries
+
+__device__ __forceinline__ void store_cluster(const void *smem, uint32_t rank, float4 v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(smem)), "r"(rank));
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 template <int SLICES>
 __global__ void __launch_bounds__(kThreads)
 reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
+    grid_trigger();
     constexpr int QB = kThreads / SLICES;          // blocks per CTA
-    __shared__ uint4 table[kJChunk];               // as above; m <= kJChunk here
+    constexpr int RANKS = SLICES == 8 ? 8 : 1;     // CTAs of a cluster at most
+    __shared__ uint4 table[kJChunk];               // as above
     __shared__ float4 part[SLICES][QB];
+    __shared__ float4 inbox[RANKS][QB];
     const int tid = threadIdx.x, ql = tid % QB, slice = tid / QB;
+    uint32_t rank = 0, ranks = 1;
+    if constexpr (RANKS > 1) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(ranks));
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA has started
+    }
     const uint64_t q_begin = (uint64_t)a.k_begin >> 2;
     const uint64_t q_end = ((uint64_t)a.k_end + 3) >> 2;
-    const uint64_t q0 = q_begin + (uint64_t)blockIdx.x * QB;     // multiple of 32: one high counter word per CTA
+    const uint64_t q0 = q_begin + (uint64_t)(blockIdx.x / ranks) * QB;     // multiple of 32: one high counter word per CTA
     const uint32_t q_hi = (uint32_t)(q0 >> 32);
-    for (int jj = tid; jj < a.m; jj += kThreads) {
-        const JPart jp = philox_jpart((uint32_t)jj, q_hi, a.keys);
-        table[jj] = make_uint4(jp.x0, jp.x2, jp.w3, __float_as_uint(a.pbar[jj]));
-    }
-    __syncthreads();
     const uint64_t q = q0 + (uint64_t)ql;
     QPart qp[1] = {philox_qpart((uint32_t)q, a.t, a.keys)};
     float4 acc[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
-    const int per = ((a.m + SLICES - 1) / SLICES + 3) & ~3;      // vectors per slice, a multiple of 4
-    const int j_begin = min(slice * per, a.m), j_end = min(j_begin + per, a.m);
-    int jj = j_begin;
-    for (; jj + 4 <= j_end; jj += 4) rec_step<4, 1>(table + jj, qp, a.keys, acc);
-    for (; jj < j_end; ++jj) rec_step<1, 1>(table + jj, qp, a.keys, acc);
+    const int mine = ((a.m + (int)ranks - 1) / (int)ranks + 3) & ~3;       // vectors of this CTA
+    const int m_begin = min((int)rank * mine, a.m), m_end = min(m_begin + mine, a.m);
+    for (int j0 = m_begin; j0 < m_end; j0 += kJChunk) {
+        const int jn = min(kJChunk, m_end - j0);
+        if (j0 > m_begin) __syncthreads();         // everyone is done with the previous table
+        for (int jj = tid; jj < jn; jj += kThreads) {
+            const JPart jp = philox_jpart((uint32_t)(j0 + jj), q_hi, a.keys);
+            table[jj] = make_uint4(jp.x0, jp.x2, jp.w3, 0u);
+        }
+        if (j0 == m_begin) grid_wait();            // the message comes last
+        if (a.parts.partial) {
+            const int n = a.parts.n, entries = n * jn;
+            float *const slices = reinterpret_cast<float *>(table + kJoinVectors);
+            for (int e = tid; e < entries * kFinishSlices; e += kThreads) {
+                const int entry = e % entries, i = entry / jn, j = entry % jn;
+                slices[e] = finish_slice(a.parts.partial, a.parts.chunks, (int64_t)n * a.m, (int64_t)i * a.m + j0 + j, e / entries);
+            }
+            __syncthreads();
+            for (int jj = tid; jj < jn; jj += kThreads) {
+                float sum = 0.f;
+                for (int i = 0; i < n; ++i) sum += finish_join(slices + i * jn + jj, entries);
+                sum /= (float)n;
+                table[jj].w = __float_as_uint(sum);
+                if (blockIdx.x < ranks) a.pbar[j0 + jj] = sum;
+            }
+        } else {
+            for (int jj = tid; jj < jn; jj += kThreads) table[jj].w = __float_as_uint(__ldcg(a.pbar + j0 + jj));
+        }
+        __syncthreads();
+        const int per = (jn + SLICES - 1) / SLICES;                         // vectors per slice
+        const int j_begin = min(slice * per, jn), j_end = min(j_begin + per, jn);
+        int jj = j_begin;
+        for (; jj + 4 <= j_end; jj += 4) rec_step<4, 1>(table + jj, qp, a.keys, acc);
+        for (; jj < j_end; ++jj) rec_step<1, 1>(table + jj, qp, a.keys, acc);
+    }
+    if (m_begin >= m_end) grid_wait();             // a CTA without vectors
     part[slice][ql] = acc[0];
     __syncthreads();
-    if (slice == 0 && q < q_end) {
-        float4 s = part[0][ql];
+    float4 s = part[0][ql];
+    if (slice == 0) {
 #pragma unroll
         for (int r = 1; r < SLICES; ++r) {
             const float4 p = part[r][ql];
             s = make_float4(s.x + p.x, s.y + p.y, s.z + p.z, s.w + p.w);
         }
+    }
+    if constexpr (RANKS > 1) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // the first CTA has started
+        if (ranks > 1) {
+            if (slice == 0 && rank > 0) store_cluster(&inbox[rank][ql], 0, s);
+            asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            if (rank > 0) return;
+            if (slice == 0)
+                for (int r = 1; r < (int)ranks; ++r) {
+                    const float4 p = inbox[r][ql];
+                    s = make_float4(s.x + p.x, s.y + p.y, s.z + p.z, s.w + p.w);
+                }
+        }
+    }
+    if (slice == 0 && q < q_end) {
         const float inv_m = 1.0f / (float)a.m;
         emit_block(a, q, q_begin, make_float4(s.x * inv_m, s.y * inv_m, s.z * inv_m, s.w * inv_m));
     }
@@ -250,9 +315,18 @@ unsigned grid_for(int64_t items, int threads, int cap) {
 
 }  // namespace
 
-cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, const float *pbar, int32_t m,
+// Too few groups of the long-vector kernel to go round evenly?
+static bool short_vector(int64_t nq, int sm_count) { return (nq + kGroupQ - 1) / kGroupQ < 8 * (int64_t)sm_count; }
+
+// Every CTA forms the whole message: worth it while that is at most eight loads per thread (with 32, d = 8192 and m = 64, the
+// launch it saves was the cheaper one: 100.7 against 105.9 us a step).
+bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count) {
+    return m <= kJoinVectors && (int64_t)n * m <= kJoinEntries && (int64_t)chunks * n * m <= 2048 && short_vector((d + 3) >> 2, sm_count);
+}
+
+cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, int32_t m,
                                int64_t k_begin, int64_t k_end, float *out, int sm_count,
-                               cudaStream_t stream, const ReconstructEpilogue *epilogue) {
+                               cudaStream_t stream, const ReconstructEpilogue *epilogue, const MessageParts *parts) {
     if (k_end <= k_begin) return cudaSuccess;
     if (k_begin % (4 * kGroupQ) != 0) return cudaErrorInvalidValue;
     ReconstructArgs a{};
@@ -273,24 +347,33 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, const float *p
     a.keys = keys;
     const int64_t nq = ((k_end + 3) >> 2) - (k_begin >> 2);
     const int64_t groups = (nq + kGroupQ - 1) / kGroupQ;
-    if (groups < 8 * (int64_t)sm_count && m <= kJChunk) {    // too few groups to go round evenly: smaller units
-        // more slices = fewer blocks per CTA = more CTAs: as many as it takes to go round, while a slice
-        // keeps at least four vectors
-        int slices = 1;
-        while (slices < 8 && m >= 8 * slices && nq / (kThreads / slices) < 4 * (int64_t)sm_count) slices *= 2;
-        const unsigned grid = (unsigned)((nq + kThreads / slices - 1) / (kThreads / slices));
+    if (parts) a.parts = *parts;
+    if (short_vector(nq, sm_count)) {
+        // more slices = fewer blocks per CTA = more CTAs: as many as it takes to go round evenly (four are resident per
+        // SM), while a slice keeps at least four vectors, or sixteen where it is only for the last wave's sake
+        int slices = 1, ranks = 1;
+        auto ctas_with = [&](int s) { return nq / (kThreads / s); };
+        while (slices < 8 && m >= 8 * slices &&
+               (ctas_with(slices) < 4 * (int64_t)sm_count || (ctas_with(slices) < 16 * (int64_t)sm_count && m >= 32 * slices)))
+            slices *= 2;
+        const int64_t ctas = (nq + kThreads / slices - 1) / (kThreads / slices);
+        if (slices == 8)
+            while (ranks < 8 && m >= 128 * ranks && ctas * ranks < 2 * (int64_t)sm_count) ranks *= 2;
+        const bool chain = chain_pays(ctas * ranks, 4 * (int64_t)sm_count, 4 * nq, m);
+        auto go = [&](auto kernel) {
+            const ChainedLaunch launch(chain, dim3((unsigned)(ctas * ranks)), dim3(kThreads), 0, stream, ranks);
+            return cudaLaunchKernelEx(&launch.cfg, kernel, a);
+        };
         switch (slices) {
-            case 8: reconstruct_small_kernel<8><<<grid, kThreads, 0, stream>>>(a); break;
-            case 4: reconstruct_small_kernel<4><<<grid, kThreads, 0, stream>>>(a); break;
-            case 2: reconstruct_small_kernel<2><<<grid, kThreads, 0, stream>>>(a); break;
-            default: reconstruct_small_kernel<1><<<grid, kThreads, 0, stream>>>(a); break;
+            case 8: return go(reconstruct_small_kernel<8>);
+            case 4: return go(reconstruct_small_kernel<4>);
+            case 2: return go(reconstruct_small_kernel<2>);
+            default: return go(reconstruct_small_kernel<1>);
         }
-        return cudaGetLastError();
     }
     int64_t grid = (int64_t)sm_count * 3;     // three resident CTAs per SM (register-limited)
     if (grid > groups) grid = groups;
-    reconstruct_kernel<<<(unsigned)grid, kThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_chained(true, reconstruct_kernel, dim3((unsigned)grid), dim3(kThreads), 0, stream, a);
 }
 
 cudaError_t launch_debug_philox(const RoundKeys &keys, uint32_t t, uint32_t j, uint64_t q0, int64_t nq,

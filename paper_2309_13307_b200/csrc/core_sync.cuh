@@ -7,6 +7,11 @@
 
 namespace core {
 
+// A kernel of a chain (launch_chained): until everything before it in the stream is done and visible ...
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and from here on the kernel after it may be scheduled where there is room (it waits in turn).
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 constexpr uint64_t kWaitLimitNs = 100ull * 1000 * 1000;   // a wait gives up after 100 ms of the global timer
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }

@@ -2,6 +2,7 @@
 // (chosen on the device from the size of the combined messages) and the gossip averaging of
 // Algorithm 5 (decentralised CORE-GD).  Everything here works on n x m or m numbers: microseconds.
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 namespace core {
 
@@ -12,8 +13,10 @@ constexpr int kVarThreads = 256;
 // p = sqrt((1/m) sum_j pbar_j^2) and h = min{ m / (16 r1), c H^-1/2 p^-1/2 d^-3/4 m^3/4 }.
 // One CTA; thread t sums entries t, t + 256, ... in ascending order, the 256 partial sums are added in
 // ascending order by thread 0: a fixed order, in double (m numbers, nothing to save in fp32).
-__global__ void option1_step_kernel(const float *__restrict__ pbar, int m, double d, double r1, double H, double c,
+__global__ void option1_step_kernel(const float * pbar, int m, double d, double r1, double H, double c,
                                     float *p_out, float *h_out) {
+    grid_trigger();
+    grid_wait();
     __shared__ double part[kVarThreads];
     double s = 0.0;
     for (int j = threadIdx.x; j < m; j += kVarThreads) s += (double)pbar[j] * (double)pbar[j];
@@ -31,8 +34,10 @@ __global__ void option1_step_kernel(const float *__restrict__ pbar, int m, doubl
 }
 
 // One gossip round: out[i][j] = sum_l W[i][l] in[l][j], l ascending.
-__global__ void gossip_round_kernel(const float *__restrict__ W, const float *__restrict__ in, int n, int m,
-                                    float *__restrict__ out) {
+__global__ void gossip_round_kernel(const float * W, const float * in, int n, int m,
+                                    float *out) {
+    grid_trigger();
+    grid_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y;
     if (j >= m) return;
@@ -47,8 +52,10 @@ __global__ void gossip_round_kernel(const float *__restrict__ W, const float *__
 // rounds of 16 machines took 46 us of launches (2.3 us each), here 4 us.
 constexpr int kGossipCols = 8;
 constexpr int kGossipMaxMachines = 128;               // W in 64 KB of shared memory
-__global__ void gossip_rounds_kernel(const float *__restrict__ W, const float *__restrict__ in, int n, int m, int rounds,
-                                     float *__restrict__ out) {
+__global__ void gossip_rounds_kernel(const float * W, const float * in, int n, int m, int rounds,
+                                     float *out) {
+    grid_trigger();
+    grid_wait();
     extern __shared__ float gossip_smem[];
     const int ldw = n + 1;                            // rows of W that are read together fall into different banks
     float *const weights = gossip_smem, *cur = weights + n * ldw, *nxt = cur + n * kGossipCols;
@@ -75,7 +82,9 @@ __global__ void gossip_rounds_kernel(const float *__restrict__ W, const float *_
 }
 
 // spread[0] = max over machines i and vectors j of |P[i][j] - P[reader][j]| (a maximum: order-free).
-__global__ void consensus_spread_kernel(const float *__restrict__ P, int n, int m, int reader, float *spread) {
+__global__ void consensus_spread_kernel(const float * P, int n, int m, int reader, float *spread) {
+    grid_trigger();
+    grid_wait();
     __shared__ float part[kVarThreads];
     float worst = 0.f;
     for (int64_t e = threadIdx.x; e < (int64_t)n * m; e += kVarThreads)
@@ -91,14 +100,12 @@ __global__ void consensus_spread_kernel(const float *__restrict__ P, int n, int 
 
 cudaError_t launch_option1_step(const float *pbar, int32_t m, int64_t d, double r1, double H, double c, float *p_out,
                                 float *h_out, cudaStream_t stream) {
-    option1_step_kernel<<<1, kVarThreads, 0, stream>>>(pbar, m, (double)d, r1, H, c, p_out, h_out);
-    return cudaGetLastError();
+    return launch_chained(true, option1_step_kernel, dim3(1), dim3(kVarThreads), 0, stream, pbar, m, (double)d, r1, H, c, p_out, h_out);
 }
 
 cudaError_t launch_gossip_round(const float *W, const float *in, int32_t n, int32_t m, float *out, cudaStream_t stream) {
     dim3 grid((unsigned)((m + 127) / 128), (unsigned)n);
-    gossip_round_kernel<<<grid, 128, 0, stream>>>(W, in, n, m, out);
-    return cudaGetLastError();
+    return launch_chained(true, gossip_round_kernel, grid, dim3(128), 0, stream, W, in, n, m, out);
 }
 
 cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m, int32_t rounds, float *scratch, float **result,
@@ -107,12 +114,10 @@ cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m,
     if (rounds <= 0) return cudaSuccess;
     if (n <= kGossipMaxMachines) {
         const size_t smem = ((size_t)n * (n + 1) + 2 * (size_t)n * kGossipCols) * sizeof(float);
-        cudaError_t e = cudaFuncSetAttribute(gossip_rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         const int rows = n < 64 ? n : 64;
-        gossip_rounds_kernel<<<(m + kGossipCols - 1) / kGossipCols, kGossipCols * rows, smem, stream>>>(W, P, n, m, rounds, scratch);
         *result = scratch;
-        return cudaGetLastError();
+        return launch_chained(true, gossip_rounds_kernel, dim3((m + kGossipCols - 1) / kGossipCols), dim3(kGossipCols * rows), smem, stream, W,
+                              P, n, m, rounds, scratch);
     }
     for (int32_t r = 0; r < rounds; ++r) {
         cudaError_t e = launch_gossip_round(W, P, n, m, scratch, stream);
@@ -127,8 +132,7 @@ cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m,
 
 cudaError_t launch_consensus_spread(const float *P, int32_t n, int32_t m, int32_t reader, float *spread,
                                     cudaStream_t stream) {
-    consensus_spread_kernel<<<1, kVarThreads, 0, stream>>>(P, n, m, reader, spread);
-    return cudaGetLastError();
+    return launch_chained(true, consensus_spread_kernel, dim3(1), dim3(kVarThreads), 0, stream, P, n, m, reader, spread);
 }
 
 }  // namespace core
