@@ -10,7 +10,8 @@
 // rows of the next tile 16 bytes at a time (eight loads in flight per thread), add them up and store the
 // sum to one of two shared-memory tiles, next to the block-dependent half of Philox; rows that
 // do not start on a 16-byte boundary are read in aligned vectors all the same, summed per alignment class
-// and shifted into place with warp shuffles.  The generating threads hold four
+// and shifted into place with warp shuffles.  Where rows are many against the vectors, every warp stages and
+// then generates (TOGETHER), and the other CTA of the SM fills the gap.  The generating threads hold four
 // vectors each and walk the blocks of the tile: thread (jl, ql) of tj x tq, where tj = the number of vector
 // quadruples of the CTA row (any number, not a power of two: 100 vectors keep 250 of 256 threads busy).  The
 // coordinates of a block are stored as (0, 2, 1, 3), so that one 16-byte read delivers the multiplicands of the
@@ -208,7 +209,7 @@ __device__ __forceinline__ void row_stage_any(int stride, const RowArgs &a, int6
     }
 }
 
-template <typename GT>
+template <typename GT, bool TOGETHER>
 __global__ void __launch_bounds__(kRowThreads, 2)
 project_row_kernel(const __grid_constant__ RowArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -261,7 +262,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     }
     __syncthreads();
 
-    if (warp >= kRowCompute / 32) {
+    if (warp >= kRowCompute / 32 && !TOGETHER) {
         // staging warps: tile i into stage i & 1 once the generating warps have left it
         for (int64_t tile = tile_begin + 1; tile < tile_end; ++tile) {
             const int i = (int)(tile - tile_begin), st = i & 1;
@@ -278,7 +279,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     }
 
     const int ql = tid / a.tj, jl = tid - ql * a.tj;
-    const bool active = ql < a.tq;
+    const bool active = ql < a.tq && tid < kRowCompute;      // (all warps are here where they stage together)
     const int jbase = blockIdx.y * a.tj * kRowJT;
     float outer[kRowJT];
     JPart jp[kRowJT];
@@ -287,9 +288,16 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     uint32_t jp_q_hi = 0;
     bool have_jp = false;
     for (int64_t tile = tile_begin; tile < tile_end; ++tile) {
-        const int i = (int)(tile - tile_begin), st = i & 1;
+        const int i = (int)(tile - tile_begin), st = TOGETHER ? 0 : i & 1;
         if (i >= 1) {
-            bar_sync(kFull + st, kRowThreads);
+            if constexpr (TOGETHER) {
+                __syncthreads();                             // everyone is done with the tile
+                row_stage_any<GT>(2, a, 4 * tile * a.tile_q, blocks_of(tile), warp, kRowWarps, 0, a.rows, lane, tile0);
+                fill_table(tile, tile0, tid, kRowThreads);
+                __syncthreads();
+            } else {
+                bar_sync(kFull + st, kRowThreads);
+            }
         }
         const float4 *cur = tile0 + 2 * st * a.tile_q;
         const int blocks = blocks_of(tile);
@@ -336,7 +344,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         }
 #pragma unroll
         for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
-        if (tile + 2 < tile_end) bar_arrive(kEmpty + st, kRowThreads);
+        if (!TOGETHER && tile + 2 < tile_end) bar_arrive(kEmpty + st, kRowThreads);
     }
 
     // The next kernel is let in only now: its CTAs, waiting beside this kernel's, would be in the way of the generating warps
@@ -427,7 +435,12 @@ cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint3
     a.keys = keys;
     const dim3 grid(plan.grid_x, plan.grid_y);
     auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(kRowThreads), plan.smem, stream, a); };
-    return dtype == 1 ? go(project_row_kernel<__nv_bfloat16>) : go(project_row_kernel<float>);
+    // Staging a row of a block costs more where rows have to be shifted into place; where rows are many against the
+    // vectors two staging warps cannot keep up and all warps stage (us, two warps -> all: n = 8, m = 8: 451 -> 375;
+    // n = 50, m = 21: 961 -> 728; unaligned n = 5, m = 8: 798 -> 484; but n = 32, m = 100: 1709 -> 1770).
+    const bool together = (int64_t)rows * (a.aligned ? 3 : 7) >= m;
+    if (dtype == 1) return together ? go(project_row_kernel<__nv_bfloat16, true>) : go(project_row_kernel<__nv_bfloat16, false>);
+    return together ? go(project_row_kernel<float, true>) : go(project_row_kernel<float, false>);
 }
 
 }  // namespace core
