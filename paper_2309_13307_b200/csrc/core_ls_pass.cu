@@ -194,6 +194,16 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     };
     constexpr int stride = 32 * W, CB = C < 4 ? C : 4;             // CB columns are tested for together
     const int first = lane + 32 * wg;
+    // The first rows on their way to L2 while the kernels before this one finish (to L2 only: whoever still writes A writes
+    // it there)
+    if (leader && !edge && a.cluster == 1)
+        for (int s = 0; s < a.slots; ++s) {
+            const int k = grp + s * GROUPS;
+            if (k >= chunks) break;
+            const uintptr_t from = (src + (int64_t)s * src_step) & ~(uintptr_t)15;
+            const uint32_t bytes = (uint32_t)min(R, nrows - first_row(k)) * row_bytes & ~15u;
+            if (bytes) bulk_prefetch(reinterpret_cast<const void *>(from), bytes);
+        }
     grid_wait();
     if (leader)
         for (int s = 0; s < a.slots; ++s)

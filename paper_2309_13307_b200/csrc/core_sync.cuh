@@ -69,6 +69,10 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
+// Asks for `bytes` (a multiple of 16, 16-byte aligned) to be brought into L2: a hint, nothing is read by the program.
+__device__ __forceinline__ void bulk_prefetch(const void *gmem_src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gmem_src), "r"(bytes) : "memory");
+}
 // `bytes` (a multiple of 16) from global to shared memory, both 16-byte aligned; completion is counted on `bar`.
 __device__ __forceinline__ void bulk_copy(uint32_t smem_dst, const void *gmem_src, uint32_t bytes, uint32_t bar, uint64_t policy) {
     asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(smem_dst),
