@@ -538,10 +538,10 @@ int32_t project_tc_max_group(int32_t m) { return tc_vector_groups(m) == 2 ? kTcM
 
 bool project_tc_applies(int32_t n_group, int32_t m) {
     // enough machines for the tensor core to pay (with five or more the multiply-adds of the scalar kernel cost
-    // more issue slots than this kernel's staging and hand-over), enough vectors to fill most of the 128 rows
-    // of the last CTA row
-    return n_group >= kTcMinMachines && n_group <= project_tc_max_group(m) && m >= 96 &&
-           (m % kTcVectors == 0 || m % kTcVectors >= 64 || m >= 1024);
+    // more issue slots than this kernel's staging and hand-over), and vectors that fill three quarters of the CTA rows
+    // (n = 30, m = 801: 94 -> 62 us a round against the warp-level kernel)
+    const int64_t rows = ((int64_t)m + kTcVectors - 1) / kTcVectors * kTcVectors;
+    return n_group >= kTcMinMachines && n_group <= project_tc_max_group(m) && (int64_t)m * 4 >= rows * 3;
 }
 
 template <int NT, int VG>
