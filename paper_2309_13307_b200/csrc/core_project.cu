@@ -306,26 +306,28 @@ __global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, floa
 
 // Both of the above in one launch for a single group of machines whose messages nobody asks for:
 // the same sums in the same order, so pbar is bitwise what the two kernels give.
-constexpr int kFinishMachines = 4;      // machines summed at a time
+// A CTA takes eight vectors, so that sixteen machines' slices are in flight together (32 vectors and four machines: 9.3 us
+// for 22 machines, 232 vectors).
+constexpr int kFinishMachines = 16;
+constexpr int kFinishVectors = 8;
 __global__ void finish_aggregate_kernel(const float *__restrict__ partial, int chunks, int n, int m,
                                         float *__restrict__ pbar) {
     grid_trigger();
     grid_wait();
-    __shared__ float slices[kFinishMachines][kFinishSlices][32];
-    const int j = blockIdx.x * 32 + threadIdx.x;
+    __shared__ float slices[kFinishMachines][kFinishSlices][kFinishVectors];
+    const int lane = threadIdx.x, slice = threadIdx.y, row = threadIdx.z;
+    const int j = blockIdx.x * kFinishVectors + lane;
     const int64_t total = (int64_t)n * m;
-    const int slice = threadIdx.y % kFinishSlices, row = threadIdx.y / kFinishSlices;
-    float sum = 0.f;                    // kept by the first 32 threads
+    float sum = 0.f;                    // kept by the first kFinishVectors threads
     for (int i0 = 0; i0 < n; i0 += kFinishMachines) {
         const int i = i0 + row;
-        slices[row][slice][threadIdx.x] =
-            i < n && j < m ? finish_slice(partial, chunks, total, (int64_t)i * m + j, slice) : 0.f;
+        slices[row][slice][lane] = i < n && j < m ? finish_slice(partial, chunks, total, (int64_t)i * m + j, slice) : 0.f;
         __syncthreads();
-        if (threadIdx.y == 0)
-            for (int r = 0; r < kFinishMachines && i0 + r < n; ++r) sum += finish_join(&slices[r][0][threadIdx.x], 32);
+        if (slice == 0 && row == 0)
+            for (int r = 0; r < kFinishMachines && i0 + r < n; ++r) sum += finish_join(&slices[r][0][lane], kFinishVectors);
         __syncthreads();
     }
-    if (threadIdx.y == 0 && j < m) pbar[j] = sum / (float)n;
+    if (slice == 0 && row == 0 && j < m) pbar[j] = sum / (float)n;
 }
 
 int ilog2(int x) {
@@ -451,8 +453,8 @@ cudaError_t launch_finish_project(const float *partial, int chunks, int32_t n, i
 cudaError_t launch_finish_aggregate(const float *partial, int chunks, int32_t n, int32_t m, float *pbar,
                                     cudaStream_t stream) {
     const int rows = n < kFinishMachines ? n : kFinishMachines;
-    return launch_chained(true, finish_aggregate_kernel, dim3((m + 31) / 32), dim3(32, kFinishSlices * rows), 0, stream, partial, chunks,
-                          n, m, pbar);
+    return launch_chained(true, finish_aggregate_kernel, dim3((m + kFinishVectors - 1) / kFinishVectors),
+                          dim3(kFinishVectors, kFinishSlices, rows), 0, stream, partial, chunks, n, m, pbar);
 }
 
 cudaError_t launch_aggregate(const float *P, int32_t n, int32_t m, float *pbar, cudaStream_t stream) {
