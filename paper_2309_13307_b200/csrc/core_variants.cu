@@ -9,6 +9,7 @@ namespace core {
 namespace {
 
 constexpr int kVarThreads = 256;
+constexpr int kSpreadThreads = 1024;
 
 // p = sqrt((1/m) sum_j pbar_j^2) and h = min{ m / (16 r1), c H^-1/2 p^-1/2 d^-3/4 m^3/4 }.
 // One CTA; thread t sums entries t, t + 256, ... in ascending order, the 256 partial sums are added in
@@ -48,29 +49,42 @@ __global__ void gossip_round_kernel(const float * W, const float * in, int n, in
 
 // All gossip rounds of a step in one launch: a column of the messages never meets another one, so a CTA takes
 // kGossipCols columns of all machines through every round in shared memory, W beside them.  Same products in the same
-// order as gossip_round_kernel, hence the same bits.  Bound by latency (n multiply-adds and a barrier per round): twenty
-// rounds of 16 machines took 46 us of launches (2.3 us each), here 4 us.
+// order as gossip_round_kernel (a zero weight on a zero row at the end changes nothing), hence the same bits.  Bound by
+// latency (n multiply-adds in a row and a barrier per round) and, with many machines, by reading shared memory: rows of W
+// and columns of the messages are read 16 bytes at a time, their strides odd multiples of 16 bytes so that the rows a warp
+// reads together fall into different banks.  Twenty rounds of 16 machines took 46 us of launches (2.3 us each).
 constexpr int kGossipCols = 8;
-constexpr int kGossipMaxMachines = 128;               // W in 64 KB of shared memory
-__global__ void gossip_rounds_kernel(const float * W, const float * in, int n, int m, int rounds,
-                                     float *out) {
+constexpr int kGossipMaxMachines = 128;               // W in 66 KB of shared memory
+__host__ __device__ constexpr int gossip_stride(int n) { return (((n + 3) / 4) | 1) * 4; }
+__global__ void gossip_rounds_kernel(const float *W, const float *in, int n, int m, int rounds, float *out) {
     grid_trigger();
     grid_wait();
-    extern __shared__ float gossip_smem[];
-    const int ldw = n + 1;                            // rows of W that are read together fall into different banks
-    float *const weights = gossip_smem, *cur = weights + n * ldw, *nxt = cur + n * kGossipCols;
-    const int tid = threadIdx.x, threads = blockDim.x;
-    const int col = tid % kGossipCols, j = blockIdx.x * kGossipCols + col;
-    for (int e = tid; e < n * n; e += threads) weights[(e / n) * ldw + e % n] = W[e];
-    for (int i = tid / kGossipCols; i < n; i += threads / kGossipCols)
-        cur[i * kGossipCols + col] = j < m ? in[(int64_t)i * m + j] : 0.f;
+    extern __shared__ __align__(16) float gossip_smem[];
+    const int ld = gossip_stride(n), n4 = (n + 3) / 4;
+    float *const weights = gossip_smem, *cur = weights + n * ld, *nxt = cur + kGossipCols * ld;    // W by rows, messages by columns
+    const int tid = threadIdx.x, threads = blockDim.x, step = threads / kGossipCols;
+    const int col = tid % kGossipCols, first = tid / kGossipCols, j = blockIdx.x * kGossipCols + col;
+    for (int i = tid / 32; i < n; i += threads / 32)
+        for (int l = tid % 32; l < ld; l += 32) weights[i * ld + l] = l < n ? W[(int64_t)i * n + l] : 0.f;
+    for (int i = first; i < ld; i += step) {
+        cur[col * ld + i] = i < n && j < m ? __ldcg(in + (int64_t)i * m + j) : 0.f;
+        nxt[col * ld + i] = 0.f;
+    }
     __syncthreads();
     for (int r = 0; r < rounds; ++r) {
-        for (int i = tid / kGossipCols; i < n; i += threads / kGossipCols) {
+        const float4 *const column = reinterpret_cast<const float4 *>(cur + col * ld);
+        for (int i = first; i < n; i += step) {
+            const float4 *const row = reinterpret_cast<const float4 *>(weights + i * ld);
             float s = 0.f;
-#pragma unroll 8
-            for (int l = 0; l < n; ++l) s = fmaf(weights[i * ldw + l], cur[l * kGossipCols + col], s);
-            nxt[i * kGossipCols + col] = s;
+#pragma unroll 4
+            for (int l = 0; l < n4; ++l) {
+                const float4 w = row[l], p = column[l];
+                s = fmaf(w.x, p.x, s);
+                s = fmaf(w.y, p.y, s);
+                s = fmaf(w.z, p.z, s);
+                s = fmaf(w.w, p.w, s);
+            }
+            nxt[col * ld + i] = s;
         }
         __syncthreads();
         float *const swap = cur;
@@ -78,22 +92,32 @@ __global__ void gossip_rounds_kernel(const float * W, const float * in, int n, i
         nxt = swap;
     }
     if (j < m)
-        for (int i = tid / kGossipCols; i < n; i += threads / kGossipCols) out[(int64_t)i * m + j] = cur[i * kGossipCols + col];
+        for (int i = first; i < n; i += step) out[(int64_t)i * m + j] = cur[col * ld + i];
 }
 
 // spread[0] = max over machines i and vectors j of |P[i][j] - P[reader][j]| (a maximum: order-free).
-__global__ void consensus_spread_kernel(const float * P, int n, int m, int reader, float *spread) {
+__global__ void __launch_bounds__(kSpreadThreads)
+consensus_spread_kernel(const float *P, int n, int m, int reader, float *spread) {
     grid_trigger();
     grid_wait();
-    __shared__ float part[kVarThreads];
+    __shared__ float part[kSpreadThreads / 32];
+    const float *const own = P + (int64_t)reader * m;
     float worst = 0.f;
-    for (int64_t e = threadIdx.x; e < (int64_t)n * m; e += kVarThreads)
-        worst = fmaxf(worst, fabsf(P[e] - P[(int64_t)reader * m + e % m]));
-    part[threadIdx.x] = worst;
+    // unit = 32 columns of one machine
+    const int groups = (m + 31) / 32, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int64_t u = warp; u < (int64_t)groups * n; u += kSpreadThreads / 32) {
+        const int i = (int)(u / groups), j = (int)(u % groups) * 32 + lane;
+        if (j < m) worst = fmaxf(worst, fabsf(__ldcg(P + (int64_t)i * m + j) - __ldcg(own + j)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o /= 2) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+    if (lane == 0) part[warp] = worst;
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    for (int r = 1; r < kVarThreads; ++r) worst = fmaxf(worst, part[r]);
-    *spread = worst;
+    if (warp != 0) return;
+    worst = part[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o /= 2) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+    if (lane == 0) *spread = worst;
 }
 
 }  // namespace
@@ -113,8 +137,8 @@ cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m,
     *result = P;
     if (rounds <= 0) return cudaSuccess;
     if (n <= kGossipMaxMachines) {
-        const size_t smem = ((size_t)n * (n + 1) + 2 * (size_t)n * kGossipCols) * sizeof(float);
-        const int rows = n < 64 ? n : 64;
+        const size_t smem = ((size_t)n + 2 * kGossipCols) * gossip_stride(n) * sizeof(float);
+        const int rows = n <= 4 ? 4 : n < 64 ? (n + 3) / 4 * 4 : 64;           // whole warps
         *result = scratch;
         return launch_chained(true, gossip_rounds_kernel, dim3((m + kGossipCols - 1) / kGossipCols), dim3(kGossipCols * rows), smem, stream, W,
                               P, n, m, rounds, scratch);
@@ -132,7 +156,7 @@ cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m,
 
 cudaError_t launch_consensus_spread(const float *P, int32_t n, int32_t m, int32_t reader, float *spread,
                                     cudaStream_t stream) {
-    return launch_chained(true, consensus_spread_kernel, dim3(1), dim3(kVarThreads), 0, stream, P, n, m, reader, spread);
+    return launch_chained(true, consensus_spread_kernel, dim3(1), dim3(kSpreadThreads), 0, stream, P, n, m, reader, spread);
 }
 
 }  // namespace core
