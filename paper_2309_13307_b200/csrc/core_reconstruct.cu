@@ -357,8 +357,13 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, i
                (ctas_with(slices) < 4 * (int64_t)sm_count || (ctas_with(slices) < 16 * (int64_t)sm_count && m >= 32 * slices)))
             slices *= 2;
         const int64_t ctas = (nq + kThreads / slices - 1) / (kThreads / slices);
-        if (slices == 8)
-            while (ranks < 8 && m >= 128 * ranks && ctas * ranks < 2 * (int64_t)sm_count) ranks *= 2;
+        if (slices == 8) {
+            // CTAs of the fullest SM, each with 1 / ranks of the vectors and the work of starting up (about six vectors a
+            // thread); every slice keeps eight vectors
+            auto cost = [&](int r) { return (double)((ctas * r + sm_count - 1) / sm_count) * (1.0 / r + 48.0 / m); };
+            for (int r = 2; r <= 8 && m >= 64 * r; ++r)
+                if (cost(r) < cost(ranks)) ranks = r;
+        }
         const bool chain = chain_pays(ctas * ranks, 4 * (int64_t)sm_count, 4 * nq, m);
         auto go = [&](auto kernel) {
             const ChainedLaunch launch(chain, dim3((unsigned)(ctas * ranks)), dim3(kThreads), 0, stream, ranks);
