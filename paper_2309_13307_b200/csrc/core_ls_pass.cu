@@ -32,15 +32,15 @@ constexpr int kPassMaxSlots = 8;
 constexpr int kPassMaxWarps = 16;
 constexpr int kPassMaxCluster = 8;
 constexpr int kPassCtaCols = 32 * 32 * kPassMaxWarps;   // columns a CTA can hold: 32 per lane
-constexpr int kPassFlushFloats = 8192;                  // room for the groups' sums while the rings are in use
+constexpr uint32_t kPassFlushBytes = 32u * 1024u;       // room for the groups' sums while the rings are in use
 constexpr uint32_t kPassRingBytes = 128u * 1024u;       // bytes in flight per SM
 
 // Rows at a time.  One warp per row: as many as 32 registers per lane hold.  Several: the chain from a row's arrival to
-// its update crosses the CTA (about 1600 cycles), so two rows go through it together, four where 20 columns per lane
-// leave the registers for it (16 x 2048 rows of 2049 columns: 125 us with one, 84 with two, 66 with four); the 512-thread
+// its update crosses the CTA (about 1600 cycles), so two rows go through it together, four where up to 24 columns
+// per lane leave the registers, and rows of up to 12 KB the shared memory, for it (16 x 2048 rows of 2049 columns: 125 us with one, 84 with two, 66 with four); the 512-thread
 // kernel has registers for two up to 24 columns.
 constexpr int pass_batch(int warps_per_row, int columns) {
-    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 24 ? 1 : 2) : columns == 20 ? 4 : 2;
+    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 24 ? 1 : 2) : warps_per_row <= 4 && columns <= 24 ? 4 : 2;
 }
 
 __device__ int g_pass_status;                           // 0, or the code of a wait that ran out
@@ -471,7 +471,7 @@ cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const floa
     a.slot_bytes = p.slot_bytes;
     a.row_stride = p.row_stride;
     a.ring_offset = p.ring_offset;
-    a.flush_floats = p.ring_offset ? kPassFlushFloats : (int)(p.smem / sizeof(float));
+    a.flush_floats = (int)((p.ring_offset ? p.ring_offset : p.smem) / sizeof(float));
     auto go = [&](auto kernel) {
         if (cudaError_t e = allow_shared(reinterpret_cast<const void *>(kernel), p.smem)) return e;
         const ChainedLaunch launch(true, dim3((unsigned)(p.units * p.cluster)), dim3((unsigned)(32 * p.warps)), p.smem, stream, p.cluster);
@@ -535,8 +535,10 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
     if (p.group_warps == 1) p.chunk_rows *= std::max(1, std::min((int)(kPassRingBytes / (3 * groups) / (row_bytes * batch)), 32 / batch));
     p.row_stride = p.cluster == 1 ? row_bytes : (row_bytes + 31) / 16 * 16 + (uint32_t)(d * 4 % 16);
     p.slot_bytes = (p.chunk_rows * p.row_stride + 12 + 15) / 16 * 16;
-    p.ring_offset = machines_apart && groups > 1 ? kPassFlushFloats * 4u : 0u;
-    const int room = (int)((220u * 1024u - p.ring_offset) / (groups * p.slot_bytes));
+    // half the room for the groups' sums (still one group's) where that makes the difference to a second ring slot
+    const uint32_t smem = 220u * 1024u, all = (uint32_t)groups * p.slot_bytes;
+    p.ring_offset = !machines_apart || groups == 1 ? 0u : kPassFlushBytes + 2 * all <= smem ? kPassFlushBytes : kPassFlushBytes / 2;
+    const int room = (int)((smem - p.ring_offset) / all);
     p.slots = std::max((int)(kPassRingBytes / (groups * p.slot_bytes)), 3);
     p.slots = std::min({p.slots, room, kPassMaxSlots});
     if (p.slots < 2) return LsPass{};
