@@ -552,7 +552,7 @@ def measure_leastsq(core_mod, local: int, min_steps: int = 50, min_seconds: floa
         "steps": steps, "ms": ms, "loss": float(ctx.core_ls_loss(ls, x).item()),
         "gpu_launches": 4 * steps,   # gradient partials, project (sums them while staging), finish+aggregate, reconstruct+update
         "gradients_ms": grad_ms, "round_and_update_ms": ms - grad_ms, "bound": "hbm", "frac": achieved / hbm_peak,
-        "roofline": {"bound": "hbm", "kernel": "ls_fused_kernel + ls_reduce_kernel", "achieved": achieved,
+        "roofline": {"bound": "hbm", "kernel": "ls_pass_kernel + ls_pass_reduce_kernel", "achieved": achieved,
                      "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": None,
                      "algorithmic_bytes": a_bytes, "ms_per_launch": grad_ms,
                      "peak_source": "of measured" if "hbm_gbs" in peaks else "of fallback",

@@ -467,8 +467,21 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
     // at least 256 KB per machine and copy
     const int64_t in_least = std::min(in_most, limit(std::max((int64_t)4 << 20, (int64_t)n << 18), es * (size_t)n));
     const int64_t out_least = std::min(out_most, limit((int64_t)1 << 20, sizeof(float)));
-    const size_t in_bytes = round_up((size_t)n * (size_t)in_most * es, 256);
-    const size_t out_bytes = round_up((size_t)out_most * sizeof(float), 256);
+    // the longest ones that occur, and the partial sums any of them needs
+    int64_t in_len = 0, out_len = 0;
+    size_t pb = 0;
+    for (int64_t k0 = 0, len = 0; k0 < d; k0 += len) {
+        len = next_slab(k0, d, in_least, in_most);
+        if (len > in_len) in_len = len;
+        pb = std::max(pb, row_partial_bytes(ctx, len));
+    }
+    for (int64_t k0 = 0, len = 0; k0 < d; k0 += len) {
+        len = next_slab(k0, d, out_least, out_most);
+        if (len > out_len) out_len = len;
+    }
+    in_len = (in_len + 7) / 8 * 8;                      // rows of a slab start on 16 bytes
+    const size_t in_bytes = round_up((size_t)n * (size_t)in_len * es, 256);
+    const size_t out_bytes = round_up((size_t)out_len * sizeof(float), 256);
     const size_t need_slab = 2 * in_bytes + 2 * out_bytes;
     if (need_slab > ctx->slab_bytes) {
         if (ctx->slab) {
@@ -484,9 +497,6 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
         }
         ctx->slab_bytes = need_slab;
     }
-    size_t pb = row_partial_bytes(ctx, in_most);       // of the longest slab, and of every shorter one
-    for (int64_t k0 = 0; k0 < d; k0 += next_slab(k0, d, in_least, in_most))
-        pb = std::max(pb, row_partial_bytes(ctx, next_slab(k0, d, in_least, in_most)));
     const size_t mb = round_up((size_t)ctx->m * sizeof(float), 256);
     if (int rc = ensure_workspace(ctx, pb + mb)) return rc;
     char *in_buf[2] = {static_cast<char *>(ctx->slab), static_cast<char *>(ctx->slab) + in_bytes};
@@ -507,15 +517,15 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
         if (s >= 2) CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->in_free[b], 0));
         const char *const from = static_cast<const char *>(G_host) + (size_t)k0 * es;
         if ((size_t)ldg * es <= (size_t)INT32_MAX)          // one copy for all rows, where the stride is a legal pitch
-            CORE_CUDA(ctx, cudaMemcpy2DAsync(in_buf[b], (size_t)in_most * es, from, (size_t)ldg * es, (size_t)len * es, (size_t)n,
+            CORE_CUDA(ctx, cudaMemcpy2DAsync(in_buf[b], (size_t)in_len * es, from, (size_t)ldg * es, (size_t)len * es, (size_t)n,
                                              cudaMemcpyHostToDevice, ctx->copy_stream));
         else
             for (int32_t i = 0; i < n; ++i)
-                CORE_CUDA(ctx, cudaMemcpyAsync(in_buf[b] + (size_t)i * (size_t)in_most * es, from + (size_t)i * (size_t)ldg * es,
+                CORE_CUDA(ctx, cudaMemcpyAsync(in_buf[b] + (size_t)i * (size_t)in_len * es, from + (size_t)i * (size_t)ldg * es,
                                                (size_t)len * es, cudaMemcpyHostToDevice, ctx->copy_stream));
         CORE_CUDA(ctx, cudaEventRecord(ctx->in_ready[b], ctx->copy_stream));
         CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->work_stream, ctx->in_ready[b], 0));
-        if (int rc = project_row_into(ctx, in_buf[b], dtype, n, in_most, 1.0f / (float)n, len, (uint64_t)k0 >> 2, partial, pbar,
+        if (int rc = project_row_into(ctx, in_buf[b], dtype, n, in_len, 1.0f / (float)n, len, (uint64_t)k0 >> 2, partial, pbar,
                                       s > 0, ctx->work_stream))
             return rc;
         CORE_CUDA(ctx, cudaEventRecord(ctx->in_free[b], ctx->work_stream));
