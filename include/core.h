@@ -146,7 +146,9 @@ int core_reconstruct(core_ctx *ctx, const float *pbar_dev, float *gtilde_dev);
 /*
  * One whole communication round (Algorithm 2, steps 1-4): project, aggregate,
  * reconstruct with the current t, then t <- t + 1.  pbar_dev (m floats) receives
- * the aggregated message; gtilde_dev (d floats) the estimate.
+ * the aggregated message; gtilde_dev (d floats) the estimate.  With several machines and at
+ * least 2^25 = d*m Gaussians the mean gradient is projected instead of every machine's (the
+ * message is linear in the gradients): the same pbar up to the order of the sums.
  */
 int core_round(core_ctx *ctx, const void *G_dev, int dtype, int32_t n, int64_t ldg, float *pbar_dev,
                float *gtilde_dev);
