@@ -4,7 +4,7 @@
 //
 // The rows of all machines are one matrix of n * rows rows, cut evenly over one CTA per SM, whatever n and rows
 // are: a CTA's range may end inside a machine and go on in the next.  Groups of W warps take the CTA's rows in
-// turn: W = 1 up to 1024 columns, then 2, 4, 8 and 16 up to 16384; beyond, a cluster of 2 to 8 CTAs shares the
+// turn: W = 1 up to 512 columns, then 2, 4, 8 and 16 up to 16384; beyond, a cluster of 2 to 8 CTAs shares the
 // columns of a row.  Lane l of warp w of a group owns columns l + 32 (w + W c): x and the partial gradient of those
 // columns stay in registers for the whole pass, the row's values between its dot product and its update.  Each
 // group has a ring of row buffers in shared memory filled by bulk copies (one lane issues them; they start and end
@@ -14,7 +14,7 @@
 // cluster every warp sends its share of the dot product to all CTAs (asynchronous remote stores counted by a barrier
 // there).  Every sum has a fixed order.
 //
-// Measured (us; pass alone unless said otherwise; before: the kernels this one replaced): n = 50, 1200 x 784: 155 -> 41;
+// Measured (us; pass alone unless said otherwise; before: the kernels this one replaced): n = 50, 1200 x 784: 155 -> 38;
 // n = 50, 11620 x 54: gradients 377 -> 31, loss 212 -> 28; n = 16, 256 x 20000: gradients 133 -> 72; n = 8, 2048 x 8192
 // (537 MB): loss 107 -> 88, gradients 87 -> 92.  Tried: cp.async instead of bulk copies (20 % slower), rings of 96 to
 // 192 KB (equal), evict_normal instead of evict_first (3 to 10 us slower), 8 warps for one-warp rows (25 % slower).
@@ -30,6 +30,7 @@ namespace {
 
 constexpr int kPassMaxSlots = 8;
 constexpr int kPassMaxWarps = 16;
+constexpr int kPassOneWarp = 512;                       // columns up to which one warp holds a row
 constexpr int kPassMaxCluster = 8;
 constexpr int kPassCtaCols = 32 * 32 * kPassMaxWarps;   // columns a CTA can hold: 32 per lane
 constexpr uint32_t kPassFlushBytes = 32u * 1024u;       // room for the groups' sums while the rings are in use
@@ -37,10 +38,11 @@ constexpr uint32_t kPassRingBytes = 128u * 1024u;       // bytes in flight per S
 
 // Rows at a time.  One warp per row: as many as 32 registers per lane hold.  Several: the chain from a row's arrival to
 // its update crosses the CTA (about 1600 cycles), so two rows go through it together, four where up to 24 columns
-// per lane leave the registers, and rows of up to 12 KB the shared memory, for it (16 x 2048 rows of 2049 columns: 125 us with one, 84 with two, 66 with four); the 512-thread
-// kernel has registers for two up to 24 columns.
+// per lane leave the registers, and rows of up to 24 KB the shared memory, for it (gradients, us: 16 x 2048 rows of
+// 2049 columns: 125 with one, 84 with two, 66 with four; 8 x 1500 x 5500: 56 with two, 46 with four); the 512-thread
+// kernel of 16 warps per row has registers for two up to 24 columns.
 constexpr int pass_batch(int warps_per_row, int columns) {
-    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 24 ? 1 : 2) : warps_per_row <= 4 && columns <= 24 ? 4 : 2;
+    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 24 ? 1 : 2) : columns <= 24 ? 4 : 2;
 }
 
 __device__ int g_pass_status;                           // 0, or the code of a wait that ran out
@@ -487,14 +489,22 @@ cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const floa
     using i2 = integral_constant<int, 2>;
     using i4 = integral_constant<int, 4>;
     using i8 = integral_constant<int, 8>;
+    using i12 = integral_constant<int, 12>;
     using i16 = integral_constant<int, 16>;
     using i20 = integral_constant<int, 20>;
     using i24 = integral_constant<int, 24>;
     using i32 = integral_constant<int, 32>;
     auto wide = [&](auto warps, auto per_row) {
-        if constexpr (decltype(per_row)::value <= 4)
+        constexpr int W = decltype(per_row)::value;
+        if constexpr (W < 16) {
+            if constexpr (W == 2)
+                if (p.columns == 12) return pick(i16{}, per_row, i12{});
+            if (p.columns == 16) return pick(warps, per_row, i16{});
             if (p.columns == 20) return pick(warps, per_row, i20{});
-        return p.columns == 24 ? pick(warps, per_row, i24{}) : pick(warps, per_row, i32{});
+        }
+        if constexpr (W >= 8)
+            if (p.columns == 32) return pick(warps, per_row, i32{});
+        return pick(warps, per_row, i24{});
     };
     switch (p.group_warps) {
         case 16: return wide(i16{}, i16{});
@@ -508,8 +518,7 @@ cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const floa
         case 2: return pick(i16{}, i1{}, i2{});
         case 4: return pick(i16{}, i1{}, i4{});
         case 8: return pick(i16{}, i1{}, i8{});
-        case 16: return pick(i16{}, i1{}, i16{});
-        default: return pick(i16{}, i1{}, i32{});
+        default: return pick(i16{}, i1{}, i16{});
     }
 }
 
@@ -522,12 +531,20 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
     while (d > (int64_t)kPassCtaCols * p.cluster) p.cluster *= 2;
     p.slice = p.cluster == 1 ? (int)d : (int)(((d + p.cluster - 1) / p.cluster + 3) / 4 * 4);
     p.group_warps = 1;
-    while (p.slice > 1024 * p.group_warps) p.group_warps *= 2;
+    // 24 columns per lane at most where several warps share a row (four rows at a time, see pass_batch), 32 where that is
+    // more than 8 warps hold.  One warp with 32 columns per lane handled one row at a time: from 513 columns two warps
+    // with four rows are faster (gradients, 50 x 1200 rows of 600: 44 -> 29 us, of 1000: 48 -> 44).  Up to 12 columns
+    // per lane 16 warps per CTA have the registers for that (37 with 8); with fewer columns per lane and more warps
+    // per row than this, longer rows were slower (784: 41 -> 46, 6100: equal).
+    if (p.slice > kPassOneWarp)
+        do p.group_warps *= 2;
+        while (p.group_warps < 8 && p.slice > 768 * p.group_warps);
+    if (p.slice > 1024 * p.group_warps) p.group_warps = kPassMaxWarps;
     const int per_lane = (p.slice + 32 * p.group_warps - 1) / (32 * p.group_warps);
     p.columns = 1;
     while (p.columns < per_lane) p.columns *= 2;
-    if (p.group_warps > 1) p.columns = per_lane <= 20 && p.group_warps <= 4 ? 20 : per_lane <= 24 ? 24 : 32;
-    p.warps = p.group_warps == 1 || p.group_warps == 16 ? 16 : 8;
+    if (p.group_warps > 1) p.columns = per_lane > 24 ? 32 : p.group_warps == kPassMaxWarps || per_lane > 20 ? 24 : per_lane > 16 ? 20 : per_lane > 12 ? 16 : 12;
+    p.warps = p.group_warps == 1 || p.columns == 12 || p.group_warps == 16 ? 16 : 8;
     const int groups = p.warps / p.group_warps;
     const uint32_t row_bytes = (uint32_t)p.slice * 4;
     const int batch = pass_batch(p.group_warps, p.columns);               // rows at a time

@@ -21,11 +21,13 @@ def core_mod():
 
 @pytest.mark.parametrize("n,rows,d,offset", [
     (1, 1, 1, 0), (3, 700, 1, 1), (2, 5, 31, 0), (50, 37, 54, 0), (7, 333, 64, 2), (64, 16, 65, 3),   # several rows at a time
-    (2, 3000, 127, 1), (5, 61, 129, 0), (3, 200, 256, 0), (2, 999, 257, 3), (4, 77, 511, 1), (6, 50, 513, 0),
-    (9, 120, 784, 0), (2, 400, 1023, 2), (1, 150, 1024, 0),                                              # one warp per row
-    (2, 90, 1025, 0), (3, 50, 2047, 1), (3, 151, 2049, 0), (2, 149, 4096, 0), (1, 40, 4097, 1),          # 2, 4, 8 warps
-    (2, 80, 8192, 0), (1, 33, 8193, 3), (2, 75, 16384, 0),                                               # 16 warps
-    (1, 80, 16385, 0), (3, 30, 20001, 1), (1, 37, 33000, 2),                                             # clusters of 2 and 4
+    (2, 3000, 127, 1), (5, 61, 129, 0), (3, 200, 256, 0), (2, 999, 257, 3), (4, 77, 511, 1), (3, 65, 512, 0),  # one warp
+    (6, 50, 513, 0), (8, 331, 600, 2), (2, 90, 768, 0), (2, 150, 769, 1), (9, 120, 784, 0), (2, 400, 1023, 2),  # per row
+    (1, 150, 1024, 0), (2, 90, 1025, 0), (3, 50, 1536, 0),                                               # 2 warps
+    (3, 50, 2047, 1), (3, 151, 2049, 0), (2, 47, 2561, 1), (3, 40, 3072, 0),                             # 4
+    (2, 70, 3073, 0), (2, 149, 4096, 0), (1, 40, 4097, 1), (3, 60, 5500, 3), (2, 51, 6145, 1), (2, 80, 8192, 0),  # 8
+    (1, 33, 8193, 3), (40, 9, 9001, 1), (5, 7, 12000, 0), (2, 75, 16384, 0),                             # 16
+    (1, 80, 16385, 0), (3, 30, 20001, 1), (16, 5, 24000, 0), (1, 37, 33000, 2),                          # clusters of 2 and 4
 ])
 def test_gradients_loss_and_step(core_mod, n, rows, d, offset):
     A = core_inputs.gradients(1, n * rows * d + offset, seed=n + rows + d, device="cuda")[0][offset:].view(n, rows, d)
