@@ -350,6 +350,16 @@ int core_debug_box_muller(core_ctx *ctx, const uint32_t *words_dev, int64_t nb, 
 int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t sm_count, int64_t out[10]);
 
 /*
+ * What one pass over the data matrices of a least-squares problem (n x rows x d floats, their address `misaligned`
+ * bytes beyond a multiple of 16) would touch beyond them, by its bulk copies and prefetches.  Host-only replay of the
+ * kernel's own index arithmetic: reads nothing, touches no device for d <= 16384.
+ * out[0..2] = CTAs (or clusters) the rows are cut over (0: the single pass does not apply), bytes touched
+ * before the matrices, bytes touched behind them (both 0 in a correct library).
+ */
+int core_debug_ls_reads(int32_t n, int32_t rows, int64_t d, int machines_apart, int32_t sm_count, uint32_t misaligned,
+                        int64_t out[3]);
+
+/*
  * Instruction-rate probes (no counterpart in the paper: they support the roofline of the round kernels,
  * which are bound by instruction issue).  Kind k < core_debug_pipe_kinds() - 3 runs a loop whose body
  * is counts_out[0..6] = (32x32-bit multiplies keeping the high word, fp32 multiply-adds, packed fp32 multiply-adds,

@@ -67,6 +67,8 @@ _SIGNATURES = {
                                 _c.POINTER(_c.c_uint32)], _c.c_int),
     "core_debug_project_plan": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32,
                                  _c.POINTER(_c.c_int64)], _c.c_int),
+    "core_debug_ls_reads": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32, _c.c_uint32,
+                             _c.POINTER(_c.c_int64)], _c.c_int),
 }
 
 
@@ -136,6 +138,14 @@ def core_debug_project_plan(n: int, m: int, d: int, dtype: int = CORE_F32, sm_co
         raise CoreError(rc, "core_debug_project_plan")
     keys = ("nb", "jt", "uq", "tile_q", "tj", "tq", "grid_x", "grid_y", "tiles", "smem")
     return dict(zip(keys, (int(v) for v in out)))
+
+
+def core_debug_ls_reads(n: int, rows: int, d: int, machines_apart: bool, misaligned: int, sm_count: int = 148) -> tuple:
+    out = (ctypes.c_int64 * 3)()
+    rc = lib().core_debug_ls_reads(n, rows, d, int(machines_apart), sm_count, misaligned, out)
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_ls_reads")
+    return tuple(out)
 
 
 def core_debug_pipe_kinds() -> int:

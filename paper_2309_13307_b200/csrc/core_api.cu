@@ -856,4 +856,14 @@ int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t 
     return CORE_OK;
 }
 
+int core_debug_ls_reads(int32_t n, int32_t rows, int64_t d, int machines_apart, int32_t sm_count, uint32_t misaligned,
+                        int64_t out[3]) {
+    if (!out || n < 1 || rows < 1 || d < 1 || sm_count < 1 || misaligned % 4 != 0) return CORE_EINVAL;
+    const LsPass pass = make_ls_pass(n, rows, d, machines_apart != 0, sm_count);
+    out[0] = pass.units;
+    out[1] = out[2] = 0;
+    ls_pass_reads(pass, d, ((uintptr_t)1 << 32) + misaligned, &out[1], &out[2]);      // any address: nothing is read here
+    return CORE_OK;
+}
+
 }  // extern "C"

@@ -211,6 +211,8 @@ cudaError_t launch_ls_pass_reduce(const LsPass &pass, const float *part, int64_t
 cudaError_t launch_ls_pass_loss(const LsPass &pass, const float *A, const float *b, const LsPoint &at, int64_t d, bool reverse,
                                 double *loss_part, cudaStream_t stream);
 cudaError_t launch_ls_loss_sum(const double *loss_part, int64_t units, double scale, double *loss, cudaStream_t stream);
+// Bytes before and behind a matrix at address a_begin that the bulk copies and prefetches of a pass would touch (host only).
+void ls_pass_reads(const LsPass &pass, int64_t d, uintptr_t a_begin, int64_t *before, int64_t *behind);
 cudaError_t ls_pass_take_status(int *status);     // after a device synchronisation; clears the word
 // Comparison step of Algorithm 3, on the device: if *f_trial < *f then x <- trial, *f <- *f_trial and the
 // flag is 1, otherwise nothing changes and the flag is 0 (a tie keeps x).  f_trial is scale times the sum of the

@@ -72,6 +72,32 @@ struct PassArgs {
     int reverse;             // rows from the last to the first (what an ascending pass left in L2 comes first)
 };
 
+// What is read of A, as the kernel computes it and ls_pass_reads checks it on the host.
+// Rows [lo, lo + count) of all machines' rows are a unit's.  `edge`: A ends less than 16 bytes before or behind them, so
+// that rounding out to 16 bytes might reach beyond it (not only for the first and the last unit: rows may be one float).
+struct UnitRows {
+    int64_t lo;
+    int count;
+    bool edge;
+};
+__host__ __device__ inline UnitRows unit_rows(int64_t total, int64_t units, int64_t unit, int64_t d) {
+    const int64_t lo = total * unit / units, hi = total * (unit + 1) / units;
+    return {lo, (int)(hi - lo), lo * d < 4 || (total - hi) * d < 4};
+}
+// The bytes [from, to) rounded out to the 16-byte units a bulk copy moves ...
+struct BulkRange {
+    uintptr_t b0, b1;
+};
+__host__ __device__ inline BulkRange bulk_range(uintptr_t from, uintptr_t to) { return {from & ~(uintptr_t)15, (to + 15) & ~(uintptr_t)15}; }
+// ... and without a first or last one that would reach beyond A (whose elements are copied one by one).
+__host__ __device__ inline BulkRange bulk_range_inside(BulkRange r, uintptr_t a_begin, uintptr_t a_end) {
+    return {r.b0 < a_begin ? r.b0 + 16 : r.b0, r.b1 > a_end ? r.b1 - 16 : r.b1};
+}
+// What a prefetch of them asks for (not at an edge).
+__host__ __device__ inline BulkRange prefetch_range(uintptr_t from, uint32_t bytes) {
+    return {from & ~(uintptr_t)15, (from & ~(uintptr_t)15) + (bytes & ~15u)};
+}
+
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -138,8 +164,10 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     const int64_t unit = MULTI && a.cluster > 1 ? blockIdx.x / a.cluster : blockIdx.x;
     const int64_t col0 = (int64_t)rank * a.slice;
     const int dn = (int)min((int64_t)a.slice, a.d - col0);
-    const int64_t lo = a.total * unit / a.units;
-    const int nrows = (int)(a.total * (unit + 1) / a.units - lo);  // rows of this unit, counted from its first
+    const UnitRows owned = unit_rows(a.total, a.units, unit, a.d);
+    const int64_t lo = owned.lo;
+    const int nrows = owned.count;                                 // rows are counted from the unit's first
+    const bool edge = owned.edge;
     const int R = a.chunk_rows;
     const int chunks = (nrows + R - 1) / R;
     const uint32_t row_bytes = (uint32_t)a.d * 4;
@@ -157,29 +185,22 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     const uintptr_t unit_base = reinterpret_cast<uintptr_t>(a.A) + (uintptr_t)(lo * a.d + col0) * 4;
     const int64_t src_step = (a.reverse ? -(int64_t)GROUPS : (int64_t)GROUPS) * R * row_bytes;
     uintptr_t src = unit_base + (uint64_t)(uint32_t)max(first_row(grp), 0) * row_bytes;
-    const bool edge = unit == 0 || unit == a.units - 1;            // may hold the first or the last bytes of A
     const uint64_t policy = l2_evict_first();
     auto issue = [&](int k, int s) {
         const uint32_t bar = bar0 + 8 * s;
         // the bytes [from, to) of A to shared memory, `from` going to `dst` (which agrees with it modulo 16)
         auto copy = [&](uintptr_t from, uintptr_t to, uint32_t dst) {
             const uint32_t origin = dst - (uint32_t)from;             // of address zero, so to say
-            uintptr_t b0 = from & ~(uintptr_t)15, b1 = (to + 15) & ~(uintptr_t)15;
+            BulkRange r = bulk_range(from, to);
             if (edge) {
-                // nothing outside A is touched: a first or last piece that would reach beyond it is copied element by element
-                const uintptr_t a_begin = reinterpret_cast<uintptr_t>(a.A), a_end = a_begin + (uintptr_t)(a.total * a.d) * 4;
-                if (b0 < a_begin) {
-                    b0 += 16;
-                    for (uintptr_t p = from; p < b0 && p < to; p += 4) store_shared(origin + (uint32_t)p, *reinterpret_cast<const float *>(p));
-                }
-                if (b1 > a_end) {
-                    b1 -= 16;
-                    for (uintptr_t p = b1 > from ? b1 : from; p < to; p += 4) store_shared(origin + (uint32_t)p, *reinterpret_cast<const float *>(p));
-                }
+                const uintptr_t a_begin = reinterpret_cast<uintptr_t>(a.A);
+                r = bulk_range_inside(r, a_begin, a_begin + (uintptr_t)(a.total * a.d) * 4);
+                for (uintptr_t p = from; p < r.b0 && p < to; p += 4) store_shared(origin + (uint32_t)p, *reinterpret_cast<const float *>(p));
+                for (uintptr_t p = r.b1 > from ? r.b1 : from; p < to; p += 4) store_shared(origin + (uint32_t)p, *reinterpret_cast<const float *>(p));
             }
-            if (b1 > b0) {
-                mbar_expect(bar, (uint32_t)(b1 - b0));
-                bulk_copy(origin + (uint32_t)b0, reinterpret_cast<const void *>(b0), (uint32_t)(b1 - b0), bar, policy);
+            if (r.b1 > r.b0) {
+                mbar_expect(bar, (uint32_t)(r.b1 - r.b0));
+                bulk_copy(origin + (uint32_t)r.b0, reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0), bar, policy);
             }
         };
         const int count = min(R, nrows - first_row(k));
@@ -202,9 +223,8 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
         for (int s = 0; s < a.slots; ++s) {
             const int k = grp + s * GROUPS;
             if (k >= chunks) break;
-            const uintptr_t from = (src + (int64_t)s * src_step) & ~(uintptr_t)15;
-            const uint32_t bytes = (uint32_t)min(R, nrows - first_row(k)) * row_bytes & ~15u;
-            if (bytes) bulk_prefetch(reinterpret_cast<const void *>(from), bytes);
+            const BulkRange r = prefetch_range(src + (int64_t)s * src_step, (uint32_t)min(R, nrows - first_row(k)) * row_bytes);
+            if (r.b1 > r.b0) bulk_prefetch(reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0));
         }
     grid_wait();
     if (leader)
@@ -613,6 +633,39 @@ cudaError_t launch_ls_pass_reduce(const LsPass &p, const float *part, int64_t d,
 
 cudaError_t launch_ls_loss_sum(const double *loss_part, int64_t units, double scale, double *loss, cudaStream_t stream) {
     return launch_chained(true, ls_loss_sum_kernel, dim3(1), dim3(32), 0, stream, loss_part, units, scale, loss);
+}
+
+// Host-side replay of the copies and prefetches of one pass over a matrix at address `a_begin`.
+void ls_pass_reads(const LsPass &p, int64_t d, uintptr_t a_begin, int64_t *before, int64_t *behind) {
+    const uintptr_t a_end = a_begin + (uintptr_t)(p.total * d) * 4;
+    const uint32_t row_bytes = (uint32_t)d * 4;
+    *before = *behind = 0;
+    auto touch = [&](BulkRange r) {
+        if (r.b1 <= r.b0) return;
+        if (r.b0 < a_begin) *before = std::max(*before, (int64_t)(a_begin - r.b0));
+        if (r.b1 > a_end) *behind = std::max(*behind, (int64_t)(r.b1 - a_end));
+    };
+    for (int64_t unit = 0; unit < p.units; ++unit) {
+        const UnitRows u = unit_rows(p.total, p.units, unit, d);
+        auto copy = [&](uintptr_t from, uintptr_t to) {
+            const BulkRange r = bulk_range(from, to);
+            touch(u.edge ? bulk_range_inside(r, a_begin, a_end) : r);
+        };
+        for (int row = 0; row < u.count; row += p.chunk_rows) {
+            const int count = std::min(p.chunk_rows, u.count - row);
+            const uintptr_t src = a_begin + (uintptr_t)((u.lo + row) * d) * 4;
+            if (p.cluster == 1) {
+                copy(src, src + (uint32_t)count * row_bytes);
+                if (!u.edge) touch(prefetch_range(src, (uint32_t)count * row_bytes));
+                continue;
+            }
+            for (int i = 0; i < count; ++i)
+                for (int64_t col = 0; col < d; col += p.slice) {
+                    const uintptr_t from = src + (uintptr_t)i * row_bytes + (uintptr_t)col * 4;
+                    copy(from, from + (uintptr_t)std::min<int64_t>(p.slice, d - col) * 4);
+                }
+        }
+    }
 }
 
 cudaError_t ls_pass_take_status(int *status) {

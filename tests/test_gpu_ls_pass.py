@@ -61,3 +61,22 @@ def test_gradients_loss_and_step(core_mod, n, rows, d, offset):
     else:
         assert torch.equal(xg, x) and f.item() == f0 and f1 >= f0 * (1 - 1e-5)
     assert core_mod.core_device_status() == 0
+
+
+@pytest.mark.parametrize("n,rows,d", [(1, 3, 1), (1, 147, 1), (7, 60, 1), (1, 443, 1), (3, 41, 2), (1, 295, 2), (1, 170, 3)])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_rows_shorter_than_a_copy_unit(core_mod, n, rows, d, offset):
+    """Rows of a few floats: the ends of the matrix lie within one 16-byte unit of CTAs that are not the first or the last."""
+    A = core_inputs.gradients(1, n * rows * d + offset, seed=n + rows + d, device="cuda")[0][offset:].view(n, rows, d)
+    b = core_inputs.gradients(n, rows, seed=5, device="cuda").contiguous()
+    x = core_inputs.gradients(1, d, seed=6, device="cuda")[0].contiguous()
+    Ah, bh, xh = A.cpu().numpy(), b.cpu().numpy(), x.cpu().numpy().astype(np.float64)
+    ctx, ls = core_mod.Core(3, d, 8), core_mod.LeastSquares(A, b)
+    G = ctx.core_ls_gradients(ls, x).cpu().numpy()
+    want = oracle.ls_grad(Ah, bh, xh)
+    # fp32 sums of `rows` products whose terms may cancel: relative to the sum of their magnitudes
+    terms = np.abs(Ah.astype(np.float64)) * np.abs(np.einsum("nrd,d->nr", Ah.astype(np.float64), xh) - bh)[:, :, None]
+    assert (np.abs(G - want) <= 1e-5 * terms.mean(axis=1) + 1e-12).all()
+    f0 = oracle.ls_loss(Ah, bh, xh)
+    assert abs(float(ctx.core_ls_loss(ls, x).item()) - f0) <= 1e-5 * f0
+    assert core_mod.core_device_status() == 0
