@@ -100,8 +100,8 @@ int core_last_cuda_error(const core_ctx *ctx);
  * Device-side status.  The tensor-memory projection kernel hands buffers between
  * its warps with barriers whose waits are bounded; a wait that runs out makes
  * the kernel finish early (its output is then meaningless) and records a
- * non-zero code in a per-device status word.  A wait gives up after 100 ms of
- * the device's global timer; waits that are served take microseconds.  This call synchronises the
+ * non-zero code in a per-device status word.  A wait gives up after 100 ms
+ * (time in which the GPU works for another program does not count); waits that are served take microseconds.  This call synchronises the
  * current device, stores the word in *status_out (host pointer; 0 = every wait
  * was served) and clears it.  Not part of the paper: run-time diagnostics.
  */
@@ -329,6 +329,13 @@ int core_debug_fail_allocations(int count);
  * saw the abort flag.  Synchronises.  Uses no tensor-core instruction.
  */
 int core_debug_wait_timeout(uint32_t limit_us, int32_t code, uint32_t observed_host[2]);
+
+/*
+ * Host-only replay of the clock of those waits: with the device timer read as readings_ns[0..count-1], the index of
+ * the reading at which a wait of limit_ns gives up, or -1.  What lies between two readings counts 1 ms at most (the
+ * timer runs on while the GPU works for somebody else).
+ */
+int core_debug_wait_clock(const uint64_t *readings_ns, int32_t count, uint64_t limit_ns, int32_t *given_up_at);
 
 /* ---- generator windows (for checking the generator itself) ------------------- */
 

@@ -55,6 +55,7 @@ _SIGNATURES = {
     "core_debug_fail_allocations": ([_c.c_int], _c.c_int),
     "core_debug_force_project_kernel": ([_c.c_int], _c.c_int),
     "core_debug_wait_timeout": ([_c.c_uint32, _c.c_int32, _c.POINTER(_c.c_uint32)], _c.c_int),
+    "core_debug_wait_clock": ([_c.POINTER(_c.c_uint64), _c.c_int32, _c.c_uint64, _c.POINTER(_c.c_int32)], _c.c_int),
     "core_ls_gradients": ([_c.c_void_p, _c.c_void_p, _c.c_void_p, _c.c_void_p], _c.c_int),
     "core_debug_philox": ([_c.c_void_p, _c.c_uint32, _c.c_uint64, _c.c_int64, _c.c_void_p], _c.c_int),
     "core_debug_gaussians": ([_c.c_void_p, _c.c_uint32, _c.c_uint64, _c.c_int64, _c.c_void_p], _c.c_int),
@@ -190,6 +191,15 @@ def core_debug_wait_timeout(limit_us: int, code: int) -> tuple:
     if rc != CORE_OK:
         raise CoreError(rc, "core_debug_wait_timeout")
     return int(out[0]), int(out[1])
+
+
+def core_debug_wait_clock(readings_ns, limit_ns: int) -> int:
+    given_up_at = ctypes.c_int32(0)
+    readings = (ctypes.c_uint64 * len(readings_ns))(*readings_ns)
+    rc = lib().core_debug_wait_clock(readings, len(readings_ns), int(limit_ns), ctypes.byref(given_up_at))
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_wait_clock")
+    return given_up_at.value
 
 
 def core_device_status() -> int:

@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "core_internal.h"
+#include "core_sync.cuh"
 
 using namespace core;
 
@@ -820,6 +821,15 @@ int core_debug_wait_timeout(uint32_t limit_us, int32_t code, uint32_t observed_h
         cudaGetLastError();
         return CORE_ECUDA;
     }
+    return CORE_OK;
+}
+
+int core_debug_wait_clock(const uint64_t *readings_ns, int32_t count, uint64_t limit_ns, int32_t *given_up_at) {
+    if (!readings_ns || !given_up_at || count < 1) return CORE_EINVAL;
+    WaitClock clock(readings_ns[0]);
+    *given_up_at = -1;
+    for (int32_t i = 1; i < count && *given_up_at < 0; ++i)
+        if (clock.over(readings_ns[i], limit_ns)) *given_up_at = i;
     return CORE_OK;
 }
 

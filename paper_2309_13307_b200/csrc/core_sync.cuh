@@ -12,7 +12,7 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 // ... and from here on the kernel after it may be scheduled where there is room (it waits in turn).
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-constexpr uint64_t kWaitLimitNs = 100ull * 1000 * 1000;   // a wait gives up after 100 ms of the global timer
+constexpr uint64_t kWaitLimitNs = 100ull * 1000 * 1000;   // a wait gives up after 100 ms
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -46,19 +46,32 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// Bounded wait: false when the phase did not complete within limit_ns of the global timer.  The timer is read only
+// Time spent waiting, from readings of the global timer.  That timer runs on while the GPU works for somebody else (time
+// slices, a debugger), so what lies between two readings counts kWaitStepNs at most: a wait is given up for the time its
+// program was there to be served, not for the time it was away.
+constexpr uint64_t kWaitStepNs = 1000ull * 1000;          // 1 ms; eight probes take some microseconds
+struct WaitClock {
+    uint64_t last, spent = 0;
+    __host__ __device__ explicit WaitClock(uint64_t now) : last(now) {}
+    __host__ __device__ bool over(uint64_t now, uint64_t limit_ns) {
+        spent += now - last < kWaitStepNs ? now - last : kWaitStepNs;
+        last = now;
+        return spent >= limit_ns;
+    }
+};
+// Bounded wait: false when the phase did not complete within limit_ns (see WaitClock).  The timer is read only
 // once a number of probes have failed (a probe waits for a while by itself): a wait for memory is normally served
 // long before.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
 #pragma unroll 1
     for (int probe = 0; probe < 64; ++probe)
         if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
+    WaitClock clock(global_timer_ns());
     do {
 #pragma unroll 1
-        for (int probe = 0; probe < 64; ++probe)
+        for (int probe = 0; probe < 8; ++probe)
             if (mbar_try_wait(bar, parity)) return true;
-    } while (global_timer_ns() - t0 < limit_ns);
+    } while (!clock.over(global_timer_ns(), limit_ns));
     return false;
 }
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
