@@ -97,10 +97,14 @@ const char *core_strerror(int code);
 int core_last_cuda_error(const core_ctx *ctx);
 
 /*
- * Device-side status.  The tensor-memory projection kernel hands buffers between
- * its warps with barriers whose waits are bounded; a wait that runs out makes
- * the kernel finish early (its output is then meaningless) and records a
- * non-zero code in a per-device status word.  A wait gives up after 100 ms
+ * Device-side status.  The tensor-memory projection kernel and the least-squares pass hand buffers
+ * between their warps with barriers whose waits are bounded; a wait that runs out makes
+ * the kernel finish early and records a non-zero code in a per-device status word.  The entry
+ * points do not see it (they return before the kernels run):
+ *   1..6    tensor-memory projection: the messages are meaningless;
+ *   21, 22  least-squares pass (rows that did not arrive; shares of a dot product from another CTA that did not):
+ *           what depends on them is NaN - gradients, loss, the x of core_gd_step, core_agd_step and
+ *           core_decentralized_step; the steps with the comparison do not take their trial point and leave x, f as they are.  A wait gives up after 100 ms
  * (time in which the GPU works for another program does not count); waits that are served take microseconds.  This call synchronises the
  * current device, stores the word in *status_out (host pointer; 0 = every wait
  * was served) and clears it.  Not part of the paper: run-time diagnostics.
@@ -329,6 +333,13 @@ int core_debug_fail_allocations(int count);
  * saw the abort flag.  Synchronises.  Uses no tensor-core instruction.
  */
 int core_debug_wait_timeout(uint32_t limit_us, int32_t code, uint32_t observed_host[2]);
+
+/*
+ * From now on the least-squares passes of this handle leave out the copies of chunks of rows (those from the `chunk`-th on,
+ * counted from 0 in each CTA, in a cluster its first CTA; -1 switches this off), so that the waits for them run out after 100 ms, as if the copies
+ * had never arrived: the passes then end by their normal exit, their results are NaN and core_device_status tells 21 or 22.
+ */
+int core_debug_ls_hold_back(core_ls *ls, int32_t chunk);
 
 /*
  * Host-only replay of the clock of those waits: with the device timer read as readings_ns[0..count-1], the index of

@@ -55,6 +55,7 @@ _SIGNATURES = {
     "core_debug_fail_allocations": ([_c.c_int], _c.c_int),
     "core_debug_force_project_kernel": ([_c.c_int], _c.c_int),
     "core_debug_wait_timeout": ([_c.c_uint32, _c.c_int32, _c.POINTER(_c.c_uint32)], _c.c_int),
+    "core_debug_ls_hold_back": ([_c.c_void_p, _c.c_int32], _c.c_int),
     "core_debug_wait_clock": ([_c.POINTER(_c.c_uint64), _c.c_int32, _c.c_uint64, _c.POINTER(_c.c_int32)], _c.c_int),
     "core_ls_gradients": ([_c.c_void_p, _c.c_void_p, _c.c_void_p, _c.c_void_p], _c.c_int),
     "core_debug_philox": ([_c.c_void_p, _c.c_uint32, _c.c_uint64, _c.c_int64, _c.c_void_p], _c.c_int),
@@ -423,6 +424,11 @@ class LeastSquares:
         if rc != CORE_OK:
             self._h = ctypes.c_void_p()
             raise CoreError(rc, "core_ls_create")
+
+    def core_debug_hold_back(self, chunk: int):
+        rc = lib().core_debug_ls_hold_back(self._h, int(chunk))
+        if rc != CORE_OK:
+            raise CoreError(rc, "core_debug_ls_hold_back")
 
     def close(self):
         if getattr(self, "_h", None) and self._h.value:

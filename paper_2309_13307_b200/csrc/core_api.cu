@@ -824,6 +824,12 @@ int core_debug_wait_timeout(uint32_t limit_us, int32_t code, uint32_t observed_h
     return CORE_OK;
 }
 
+int core_debug_ls_hold_back(core_ls *ls, int32_t chunk) {
+    if (!ls || chunk < -1) return CORE_EINVAL;
+    ls->step_pass.hold_back = ls->machine_pass.hold_back = chunk < 0 ? INT32_MAX : chunk;
+    return CORE_OK;
+}
+
 int core_debug_wait_clock(const uint64_t *readings_ns, int32_t count, uint64_t limit_ns, int32_t *given_up_at) {
     if (!readings_ns || !given_up_at || count < 1) return CORE_EINVAL;
     WaitClock clock(readings_ns[0]);

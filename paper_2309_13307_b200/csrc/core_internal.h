@@ -195,6 +195,7 @@ struct LsPass {
     int cluster, slice, warps, group_warps, columns, chunk_rows, slots;
     uint32_t slot_bytes, row_stride, ring_offset;
     size_t smem;
+    int hold_back = INT32_MAX;   // test: chunks of rows from this one on are never copied, so that a wait runs out
 };
 struct LsPoint {              // x, or x + gamma (x - x_prev) (the look-ahead point of Algorithm 4)
     const float *x;

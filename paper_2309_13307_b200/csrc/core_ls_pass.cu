@@ -70,6 +70,7 @@ struct PassArgs {
     uint32_t ring_offset;    // of the rings in shared memory, behind a buffer for the groups' sums where machines are kept apart
     int flush_floats;        // room for the groups' sums: that buffer, or the rings once the last row is done
     int reverse;             // rows from the last to the first (what an ascending pass left in L2 comes first)
+    int hold_back;           // test: chunks from this one on are never copied (by the first CTA of a cluster)
 };
 
 // What is read of A, as the kernel computes it and ls_pass_reads checks it on the host.
@@ -155,6 +156,8 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     __shared__ float xch[2][RB][WARPS * kPassMaxCluster];         // [parity][row][group][CTA][warp of the group]
     __shared__ __align__(8) uint64_t xch_bars[2][WARPS];          // [row parity][group]
     __shared__ double loss_sums[WARPS];
+    __shared__ int last_issued[WARPS];                            // [group] chunk copied last
+    __shared__ volatile int gave_up;                              // a wait ran out
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -170,11 +173,14 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     const bool edge = owned.edge;
     const int R = a.chunk_rows;
     const int chunks = (nrows + R - 1) / R;
+    int copied = rank == 0 ? min(chunks, a.hold_back) : chunks;    // chunks the leaders copy: all, but for a test, until a wait runs out
     const uint32_t row_bytes = (uint32_t)a.d * 4;
     const uint32_t ring = smem_u32(pass_smem) + a.ring_offset + (uint32_t)grp * a.slots * a.slot_bytes;
     const uint32_t bar0 = smem_u32(bars) + 8u * grp * a.slots;
     float *const flush = reinterpret_cast<float *>(pass_smem);
+    if (tid == 0) gave_up = 0;
     if (leader) {
+        last_issued[grp] = grp - GROUPS;
         for (int s = 0; s < a.slots; ++s) mbar_init(bar0 + 8 * s, 1);
         for (int f = 0; f < 2; ++f) mbar_init(smem_u32(&xch_bars[f][grp]), 1);
         fence_barrier_init();
@@ -214,6 +220,7 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
             copy(src, src + (uint32_t)count * row_bytes, dst);
         mbar_arrive(bar);
         src += src_step;
+        last_issued[grp] = k;
     };
     constexpr int stride = 32 * W, CB = C < 4 ? C : 4;             // CB columns are tested for together
     const int first = lane + 32 * wg;
@@ -229,7 +236,7 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     grid_wait();
     if (leader)
         for (int s = 0; s < a.slots; ++s)
-            if (grp + s * GROUPS < chunks) issue(grp + s * GROUPS, s);
+            if (grp + s * GROUPS < copied) issue(grp + s * GROUPS, s);
 
     float xv[C], acc[GRAD ? C : 1];
 #pragma unroll
@@ -247,8 +254,19 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     __syncthreads();                                    // barriers initialised, for every warp of a group
     if (MULTI && a.cluster > 1) cluster_sync();         // and every CTA of the cluster has started
 
+    // A wait that runs out ends its warp's part (lane by lane): it waits for nothing more, its leader copies nothing more, it
+    // sends nothing to the cluster (whose other warps then run out of time in turn), and the CTA's results become NaN, so
+    // that no wrong gradient or loss passes for a right one.  It goes on through its rows all the same, because the
+    // barriers it shares with other warps count it.  (Each of these conditions is on the path of every chunk or row: a test of
+    // `alive` before the refill in place of `copied`, or state kept in shared memory, cost 2 to 10 %.)
     bool alive = true;
     int flip = 0, xch_parity = 0;
+    auto give_up = [&](int code) {
+        alive = false;
+        copied = 0;
+        gave_up = 1;
+        atomicMax(&g_pass_status, code);
+    };
 
     // RBX rows whose first one starts at shared-memory address `at`, right-hand side bv in the lanes that get its sum.
     auto process = [&](auto batch, uint32_t at, float bv) {
@@ -303,12 +321,9 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
                 const int parts = W * a.cluster;                      // shares of a dot product
                 const uint32_t bar = smem_u32(&xch_bars[flip][grp]);
                 float *const share = &xch[flip][mine][grp * parts];
-                if (leader) mbar_arrive_expect(bar, 4u * parts * RBX);
-                if (sub < a.cluster) send_remote(smem_u32(share + rank * W + wg), bar, (uint32_t)sub, dot);
-                if (alive && !mbar_wait(bar, xch_parity)) {
-                    alive = false;
-                    atomicMax(&g_pass_status, 22);
-                }
+                if (leader && alive) mbar_arrive_expect(bar, 4u * parts * RBX);
+                if (sub < a.cluster && alive) send_remote(smem_u32(share + rank * W + wg), bar, (uint32_t)sub, dot);
+                if (alive && !mbar_wait(bar, xch_parity)) give_up(22);
                 __syncwarp();
                 dot = 0.f;
                 for (int q = sub; q < parts; q += SHARE) dot += share[q];
@@ -362,10 +377,7 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
         while (k < chunks && row < seg_end) {
             const int r0 = first_row(k), r1 = min(r0 + R, nrows);
             if (!loaded) {
-                if (alive && !mbar_wait(bar0 + 8 * slot, parity)) {
-                    alive = false;                      // no further waits: the CTA runs to its end and is reported
-                    atomicMax(&g_pass_status, 21);
-                }
+                if (alive && !mbar_wait(bar0 + 8 * slot, parity)) give_up(21);
                 loaded = true;
             }
             const uint32_t mis = ((uint32_t)unit_base + (uint32_t)r0 * row_bytes) & 15;
@@ -385,7 +397,7 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
                 // every warp of the group has read its part of the rows (in a cluster and between warps the exchange of
                 // the last row's shares told so): the slot may be refilled
                 __syncwarp();
-                if (leader && k + a.slots * GROUPS < chunks) issue(k + a.slots * GROUPS, slot);
+                if (leader && k + a.slots * GROUPS < copied) issue(k + a.slots * GROUPS, slot);
                 k += GROUPS;
                 b_now = b_next;
                 b_next = fetch_rhs(k + GROUPS);
@@ -421,6 +433,14 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
                     __syncthreads();
                 }
             }
+            if (gave_up) {                              // (threads overwrite what they wrote themselves)
+                if constexpr (GROUPS == 1) {
+#pragma unroll 1
+                    for (int col = first; col < dn; col += stride) out[col] = __int_as_float(0x7fffffff);
+                } else
+#pragma unroll 1
+                    for (int col = tid; col < dn; col += THREADS) out[col] = __int_as_float(0x7fffffff);
+            }
 #pragma unroll
             for (int c = 0; c < C; ++c) acc[c] = 0.f;
         }
@@ -436,12 +456,20 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
         if (tid == 0 && rank == 0) {
             double sum = 0.0;
             for (int w = 0; w < WARPS; ++w) sum += loss_sums[w];
-            a.loss_part[unit] = sum;
+            a.loss_part[unit] = gave_up ? __longlong_as_double(0x7fffffffffffffffll) : sum;
         }
     }
-    if (!alive && leader)                               // copies in flight must not outlive the CTA's shared memory
-        for (int s = 0; s < a.slots; ++s) mbar_wait(bar0 + 8 * s, parity);
-    if (MULTI && a.cluster > 1) cluster_sync();         // a CTA stays while others may still send to it
+    if (leader && !alive) {
+        // Copies in flight must not outlive the CTA's shared memory: the last ones issued, one per slot at most (the i-th
+        // went to slot i % slots and completes its phase i / slots).
+        const int issued = (last_issued[grp] - grp) / GROUPS + 1;
+        for (int i = max(issued - a.slots, 0); i < issued; ++i) mbar_wait(bar0 + 8 * (i % a.slots), (i / a.slots) & 1);
+    }
+    if (MULTI && a.cluster > 1) {
+        cluster_sync();                                 // a CTA stays while others may still send to it
+        if (!alive)                                     // ... and until what nobody waited for has arrived
+            for (int i = 0; i < 100; ++i) __nanosleep(1000);
+    }
 }
 
 // G[i][k] = inv_rows * sum of machine i's partial gradients, in the order of its units.
@@ -490,6 +518,7 @@ cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const floa
     a.slice = p.slice;
     a.chunk_rows = p.chunk_rows;
     a.slots = p.slots;
+    a.hold_back = p.hold_back;
     a.slot_bytes = p.slot_bytes;
     a.row_stride = p.row_stride;
     a.ring_offset = p.ring_offset;
