@@ -368,6 +368,13 @@ int core_debug_box_muller(core_ctx *ctx, const uint32_t *words_dev, int64_t nb, 
 int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t sm_count, int64_t out[10]);
 
 /*
+ * How core_round_host cuts the vectors: the number of slabs of the input (output = 0) or of the estimate (output != 0)
+ * in *count, and the lengths of the first `room` of them.  Host-only.
+ */
+int core_debug_host_slabs(int64_t d, int32_t n, int dtype, int32_t sm_count, int output, int64_t *lengths, int32_t room,
+                          int32_t *count);
+
+/*
  * What one pass over the data matrices of a least-squares problem (n x rows x d floats, their address `misaligned`
  * bytes beyond a multiple of 16) would touch beyond them, by its bulk copies and prefetches.  Host-only replay of the
  * kernel's own index arithmetic: reads nothing, touches no device for d <= 16384.

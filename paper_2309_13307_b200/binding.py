@@ -69,6 +69,8 @@ _SIGNATURES = {
                                 _c.POINTER(_c.c_uint32)], _c.c_int),
     "core_debug_project_plan": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32,
                                  _c.POINTER(_c.c_int64)], _c.c_int),
+    "core_debug_host_slabs": ([_c.c_int64, _c.c_int32, _c.c_int, _c.c_int32, _c.c_int, _c.POINTER(_c.c_int64), _c.c_int32,
+                               _c.POINTER(_c.c_int32)], _c.c_int),
     "core_debug_ls_reads": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32, _c.c_uint32,
                              _c.POINTER(_c.c_int64)], _c.c_int),
 }
@@ -140,6 +142,19 @@ def core_debug_project_plan(n: int, m: int, d: int, dtype: int = CORE_F32, sm_co
         raise CoreError(rc, "core_debug_project_plan")
     keys = ("nb", "jt", "uq", "tile_q", "tj", "tq", "grid_x", "grid_y", "tiles", "smem")
     return dict(zip(keys, (int(v) for v in out)))
+
+
+def core_debug_host_slabs(d: int, n: int = 1, dtype: int = CORE_F32, output: bool = False, sm_count: int = 148) -> list:
+    count = ctypes.c_int32(0)
+    args = (d, n, dtype, sm_count, int(output))
+    room = (ctypes.c_int64 * 1)()
+    rc = lib().core_debug_host_slabs(*args, room, 0, ctypes.byref(count))
+    if rc == CORE_OK:
+        room = (ctypes.c_int64 * count.value)()
+        rc = lib().core_debug_host_slabs(*args, room, count.value, ctypes.byref(count))
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_host_slabs")
+    return list(room)
 
 
 def core_debug_ls_reads(n: int, rows: int, d: int, machines_apart: bool, misaligned: int, sm_count: int = 148) -> tuple:

@@ -422,13 +422,37 @@ int core_round_host(core_ctx *ctx, const void *G_host, int dtype, int32_t n, int
     return rc;
 }
 
-// Length of the slab that starts at coordinate k0 of d: growing from `least` with what is behind it, shrinking to
-// `least` with what is ahead, multiples of 4096 but for the end of the vector.
-static int64_t next_slab(int64_t k0, int64_t d, int64_t least, int64_t most) {
+// How a vector of a host round is cut into slabs: growing from `least` with what is behind them, shrinking to `least` with
+// what is ahead, `most` at most, multiples of 4096 but for the end of the vector; from `whole_from` on whole multiples of `whole`.
+struct SlabRule {
+    int64_t least, most, whole_from, whole;
+};
+static int64_t next_slab(int64_t k0, int64_t d, const SlabRule &r) {
     const int64_t left = d - k0;
-    int64_t len = std::min(most, std::min(k0 + least, std::max(left / 2, least)));
+    int64_t len = std::min(r.most, std::min(k0 + r.least, std::max(left / 2, r.least)));
     len = std::max<int64_t>(len / 4096 * 4096, 4096);
-    return left - len < least / 2 ? (left <= most ? left : len) : len;
+    if (len >= r.whole_from) len = len / r.whole * r.whole;
+    return left - len < r.least / 2 ? (left <= r.most ? left : len) : len;
+}
+static int64_t slab_limit(int64_t d, int64_t bytes, size_t per_coordinate) {
+    const int64_t whole = (d + 4095) / 4096 * 4096, slab = bytes / (int64_t)per_coordinate / 4096 * 4096;
+    return slab < 4096 ? 4096 : slab > whole ? whole : slab;
+}
+// Slabs of at most 64 MiB of input over all machines and 16 MiB of output.  The first and the last ones are shorter: what is
+// not overlapped is the projection of the last slab and the reconstruction of the first one (and, where the kernels
+// are the slower side, the first copy in and the last out).
+static SlabRule input_slabs(int64_t d, int32_t n, size_t es) {
+    const int64_t most = slab_limit(d, (int64_t)64 << 20, es * (size_t)n);
+    // at least 256 KB per machine and copy
+    return {std::min(most, slab_limit(d, std::max((int64_t)4 << 20, (int64_t)n << 18), es * (size_t)n)), most, INT64_MAX, 1};
+}
+// Every slab is one launch of the reconstruction: those that its kernel for long vectors takes are whole waves of its CTAs, four
+// of them on 148 SMs.  (Slabs of 16 MiB, 4.6 waves, all ended in a wave that was not full: 2e8 coordinates at m = 4096
+// took 697 ms of kernels instead of 645.  Nine waves: the same there, but longer
+// steps up to them where the copies are the slower side: n = 1, d = 3e7, m = 64: 4.80 -> 4.90 ms.)
+static SlabRule output_slabs(int64_t d, int sm_count) {
+    const int64_t most = slab_limit(d, (int64_t)16 << 20, sizeof(float));
+    return {std::min(most, slab_limit(d, (int64_t)1 << 20, sizeof(float))), most, reconstruct_long(sm_count), reconstruct_wave(sm_count)};
 }
 
 static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t n, int64_t ldg, float *pbar_host,
@@ -456,28 +480,17 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
     }
     const size_t es = elem_size(dtype);
     const int64_t d = ctx->d;
-    // Slabs of at most 64 MiB of input over all machines and 16 MiB of output, all multiples of 4096 coordinates.  The
-    // first and the last ones are shorter (next_slab): what is not overlapped is the projection of the last slab and the
-    // reconstruction of the first one (and, where the kernels are the slower side, the first copy in and the last out).
-    const int64_t whole = (d + 4095) / 4096 * 4096;
-    auto limit = [&](int64_t bytes, size_t per_coordinate) {
-        int64_t slab = bytes / (int64_t)per_coordinate / 4096 * 4096;
-        return slab < 4096 ? 4096 : slab > whole ? whole : slab;
-    };
-    const int64_t in_most = limit((int64_t)64 << 20, es * (size_t)n), out_most = limit((int64_t)16 << 20, sizeof(float));
-    // at least 256 KB per machine and copy
-    const int64_t in_least = std::min(in_most, limit(std::max((int64_t)4 << 20, (int64_t)n << 18), es * (size_t)n));
-    const int64_t out_least = std::min(out_most, limit((int64_t)1 << 20, sizeof(float)));
+    const SlabRule in = input_slabs(d, n, es), out = output_slabs(d, ctx->sm_count);
     // the longest ones that occur, and the partial sums any of them needs
     int64_t in_len = 0, out_len = 0;
     size_t pb = 0;
     for (int64_t k0 = 0, len = 0; k0 < d; k0 += len) {
-        len = next_slab(k0, d, in_least, in_most);
+        len = next_slab(k0, d, in);
         if (len > in_len) in_len = len;
         pb = std::max(pb, row_partial_bytes(ctx, len));
     }
     for (int64_t k0 = 0, len = 0; k0 < d; k0 += len) {
-        len = next_slab(k0, d, out_least, out_most);
+        len = next_slab(k0, d, out);
         if (len > out_len) out_len = len;
     }
     in_len = (in_len + 7) / 8 * 8;                      // rows of a slab start on 16 bytes
@@ -514,7 +527,7 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
     int s = 0;
     for (int64_t k0 = 0; k0 < d; k0 += len, ++s) {
         const int b = s & 1;
-        len = next_slab(k0, d, in_least, in_most);
+        len = next_slab(k0, d, in);
         if (s >= 2) CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->in_free[b], 0));
         const char *const from = static_cast<const char *>(G_host) + (size_t)k0 * es;
         if ((size_t)ldg * es <= (size_t)INT32_MAX)          // one copy for all rows, where the stride is a legal pitch
@@ -538,7 +551,7 @@ static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t
     s = 0;
     for (int64_t k0 = 0; k0 < d; k0 += len, ++s) {
         const int b = s & 1;
-        len = next_slab(k0, d, out_least, out_most);
+        len = next_slab(k0, d, out);
         if (s >= 2) CORE_CUDA(ctx, cudaStreamWaitEvent(ctx->work_stream, ctx->out_free[b], 0));
         CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar, ctx->m, k0, k0 + len, out_buf[b], ctx->sm_count,
                                           ctx->work_stream));
@@ -869,6 +882,17 @@ int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t 
     const ProjectPlan p = make_project_plan(project_group(n, m), m, d, dtype, sm_count);
     const int64_t v[10] = {p.nb, p.jt, p.uq, p.tile_q, p.tj, p.tq, p.grid_x, p.grid_y, p.tiles, (int64_t)p.smem};
     for (int i = 0; i < 10; ++i) out[i] = v[i];
+    return CORE_OK;
+}
+
+int core_debug_host_slabs(int64_t d, int32_t n, int dtype, int32_t sm_count, int output, int64_t *lengths, int32_t room, int32_t *count) {
+    if (!lengths || !count || d < 1 || n < 1 || !valid_dtype(dtype) || sm_count < 1 || room < 0) return CORE_EINVAL;
+    const SlabRule rule = output ? output_slabs(d, sm_count) : input_slabs(d, n, elem_size(dtype));
+    *count = 0;
+    for (int64_t k0 = 0, len = 0; k0 < d; k0 += len, ++*count) {
+        len = next_slab(k0, d, rule);
+        if (*count < room) lengths[*count] = len;
+    }
     return CORE_OK;
 }
 

@@ -157,6 +157,9 @@ struct MessageParts {
     int chunks;
     int n;
 };
+// Coordinates from which the kernel for long vectors takes over, and those that one wave of its CTAs covers.
+int64_t reconstruct_long(int sm_count);
+int64_t reconstruct_wave(int sm_count);
 bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count);
 cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, int32_t m,
                                int64_t k_begin, int64_t k_end, float *out, int sm_count,

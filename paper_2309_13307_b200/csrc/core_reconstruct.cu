@@ -317,6 +317,9 @@ unsigned grid_for(int64_t items, int threads, int cap) {
 
 // Too few groups of the long-vector kernel to go round evenly?
 static bool short_vector(int64_t nq, int sm_count) { return (nq + kGroupQ - 1) / kGroupQ < 8 * (int64_t)sm_count; }
+constexpr int kRecCtas = 3;                       // resident CTAs of the long-vector kernel per SM (register-limited)
+int64_t reconstruct_long(int sm_count) { return 8 * (int64_t)sm_count * kGroupQ * 4; }
+int64_t reconstruct_wave(int sm_count) { return kRecCtas * (int64_t)sm_count * kGroupQ * 4; }
 
 // Every CTA forms the whole message: worth it while that is at most eight loads per thread (with 32, d = 8192 and m = 64, the
 // launch it saves was the cheaper one: 100.7 against 105.9 us a step).
@@ -376,7 +379,7 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, i
             default: return go(reconstruct_small_kernel<1>);
         }
     }
-    int64_t grid = (int64_t)sm_count * 3;     // three resident CTAs per SM (register-limited)
+    int64_t grid = (int64_t)sm_count * kRecCtas;
     if (grid > groups) grid = groups;
     return launch_chained(true, reconstruct_kernel, dim3((unsigned)grid), dim3(kThreads), 0, stream, a);
 }
