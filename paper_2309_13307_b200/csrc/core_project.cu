@@ -10,7 +10,6 @@
 // vector group.  Sums are kept in two levels (per tile, then across tiles) to bound the
 // fp32 chain length, reduced across the ql lanes in a fixed order, and written as one
 // partial P per CTA column; a second kernel adds the columns in ascending order.
-#include "core_finish.cuh"
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -280,56 +279,6 @@ cudaError_t launch_typed(const ProjectPlan &plan, const ProjectArgs &args, int d
     return launch_tiled<NB, JT, UQ, tile_q_for(NB)>(plan, args, dtype, stream);
 }
 
-__global__ void finish_project_kernel(const float *__restrict__ partial, int chunks, int n, int m,
-                                      float *__restrict__ P, int accumulate) {
-    grid_trigger();
-    grid_wait();
-    __shared__ float slices[kFinishSlices][32];
-    const int64_t idx = (int64_t)blockIdx.x * 32 + threadIdx.x;
-    const int64_t total = (int64_t)n * m;
-    slices[threadIdx.y][threadIdx.x] = idx < total ? finish_slice(partial, chunks, total, idx, threadIdx.y) : 0.f;
-    __syncthreads();
-    if (threadIdx.y != 0 || idx >= total) return;
-    const float s = finish_join(&slices[0][threadIdx.x], 32);
-    P[idx] = accumulate ? P[idx] + s : s;
-}
-
-__global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, float *__restrict__ pbar) {
-    grid_trigger();
-    grid_wait();
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
-    float s = 0.f;
-    for (int i = 0; i < n; ++i) s += __ldcg(P + (int64_t)i * m + j);
-    pbar[j] = s / (float)n;
-}
-
-// Both of the above in one launch for a single group of machines whose messages nobody asks for:
-// the same sums in the same order, so pbar is bitwise what the two kernels give.
-// A CTA takes eight vectors, so that sixteen machines' slices are in flight together (32 vectors and four machines: 9.3 us
-// for 22 machines, 232 vectors).
-constexpr int kFinishMachines = 16;
-constexpr int kFinishVectors = 8;
-__global__ void finish_aggregate_kernel(const float *__restrict__ partial, int chunks, int n, int m,
-                                        float *__restrict__ pbar) {
-    grid_trigger();
-    grid_wait();
-    __shared__ float slices[kFinishMachines][kFinishSlices][kFinishVectors];
-    const int lane = threadIdx.x, slice = threadIdx.y, row = threadIdx.z;
-    const int j = blockIdx.x * kFinishVectors + lane;
-    const int64_t total = (int64_t)n * m;
-    float sum = 0.f;                    // kept by the first kFinishVectors threads
-    for (int i0 = 0; i0 < n; i0 += kFinishMachines) {
-        const int i = i0 + row;
-        slices[row][slice][lane] = i < n && j < m ? finish_slice(partial, chunks, total, (int64_t)i * m + j, slice) : 0.f;
-        __syncthreads();
-        if (slice == 0 && row == 0)
-            for (int r = 0; r < kFinishMachines && i0 + r < n; ++r) sum += finish_join(&slices[r][0][lane], kFinishVectors);
-        __syncthreads();
-    }
-    if (slice == 0 && row == 0 && j < m) pbar[j] = sum / (float)n;
-}
-
 int ilog2(int x) {
     int l = 0;
     while ((1 << l) < x) ++l;
@@ -441,25 +390,6 @@ cudaError_t launch_project(const ProjectPlan &plan, const RoundKeys &keys, uint3
         case 8: return launch_typed<8, 2, 2>(plan, a, dtype, stream);
         default: return launch_typed<16, 2, 1>(plan, a, dtype, stream);
     }
-}
-
-cudaError_t launch_finish_project(const float *partial, int chunks, int32_t n, int32_t m, float *P,
-                                  bool accumulate, cudaStream_t stream) {
-    const int64_t total = (int64_t)n * m;
-    return launch_chained(true, finish_project_kernel, dim3((unsigned)((total + 31) / 32)), dim3(32, kFinishSlices), 0, stream, partial,
-                          chunks, n, m, P, accumulate ? 1 : 0);
-}
-
-cudaError_t launch_finish_aggregate(const float *partial, int chunks, int32_t n, int32_t m, float *pbar,
-                                    cudaStream_t stream) {
-    const int rows = n < kFinishMachines ? n : kFinishMachines;
-    return launch_chained(true, finish_aggregate_kernel, dim3((m + kFinishVectors - 1) / kFinishVectors),
-                          dim3(kFinishVectors, kFinishSlices, rows), 0, stream, partial, chunks, n, m, pbar);
-}
-
-cudaError_t launch_aggregate(const float *P, int32_t n, int32_t m, float *pbar, cudaStream_t stream) {
-    const int threads = 128;
-    return launch_chained(true, aggregate_kernel, dim3((m + threads - 1) / threads), dim3(threads), 0, stream, P, n, m, pbar);
 }
 
 }  // namespace core
