@@ -74,10 +74,9 @@ def test_least_squares_workload_200_iterations(core_mod):
 
 @pytest.mark.parametrize("n,rows,d,m", [(8, 256, 4096, 64), (3, 50, 1001, 8)])
 def test_step_equals_its_parts(core_mod, n, rows, d, m):
-    """core_gd_step never stores the machine gradients (where the single-pass gradient kernel applies the
-    projection adds their partial sums while it stages its tiles).  Building the same step from the entry
-    points that do store them - gradients, round, update - must give the same iterate: the sums are the same
-    and taken in the same order, so only the final multiply-add may round differently."""
+    """core_gd_step never stores the machine gradients (where the single pass over A applies the
+    projection adds the partial sums of its CTAs while it stages its tiles).  Building the same step from the entry
+    points that do store them - gradients, round, update - must give the same iterate up to the order of the sums."""
     ls_in = core_inputs.least_squares(n=n, rows=rows, d=d, seed=3, device="cuda")
     h = 0.37
     x0 = core_inputs.gradients(1, d, seed=5, device="cuda")[0].contiguous()
