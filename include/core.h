@@ -118,12 +118,15 @@ int core_device_status(int32_t *status_out);
  * step; Algorithm 2, "machine i sends p_ij").
  *   G_dev   n rows of d elements, row i at element offset i*ldg (ldg >= d),
  *           dtype CORE_F32 (float) or CORE_BF16 (bfloat16, widened exactly).
- *           Rows whose byte address and stride are multiples of 16 take the
- *           asynchronous-copy path; any other alignment is handled by an
- *           element-wise path with the same result.
+ *           Rows may have any alignment.  Several rows whose byte addresses and
+ *           stride are multiples of 16 are copied asynchronously, others element by
+ *           element, with the same result; a single row is read 16 bytes at a time
+ *           wherever it starts.
  *   P_dev   n*m floats, row-major.
  * fp32 multiply-add with two-level fp32 accumulation and a fixed reduction
- * order: results are bitwise reproducible for a given (n, m, d, dtype).
+ * order: results are bitwise reproducible for a given (n, m, d, dtype).  (A row's
+ * message may differ in the last bits from the same row's among others: one row and
+ * several take different kernels.)
  * Machines are processed in groups: up to 64 per pass where the tensor-memory
  * kernel applies (9 or more machines, m >= 96; more than 32 only when m lets a CTA
  * hold 256 vectors, about m >= 256), otherwise up to 16.  The
@@ -152,7 +155,9 @@ int core_reconstruct(core_ctx *ctx, const float *pbar_dev, float *gtilde_dev);
  * reconstruct with the current t, then t <- t + 1.  pbar_dev (m floats) receives
  * the aggregated message; gtilde_dev (d floats) the estimate.  With several machines and at
  * least 2^25 = d*m Gaussians the mean gradient is projected instead of every machine's (the
- * message is linear in the gradients): the same pbar up to the order of the sums.
+ * message is linear in the gradients): the same pbar as core_project and core_aggregate give up
+ * to the order of the sums, and below that size the same bits.  From that size on the rows are
+ * added up by alignment class, so the last bits of pbar also depend on G_dev modulo 16 and on ldg.
  */
 int core_round(core_ctx *ctx, const void *G_dev, int dtype, int32_t n, int64_t ldg, float *pbar_dev,
                float *gtilde_dev);
@@ -358,8 +363,10 @@ int core_debug_gaussians(core_ctx *ctx, uint32_t j, uint64_t q0, int64_t nq, flo
 int core_debug_box_muller(core_ctx *ctx, const uint32_t *words_dev, int64_t nb, float *z_dev);
 
 /*
- * Launch geometry the projection would use for the first pass over n machines (at most 64 per pass),
- * m vectors and d coordinates on a device with sm_count SMs.  Host-only: touches no device.
+ * Launch geometry the projection of separate messages would use for the first pass over n machines (at most
+ * 64 per pass), m vectors and d coordinates on a device with sm_count SMs.  Host-only: touches no device.  n = 1
+ * gives the plan of the scalar kernel, which a single row takes only where core_debug_force_project_kernel asks for
+ * it: one row, and the combined row of a round, go through a kernel of their own.
  * out[0..9] = machines per pass (rounded up to a power of two; 16, 32 or 64 for the tensor-memory kernel), vectors per thread,
  * coordinate blocks per thread step, blocks per shared-memory tile, threads across
  * vectors, threads across blocks, CTAs across coordinates, CTAs across vectors,

@@ -14,7 +14,9 @@ cudaError_t allow_shared(const void *kernel, size_t bytes);
 
 // Launches a kernel of a chain: it may be scheduled while its predecessor in the stream drains (programmatic stream
 // serialisation), which hides its launch latency (1 to 1.5 us a kernel).  Such a kernel calls grid_wait() before it touches
-// global memory and reads what an earlier kernel wrote past the L1 cache (__ldcg).
+// global memory: what every earlier kernel of the stream wrote is then visible to its ordinary loads, cached in L1 or not.  It
+// is not to the read-only path, so no __ldg there, and no plain reads through `const T *__restrict__`, which the compiler
+// may turn into such loads: __ldcg, or pointers without __restrict__.
 struct ChainedLaunch {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attrs[2];

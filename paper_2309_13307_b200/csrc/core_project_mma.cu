@@ -231,6 +231,11 @@ project_mma_kernel(const __grid_constant__ MmaArgs a) {
 
 }  // namespace
 
+// Taken where the tensor-memory kernel's own rule declines (m = 64..95, 129..191).  Measured there (us at d = 8e6, n = 16: scalar,
+// this kernel, the tensor-memory kernel): fp32 m = 64 818, 1622, 1294; m = 80 1586, 1622, 1294; m = 150 3114, 3235, 2573; bf16
+// m = 64 821, 1368, 1267; m = 80 1591, 1368, 1266; m = 150 3130, 2726, 2517; the order is the same down to d = 2e4.  A CTA spans
+// 128 vectors and its warps generate for those that do not exist as well, so another kernel is the faster one
+// throughout this range: the line between them does not lie where it should.
 bool project_mma_applies(int32_t n_group, int32_t m) { return n_group > 8 && m >= 64; }
 
 void fill_project_mma_plan(ProjectPlan &p, int32_t m, int64_t d, int dtype, int sm_count) {

@@ -6,7 +6,8 @@ from it with the common vectors.  Here a rank is a machine (one process per GPU)
 local gradient and the reconstruction run in the library's kernels on the rank's GPU, and the exchange
 is one collective of m floats per rank over ``torch.distributed`` (NCCL on GPUs).  The messages are
 gathered, not summed in flight, and combined by ``core_aggregate`` in ascending machine order, so every
-rank holds bitwise the same mean, and the same one the single-GPU simulation of n machines produces.
+rank holds bitwise the same mean.  The single-GPU simulation of n machines produces the same one up to the
+order of its sums (it projects several rows, or their mean, where a rank projects one).
 
 Algorithm 5 (decentralised): no central machine.  In a gossip round every rank sends its current
 estimate of the mean message to its neighbours in the network W (the machines l with W[i][l] != 0) and
