@@ -220,7 +220,8 @@ int core_project_static(uint64_t seed, uint32_t t, int64_t d, int32_t m, const v
  * f(x) = (1/n) sum_i 1/(2 rows) ||A_i x - b_i||^2 : the ridge-separable form of
  * Section 4 with quadratic loss and no ridge term.  A_dev is n x rows x d floats
  * row-major, b_dev n x rows floats; both are borrowed (must outlive the handle).
- * The handle owns the gradient matrix G[n x d] and its partial sums.
+ * The handle owns the gradient matrix G[n x d] and its partial sums.  Rows of up to 131072 columns go through
+ * a pass whose waits are bounded: should one run out, results are NaN (see core_device_status).
  */
 int core_ls_create(core_ls **out, const float *A_dev, const float *b_dev, int32_t n, int32_t rows,
                    int64_t d);
