@@ -144,8 +144,7 @@ bool combine_first(const core_ctx *ctx, int32_t n) {
 }
 
 size_t row_partial_bytes(const core_ctx *ctx, int64_t d) {
-    const RowPlan plan = make_row_plan(ctx->m, d, ctx->sm_count);
-    return round_up((size_t)plan.grid_x * ctx->m * sizeof(float), 256);
+    return round_up((size_t)row_plan_columns(ctx->m, d, ctx->sm_count) * ctx->m * sizeof(float), 256);
 }
 
 // Bytes of partial sums the projection of n machines needs (largest group of a pass).
@@ -163,7 +162,7 @@ size_t partial_bytes(const core_ctx *ctx, int32_t n, int64_t d, int dtype) {
 // message (m floats) = <scale * sum of `rows` rows, xi_j> over coordinates [0, d), added to what is there if asked.
 int project_row_into(core_ctx *ctx, const void *G, int dtype, int32_t rows, int64_t ldg, float scale, int64_t d,
                      uint64_t q_base, float *partial, float *message, bool accumulate, cudaStream_t stream) {
-    const RowPlan plan = make_row_plan(ctx->m, d, ctx->sm_count);
+    const RowPlan plan = make_row_plan(G, dtype, rows, ldg, ctx->m, d, ctx->sm_count);
     CORE_CUDA(ctx, launch_project_row(plan, ctx->keys, ctx->t, G, dtype, rows, ldg, scale, d, ctx->m, q_base, partial, stream));
     CORE_CUDA(ctx, launch_finish_project(partial, plan.grid_x, 1, ctx->m, message, accumulate, stream));
     return CORE_OK;
@@ -346,7 +345,7 @@ static int apply_step_rule(core_ctx *ctx, const StepRule *rule, const float *pba
 // round leaves it to the reconstruction to finish the message.
 static int finish_round(core_ctx *ctx, const void *G, int dtype, int32_t rows, int64_t ldg, float scale, float *partial,
                         float *pbar_dev, float *out, const ReconstructEpilogue *epilogue, const StepRule *rule) {
-    const RowPlan plan = make_row_plan(ctx->m, ctx->d, ctx->sm_count);
+    const RowPlan plan = make_row_plan(G, dtype, rows, ldg, ctx->m, ctx->d, ctx->sm_count);
     CORE_CUDA(ctx, launch_project_row(plan, ctx->keys, ctx->t, G, dtype, rows, ldg, scale, ctx->d, ctx->m, 0, partial, ctx->stream));
     const MessageParts parts{partial, plan.grid_x, 1};
     const bool join = !rule && reconstruct_joins(plan.grid_x, 1, ctx->m, ctx->d, ctx->sm_count);
@@ -446,13 +445,14 @@ static SlabRule input_slabs(int64_t d, int32_t n, size_t es) {
     // at least 256 KB per machine and copy
     return {std::min(most, slab_limit(d, std::max((int64_t)4 << 20, (int64_t)n << 18), es * (size_t)n)), most, INT64_MAX, 1};
 }
-// Every slab is one launch of the reconstruction: those that its kernel for long vectors takes are whole waves of its CTAs, four
-// of them on 148 SMs.  (Slabs of 16 MiB, 4.6 waves, all ended in a wave that was not full: 2e8 coordinates at m = 4096
-// took 697 ms of kernels instead of 645.  Nine waves: the same there, but longer
-// steps up to them where the copies are the slower side: n = 1, d = 3e7, m = 64: 4.80 -> 4.90 ms.)
+// Every slab is one launch of the reconstruction.  Its kernel for long vectors shares any length out evenly; long slabs are
+// whole multiples of 96 units of 32 blocks per SM all the same, four of those multiples on 148 SMs, so that SMs have the same
+// number of units, three per warp.  (Twice as long: longer steps up to them where the copies are the slower
+// side: n = 1, d = 3e7, m = 64: 4.80 -> 4.90 ms.)
 static SlabRule output_slabs(int64_t d, int sm_count) {
     const int64_t most = slab_limit(d, (int64_t)16 << 20, sizeof(float));
-    return {std::min(most, slab_limit(d, (int64_t)1 << 20, sizeof(float))), most, reconstruct_long(sm_count), reconstruct_wave(sm_count)};
+    return {std::min(most, slab_limit(d, (int64_t)1 << 20, sizeof(float))), most,
+            (int64_t)sm_count << 14, 3 * ((int64_t)sm_count << 11)};
 }
 
 static int round_host_body(core_ctx *ctx, const void *G_host, int dtype, int32_t n, int64_t ldg, float *pbar_host,

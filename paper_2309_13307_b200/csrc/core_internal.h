@@ -118,8 +118,10 @@ struct RowPlan {
     int64_t tiles;
     size_t smem;
     bool chain;       // see chain_pays
+    bool turn;        // angles from the table (core_rng.cuh)
 };
-RowPlan make_row_plan(int32_t m, int64_t d, int sm_count);
+RowPlan make_row_plan(const void *G, int dtype, int32_t rows, int64_t ldg, int32_t m, int64_t d, int sm_count);
+int row_plan_columns(int32_t m, int64_t d, int sm_count);      // most CTA columns of any rows' plan
 cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype,
                                int32_t rows, int64_t ldg, float scale, int64_t d, int32_t m, uint64_t q_base,
                                float *partial, cudaStream_t stream);
@@ -159,9 +161,6 @@ struct MessageParts {
     int chunks;
     int n;
 };
-// Coordinates from which the kernel for long vectors takes over, and those that one wave of its CTAs covers.
-int64_t reconstruct_long(int sm_count);
-int64_t reconstruct_wave(int sm_count);
 bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count);
 cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, int32_t m,
                                int64_t k_begin, int64_t k_end, float *out, int sm_count,

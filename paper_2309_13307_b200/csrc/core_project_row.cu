@@ -6,31 +6,48 @@
 // are staged (n d additions) replaces the n d m multiply-adds of n separate messages by d m.
 //
 // What bounds it: the generator (see core_rng.cuh), like the other round kernels; with few vectors and many
-// rows, the reading of G.  A CTA has 8 generating warps and 2 staging warps.  The staging warps read the
+// rows, the reading of G.  A CTA has generating warps and a few staging warps.  The staging warps read the
 // rows of the next tile 16 bytes at a time (eight loads in flight per thread), add them up and store the
 // sum to one of two shared-memory tiles, next to the block-dependent half of Philox; rows that
 // do not start on a 16-byte boundary are read in aligned vectors all the same, summed per alignment class
 // and shifted into place with warp shuffles.  Where rows are many against the vectors, every warp stages and
-// then generates (TOGETHER), and the other CTA of the SM fills the gap.  The generating threads hold four
+// then generates, and the other CTA of the SM fills the gap.  The generating threads hold four
 // vectors each and walk the blocks of the tile: thread (jl, ql) of tj x tq, where tj = the number of vector
-// quadruples of the CTA row (any number, not a power of two: 100 vectors keep 250 of 256 threads busy).  The
+// quadruples of the CTA row (any number, not a power of two: 100 vectors keep 750 of 768 threads busy).  The
 // coordinates of a block are stored as (0, 2, 1, 3), so that one 16-byte read delivers the multiplicands of the
-// cosine and of the sine lanes of both pairs as ready register pairs and S (g_c (y sp) + g_s cs) is four packed
-// instructions per counter.  d = 2.5e7, m = 256: 5204 us = 1.23e12 Gaussians/s.
+// cosine and of the sine lanes of both pairs as ready register pairs and S (g_c cos + g_s sin) is two packed and two
+// scalar instructions per counter.
+//
+// Three modes.  kRowTurn, wherever there is work for it: angles from the table, one CTA of 24 generating and 4 staging warps
+// per SM, d = 2.5e7, m = 256: 5048 us = 1.30e12 Gaussians/s.  kRowShort: angles from the polynomials, two CTAs of 8 and 2
+// warps per SM (5325 us there), for short work.  kRowTogether: the same, all warps stage.  In kRowTurn the registers decide:
+// 72 per thread hold the loop only because the sums over tiles live in shared memory and scalar accumulators
+// (packed ones need pairs: 5138 us) and 32-bit counts go around it (64-bit tile numbers: 5095); 20 generating warps of 80 registers:
+// 5169, 28 of 64: 5144, two counters at a time: 5379.
 #include "core_internal.h"
 #include "core_sync.cuh"
 
 #include <cuda_bf16.h>
 
+#include <climits>
+#include <type_traits>
+
 namespace core {
 
 namespace {
 
-constexpr int kRowCompute = 256;                 // generating threads
-constexpr int kRowStagers = 64;                  // staging threads
-constexpr int kRowThreads = kRowCompute + kRowStagers;
 constexpr int kRowJT = 4;                        // vectors per generating thread
-constexpr int kRowWarps = kRowThreads / 32;
+
+// With the table of angles one CTA fills an SM, without it two do.
+template <bool TURN>
+struct RowCta {
+    static constexpr int kCompute = TURN ? 768 : 256;        // generating threads
+    static constexpr int kStagers = TURN ? 128 : 64;         // staging threads
+    static constexpr int kThreads = kCompute + kStagers;
+    static constexpr int kWarps = kThreads / 32;
+    static constexpr int kPerSm = TURN ? 1 : 2;
+    static constexpr int kTileBlocks = TURN ? 2048 : 1024;   // most blocks of a tile
+};
 
 struct RowArgs {
     const void *G;
@@ -209,15 +226,22 @@ __device__ __forceinline__ void row_stage_any(int stride, const RowArgs &a, int6
     }
 }
 
-template <typename GT, bool TOGETHER>
-__global__ void __launch_bounds__(kRowThreads, 2)
+enum RowMode { kRowShort, kRowTogether, kRowTurn };
+
+template <typename GT, RowMode MODE>
+__global__ void __launch_bounds__(RowCta<MODE == kRowTurn>::kThreads, RowCta<MODE == kRowTurn>::kPerSm)
 project_row_kernel(const __grid_constant__ RowArgs a) {
+    constexpr bool TOGETHER = MODE == kRowTogether, TURN = MODE == kRowTurn;
+    constexpr int kRowCompute = RowCta<TURN>::kCompute, kRowStagers = RowCta<TURN>::kStagers, kRowThreads = RowCta<TURN>::kThreads,
+                  kRowWarps = RowCta<TURN>::kWarps;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // two tiles of {coordinates of the combined row, QPart} per block, side by side so that a step addresses both
     // with one pointer (two separate arrays: 5426 against 5276 us at d = 2.5e7, m = 256)
-    float4 *const tile0 = reinterpret_cast<float4 *>(smem_raw);
+    float4 *const tile0 = reinterpret_cast<float4 *>(smem_raw + (TURN ? kTurnBytes + kRowJT * 4 * RowCta<true>::kCompute : 0));
+    const float2 *const turns = reinterpret_cast<const float2 *>(smem_raw);
+    float *const totals = reinterpret_cast<float *>(smem_raw + kTurnBytes);
     constexpr int kSegBlocks = 8 * RowVec<GT>::V;
-    constexpr int kFull = 1, kEmpty = 3;                     // barrier ids: kFull + stage, kEmpty + stage
+    constexpr int kFull = 1, kEmpty = 3, kLast = 5;          // barrier ids: kFull + stage, kEmpty + stage
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t tile_begin = a.tiles * (int64_t)blockIdx.x / gridDim.x;
@@ -232,6 +256,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         }
     };
 
+    if constexpr (TURN) fill_turn_table<kRowWarps>(reinterpret_cast<float2 *>(smem_raw), warp, lane);
     if (tile_begin < tile_end) fill_table(tile_begin, tile0, tid, kRowThreads);
     grid_wait();
 
@@ -283,68 +308,90 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     const int jbase = blockIdx.y * a.tj * kRowJT;
     float outer[kRowJT];
     JPart jp[kRowJT];
+    auto make_jp = [&](uint32_t q_hi) {
 #pragma unroll
-    for (int v = 0; v < kRowJT; ++v) outer[v] = 0.f;
-    uint32_t jp_q_hi = 0;
-    bool have_jp = false;
-    for (int64_t tile = tile_begin; tile < tile_end; ++tile) {
-        const int i = (int)(tile - tile_begin), st = TOGETHER ? 0 : i & 1;
+        for (int v = 0; v < kRowJT; ++v) jp[v] = philox_jpart((uint32_t)(jbase + jl + v * a.tj), q_hi, a.keys);
+    };
+#pragma unroll
+    for (int v = 0; v < kRowJT; ++v) {
+        outer[v] = 0.f;
+        if (TURN && tid < kRowCompute) totals[v * kRowCompute + tid] = 0.f;
+    }
+    // Few and short variables are carried around the loop: the registers are what limits the warps of an SM.
+    const int my_tiles = (int)(tile_end - tile_begin);
+    const int last_blocks = my_tiles > 0 ? blocks_of(tile_end - 1) : 0;
+    // the block, counted from this CTA's first, at which the high counter word changes (once in 2^32 blocks)
+    auto first_q = [&] { return a.q_base + (uint64_t)tile_begin * a.tile_q; };
+    const uint64_t to_change = 0x100000000ull - (first_q() & 0xFFFFFFFFull);
+    int change = to_change < (uint64_t)INT_MAX ? (int)to_change : INT_MAX;
+    make_jp((uint32_t)(first_q() >> 32));
+    for (int i = 0; i < my_tiles; ++i) {
+        const int st = TOGETHER ? 0 : i & 1;
+        const int blocks = i == my_tiles - 1 ? last_blocks : a.tile_q;
         if (i >= 1) {
             if constexpr (TOGETHER) {
                 __syncthreads();                             // everyone is done with the tile
-                row_stage_any<GT>(2, a, 4 * tile * a.tile_q, blocks_of(tile), warp, kRowWarps, 0, a.rows, lane, tile0);
-                fill_table(tile, tile0, tid, kRowThreads);
+                row_stage_any<GT>(2, a, 4 * (tile_begin + i) * a.tile_q, blocks, warp, kRowWarps, 0, a.rows, lane, tile0);
+                fill_table(tile_begin + i, tile0, tid, kRowThreads);
                 __syncthreads();
             } else {
                 bar_sync(kFull + st, kRowThreads);
             }
         }
-        const float4 *cur = tile0 + 2 * st * a.tile_q;
-        const int blocks = blocks_of(tile);
-        const uint64_t q0 = a.q_base + (uint64_t)tile * a.tile_q;
-        // blocks of this tile that share the high counter word of the first one (all of them but once in 2^32)
-        const uint64_t left = 0x100000000ull - (q0 & 0xFFFFFFFFull);
-        int upto = left < (uint64_t)blocks ? (int)left : blocks;
-        uint32_t q_hi = (uint32_t)(q0 >> 32);
-        float2 acc[kRowJT];
+        const float4 *const cur = tile0 + 2 * st * a.tile_q;
+        std::conditional_t<TURN, float, float2> acc[kRowJT];
 #pragma unroll
-        for (int v = 0; v < kRowJT; ++v) acc[v] = make_float2(0.f, 0.f);
-        int qq = ql;
+        for (int v = 0; v < kRowJT; ++v) acc[v] = {};
         if (active) {
-            for (;;) {
-                if (!have_jp || q_hi != jp_q_hi) {
-#pragma unroll
-                    for (int v = 0; v < kRowJT; ++v) jp[v] = philox_jpart((uint32_t)(jbase + jl + v * a.tj), q_hi, a.keys);
-                    jp_q_hi = q_hi;
-                    have_jp = true;
-                }
-                const float4 *entry = cur + 2 * qq;
-                for (; qq < upto; qq += a.tq, entry += 2 * a.tq) {
+            const float4 *entry = cur + 2 * ql;
+            for (int upto = min(blocks, change - i * a.tile_q);;) {
+                for (const float4 *const stop = cur + 2 * upto; entry < stop; entry += 2 * a.tq) {
                     const float4 g = entry[0], e = entry[1];
                     QPart qp;
                     qp.hi_b = __float_as_uint(e.x);
                     qp.lo_b = __float_as_uint(e.y);
                     qp.w3 = __float_as_uint(e.z);
-                    uint4 w[kRowJT];
-#pragma unroll
-                    for (int v = 0; v < kRowJT; ++v) w[v] = philox_combine(jp[v], qp, a.keys);
-                    BmParts r[kRowJT];
-                    box_muller_parts<kRowJT>(w, r);
                     const float2 gc = make_float2(g.x, g.y), gs = make_float2(g.z, g.w);
+                    if constexpr (TURN) {
+                        uint4 w[kRowJT];
+                        float2 l[kRowJT];
 #pragma unroll
-                    for (int v = 0; v < kRowJT; ++v) {
-                        const float2 c = __fmul2_rn(__fmul2_rn(r[v].y, r[v].sp), gc);
-                        acc[v] = __ffma2_rn(r[v].s, __ffma2_rn(r[v].cs, gs, c), acc[v]);
+                        for (int v = 0; v < kRowJT; ++v) w[v] = philox_combine(jp[v], qp, a.keys);
+                        bm_logs<kRowJT, true>(w, l);
+#pragma unroll
+                        for (int v = 0; v < kRowJT; ++v) {
+                            const TurnParts r = turn_parts(w[v], l[v], turns);
+                            const float2 t = __ffma2_rn(r.n, gs, __fmul2_rn(r.c, gc));
+                            acc[v] = fmaf(r.s.x, t.x, fmaf(r.s.y, t.y, acc[v]));
+                        }
+                    } else {
+                        uint4 w[kRowJT];
+                        BmParts r[kRowJT];
+#pragma unroll
+                        for (int v = 0; v < kRowJT; ++v) w[v] = philox_combine(jp[v], qp, a.keys);
+                        box_muller_parts<kRowJT>(w, r);
+#pragma unroll
+                        for (int v = 0; v < kRowJT; ++v) {
+                            const float2 c = __fmul2_rn(__fmul2_rn(r[v].y, r[v].sp), gc);
+                            acc[v] = __ffma2_rn(r[v].s, __ffma2_rn(r[v].cs, gs, c), acc[v]);
+                        }
                     }
                 }
                 if (upto == blocks) break;
                 upto = blocks;
-                ++q_hi;
+                change = INT_MAX;
+                make_jp((uint32_t)(first_q() >> 32) + 1);
             }
         }
 #pragma unroll
-        for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
-        if (!TOGETHER && tile + 2 < tile_end) bar_arrive(kEmpty + st, kRowThreads);
+        for (int v = 0; v < kRowJT; ++v) {
+            if constexpr (TURN) {
+                if (active) totals[v * kRowCompute + tid] += acc[v];
+            } else {
+                outer[v] += acc[v].x + acc[v].y;
+            }
+        }
+        if (!TOGETHER && i + 2 < my_tiles) bar_arrive(kEmpty + st, kRowThreads);
     }
 
     // The next kernel is let in only now: its CTAs, waiting beside this kernel's, would be in the way of the generating warps
@@ -353,30 +400,69 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
 
     // fixed-order sum over the ql lanes
     __syncthreads();
-    float *red = reinterpret_cast<float *>(smem_raw);
+    float *red = reinterpret_cast<float *>(tile0);
     const int plane = kRowJT * a.tj;
     if (active)
 #pragma unroll
-        for (int v = 0; v < kRowJT; ++v) red[ql * plane + v * a.tj + jl] = outer[v];
+        for (int v = 0; v < kRowJT; ++v) red[ql * plane + v * a.tj + jl] = TURN ? totals[v * kRowCompute + tid] : outer[v];
     __syncthreads();
+    int lanes = a.tq;
+    if constexpr (TURN) {
+        // in two levels where there are threads for it (one would add 384 lanes at m = 8: 5 us)
+        const int ranges = min(kRowCompute / plane, a.tq / 4);
+        if (ranges > 1) {
+            const int idx = tid % plane, range = tid / plane;
+            float s = 0.f;
+            if (range < ranges)
+                for (int l = a.tq * range / ranges; l < a.tq * (range + 1) / ranges; ++l) s += red[l * plane + idx];
+            bar_sync(kLast, kRowCompute);                    // the staging warps have gone
+            if (range < ranges) red[range * plane + idx] = s;
+            bar_sync(kLast, kRowCompute);
+            lanes = ranges;
+        }
+    }
     for (int idx = tid; idx < plane; idx += kRowCompute) {
         float s = 0.f;
-        for (int l = 0; l < a.tq; ++l) s += red[l * plane + idx];
-        if (jbase + idx < a.m) a.partial[(int64_t)blockIdx.x * a.m + jbase + idx] = s;
+        for (int l = 0; l < lanes; ++l) s += red[l * plane + idx];
+        if (jbase + idx < a.m) a.partial[(int64_t)blockIdx.x * a.m + jbase + idx] = TURN ? kTurnScale * s : s;
     }
 }
 
 }  // namespace
 
-RowPlan make_row_plan(int32_t m, int64_t d, int sm_count) {
+// Rows r and r + period have the same alignment; do all of them start on a 16-byte boundary?
+static int row_period(int dtype, int64_t ldg) {
+    int period = 1;
+    while ((int64_t)period * ldg % (dtype == 1 ? 8 : 4) != 0) period *= 2;
+    return period;
+}
+// Staging a row of a block costs more where rows have to be shifted into place; where rows are many against the
+// vectors the staging warps cannot keep up and all warps stage (us, two warps -> all: n = 8, m = 8: 451 -> 375;
+// n = 50, m = 21: 961 -> 728; unaligned n = 5, m = 8: 798 -> 484; but n = 32, m = 100: 1709 -> 1770).
+static bool row_together(int32_t rows, bool aligned, int32_t m) { return (int64_t)rows * (aligned ? 3 : 7) >= m; }
+
+// The table of angles pays from the microsecond it takes on, where the staging warps keep up with the faster
+// generation (one in seven instead of one in five): lines through measured shapes (us, without -> with; aligned rows, d = 1e7: n = 1,
+// m = 16: 145 -> 140; n = 5, m = 32: 537 -> 522 the round; n = 32, m = 100: 1649 -> 1584; but n = 4, m = 16: 300 -> 330, n = 8,
+// m = 32: 539 -> 549; shifted, d = 1e7: n = 7, m = 64: 1073 -> 1063; n = 5, m = 100 at d = 1e6: 178 -> 171; but n = 3, m = 32: 579 -> 603,
+// n = 16, m = 128: 2147 -> 2190).  By size (n = 1): d = 3e5, m = 64: 23.3 -> 21.8; d = 5e4, m = 400: 23.0 -> 22.8.
+static bool row_turn(int32_t rows, bool aligned, int32_t m, int64_t d) {
+    return d >= ((int64_t)1 << 24) / m && (aligned ? 11 * (int64_t)rows + 40 < 4 * (int64_t)m : 8 * (int64_t)rows + 10 < m);
+}
+
+static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
     RowPlan p{};
+    p.turn = turn;
+    const int compute = turn ? RowCta<true>::kCompute : RowCta<false>::kCompute, warps = turn ? RowCta<true>::kWarps : RowCta<false>::kWarps;
+    const int per_sm = turn ? RowCta<true>::kPerSm : RowCta<false>::kPerSm;
+    const int room = turn ? RowCta<true>::kTileBlocks : RowCta<false>::kTileBlocks;
     // Threads across vectors: one per quadruple, in as few CTA rows as keep at least 15/16 of the generating
     // threads busy (every CTA row stages the gradients again)
     const int quads = (m + kRowJT - 1) / kRowJT;
     double best = -1.0;
-    for (int g = (quads + kRowCompute - 1) / kRowCompute, tried = 0; tried < 8 && g <= quads; ++g, ++tried) {
-        const int tj = (quads + g - 1) / g, tq = kRowCompute / tj;
-        const double busy = (double)quads / g * tq / kRowCompute;
+    for (int g = (quads + compute - 1) / compute, tried = 0; tried < 8 && g <= quads; ++g, ++tried) {
+        const int tj = (quads + g - 1) / g, tq = compute / tj;
+        const double busy = (double)quads / g * tq / compute;
         if (busy > best + 0.02) {
             best = busy;
             p.grid_y = g;
@@ -386,12 +472,12 @@ RowPlan make_row_plan(int32_t m, int64_t d, int sm_count) {
         if (busy >= 15.0 / 16.0) break;
     }
     const int64_t nq = (d + 3) >> 2;
-    int64_t slots = (int64_t)sm_count * 2 / p.grid_y;             // CTAs across coordinates that are resident together
+    int64_t slots = (int64_t)sm_count * per_sm / p.grid_y;             // CTAs across coordinates that are resident together
     if (slots < 1) slots = 1;
     // blocks per tile: as many steps per tile and generating thread as fit (32, or 1024 blocks: two tiles take 64 KB),
     // and of the tile counts per CTA from there on the one that leaves the fewest steps to the CTA with most of them
     // (d = 1e6, m = 100: 104 -> 98 us)
-    const int64_t most = 32 * p.tq < 1024 ? 32 * p.tq : 1024 / p.tq * p.tq;
+    const int64_t most = 32 * p.tq < room ? 32 * p.tq : room / p.tq * p.tq;
     const int64_t least_tiles = (nq + slots * most - 1) / (slots * most);
     int64_t best_steps = -1;
     for (int64_t k = least_tiles; k <= 2 * least_tiles && k < least_tiles + 16; ++k) {
@@ -403,12 +489,22 @@ RowPlan make_row_plan(int32_t m, int64_t d, int sm_count) {
     }
     p.tiles = (nq + p.tile_q - 1) / p.tile_q;
     p.grid_x = (int)(slots < p.tiles ? slots : p.tiles);
-    p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * 2, d, m);
-    // two tiles, two tables, and the row ranges of a short first tile (at most kRowWarps segments of 64 blocks)
-    const size_t stage = 2 * (size_t)p.tile_q * (16 + 16) + (size_t)kRowWarps * 64 * 16;
+    p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * per_sm, d, m);
+    // two tiles, two tables, and the row ranges of a short first tile (at most warps segments of 64 blocks)
+    const size_t stage = 2 * (size_t)p.tile_q * (16 + 16) + (size_t)warps * 64 * 16;
     const size_t red = (size_t)p.tj * p.tq * kRowJT * 4;
-    p.smem = stage > red ? stage : red;
+    p.smem = (stage > red ? stage : red) + (turn ? kTurnBytes + kRowJT * 4 * RowCta<true>::kCompute : 0);
     return p;
+}
+
+RowPlan make_row_plan(const void *G, int dtype, int32_t rows, int64_t ldg, int32_t m, int64_t d, int sm_count) {
+    const bool aligned = row_period(dtype, ldg) == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
+    return plan_rows(row_turn(rows, aligned, m, d), m, d, sm_count);
+}
+
+int row_plan_columns(int32_t m, int64_t d, int sm_count) {
+    const int with = plan_rows(true, m, d, sm_count).grid_x, without = plan_rows(false, m, d, sm_count).grid_x;
+    return with > without ? with : without;
 }
 
 cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype, int32_t rows,
@@ -422,10 +518,8 @@ cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint3
     a.q_base = q_base;
     a.partial = partial;
     a.rows = rows;
-    const int v = dtype == 1 ? 8 : 4;
-    a.period = 1;
-    while ((int64_t)a.period * ldg % v != 0) a.period *= 2;
-    a.aligned = a.period == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0 && 4 * plan.tile_q % v == 0;
+    a.period = row_period(dtype, ldg);
+    a.aligned = a.period == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0 && 4 * plan.tile_q % (dtype == 1 ? 8 : 4) == 0;
     a.scale = scale;
     a.m = m;
     a.tile_q = plan.tile_q;
@@ -434,13 +528,14 @@ cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint3
     a.t = t;
     a.keys = keys;
     const dim3 grid(plan.grid_x, plan.grid_y);
-    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(kRowThreads), plan.smem, stream, a); };
-    // Staging a row of a block costs more where rows have to be shifted into place; where rows are many against the
-    // vectors two staging warps cannot keep up and all warps stage (us, two warps -> all: n = 8, m = 8: 451 -> 375;
-    // n = 50, m = 21: 961 -> 728; unaligned n = 5, m = 8: 798 -> 484; but n = 32, m = 100: 1709 -> 1770).
-    const bool together = (int64_t)rows * (a.aligned ? 3 : 7) >= m;
-    if (dtype == 1) return together ? go(project_row_kernel<__nv_bfloat16, true>) : go(project_row_kernel<__nv_bfloat16, false>);
-    return together ? go(project_row_kernel<float, true>) : go(project_row_kernel<float, false>);
+    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(plan.turn ? RowCta<true>::kThreads : RowCta<false>::kThreads), plan.smem, stream, a); };
+    const bool together = row_together(rows, a.aligned, m);
+    auto pick = [&](auto element) {
+        using GT = decltype(element);
+        if (plan.turn) return go(project_row_kernel<GT, kRowTurn>);
+        return together ? go(project_row_kernel<GT, kRowTogether>) : go(project_row_kernel<GT, kRowShort>);
+    };
+    return dtype == 1 ? pick(__nv_bfloat16{}) : pick(float{});
 }
 
 }  // namespace core

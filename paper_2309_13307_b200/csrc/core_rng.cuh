@@ -153,6 +153,8 @@ __device__ __forceinline__ uint4 philox_combine(const JPart &jp, const QPart &qp
 
 constexpr uint32_t kNearOneWord = 0xFFC00000u;   // words with v = 1 - u < 2^-10
 
+__device__ __forceinline__ float2 bm_splat(float c) { return make_float2(c, c); }
+
 // -log2(1 - v) = (v + v^2/2 + v^3/3 + v^4/4 + ...) / ln 2
 __device__ __forceinline__ float bm_near_one(float v) {
     float s = fmaf(v, 0.36067376f, 0.48089835f);
@@ -160,8 +162,12 @@ __device__ __forceinline__ float bm_near_one(float v) {
     s = fmaf(s, v, 1.44269504f);
     return s * v;
 }
-
-__device__ __forceinline__ float2 bm_splat(float c) { return make_float2(c, c); }
+__device__ __forceinline__ float2 bm_near_one(float2 v) {
+    float2 s = __ffma2_rn(v, bm_splat(0.36067376f), bm_splat(0.48089835f));
+    s = __ffma2_rn(s, v, bm_splat(0.72134752f));
+    s = __ffma2_rn(s, v, bm_splat(1.44269504f));
+    return __fmul2_rn(s, v);
+}
 
 // log2 u (negative) of the two radius words of a call (lanes x, y = pair a, pair b) by the
 // hardware log2; u itself is returned for the rare correction.
@@ -175,9 +181,34 @@ __device__ __forceinline__ float2 bm_log2(uint4 w, float2 &u) {
     return l;
 }
 
-__device__ __forceinline__ void bm_fix_near_one(uint4 w, float2 u, float2 &l) {
-    if (w.x >= kNearOneWord) l.x = bm_near_one(1.0f - u.x);
-    if (w.z >= kNearOneWord) l.y = bm_near_one(1.0f - u.y);
+// l of N calls.  The rare near-one correction of all 2N radii sits behind one test, which leaves the N evaluations in one
+// straight-line block for the instruction scheduler.  A warp finds some radius of its 64 N near one in a fifth of the cases,
+// but rarely more than one: with EACH the calls are then tested one by one, which suits the kernels that take the angle
+// from the table (0.9 % faster; those with the polynomials are 1 to 2 % slower with it).
+template <int N, bool EACH>
+__device__ __forceinline__ void bm_logs(const uint4 (&w)[N], float2 (&l)[N]) {
+    float2 u[N];
+    uint32_t top = 0u;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        l[c] = bm_log2(w[c], u[c]);
+        top = __vimax3_u32(top, w[c].x, w[c].z);
+    }
+    if (EACH ? __builtin_expect(top >= kNearOneWord, 0) : top >= kNearOneWord) {
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            if constexpr (EACH) {
+                if (__builtin_expect(max(w[c].x, w[c].z) >= kNearOneWord, 0)) {
+                    const float2 s = bm_near_one(__fadd2_rn(bm_splat(1.0f), make_float2(-u[c].x, -u[c].y)));
+                    if (w[c].x >= kNearOneWord) l[c].x = s.x;
+                    if (w[c].z >= kNearOneWord) l[c].y = s.y;
+                }
+            } else {
+                if (w[c].x >= kNearOneWord) l[c].x = bm_near_one(1.0f - u[c].x);
+                if (w[c].z >= kNearOneWord) l[c].y = bm_near_one(1.0f - u[c].y);
+            }
+        }
+    }
 }
 
 // The rest of Box-Muller given l with |l| = -log2 u of the two pairs (the sign of l is ignored:
@@ -225,39 +256,20 @@ __device__ __forceinline__ float4 bm_finish(uint4 w, float2 l) {
     return make_float4(zc.x, zs.x, zc.y, zs.y);
 }
 
-// N calls at once: the rare near-one correction of all 2N radii sits behind one test, which
-// leaves the N evaluations in one straight-line block for the instruction scheduler.
+// N calls at once.
 template <int N>
 __device__ __forceinline__ void box_muller4xN(const uint4 (&w)[N], float4 (&z)[N]) {
-    float2 u[N], l[N];
-    uint32_t top = 0u;
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-        l[c] = bm_log2(w[c], u[c]);
-        top = __vimax3_u32(top, w[c].x, w[c].z);
-    }
-    if (top >= kNearOneWord) {
-#pragma unroll
-        for (int c = 0; c < N; ++c) bm_fix_near_one(w[c], u[c], l[c]);
-    }
+    float2 l[N];
+    bm_logs<N, false>(w, l);
 #pragma unroll
     for (int c = 0; c < N; ++c) z[c] = bm_finish(w[c], l[c]);
 }
 
-// The factors of N calls (same near-one handling as box_muller4xN).
+// The factors of N calls.
 template <int N>
 __device__ __forceinline__ void box_muller_parts(const uint4 (&w)[N], BmParts (&r)[N]) {
-    float2 u[N], l[N];
-    uint32_t top = 0u;
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-        l[c] = bm_log2(w[c], u[c]);
-        top = __vimax3_u32(top, w[c].x, w[c].z);
-    }
-    if (top >= kNearOneWord) {
-#pragma unroll
-        for (int c = 0; c < N; ++c) bm_fix_near_one(w[c], u[c], l[c]);
-    }
+    float2 l[N];
+    bm_logs<N, false>(w, l);
 #pragma unroll
     for (int c = 0; c < N; ++c) r[c] = bm_parts(w[c], l[c]);
 }
@@ -267,6 +279,99 @@ __device__ __forceinline__ float4 box_muller4(uint4 w) {
     float4 zs[1];
     box_muller4xN<1>(ws, zs);
     return zs[0];
+}
+
+// ---- Box-Muller with the angle from a table ----------------------------------------------
+// Long launches take sine and cosine from a table of kTurnEntries angles in shared memory (64 KB): the 13 top bits of the
+// word name the entry, the other ten bits used an angle delta of at most pi/8192 about its middle, and
+//   cos(theta) = C - S delta,   sin(theta) = S + C delta.
+// What is left out, 1 - cos(delta) <= 7.4e-8, is met by its mean in the scale of the entries.  Every integer and every fp32
+// instruction costs the schedulers two cycles here (scalar fp32: one; wide multiplies: two of their four; loads from shared
+// memory: about one), so it is their number that counts: 3 integer, 2.5 fp32 instructions and a load per angle in place of
+// 3 and 6.5.  116 -> 108 cycles per counter in the reconstruction, and closer to Box-Muller than the polynomials: rms error
+// 7.5e-8 against 1.02e-7, worst 1.2e-6 as there.  (A copy of 512 entries per lane, free of bank conflicts but in need of
+// second-order terms: 117.  Two loads of 4 bytes instead of one of 8, the products packed: 110.  4096 entries: rms error 1.27e-7.)
+//
+// The table comes without the factor kTurnScale = sqrt(2 ln 2): values below 1 are twice as finely spaced, and the factor is
+// applied where a sum ends.  Its fp32 rounding, and the bias of the hardware's log2 and square root (the radius is 1.5e-7
+// too small at first order, of which 3e-8 is best taken back: more makes the longest radii worse), are in the entries.
+constexpr int kTurnBits = 13;
+constexpr int kTurnEntries = 1 << kTurnBits;
+constexpr int kTurnBytes = kTurnEntries * 8;
+constexpr float kTurnScale = 1.1774100225154747f;
+
+constexpr double turn_series(double x, double term, int k) {      // x^k/k! - x^(k+2)/(k+2)! + ...
+    double sum = 0.0;
+    for (; k < 40; k += 2) {
+        sum += term;
+        term = -term * x * x / ((k + 1) * (k + 2));
+    }
+    return sum;
+}
+// The entries are made in place by an angle addition: 256 coarse angles in two floats each, 32 fine ones (cosine minus one).
+constexpr int kTurnFine = 32;
+struct TurnSeed {
+    float4 coarse[kTurnEntries / kTurnFine];      // {C, C's remainder, S, S's remainder}
+    float2 fine[kTurnFine];                       // {cos - 1, sin}
+};
+constexpr TurnSeed make_turn_seed() {
+    constexpr double pi = 3.14159265358979323846, delta = pi / kTurnEntries;
+    constexpr double scale = 1.17741002251547469101 / (double)kTurnScale * (1.0 - delta * delta / 6.0) * (1.0 + 3e-8);
+    TurnSeed t{};
+    for (int h = 0; h < kTurnEntries / kTurnFine; ++h) {
+        const double a = 2.0 * pi * (h + 0.5) / (kTurnEntries / kTurnFine) - pi;        // series in (-pi, pi), then negated
+        const double c = -scale * turn_series(a, 1.0, 0), s = -scale * turn_series(a, a, 1);
+        t.coarse[h].x = (float)c;
+        t.coarse[h].y = (float)(c - (double)t.coarse[h].x);
+        t.coarse[h].z = (float)s;
+        t.coarse[h].w = (float)(s - (double)t.coarse[h].z);
+    }
+    for (int l = 0; l < kTurnFine; ++l) {
+        const double a = 2.0 * pi * (l + 0.5 - kTurnFine / 2) / kTurnEntries;
+        t.fine[l].x = (float)-(a * a / 2.0 - a * a * a * a / 24.0);
+        t.fine[l].y = (float)turn_series(a, a, 1);
+    }
+    return t;
+}
+static __device__ const TurnSeed kTurnSeed = make_turn_seed();
+
+// Filled by WARPS warps of a CTA; the caller synchronises.  A warp reads its coarse angles in one load, a lane each.
+template <int WARPS>
+__device__ __forceinline__ void fill_turn_table(float2 *table, int warp, int lane) {
+    constexpr int kCoarse = kTurnEntries / kTurnFine, kMine = (kCoarse + WARPS - 1) / WARPS;
+    static_assert(kMine <= 32, "a coarse angle per lane");
+    const float2 f = __ldg(&kTurnSeed.fine[lane]);
+    const float4 mine = __ldg(&kTurnSeed.coarse[min(warp + lane * WARPS, kCoarse - 1)]);
+#pragma unroll 4
+    for (int i = 0; i < kMine; ++i) {
+        const int h = warp + i * WARPS;
+        const float4 g = make_float4(__shfl_sync(0xffffffffu, mine.x, i), __shfl_sync(0xffffffffu, mine.y, i),
+                                     __shfl_sync(0xffffffffu, mine.z, i), __shfl_sync(0xffffffffu, mine.w, i));
+        // C cos - S sin = C + (C (cos - 1) - S sin + C's remainder): what is rounded before the last sum is small
+        if (h < kCoarse)
+            table[h * kTurnFine + lane] = make_float2(g.x + fmaf(g.x, f.x, fmaf(-g.z, f.y, g.y)), g.z + fmaf(g.z, f.x, fmaf(g.x, f.y, g.w)));
+    }
+}
+
+// The four values of a call are kTurnScale times (s c, s n) of pair a (lanes x) and of pair b (lanes y).
+struct TurnParts {
+    float2 s;     // sqrt(-log2 u)
+    float2 c;     // cosine
+    float2 n;     // sine
+};
+__device__ __forceinline__ TurnParts turn_parts(uint4 w, float2 l, const float2 *table) {
+    constexpr uint32_t kFraction = ((1u << (32 - kTurnBits)) - 1u) & ~511u;
+    constexpr float kUnit = (float)(1u << (32 - kTurnBits)) / 8388608.0f;               // an entry's share of the mantissa
+    constexpr float kSlope = 6.283185307179586f / kTurnEntries / kUnit;
+    const float2 ta = table[w.y >> (32 - kTurnBits)], tb = table[w.w >> (32 - kTurnBits)];
+    const float2 f = make_float2(__uint_as_float((w.y & kFraction) | 0x3F800100u), __uint_as_float((w.w & kFraction) | 0x3F800100u));
+    const float2 delta = __ffma2_rn(f, bm_splat(kSlope), bm_splat(-(1.0f + 0.5f * kUnit) * kSlope));
+    TurnParts r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r.s.x) : "f"(fabsf(l.x)));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r.s.y) : "f"(fabsf(l.y)));
+    r.c = make_float2(fmaf(-ta.y, delta.x, ta.x), fmaf(-tb.y, delta.y, tb.x));
+    r.n = make_float2(fmaf(ta.x, delta.x, ta.y), fmaf(tb.x, delta.y, tb.y));
+    return r;
 }
 
 }  // namespace core

@@ -97,7 +97,7 @@ int core_project_static(uint64_t seed, uint32_t t, int64_t d, int32_t m, const v
     }
     const bool single = n == 1 && !project_kernel_forced();           // as core_project does
     ProjectPlan plan = make_project_plan(n, m, d, dtype, sm_count);
-    RowPlan row_plan = make_row_plan(m, d, sm_count);
+    RowPlan row_plan = make_row_plan(G_dev, dtype, 1, ldg, m, d, sm_count);
     // fewer CTA columns if the usual number would overflow the array (slower, same result up to
     // the order of the final additions)
     const size_t per_column = (size_t)n * (size_t)m;

@@ -1,0 +1,81 @@
+"""The kernels that take the angles from a table: the Gaussians they use, the reconstruction's line of (unit, vector) pairs over
+the warps, and the single-row projection's tiles, at sizes around the edges of units, warps, tables and CTA rows."""
+import numpy as np
+import pytest
+import torch
+
+import core_inputs
+import oracle
+from helpers import P_TOL, REC_TOL, rel_l2, row_norms
+
+pytestmark = pytest.mark.gpu
+
+XI_TOL = 4e-6       # |xi_gpu - xi_oracle|, element by element
+
+
+@pytest.fixture(scope="module")
+def core_mod():
+    import paper_2309_13307_b200 as core_mod
+    core_mod.lib()
+    return core_mod
+
+
+def windows(d, width=4096):
+    """First, middle and last coordinates of a vector, starting on whole blocks."""
+    middle, last = d // 2 // 4 * 4, max(0, d - width) // 4 * 4
+    return [(0, min(width, d)), (middle, min(middle + width, d)), (last, d)]
+
+
+@pytest.mark.parametrize("d,m,j", [(3_000_001, 9, 4), (94_720, 178, 0), (1_000_003, 100, 99)])
+def test_gaussians(core_mod, d, m, j):
+    """A message of one entry m reconstructs the vector of that entry itself; 3e6 coordinates hold radii down to 1e-3 and
+    up to 5.6 and every entry of the table some hundred times."""
+    pbar = torch.zeros(m, dtype=torch.float32, device="cuda")
+    pbar[j] = m
+    ctx = core_mod.Core(11, d, m)
+    ctx.core_set_round(6)
+    got = ctx.core_reconstruct(pbar).cpu().numpy().astype(np.float64)
+    want = oracle.xi_range(11, 6, j, 0, d)
+    assert np.abs(got - want).max() <= XI_TOL
+
+
+@pytest.mark.parametrize("d,m", [
+    (94_717, 178), (94_720, 1025), (94_721, 2049), (151_552, 111), (151_553, 112), (303_100, 64), (1_000_003, 17), (6_000_000, 3),
+    (17_000_001, 1), (17_000_001, 2), (100_003, 8192), (100_003, 8195), (700_001, 131),
+])
+def test_long_reconstructions(core_mod, d, m):
+    pbar = core_inputs.gradients(1, m, seed=d % 1000 + m).numpy()[0]
+    ctx = core_mod.Core(5, d, m)
+    ctx.core_set_round(2)
+    gt = ctx.core_reconstruct(torch.from_numpy(pbar).cuda()).cpu().numpy()
+    for k0, k1 in windows(d, 4096 if m < 1000 else 640):
+        assert rel_l2(gt[k0:k1], oracle.reconstruct_slice(5, 2, pbar.astype(np.float64), k0, k1)) <= REC_TOL
+
+
+def test_reconstructions_do_not_depend_on_what_ran_before(core_mod):
+    """Warps that share a unit meet in shared memory: the same bits on every launch."""
+    d, m = 151_600, 333
+    pbar = core_inputs.gradients(1, m, seed=1, device="cuda")[0]
+    ctx = core_mod.Core(5, d, m)
+    first = ctx.core_reconstruct(pbar).clone()
+    for _ in range(20):
+        assert torch.equal(ctx.core_reconstruct(pbar), first)
+
+
+@pytest.mark.parametrize("n,d,m,dtype,offset,pad", [
+    (1, 16_385, 1024, "f32", 0, 0), (1, 16_400, 1030, "bf16", 0, 8), (1, 5_600, 3073, "f32", 3, 0), (1, 100_003, 170, "bf16", 5, 0),
+    (1, 1_200_001, 14, "f32", 0, 0), (3, 600_001, 61, "f32", 0, 3), (4, 262_147, 130, "bf16", 1, 6), (20, 335_546, 101, "f32", 0, 2),
+])
+def test_projections(core_mod, n, d, m, dtype, offset, pad):
+    """One row through core_project, several through the mean gradient of a round."""
+    G = core_inputs.gradients(n, d + offset, seed=d + m, dtype=dtype, device="cuda", ld=d + offset + pad)[:, offset:]
+    ctx = core_mod.Core(7, d, m)
+    ctx.core_set_round(3)
+    mean = G.float().cpu().numpy().astype(np.float64).mean(axis=0, keepdims=True)
+    if n == 1:
+        got = ctx.core_project(G).cpu().numpy()[0]
+    else:
+        got = ctx.core_round(G)[0].cpu().numpy()
+    want = oracle.project(7, 3, m, np.ascontiguousarray(mean.astype(np.float32)))[0]
+    # fp32 rounding of the mean itself: 2^-24 of its norm at most, four decimal digits below the bar
+    assert np.abs(got - want).max() <= P_TOL * row_norms(mean.astype(np.float32))[0]
