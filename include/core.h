@@ -315,9 +315,8 @@ int core_ls_gradients(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G_o
 /* ---- failure paths, made on the host or bounded on the device (no counterpart in the paper) ---- */
 
 /*
- * Which projection kernel later calls use: -1 the library's choice by shape (default), 0 the scalar
- * kernel, 1 the warp-level tensor-core kernel where its shape limits allow, 2 the tensor-memory
- * (tcgen05) kernel for every group of machines it can take (up to 64).  Process-wide; for measuring where one kernel
+ * Which projection kernel later calls use: -1 the library's choice by shape (default), 0 or 1 the scalar
+ * kernel, 2 the tensor-memory (tcgen05) kernel for every group of machines it can take (up to 64).  Process-wide; for measuring where one kernel
  * overtakes the other and for testing each on shapes the default would not give it.
  */
 int core_debug_force_project_kernel(int kind);

@@ -187,7 +187,7 @@ def core_debug_pipe_cycles(kind: int, warps_per_scheduler: int = 4, iters: int =
 
 
 def core_debug_force_project_kernel(kind: int) -> None:
-    """-1: by shape (default); 0: scalar; 1: warp-level tensor cores; 2: tensor-memory kernel."""
+    """-1: by shape (default); 0 or 1: scalar; 2: tensor-memory kernel."""
     rc = lib().core_debug_force_project_kernel(int(kind))
     if rc != CORE_OK:
         raise CoreError(rc, "core_debug_force_project_kernel")

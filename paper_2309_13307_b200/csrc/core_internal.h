@@ -54,8 +54,8 @@ constexpr int kMaxGroupTc = 64;      // most machines one pass of the tensor-mem
 // Machines the next projection pass takes when n_left remain: up to 64 (32 where a CTA holds one group of
 // 128 vectors only) where the tensor-memory kernel applies to more than 16, otherwise at most 16.
 int32_t project_group(int32_t n_left, int32_t m);
-// Test hook: -1 = choose by shape (default); 0 = always the scalar kernel; 1 = the warp-level tensor-core
-// kernel where its shape limits allow; 2 = the tensor-memory kernel for any group of machines it can take.
+// Test hook: -1 = choose by shape (default); 0 or 1 = always the scalar kernel; 2 = the tensor-memory kernel for any group
+// of machines it can take.
 void project_force_kernel(int kind);
 bool project_kernel_forced();      // anything but -1
 
@@ -71,18 +71,11 @@ struct ProjectPlan {
     int grid_y;       // CTAs across vectors
     int64_t tiles;    // ceil(d / (4 * tile_q))
     size_t smem;      // dynamic shared memory per CTA
-    int mma;          // 0: scalar kernel; 1: warp-level tensor-core kernel; 2: tcgen05 kernel
+    bool tc;          // the tcgen05 kernel
     bool chain;       // see chain_pays
 };
 
 ProjectPlan make_project_plan(int32_t n_group, int32_t m, int64_t d, int dtype, int sm_count);
-
-// Tensor-core variant of the projection pass (core_project_mma.cu); same partial-sum layout.
-bool project_mma_applies(int32_t n_group, int32_t m);
-void fill_project_mma_plan(ProjectPlan &plan, int32_t m, int64_t d, int dtype, int sm_count);
-cudaError_t launch_project_mma(const ProjectPlan &plan, const RoundKeys &keys, uint32_t t, const void *G,
-                               int dtype, int32_t n, int64_t ldg, int64_t d, int32_t m, uint64_t q_base,
-                               float *partial, cudaStream_t stream);
 
 // tcgen05 variant (core_project_tc.cu): 128 or 256 vectors per CTA, up to project_tc_max_group(m) machines per
 // pass (N = 16, 32 or 64 of the instruction), accumulators in tensor memory; same partial-sum layout.  q_base must be a multiple of 64 blocks.  Its waits are bounded: a wait that

@@ -537,11 +537,12 @@ static int tc_vector_groups(int32_t m) {
 int32_t project_tc_max_group(int32_t m) { return tc_vector_groups(m) == 2 ? kTcMaxN : 32; }
 
 bool project_tc_applies(int32_t n_group, int32_t m) {
-    // enough machines for the tensor core to pay (with five or more the multiply-adds of the scalar kernel cost
-    // more issue slots than this kernel's staging and hand-over), and vectors that fill three quarters of the CTA rows
-    // (n = 30, m = 801: 94 -> 62 us a round against the warp-level kernel)
-    const int64_t rows = ((int64_t)m + kTcVectors - 1) / kTcVectors * kTcVectors;
-    return n_group >= kTcMinMachines && n_group <= project_tc_max_group(m) && (int64_t)m * 4 >= rows * 3;
+    // Enough machines for the tensor core to pay (with five or more the multiply-adds of the scalar kernel cost
+    // more issue slots than this kernel's staging and hand-over), and more vectors than the scalar kernel takes at half this
+    // one's rate: a CTA here generates for 128 whether they exist or not, one there for 64.  us a projection, scalar / this
+    // one, n = 16 fp32: d = 1e6, m = 64: 115 / 180, m = 65: 217 / 180, m = 129: 420 / 337, m = 300: 827 / 492; d = 2e4: 11.3 / 13.9,
+    // 15.6 / 13.8, 25.2 / 20.8, 42.8 / 20.8.  Passes of more than 16 machines stay with at least 96 vectors.
+    return n_group >= kTcMinMachines && n_group <= project_tc_max_group(m) && m > 64 && (n_group <= kMaxGroup || m >= 96);
 }
 
 template <int NT, int VG>
@@ -551,7 +552,7 @@ static size_t tc_smem_bytes(bool bf16) {
 
 void fill_project_tc_plan(ProjectPlan &p, int32_t n_group, int32_t m, int64_t d, int dtype, int sm_count) {
     const int vg = tc_vector_groups(m);
-    p.mma = 2;
+    p.tc = true;
     p.nb = n_group > 32 ? 64 : n_group > 16 ? 32 : 16;     // N of the instruction
     p.jt = 4 * vg;                     // producer thread = (lane, warp): 4 or 8 vectors x 1 block per stage
     p.uq = 1;
