@@ -360,7 +360,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                         bm_logs<kRowJT, true>(w, l);
 #pragma unroll
                         for (int v = 0; v < kRowJT; ++v) {
-                            const TurnParts r = turn_parts(w[v], l[v], turns);
+                            const TurnParts r = turn_parts(w[v], l[v], turns, a.keys);
                             const float2 t = __ffma2_rn(r.n, gs, __fmul2_rn(r.c, gc));
                             acc[v] = fmaf(r.s.x, t.x, fmaf(r.s.y, t.y, acc[v]));
                         }

@@ -131,7 +131,7 @@ __device__ __forceinline__ void turn_step(const uint4 *entries, const float2 *tu
     float2 c, n;
 #pragma unroll
     for (int s = 0; s < JS; ++s) {
-        const TurnParts r = turn_parts(w[s], l[s], turns);
+        const TurnParts r = turn_parts(w[s], l[s], turns, keys);
         const float2 ps = __fmul2_rn(make_float2(p[s], p[s]), r.s);
         c = s == 0 ? __fmul2_rn(ps, r.c) : __ffma2_rn(ps, r.c, c);
         n = s == 0 ? __fmul2_rn(ps, r.n) : __ffma2_rn(ps, r.n, n);

@@ -22,10 +22,13 @@ constexpr uint32_t kPhiloxMulB = 0xCD9E8D57u;  // multiplies counter word 2
 constexpr uint32_t kPhiloxKeyA = 0x9E3779B9u;  // key word 0 increment per round
 constexpr uint32_t kPhiloxKeyB = 0xBB67AE85u;  // key word 1 increment per round
 
-// Key schedule, expanded once on the host: a[r], b[r] are the key words of round r.
+// Key schedule, expanded once on the host: a[r], b[r] are the key words of round r.  The last word is a
+// constant that turn_parts() wants as a run-time value.
+constexpr uint32_t kTurnUnder = 0x3F800100u;
 struct RoundKeys {
     uint32_t a[10];
     uint32_t b[10];
+    uint32_t turn_under;
 };
 
 inline RoundKeys expand_keys(uint64_t seed) {
@@ -37,6 +40,7 @@ inline RoundKeys expand_keys(uint64_t seed) {
         a += kPhiloxKeyA;
         b += kPhiloxKeyB;
     }
+    k.turn_under = kTurnUnder;
     return k;
 }
 
@@ -152,6 +156,14 @@ __device__ __forceinline__ uint4 philox_combine(const JPart &jp, const QPart &qp
 // Worst absolute error over all 2^23 radius words and all 2^23 angle words: 1.2e-6.
 
 constexpr uint32_t kNearOneWord = 0xFFC00000u;   // words with v = 1 - u < 2^-10
+
+// (w & MASK) | under in one instruction: one holds a single constant, so where `under` is known to the compiler it makes two.
+template <uint32_t MASK>
+__device__ __forceinline__ float insert_bits(uint32_t w, uint32_t under) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(w), "n"(MASK), "r"(under));
+    return __uint_as_float(r);
+}
 
 __device__ __forceinline__ float2 bm_splat(float c) { return make_float2(c, c); }
 
@@ -289,7 +301,9 @@ __device__ __forceinline__ float4 box_muller4(uint4 w) {
 // instruction costs the schedulers two cycles here (scalar fp32: one; wide multiplies: two of their four; loads from shared
 // memory: about one), so it is their number that counts: 3 integer, 2.5 fp32 instructions and a load per angle in place of
 // 3 and 6.5.  116 -> 108 cycles per counter in the reconstruction, and closer to Box-Muller than the polynomials: rms error
-// 7.5e-8 against 1.02e-7, worst 1.2e-6 as there.  (A copy of 512 entries per lane, free of bank conflicts but in need of
+// 7.5e-8 against 1.02e-7, worst 1.2e-6 as there.  The two integer instructions that cut out the fraction are one where its upper bits
+// come from a kernel parameter (insert_bits): 107.4 -> 105.6 cycles, d = 2.5e7, m = 256: 4607 -> 4536 us; the same in the angles
+// of the polynomials made the tcgen05 projection 3 to 6 % slower and changed nothing elsewhere.  (A copy of 512 entries per lane, free of bank conflicts but in need of
 // second-order terms: 117.  Two loads of 4 bytes instead of one of 8, the products packed: 110.  4096 entries: rms error 1.27e-7.)
 //
 // The table comes without the factor kTurnScale = sqrt(2 ln 2): values below 1 are twice as finely spaced, and the factor is
@@ -359,12 +373,12 @@ struct TurnParts {
     float2 c;     // cosine
     float2 n;     // sine
 };
-__device__ __forceinline__ TurnParts turn_parts(uint4 w, float2 l, const float2 *table) {
+__device__ __forceinline__ TurnParts turn_parts(uint4 w, float2 l, const float2 *table, const RoundKeys &k) {
     constexpr uint32_t kFraction = ((1u << (32 - kTurnBits)) - 1u) & ~511u;
     constexpr float kUnit = (float)(1u << (32 - kTurnBits)) / 8388608.0f;               // an entry's share of the mantissa
     constexpr float kSlope = 6.283185307179586f / kTurnEntries / kUnit;
     const float2 ta = table[w.y >> (32 - kTurnBits)], tb = table[w.w >> (32 - kTurnBits)];
-    const float2 f = make_float2(__uint_as_float((w.y & kFraction) | 0x3F800100u), __uint_as_float((w.w & kFraction) | 0x3F800100u));
+    const float2 f = make_float2(insert_bits<kFraction>(w.y, k.turn_under), insert_bits<kFraction>(w.w, k.turn_under));
     const float2 delta = __ffma2_rn(f, bm_splat(kSlope), bm_splat(-(1.0f + 0.5f * kUnit) * kSlope));
     TurnParts r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r.s.x) : "f"(fabsf(l.x)));
