@@ -19,11 +19,14 @@
 // scalar instructions per counter.
 //
 // Three modes.  kRowTurn, wherever there is work for it: angles from the table, one CTA of 24 generating and 4 staging warps
-// per SM, d = 2.5e7, m = 256: 5048 us = 1.30e12 Gaussians/s.  kRowShort: angles from the polynomials, two CTAs of 8 and 2
+// per SM, d = 2.5e7, m = 256: 4904 us = 1.31e12 Gaussians/s.  kRowShort: angles from the polynomials, two CTAs of 8 and 2
 // warps per SM (5325 us there), for short work.  kRowTogether: the same, all warps stage.  In kRowTurn the registers decide:
 // 72 per thread hold the loop only because the sums over tiles live in shared memory and scalar accumulators
 // (packed ones need pairs: 5138 us) and 32-bit counts go around it (64-bit tile numbers: 5095); 20 generating warps of 80 registers:
 // 5169, 28 of 64: 5144, two counters at a time: 5379.
+// The generating warps take tiles over in three groups of eight, each with barriers of its own: with one barrier for all, every warp
+// waited for the slowest one at each tile (us, one group -> three: d = 2.5e7, m = 256: 4958 -> 4904; d = 1e6, m = 100:
+// 88.7 -> 87.9; eight rows, d = 1e7, the whole round: 3838 -> 3805).
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -44,6 +47,7 @@ struct RowCta {
     static constexpr int kCompute = TURN ? 768 : 256;        // generating threads
     static constexpr int kStagers = TURN ? 128 : 64;         // staging threads
     static constexpr int kThreads = kCompute + kStagers;
+    static constexpr int kGroups = TURN ? 3 : 1;             // of generating warps that take a tile over by themselves
     static constexpr int kWarps = kThreads / 32;
     static constexpr int kPerSm = TURN ? 1 : 2;
     static constexpr int kTileBlocks = TURN ? 2048 : 1024;   // most blocks of a tile
@@ -241,7 +245,9 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     const float2 *const turns = reinterpret_cast<const float2 *>(smem_raw);
     float *const totals = reinterpret_cast<float *>(smem_raw + kTurnBytes);
     constexpr int kSegBlocks = 8 * RowVec<GT>::V;
-    constexpr int kFull = 1, kEmpty = 3, kLast = 5;          // barrier ids: kFull + stage, kEmpty + stage
+    constexpr int kGroups = RowCta<TURN>::kGroups, kHandOver = kRowCompute / kGroups + kRowStagers;     // threads of a group's barriers
+    constexpr int kFull = 1, kEmpty = kFull + 2 * kGroups, kLast = kEmpty + 2 * kGroups;                // barrier ids: + 2 group + stage
+    static_assert(kLast < 16, "barriers of a CTA");
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t tile_begin = a.tiles * (int64_t)blockIdx.x / gridDim.x;
@@ -291,12 +297,13 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         // staging warps: tile i into stage i & 1 once the generating warps have left it
         for (int64_t tile = tile_begin + 1; tile < tile_end; ++tile) {
             const int i = (int)(tile - tile_begin), st = i & 1;
-            if (i >= 2) bar_sync(kEmpty + st, kRowThreads);
+            if (i >= 2)
+                for (int g = 0; g < kGroups; ++g) bar_sync(kEmpty + 2 * g + st, kHandOver);
             row_stage_any<GT>(2, a, 4 * tile * a.tile_q, blocks_of(tile), warp - kRowCompute / 32, kRowStagers / 32, 0, a.rows, lane,
                               tile0 + 2 * st * a.tile_q);
             fill_table(tile, tile0 + 2 * st * a.tile_q, tid - kRowCompute, kRowStagers);
             __threadfence_block();
-            bar_arrive(kFull + st, kRowThreads);
+            for (int g = 0; g < kGroups; ++g) bar_arrive(kFull + 2 * g + st, kHandOver);
         }
         __syncthreads();
         __syncthreads();
@@ -319,6 +326,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     }
     // Few and short variables are carried around the loop: the registers are what limits the warps of an SM.
     const int my_tiles = (int)(tile_end - tile_begin);
+    const int group2 = kGroups > 1 ? warp / (kRowCompute / 32 / kGroups) * 2 : 0;
     const int last_blocks = my_tiles > 0 ? blocks_of(tile_end - 1) : 0;
     // the block, counted from this CTA's first, at which the high counter word changes (once in 2^32 blocks)
     auto first_q = [&] { return a.q_base + (uint64_t)tile_begin * a.tile_q; };
@@ -335,7 +343,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                 fill_table(tile_begin + i, tile0, tid, kRowThreads);
                 __syncthreads();
             } else {
-                bar_sync(kFull + st, kRowThreads);
+                bar_sync(kFull + group2 + st, kHandOver);
             }
         }
         const float4 *const cur = tile0 + 2 * st * a.tile_q;
@@ -391,7 +399,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                 outer[v] += acc[v].x + acc[v].y;
             }
         }
-        if (!TOGETHER && i + 2 < my_tiles) bar_arrive(kEmpty + st, kRowThreads);
+        if (!TOGETHER && i + 2 < my_tiles) bar_arrive(kEmpty + group2 + st, kHandOver);
     }
 
     // The next kernel is let in only now: its CTAs, waiting beside this kernel's, would be in the way of the generating warps
