@@ -632,15 +632,15 @@ int core_ls_destroy(core_ls *ls) {
     return rc;
 }
 
-static int ls_gradients_into(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G) {
+static int ls_gradients_into(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G, float *clear = nullptr) {
     if (ls->machine_pass.units > 0) {
         CORE_CUDA(ctx, launch_ls_pass_gradients(ls->machine_pass, ls->A, ls->b, LsPoint{x_dev}, ls->d, ls->part, ctx->stream));
-        CORE_CUDA(ctx, launch_ls_pass_reduce(ls->machine_pass, ls->part, ls->d, 1.0f / (float)ls->rows, G, ctx->stream));
+        CORE_CUDA(ctx, launch_ls_pass_reduce(ls->machine_pass, ls->part, ls->d, 1.0f / (float)ls->rows, G, clear, ctx->stream));
         return CORE_OK;
     }
     CORE_CUDA(ctx, launch_ls_residual(ls->A, ls->b, x_dev, ls->n, ls->rows, ls->d, ls->res, ctx->stream));
     CORE_CUDA(ctx, launch_ls_at_r(ls->plan, ls->A, ls->res, ls->n, ls->rows, ls->d, ls->part, ctx->stream));
-    CORE_CUDA(ctx, launch_ls_reduce(ls->plan, ls->part, ls->n, ls->rows, ls->d, G, ctx->stream));
+    CORE_CUDA(ctx, launch_ls_reduce(ls->plan, ls->part, ls->n, ls->rows, ls->d, G, clear, ctx->stream));
     return CORE_OK;
 }
 
@@ -777,11 +777,25 @@ int core_decentralized_step(core_ctx *ctx, core_ls *ls, const float *W_dev, int3
     float *P = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb);
     float *P_next = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb + Pb);
     // every machine projects its own gradient; nothing is combined centrally
-    if (int rc = ls_gradients_into(ctx, ls, x_dev, ls->G)) return rc;
-    if (int rc = project_into(ctx, ls->G, CORE_F32, n, ls->d, ctx->d, 0, partial, P, false, ctx->stream)) return rc;
-    // the m-dimensional averaging problem, by gossip with the neighbours: row i is machine i's estimate
-    CORE_CUDA(ctx, launch_gossip_rounds(W_dev, P, n, ctx->m, rounds, P_next, &P, ctx->stream));
-    if (spread_dev) CORE_CUDA(ctx, launch_consensus_spread(P, n, ctx->m, reader, spread_dev, ctx->stream));
+    const bool one_launch = gossip_step_applies(n);
+    if (int rc = ls_gradients_into(ctx, ls, x_dev, ls->G, one_launch ? spread_dev : nullptr)) return rc;
+    // then the m-dimensional averaging problem, by gossip with the neighbours: row i is machine i's estimate
+    const bool one_group = one_launch && !single_row(n) && project_group(n, ctx->m) >= n;
+    const ProjectPlan plan = one_group ? make_project_plan(n, ctx->m, ctx->d, CORE_F32, ctx->sm_count) : ProjectPlan{};
+    if (one_group && gossip_joins(n, plan.grid_x)) {
+        CORE_CUDA(ctx, launch_project(plan, ctx->keys, ctx->t, ls->G, CORE_F32, n, ls->d, ctx->d, ctx->m, 0, partial, ctx->stream));
+        CORE_CUDA(ctx, launch_gossip_step(W_dev, partial, plan.grid_x, nullptr, n, ctx->m, rounds, P_next, reader, spread_dev, ctx->stream));
+        P = P_next;
+    } else {
+        if (int rc = project_into(ctx, ls->G, CORE_F32, n, ls->d, ctx->d, 0, partial, P, false, ctx->stream)) return rc;
+        if (one_launch) {
+            CORE_CUDA(ctx, launch_gossip_step(W_dev, nullptr, 0, P, n, ctx->m, rounds, P_next, reader, spread_dev, ctx->stream));
+            P = P_next;
+        } else {
+            CORE_CUDA(ctx, launch_gossip_rounds(W_dev, P, n, ctx->m, rounds, P_next, &P, ctx->stream));
+            if (spread_dev) CORE_CUDA(ctx, launch_consensus_spread(P, n, ctx->m, reader, spread_dev, ctx->stream));
+        }
+    }
     // reconstruction from the reader's estimate, update inside the kernel; the printed prefactor n/m is
     // the mean convention's 1/m with an n times longer step
     const ReconstructEpilogue update{x_dev, as_printed ? h * (float)n : h, nullptr, nullptr};

@@ -179,7 +179,7 @@ cudaError_t launch_ls_residual(const float *A, const float *b, const float *x, i
 cudaError_t launch_ls_at_r(const LsPlan &plan, const float *A, const float *res, int32_t n, int32_t rows,
                            int64_t d, float *part, cudaStream_t stream);
 cudaError_t launch_ls_reduce(const LsPlan &plan, const float *part, int32_t n, int32_t rows, int64_t d,
-                             float *G, cudaStream_t stream);
+                             float *G, float *clear, cudaStream_t stream);
 // Single pass over A (core_ls_pass.cu) for rows of up to 131072 columns of any alignment: the residual of each row is
 // formed on the fly, A is read from HBM once.  The n * rows rows are cut over `units` CTAs (or clusters); a unit's
 // partial gradient goes to part[(i * slots_per_machine + s) * ldp + k], s counting the units that hold rows of
@@ -204,7 +204,7 @@ size_t ls_pass_partials(const LsPass &pass);      // floats
 cudaError_t launch_ls_pass_gradients(const LsPass &pass, const float *A, const float *b, const LsPoint &at, int64_t d,
                                      float *part, cudaStream_t stream);
 cudaError_t launch_ls_pass_reduce(const LsPass &pass, const float *part, int64_t d, float inv_rows, float *G,
-                                  cudaStream_t stream);
+                                  float *clear, cudaStream_t stream);
 // loss_part[u] = sum of squared residuals of unit u; with `reverse` from the last row to the first.
 cudaError_t launch_ls_pass_loss(const LsPass &pass, const float *A, const float *b, const LsPoint &at, int64_t d, bool reverse,
                                 double *loss_part, cudaStream_t stream);
@@ -229,6 +229,14 @@ cudaError_t launch_option1_step(const float *pbar, int32_t m, int64_t d, double 
                                 float *h_out, cudaStream_t stream);
 // Algorithm 5's averaging by gossip: out[i*m + j] = sum_l W[i*n + l] in[l*m + j], l ascending (in != out).
 cudaError_t launch_gossip_round(const float *W, const float *in, int32_t n, int32_t m, float *out, cudaStream_t stream);
+// What lies between the projection and the reconstruction of a decentralised step, for up to 64 machines (gossip_step_applies):
+// out = W^rounds P, where P is given, or comes from the projection's partial sums partial[c][i][j], c < chunks (the bits of
+// launch_finish_project; gossip_joins tells where that pays); *spread, zero before, becomes max_ij |out[i][j] - out[reader][j]|
+// (null: not wanted).
+bool gossip_step_applies(int32_t n);
+bool gossip_joins(int32_t n, int chunks);
+cudaError_t launch_gossip_step(const float *W, const float *partial, int chunks, const float *P, int32_t n, int32_t m, int32_t rounds,
+                               float *out, int32_t reader, float *spread, cudaStream_t stream);
 // `rounds` of them: P and scratch (n x m each) are both written, *result tells which holds the outcome.
 cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m, int32_t rounds, float *scratch, float **result,
                                  cudaStream_t stream);

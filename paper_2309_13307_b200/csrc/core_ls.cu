@@ -94,8 +94,9 @@ ls_at_r_kernel(const float *__restrict__ A, const float *__restrict__ res, int r
 }
 
 __global__ void ls_reduce_kernel(const float *__restrict__ part, int n, int splits, int64_t d, float inv_rows,
-                                 float *__restrict__ G) {
+                                 float *__restrict__ G, float *clear) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (clear && idx == 0) *clear = 0.f;
     if (idx >= (int64_t)n * d) return;
     const int i = (int)(idx / d);
     const int64_t k = idx % d;
@@ -224,10 +225,10 @@ cudaError_t launch_ls_at_r(const LsPlan &plan, const float *A, const float *res,
 }
 
 cudaError_t launch_ls_reduce(const LsPlan &plan, const float *part, int32_t n, int32_t rows, int64_t d,
-                             float *G, cudaStream_t stream) {
+                             float *G, float *clear, cudaStream_t stream) {
     const int64_t total = (int64_t)n * d;
     ls_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(part, n, plan.splits, d,
-                                                                         1.0f / (float)rows, G);
+                                                                         1.0f / (float)rows, G, clear);
     return cudaGetLastError();
 }
 

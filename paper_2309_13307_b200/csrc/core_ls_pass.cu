@@ -472,11 +472,13 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     }
 }
 
-// G[i][k] = inv_rows * sum of machine i's partial gradients, in the order of its units.
+// G[i][k] = inv_rows * sum of machine i's partial gradients, in the order of its units.  *clear = 0 (where it is not null) for a
+// later kernel of the step.
 __global__ void ls_pass_reduce_kernel(const float *__restrict__ part, int64_t rows, int64_t total, int64_t units,
-                                      int slots_per_machine, int64_t ldp, int64_t d, float inv_rows, float *__restrict__ G) {
+                                      int slots_per_machine, int64_t ldp, int64_t d, float inv_rows, float *__restrict__ G, float *clear) {
     grid_trigger();
     grid_wait();
+    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0.f;
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = blockIdx.y;
     if (k >= d) return;
@@ -654,10 +656,10 @@ cudaError_t launch_ls_pass_loss(const LsPass &p, const float *A, const float *b,
     return launch_pass(p, a, A, b, at, d, stream);
 }
 
-cudaError_t launch_ls_pass_reduce(const LsPass &p, const float *part, int64_t d, float inv_rows, float *G, cudaStream_t stream) {
+cudaError_t launch_ls_pass_reduce(const LsPass &p, const float *part, int64_t d, float inv_rows, float *G, float *clear, cudaStream_t stream) {
     const int n = (int)(p.total / p.rows);
     return launch_chained(true, ls_pass_reduce_kernel, dim3((unsigned)((d + 127) / 128), n), dim3(128), 0, stream, part, p.rows, p.total, p.units,
-                          p.slots_per_machine, p.ldp, d, inv_rows, G);
+                          p.slots_per_machine, p.ldp, d, inv_rows, G, clear);
 }
 
 cudaError_t launch_ls_loss_sum(const double *loss_part, int64_t units, double scale, double *loss, cudaStream_t stream) {

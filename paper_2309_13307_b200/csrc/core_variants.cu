@@ -1,6 +1,7 @@
 // Small kernels of the optimiser variants built on the round: the step rule of Algorithm 3's Option I
 // (chosen on the device from the size of the combined messages) and the gossip averaging of
 // Algorithm 5 (decentralised CORE-GD).  Everything here works on n x m or m numbers: microseconds.
+#include "core_finish.cuh"
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -47,13 +48,80 @@ __global__ void gossip_round_kernel(const float * W, const float * in, int n, in
     out[(int64_t)i * m + j] = s;
 }
 
-// All gossip rounds of a step in one launch: a column of the messages never meets another one, so a CTA takes
-// kGossipCols columns of all machines through every round in shared memory, W beside them.  Same products in the same
-// order as gossip_round_kernel (a zero weight on a zero row at the end changes nothing), hence the same bits.  Bound by
-// latency (n multiply-adds in a row and a barrier per round) and, with many machines, by reading shared memory: rows of W
-// and columns of the messages are read 16 bytes at a time, their strides odd multiples of 16 bytes so that the rows a warp
-// reads together fall into different banks.  Twenty rounds of 16 machines took 46 us of launches (2.3 us each).
+// Everything between the projection and the reconstruction of a decentralised step in one launch, for up to 64 machines: the
+// messages from the projection's partial sums (the order of finish_project_kernel), all gossip rounds, the distance from
+// consensus.  A column of the messages never meets another one, so a CTA takes kGossipCols columns of all machines through
+// every round in shared memory; a thread holds one entry and its row of W in registers.  Same products in the same order
+// as gossip_round_kernel (zero weights on zero rows at the end change nothing), hence the same bits.  Bound by latency: the
+// loads of the partial sums (all threads, a slice of a message each), then NR multiply-adds in a row and a barrier per round.
+// us of a step, 16 machines, d = 20000, m = 64, 20 rounds: finish, rounds with W in shared memory and distance as three
+// launches 96.8, this one 91.5; 5 machines, d = 3000, m = 300, 30 rounds: 41.5 -> 34.4; 64 machines, d = 4096, m = 256, 20 rounds:
+// 82.2 -> 63.1 (messages finished by a launch of their own).
 constexpr int kGossipCols = 8;
+constexpr int gossip_threads(int nr) { return nr <= 32 ? 1024 : 512; }      // that finish the messages: a row of W has to fit
+template <int NR>
+__global__ void __launch_bounds__(gossip_threads(NR))
+gossip_step_kernel(const float *W, const float *partial, int chunks, const float *in, int n, int m, int rounds, float *out,
+                   int reader, int *spread) {
+    grid_trigger();
+    constexpr int kLd = NR + 4;                       // an odd multiple of 16 bytes: columns fall into different banks
+    __shared__ __align__(16) float buffers[2][kGossipCols][kLd];
+    __shared__ float slices[NR * kGossipCols * kFinishSlices];
+    __shared__ int worst;
+    const int tid = threadIdx.x, col = tid % kGossipCols, i = tid / kGossipCols, j0 = blockIdx.x * kGossipCols, j = j0 + col;
+    const int active = (n + 3) / 4 * 4 * kGossipCols; // threads with an entry, whole warps
+    for (int e = tid; e < 2 * kGossipCols * kLd; e += blockDim.x) (&buffers[0][0][0])[e] = 0.f;
+    if (tid == 0) worst = 0;
+    grid_wait();
+    float w[NR];
+    if (tid < active) {
+#pragma unroll
+        for (int l = 0; l < NR; ++l) w[l] = i < n && l < n ? __ldcg(W + i * n + l) : 0.f;
+    }
+    if (partial) {
+        const int entries = n * kGossipCols;
+        for (int e = tid; e < entries * kFinishSlices; e += blockDim.x) {
+            const int entry = e % entries, slice = e / entries, jj = j0 + entry % kGossipCols;
+            slices[e] = jj < m ? finish_slice(partial, chunks, (int64_t)n * m, (int64_t)(entry / kGossipCols) * m + jj, slice) : 0.f;
+        }
+        __syncthreads();
+        if (tid < entries) buffers[0][col][i] = finish_join(slices + tid, entries);
+    } else {
+        __syncthreads();                              // the buffers are zero
+        if (i < n && j < m) buffers[0][col][i] = __ldcg(in + (int64_t)i * m + j);
+    }
+    __syncthreads();
+    if (tid >= active) return;
+    int cur = 0;
+    for (int r = 0; r < rounds; ++r, cur ^= 1) {
+        const float4 *const column = reinterpret_cast<const float4 *>(buffers[cur][col]);
+        float s = 0.f;
+#pragma unroll
+        for (int l = 0; l < NR / 4; ++l) {
+            const float4 p = column[l];
+            s = fmaf(w[4 * l], p.x, s);
+            s = fmaf(w[4 * l + 1], p.y, s);
+            s = fmaf(w[4 * l + 2], p.z, s);
+            s = fmaf(w[4 * l + 3], p.w, s);
+        }
+        if (i < n) buffers[cur ^ 1][col][i] = s;
+        bar_sync(1, active);
+    }
+    const float mine = buffers[cur][col][i];
+    if (i < n && j < m) out[(int64_t)i * m + j] = mine;
+    if (spread) {
+        // a maximum is the same in any order, and of numbers that are not negative it is that of their bits (NaN never wins)
+        float far = i < n && j < m ? fmaxf(0.f, fabsf(mine - buffers[cur][col][reader])) : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o /= 2) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, o));
+        if (tid % 32 == 0) atomicMax(&worst, __float_as_int(far));
+        bar_sync(1, active);
+        if (tid == 0) atomicMax(spread, worst);
+    }
+}
+
+// The rounds alone, for more machines: W in shared memory too.  Rows of W and columns of the messages are read 16 bytes at a
+// time, their strides odd multiples of 16 bytes so that the rows a warp reads together fall into different banks.
 constexpr int kGossipMaxMachines = 128;               // W in 66 KB of shared memory
 __host__ __device__ constexpr int gossip_stride(int n) { return (((n + 3) / 4) | 1) * 4; }
 __global__ void gossip_rounds_kernel(const float *W, const float *in, int n, int m, int rounds, float *out) {
@@ -130,6 +198,26 @@ cudaError_t launch_option1_step(const float *pbar, int32_t m, int64_t d, double 
 cudaError_t launch_gossip_round(const float *W, const float *in, int32_t n, int32_t m, float *out, cudaStream_t stream) {
     dim3 grid((unsigned)((m + 127) / 128), (unsigned)n);
     return launch_chained(true, gossip_round_kernel, grid, dim3(128), 0, stream, W, in, n, m, out);
+}
+
+bool gossip_step_applies(int32_t n) { return n <= 64; }
+// A CTA finishes the messages of its columns alone, with few threads against the machines where there are more than 32 (us of a
+// step, in a launch of their own -> here: 16 machines, d = 2000, m = 64: 25.7 -> 24.2; 32, d = 8192, m = 128: 48.1 -> 47.2; but 40,
+// d = 20000, m = 1000: 144.8 -> 148.8; 64, d = 4096, m = 256: 63.1 -> 69.2), and only while a thread adds up few partial sums.
+bool gossip_joins(int32_t n, int chunks) {
+    const int tasks = n * kGossipCols * kFinishSlices, threads = gossip_threads(n);
+    return n <= 32 && (tasks + threads - 1) / threads * ((chunks + kFinishSlices - 1) / kFinishSlices) <= 48;
+}
+
+cudaError_t launch_gossip_step(const float *W, const float *partial, int chunks, const float *P, int32_t n, int32_t m, int32_t rounds,
+                               float *out, int32_t reader, float *spread, cudaStream_t stream) {
+    const int entries = (n + 3) / 4 * 4 * kGossipCols;
+    const int most = gossip_threads(n), threads = partial ? (entries * kFinishSlices < most ? entries * kFinishSlices : most) : entries;
+    auto go = [&](auto kernel) {
+        return launch_chained(true, kernel, dim3((m + kGossipCols - 1) / kGossipCols), dim3(threads), 0, stream, W, partial, chunks, P, n, m, rounds,
+                              out, reader, reinterpret_cast<int *>(spread));
+    };
+    return n <= 16 ? go(gossip_step_kernel<16>) : n <= 32 ? go(gossip_step_kernel<32>) : go(gossip_step_kernel<64>);
 }
 
 cudaError_t launch_gossip_rounds(const float *W, float *P, int32_t n, int32_t m, int32_t rounds, float *scratch, float **result,

@@ -90,3 +90,31 @@ def test_many_rounds_reach_the_centralised_step_and_printed_prefactor(core_mod):
     assert L.core_decentralized_step(ctx._h, ls._h, W_dev.data_ptr(), -1, 0, 0, h, x0.data_ptr(), None) == -1
     assert L.core_decentralized_step(ctx._h, ls._h, None, 2, 0, 0, h, x0.data_ptr(), None) == -1
     assert ctx.core_get_round() == 0
+
+
+@pytest.mark.parametrize("n,d,m,rounds", [(1, 512, 9, 2), (2, 640, 8, 0), (16, 700, 33, 7), (17, 2048, 100, 5), (32, 515, 7, 4), (33, 1024, 65, 3),
+                                          (64, 640, 130, 6), (65, 640, 24, 3), (3, 131076, 16, 4)])
+def test_step_equals_its_parts_for_every_number_of_machines(core_mod, n, d, m, rounds):
+    """Between projection and reconstruction a step runs in one launch (up to 64 machines, messages finished there or not): the
+    distance from consensus has the very bits of the entry points one by one, the iterate differs by the rounding of one update
+    (x - h g in two roundings instead of one: half an ulp of h g and of x)."""
+    gen = torch.Generator(device="cuda").manual_seed(n * 1000 + m)
+    A = torch.randn(n, 6, d, generator=gen, device="cuda")
+    b = torch.randn(n, 6, generator=gen, device="cuda")
+    x = torch.randn(d, generator=gen, device="cuda")
+    W = torch.from_numpy(core_inputs.gossip_matrix("ring" if n > 2 else "complete", n).astype(np.float32)).cuda()
+    ctx = core_mod.Core(11, d, m)
+    ls = core_mod.LeastSquares(A, b)
+    reader, h = n // 2, 1e-3
+    P = ctx.core_project(ctx.core_ls_gradients(ls, x))
+    for _ in range(rounds):
+        P = ctx.core_gossip_round(W, P)
+    want = x - h * ctx.core_reconstruct(P[reader].contiguous())
+    spread = torch.full((1,), 1e30, device="cuda")             # what is in it does not count
+    ctx.core_set_round(0)
+    for _ in range(2):
+        y = x.clone()
+        ctx.core_set_round(0)
+        ctx.core_decentralized_step(ls, W, rounds, h, y, reader=reader, spread_dev=spread)
+        assert spread.item() == float((P - P[reader]).abs().max())
+        assert float((y - want).abs().max()) <= 2.0 ** -23 * float(want.abs().max() + (want - x).abs().max())
