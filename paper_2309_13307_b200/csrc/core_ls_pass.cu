@@ -40,9 +40,11 @@ constexpr uint32_t kPassRingBytes = 128u * 1024u;       // bytes in flight per S
 // its update crosses the CTA (about 1600 cycles), so two rows go through it together, four where up to 24 columns
 // per lane leave the registers, and rows of up to 24 KB the shared memory, for it (gradients, us: 16 x 2048 rows of
 // 2049 columns: 125 with one, 84 with two, 66 with four; 8 x 1500 x 5500: 56 with two, 46 with four); the 512-thread
-// kernel of 16 warps per row has registers for two up to 24 columns.
+// kernel of 16 warps per row has registers for two up to 24 columns, and gains by two up to 28, as far as the shared memory has
+// room for two slots of them (14064 columns), although some registers are then spilled (8 x 64 rows of 100000: 80 with one, 70 with two; 16 x 512
+// of 14000: 89, 80).
 constexpr int pass_batch(int warps_per_row, int columns) {
-    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 24 ? 1 : 2) : columns <= 24 ? 4 : 2;
+    return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 28 ? 1 : 2) : columns <= 24 ? 4 : 2;
 }
 
 __device__ int g_pass_status;                           // 0, or the code of a wait that ran out
@@ -544,15 +546,17 @@ cudaError_t launch_pass(const LsPass &p, PassArgs &a, const float *A, const floa
     using i16 = integral_constant<int, 16>;
     using i20 = integral_constant<int, 20>;
     using i24 = integral_constant<int, 24>;
+    using i28 = integral_constant<int, 28>;
     using i32 = integral_constant<int, 32>;
     auto wide = [&](auto warps, auto per_row) {
         constexpr int W = decltype(per_row)::value;
-        if constexpr (W < 16) {
-            if constexpr (W == 2)
-                if (p.columns == 12) return pick(i16{}, per_row, i12{});
+        if constexpr (W == 2)
+            if (p.columns == 12) return pick(i16{}, per_row, i12{});
+        if constexpr (W < 16)
             if (p.columns == 16) return pick(warps, per_row, i16{});
-            if (p.columns == 20) return pick(warps, per_row, i20{});
-        }
+        if (p.columns == 20) return pick(warps, per_row, i20{});
+        if constexpr (W == 16)
+            if (p.columns == 28) return pick(warps, per_row, i28{});
         if constexpr (W >= 8)
             if (p.columns == 32) return pick(warps, per_row, i32{});
         return pick(warps, per_row, i24{});
@@ -582,7 +586,8 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
     while (d > (int64_t)kPassCtaCols * p.cluster) p.cluster *= 2;
     p.slice = p.cluster == 1 ? (int)d : (int)(((d + p.cluster - 1) / p.cluster + 3) / 4 * 4);
     p.group_warps = 1;
-    // 24 columns per lane at most where several warps share a row (four rows at a time, see pass_batch), 32 where that is
+    // (16 warps with 20 columns per lane instead of 24 where they suffice, us: 16 x 256 rows of 20000: 72.5 -> 70.5, 16 x 512 of
+    // 8200: 53.2 -> 50.6.)  24 columns per lane at most where several warps share a row (four rows at a time, see pass_batch), 32 where that is
     // more than 8 warps hold.  One warp with 32 columns per lane handled one row at a time: from 513 columns two warps
     // with four rows are faster (gradients, 50 x 1200 rows of 600: 44 -> 29 us, of 1000: 48 -> 44).  Up to 12 columns
     // per lane 16 warps per CTA have the registers for that (37 with 8); with fewer columns per lane and more warps
@@ -594,7 +599,9 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
     const int per_lane = (p.slice + 32 * p.group_warps - 1) / (32 * p.group_warps);
     p.columns = 1;
     while (p.columns < per_lane) p.columns *= 2;
-    if (p.group_warps > 1) p.columns = per_lane > 24 ? 32 : p.group_warps == kPassMaxWarps || per_lane > 20 ? 24 : per_lane > 16 ? 20 : per_lane > 12 ? 16 : 12;
+    if (p.group_warps > 1) p.columns = per_lane > 20 ? (per_lane + 3) / 4 * 4 : per_lane > 16 || p.group_warps == kPassMaxWarps ? 20 : per_lane > 12 ? 16 : 12;
+    const uint32_t smem = 220u * 1024u;
+    if (p.columns == 28 && (p.group_warps < kPassMaxWarps || 4 * (p.slice * 4 + 56) > (int)smem)) p.columns = 32;      // no room for two slots of two rows
     p.warps = p.group_warps == 1 || p.columns == 12 || p.group_warps == 16 ? 16 : 8;
     const int groups = p.warps / p.group_warps;
     const uint32_t row_bytes = (uint32_t)p.slice * 4;
@@ -604,7 +611,7 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
     p.row_stride = p.cluster == 1 ? row_bytes : (row_bytes + 31) / 16 * 16 + (uint32_t)(d * 4 % 16);
     p.slot_bytes = (p.chunk_rows * p.row_stride + 12 + 15) / 16 * 16;
     // half the room for the groups' sums (still one group's) where that makes the difference to a second ring slot
-    const uint32_t smem = 220u * 1024u, all = (uint32_t)groups * p.slot_bytes;
+    const uint32_t all = (uint32_t)groups * p.slot_bytes;
     p.ring_offset = !machines_apart || groups == 1 ? 0u : kPassFlushBytes + 2 * all <= smem ? kPassFlushBytes : kPassFlushBytes / 2;
     const int room = (int)((smem - p.ring_offset) / all);
     p.slots = std::max((int)(kPassRingBytes / (groups * p.slot_bytes)), 3);

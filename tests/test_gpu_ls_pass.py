@@ -80,3 +80,11 @@ def test_rows_shorter_than_a_copy_unit(core_mod, n, rows, d, offset):
     f0 = oracle.ls_loss(Ah, bh, xh)
     assert abs(float(ctx.core_ls_loss(ls, x).item()) - f0) <= 1e-5 * f0
     assert core_mod.core_device_status() == 0
+
+
+@pytest.mark.parametrize("n,rows,d,offset", [
+    (2, 75, 10240, 0), (1, 40, 10241, 1), (2, 150, 12288, 0), (3, 50, 12289, 1), (1, 160, 13824, 0), (2, 30, 14064, 2), (2, 75, 14065, 3),   # a CTA
+    (2, 40, 20480, 0), (1, 37, 20481, 1), (2, 37, 28126, 0), (1, 30, 28133, 3), (1, 20, 100003, 0)])                                  # clusters
+def test_columns_per_lane_of_long_rows(core_mod, n, rows, d, offset):
+    """20, 24, 28 and 32 columns per lane, two rows at a time or one, up to the last row length of each."""
+    test_gradients_loss_and_step(core_mod, n, rows, d, offset)

@@ -27,3 +27,10 @@ def test_rows_of_several_machines_stay_inside(n, rows, d):
             for misaligned in (0, 4, 8, 12):
                 units, before, behind = binding.core_debug_ls_reads(n, rows, d, apart, misaligned, sm_count)
                 assert units > 0 and (before, behind) == (0, 0), (apart, sm_count, misaligned)
+
+
+def test_long_rows_of_one_cta_have_room_for_two_slots():
+    """Every length up to 16384 takes the single pass (no unit would mean two passes over A)."""
+    for d in [*range(8193, 16384, 61), 13824, 13825, *range(14050, 14090), 14336, 16384]:
+        for apart in (False, True):
+            assert binding.core_debug_ls_reads(3, 60, d, apart, 4)[0] > 0, d
