@@ -263,7 +263,16 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     };
 
     if constexpr (TURN) fill_turn_table<kRowWarps>(reinterpret_cast<float2 *>(smem_raw), warp, lane);
+    const int ql = tid / a.tj, jl = tid - ql * a.tj, jbase = blockIdx.y * a.tj * kRowJT;
+    auto first_q = [&] { return a.q_base + (uint64_t)tile_begin * a.tile_q; };
+    JPart jp[kRowJT];
+    auto make_jp = [&](uint32_t q_hi) {
+#pragma unroll
+        for (int v = 0; v < kRowJT; ++v) jp[v] = philox_jpart((uint32_t)(jbase + jl + v * a.tj), q_hi, a.keys);
+    };
     if (tile_begin < tile_end) fill_table(tile_begin, tile0, tid, kRowThreads);
+    // in short launches while the kernel before this one ends; in long ones the registers are wanted for staging
+    if constexpr (!TURN) make_jp((uint32_t)(first_q() >> 32));
     grid_wait();
 
     // the first tile is staged by all warps, nobody having anything else to do yet; a short tile with many rows (the
@@ -310,15 +319,8 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         return;
     }
 
-    const int ql = tid / a.tj, jl = tid - ql * a.tj;
     const bool active = ql < a.tq && tid < kRowCompute;      // (all warps are here where they stage together)
-    const int jbase = blockIdx.y * a.tj * kRowJT;
     float outer[kRowJT];
-    JPart jp[kRowJT];
-    auto make_jp = [&](uint32_t q_hi) {
-#pragma unroll
-        for (int v = 0; v < kRowJT; ++v) jp[v] = philox_jpart((uint32_t)(jbase + jl + v * a.tj), q_hi, a.keys);
-    };
 #pragma unroll
     for (int v = 0; v < kRowJT; ++v) {
         outer[v] = 0.f;
@@ -329,10 +331,9 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
     const int group2 = kGroups > 1 ? warp / (kRowCompute / 32 / kGroups) * 2 : 0;
     const int last_blocks = my_tiles > 0 ? blocks_of(tile_end - 1) : 0;
     // the block, counted from this CTA's first, at which the high counter word changes (once in 2^32 blocks)
-    auto first_q = [&] { return a.q_base + (uint64_t)tile_begin * a.tile_q; };
     const uint64_t to_change = 0x100000000ull - (first_q() & 0xFFFFFFFFull);
     int change = to_change < (uint64_t)INT_MAX ? (int)to_change : INT_MAX;
-    make_jp((uint32_t)(first_q() >> 32));
+    if constexpr (TURN) make_jp((uint32_t)(first_q() >> 32));
     for (int i = 0; i < my_tiles; ++i) {
         const int st = TOGETHER ? 0 : i & 1;
         const int blocks = i == my_tiles - 1 ? last_blocks : a.tile_q;
