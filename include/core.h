@@ -375,6 +375,15 @@ int core_debug_box_muller(core_ctx *ctx, const uint32_t *words_dev, int64_t nb, 
 int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t sm_count, int64_t out[10]);
 
 /*
+ * Launch geometry of the kernel that projects one row, or the sum of `rows` rows, which start `misaligned` bytes beyond a multiple
+ * of 16 and `ldg` elements apart.  Host-only.  out[0..9] = blocks per shared-memory tile, threads across vectors (four vectors
+ * each), threads across blocks, CTAs across coordinates, CTAs across vectors, tiles of d, dynamic shared memory bytes, 1 if the angles
+ * come from a table (0: polynomials), CTAs across coordinates that the workspace has room for, generating threads per CTA.
+ */
+int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligned, int32_t m, int64_t d, int32_t sm_count,
+                        int64_t out[10]);
+
+/*
  * How core_round_host cuts the vectors: the number of slabs of the input (output = 0) or of the estimate (output != 0)
  * in *count, and the lengths of the first `room` of them.  Host-only.
  */

@@ -69,6 +69,8 @@ _SIGNATURES = {
                                 _c.POINTER(_c.c_uint32)], _c.c_int),
     "core_debug_project_plan": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32,
                                  _c.POINTER(_c.c_int64)], _c.c_int),
+    "core_debug_row_plan": ([_c.c_int, _c.c_int32, _c.c_int64, _c.c_uint32, _c.c_int32, _c.c_int64, _c.c_int32,
+                             _c.POINTER(_c.c_int64)], _c.c_int),
     "core_debug_host_slabs": ([_c.c_int64, _c.c_int32, _c.c_int, _c.c_int32, _c.c_int, _c.POINTER(_c.c_int64), _c.c_int32,
                                _c.POINTER(_c.c_int32)], _c.c_int),
     "core_debug_ls_reads": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32, _c.c_uint32,
@@ -141,6 +143,16 @@ def core_debug_project_plan(n: int, m: int, d: int, dtype: int = CORE_F32, sm_co
     if rc != CORE_OK:
         raise CoreError(rc, "core_debug_project_plan")
     keys = ("nb", "jt", "uq", "tile_q", "tj", "tq", "grid_x", "grid_y", "tiles", "smem")
+    return dict(zip(keys, (int(v) for v in out)))
+
+
+def core_debug_row_plan(m: int, d: int, rows: int = 1, ldg: int | None = None, dtype: int = CORE_F32, misaligned: int = 0,
+                        sm_count: int = 148) -> dict:
+    out = (ctypes.c_int64 * 10)()
+    rc = lib().core_debug_row_plan(dtype, rows, d if ldg is None else ldg, misaligned, m, d, sm_count, out)
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_row_plan")
+    keys = ("tile_q", "tj", "tq", "grid_x", "grid_y", "tiles", "smem", "turn", "columns", "compute")
     return dict(zip(keys, (int(v) for v in out)))
 
 

@@ -899,6 +899,15 @@ int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t 
     return CORE_OK;
 }
 
+int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligned, int32_t m, int64_t d, int32_t sm_count, int64_t out[10]) {
+    if (!out || !valid_dtype(dtype) || rows < 1 || ldg < d || m < 1 || d < 1 || sm_count < 1 || misaligned % elem_size(dtype) != 0) return CORE_EINVAL;
+    const void *const G = reinterpret_cast<const void *>(((uintptr_t)1 << 32) + misaligned);      // any address: nothing is read here
+    const RowPlan p = make_row_plan(G, dtype, rows, ldg, m, d, sm_count);
+    const int64_t v[10] = {p.tile_q, p.tj, p.tq, p.grid_x, p.grid_y, p.tiles, (int64_t)p.smem, p.turn ? 1 : 0, row_plan_columns(m, d, sm_count), p.compute};
+    for (int i = 0; i < 10; ++i) out[i] = v[i];
+    return CORE_OK;
+}
+
 int core_debug_host_slabs(int64_t d, int32_t n, int dtype, int32_t sm_count, int output, int64_t *lengths, int32_t room, int32_t *count) {
     if (!lengths || !count || d < 1 || n < 1 || !valid_dtype(dtype) || sm_count < 1 || room < 0) return CORE_EINVAL;
     const SlabRule rule = output ? output_slabs(d, sm_count) : input_slabs(d, n, elem_size(dtype));

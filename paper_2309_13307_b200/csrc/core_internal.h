@@ -108,6 +108,7 @@ struct RowPlan {
     int tq;           // threads across coordinate blocks
     int grid_x;       // CTAs across coordinates
     int grid_y;       // CTAs across vectors
+    int compute;      // generating threads of a CTA
     int64_t tiles;
     size_t smem;
     bool chain;       // see chain_pays

@@ -67,7 +67,7 @@ struct RowArgs {
     int m;
     int tile_q;      // coordinate blocks per tile
     int tj;          // threads across vectors
-    int tq;          // threads across blocks: tj * tq <= 256
+    int tq;          // threads across blocks: tj * tq generating threads at most
     uint32_t t;
     RoundKeys keys;
 };
@@ -281,7 +281,7 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         const int blocks = blocks_of(tile_begin), segments = (blocks + kSegBlocks - 1) / kSegBlocks;
         const int ranges = a.rows >= 2 * kRowWarps ? kRowWarps / segments : 1;
         if (ranges > 1) {
-            float4 *const scratch = tile0 + 4 * a.tile_q;
+            float4 *const scratch = tile0 + 2 * a.tile_q;    // the second tile's place: it is staged after the barrier below
             const int range = warp / segments;
             const int per = ((a.rows + ranges - 1) / ranges + a.period - 1) / a.period * a.period;
             if (range < ranges)
@@ -459,10 +459,24 @@ static bool row_turn(int32_t rows, bool aligned, int32_t m, int64_t d) {
     return d >= ((int64_t)1 << 24) / m && (aligned ? 11 * (int64_t)rows + 40 < 4 * (int64_t)m : 8 * (int64_t)rows + 10 < m);
 }
 
+// Bytes of dynamic shared memory: two tiles with their tables (or, while the first one is staged, one and the row ranges it is
+// added up from, at most a segment of 64 blocks per warp), in whose place the last sums meet; with the table of angles, it and the sums
+// over tiles.
+template <bool TURN>
+static constexpr size_t row_shared(int tile_q, int threads) {
+    const size_t tile = (size_t)tile_q * (16 + 16), ranges = (size_t)RowCta<TURN>::kWarps * 64 * 16, red = (size_t)threads * kRowJT * 4;
+    const size_t stage = tile + (tile > ranges ? tile : ranges);
+    return (stage > red ? stage : red) + (TURN ? kTurnBytes + kRowJT * 4 * RowCta<true>::kCompute : 0);
+}
+constexpr size_t kSharedPerCta = 227 * 1024, kSharedPerSm = 228 * 1024;
+static_assert(row_shared<true>(RowCta<true>::kTileBlocks, RowCta<true>::kCompute) <= kSharedPerCta, "the longest tile fits a CTA");
+static_assert(RowCta<false>::kPerSm * (row_shared<false>(RowCta<false>::kTileBlocks, RowCta<false>::kCompute) + 1024) <= kSharedPerSm, "and an SM");
+
 static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
     RowPlan p{};
     p.turn = turn;
-    const int compute = turn ? RowCta<true>::kCompute : RowCta<false>::kCompute, warps = turn ? RowCta<true>::kWarps : RowCta<false>::kWarps;
+    const int compute = turn ? RowCta<true>::kCompute : RowCta<false>::kCompute;
+    p.compute = compute;
     const int per_sm = turn ? RowCta<true>::kPerSm : RowCta<false>::kPerSm;
     const int room = turn ? RowCta<true>::kTileBlocks : RowCta<false>::kTileBlocks;
     // Threads across vectors: one per quadruple, in as few CTA rows as keep at least 15/16 of the generating
@@ -499,10 +513,7 @@ static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
     p.tiles = (nq + p.tile_q - 1) / p.tile_q;
     p.grid_x = (int)(slots < p.tiles ? slots : p.tiles);
     p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * per_sm, d, m);
-    // two tiles, two tables, and the row ranges of a short first tile (at most warps segments of 64 blocks)
-    const size_t stage = 2 * (size_t)p.tile_q * (16 + 16) + (size_t)warps * 64 * 16;
-    const size_t red = (size_t)p.tj * p.tq * kRowJT * 4;
-    p.smem = (stage > red ? stage : red) + (turn ? kTurnBytes + kRowJT * 4 * RowCta<true>::kCompute : 0);
+    p.smem = turn ? row_shared<true>(p.tile_q, p.tj * p.tq) : row_shared<false>(p.tile_q, p.tj * p.tq);
     return p;
 }
 

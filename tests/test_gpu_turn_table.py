@@ -79,3 +79,42 @@ def test_projections(core_mod, n, d, m, dtype, offset, pad):
     want = oracle.project(7, 3, m, np.ascontiguousarray(mean.astype(np.float32)))[0]
     # fp32 rounding of the mean itself: 2^-24 of its norm at most, four decimal digits below the bar
     assert np.abs(got - want).max() <= P_TOL * row_norms(mean.astype(np.float32))[0]
+
+
+@pytest.mark.parametrize("n,d,m", [(1, 1_130_988, 18), (1, 1_090_804, 17), (2, 1_136_948, 24), (1, 1_138_688, 32), (2, 2_324_170, 34),
+                                   (1, 1_175_641, 45), (1, 1_174_605, 48), (2, 1_174_604, 48)])
+def test_projections_with_the_longest_tiles(core_mod, n, d, m):
+    """Tiles close to the longest of 2048 blocks: beside the table of angles they take most of a CTA's shared memory."""
+    from paper_2309_13307_b200 import binding
+    G = core_inputs.gradients(n, d, seed=d + m, device="cuda", ld=(d + 3) // 4 * 4)
+    plan = binding.core_debug_row_plan(m, d, rows=n, ldg=G.stride(0))
+    assert plan["turn"] and plan["tile_q"] > 1968
+    ctx = core_mod.Core(7, d, m)
+    ctx.core_set_round(3)
+    mean = np.ascontiguousarray(G.cpu().numpy().astype(np.float64).mean(axis=0, keepdims=True).astype(np.float32))
+    want = oracle.project(7, 3, m, mean)[0]
+    got = [ctx.core_round(G)[0]]
+    if n == 1:
+        ctx.core_set_round(3)
+        P = torch.empty((1, m), dtype=torch.float32, device="cuda")
+        binding.core_project_static(7, 3, m, G, P)
+        got += [ctx.core_project(G)[0], P[0]]
+    for p in got:
+        assert np.abs(p.cpu().numpy() - want).max() <= P_TOL * row_norms(mean)[0]
+        assert torch.equal(p, got[0])
+
+
+@pytest.mark.parametrize("n,d,m", [(1, 2_200_673, 45), (2, 3_801_345, 20)])
+def test_host_rounds_with_the_longest_tiles(core_mod, n, d, m):
+    from paper_2309_13307_b200 import binding
+    plans = [binding.core_debug_row_plan(m, s, rows=n, ldg=(s + 7) // 8 * 8) for s in binding.core_debug_host_slabs(d, n)]
+    assert any(p["turn"] and p["tile_q"] > 1968 for p in plans)
+    G = core_inputs.gradients(n, d, seed=d, device="cuda")
+    ctx = core_mod.Core(7, d, m)
+    pbar, gt = torch.empty(m, dtype=torch.float32), torch.empty(d, dtype=torch.float32)
+    ctx.core_round_host(G.cpu(), pbar, gt)
+    ctx.core_set_round(0)
+    want, want_gt = ctx.core_round(G)
+    # two orders of fp32 sums over the same Gaussians
+    assert float((pbar - want.cpu()).norm()) <= 2e-5 * float(want.norm())
+    assert rel_l2(gt.numpy(), want_gt.cpu().numpy()) <= 2e-5

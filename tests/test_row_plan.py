@@ -1,0 +1,49 @@
+"""Launch geometry of the kernel that projects one row or the sum of several (host logic only): every plan fits a CTA's shared
+memory and covers all vectors and coordinates, and the workspace has room for its partial sums."""
+import pytest
+
+from paper_2309_13307_b200 import binding
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2309_13307_b200 import build
+    build.build()
+
+
+def check_plan(p, m, d):
+    assert p["smem"] <= 227 * 1024
+    assert p["smem"] >= 64 * p["tile_q"] and p["smem"] >= 16 * p["tj"] * p["tq"]     # two tiles; the final reduction
+    assert 1 <= p["tj"] * p["tq"] <= p["compute"] and p["tile_q"] % p["tq"] == 0
+    assert p["grid_y"] * p["tj"] * 4 >= m
+    assert p["tiles"] * 4 * p["tile_q"] >= d > (p["tiles"] - 1) * 4 * p["tile_q"]
+    assert 1 <= p["grid_x"] <= min(p["tiles"], p["columns"])
+
+
+LENGTHS = sorted({int(1e9 ** (i / 150)) for i in range(1, 151)} | {1_130_000, 2_324_170, 25_557_032, 124_439_808, 1_000_000_000})
+
+
+@pytest.mark.parametrize("sm_count", [148, 132, 1])
+def test_every_plan_fits(sm_count):
+    turns = 0
+    for m in [*range(1, 131), 170, 191, 256, 400, 511, 512, 513, 1000, 1024, 1030, 2048, 3073, 4096, 4200, 8192, 100_000]:
+        for d in LENGTHS:
+            for rows, misaligned in ((1, 0), (1, 4), (2, 0), (5, 4)):
+                p = binding.core_debug_row_plan(m, d, rows=rows, misaligned=misaligned, sm_count=sm_count)
+                check_plan(p, m, d)
+                turns += p["turn"]
+    assert turns > 1000
+
+
+@pytest.mark.parametrize("rows", [55, 56, 148, 2368])
+@pytest.mark.parametrize("dtype", [binding.CORE_F32, binding.CORE_BF16])
+def test_many_rows_have_room_for_their_ranges(rows, dtype):
+    """From twice as many rows as warps on, the first tile is added up from ranges of the rows, at most a segment of 64 blocks
+    per warp, beside the first tile."""
+    for m in (1, 16, 64, 165, 459, 700, 1024, 4096, 20_000):
+        for d in LENGTHS[::3]:
+            for ldg in ((d + 7) // 8 * 8, d + 1):
+                p = binding.core_debug_row_plan(m, d, rows=rows, ldg=ldg, dtype=dtype)
+                check_plan(p, m, d)
+                warps, table = (28, 65_536 + 12_288) if p["turn"] else (10, 0)
+                assert p["smem"] >= table + 32 * p["tile_q"] + warps * 64 * 16
