@@ -124,7 +124,8 @@ int core_device_status(int32_t *status_out);
  *           wherever it starts.
  *   P_dev   n*m floats, row-major.
  * fp32 multiply-add with two-level fp32 accumulation and a fixed reduction
- * order: results are bitwise reproducible for a given (n, m, d, dtype).  (A row's
+ * order: results are bitwise reproducible for a given (n, m, d, dtype), wherever the rows start
+ * and whatever ldg is.  (A row's
  * message may differ in the last bits from the same row's among others: one row and
  * several take different kernels.)
  * Machines are processed in groups: up to 64 per pass where the tensor-memory

@@ -439,8 +439,9 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
 
 }  // namespace
 
-// Rows r and r + period have the same alignment; do all of them start on a 16-byte boundary?
-static int row_period(int dtype, int64_t ldg) {
+// Rows r and r + period have the same alignment; do all of them start on a 16-byte boundary?  (A single row has no stride.)
+static int row_period(int dtype, int32_t rows, int64_t ldg) {
+    if (rows == 1) return 1;
     int period = 1;
     while ((int64_t)period * ldg % (dtype == 1 ? 8 : 4) != 0) period *= 2;
     return period;
@@ -451,12 +452,17 @@ static int row_period(int dtype, int64_t ldg) {
 static bool row_together(int32_t rows, bool aligned, int32_t m) { return (int64_t)rows * (aligned ? 3 : 7) >= m; }
 
 // The table of angles pays from the microsecond it takes on, where the staging warps keep up with the faster
-// generation (one in seven instead of one in five): lines through measured shapes (us, without -> with; aligned rows, d = 1e7: n = 1,
-// m = 16: 145 -> 140; n = 5, m = 32: 537 -> 522 the round; n = 32, m = 100: 1649 -> 1584; but n = 4, m = 16: 300 -> 330, n = 8,
-// m = 32: 539 -> 549; shifted, d = 1e7: n = 7, m = 64: 1073 -> 1063; n = 5, m = 100 at d = 1e6: 178 -> 171; but n = 3, m = 32: 579 -> 603,
+// generation (one in seven instead of one in five): lines through measured shapes (us, without -> with; aligned rows, d = 1e7: n = 5,
+// m = 32: 537 -> 522 the round; n = 32, m = 100: 1649 -> 1584; but n = 4, m = 16: 300 -> 330, n = 8, m = 32: 539 -> 549;
+// shifted, d = 1e7: n = 7, m = 64: 1073 -> 1063; n = 5, m = 100 at d = 1e6: 178 -> 171; but n = 3, m = 32: 579 -> 603,
 // n = 16, m = 128: 2147 -> 2190).  By size (n = 1): d = 3e5, m = 64: 23.3 -> 21.8; d = 5e4, m = 400: 23.0 -> 22.8.
+// The message of a single row must not depend on where the row starts, so there the line asks for the number of vectors alone, and lies
+// where aligned and shifted rows both gain (d = 1e7, aligned / shifted: m = 24: 216 -> 198 / 226 -> 205; but m = 13, d = 1e8: 1387 -> 1302 /
+// 1548 -> 1707; m = 20, d = 3e6: 60 -> 60 / 62 -> 66).
 static bool row_turn(int32_t rows, bool aligned, int32_t m, int64_t d) {
-    return d >= ((int64_t)1 << 24) / m && (aligned ? 11 * (int64_t)rows + 40 < 4 * (int64_t)m : 8 * (int64_t)rows + 10 < m);
+    if (d < ((int64_t)1 << 24) / m) return false;
+    if (rows == 1) return m > 20;
+    return aligned ? 11 * (int64_t)rows + 40 < 4 * (int64_t)m : 8 * (int64_t)rows + 10 < m;
 }
 
 // Bytes of dynamic shared memory: two tiles with their tables (or, while the first one is staged, one and the row ranges it is
@@ -518,7 +524,7 @@ static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
 }
 
 RowPlan make_row_plan(const void *G, int dtype, int32_t rows, int64_t ldg, int32_t m, int64_t d, int sm_count) {
-    const bool aligned = row_period(dtype, ldg) == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
+    const bool aligned = row_period(dtype, rows, ldg) == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
     return plan_rows(row_turn(rows, aligned, m, d), m, d, sm_count);
 }
 
@@ -538,7 +544,7 @@ cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint3
     a.q_base = q_base;
     a.partial = partial;
     a.rows = rows;
-    a.period = row_period(dtype, ldg);
+    a.period = row_period(dtype, rows, ldg);
     a.aligned = a.period == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0 && 4 * plan.tile_q % (dtype == 1 ? 8 : 4) == 0;
     a.scale = scale;
     a.m = m;

@@ -81,7 +81,7 @@ def test_projections(core_mod, n, d, m, dtype, offset, pad):
     assert np.abs(got - want).max() <= P_TOL * row_norms(mean.astype(np.float32))[0]
 
 
-@pytest.mark.parametrize("n,d,m", [(1, 1_130_988, 18), (1, 1_090_804, 17), (2, 1_136_948, 24), (1, 1_138_688, 32), (2, 2_324_170, 34),
+@pytest.mark.parametrize("n,d,m", [(2, 1_130_988, 18), (2, 1_090_804, 17), (2, 1_136_948, 24), (1, 1_138_688, 32), (2, 2_324_170, 34),
                                    (1, 1_175_641, 45), (1, 1_174_605, 48), (2, 1_174_604, 48)])
 def test_projections_with_the_longest_tiles(core_mod, n, d, m):
     """Tiles close to the longest of 2048 blocks: beside the table of angles they take most of a CTA's shared memory."""
@@ -118,3 +118,23 @@ def test_host_rounds_with_the_longest_tiles(core_mod, n, d, m):
     # two orders of fp32 sums over the same Gaussians
     assert float((pbar - want.cpu()).norm()) <= 2e-5 * float(want.norm())
     assert rel_l2(gt.numpy(), want_gt.cpu().numpy()) <= 2e-5
+
+
+@pytest.mark.parametrize("m", [2, 3, 7, 8, *range(12, 21)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_one_row_gives_the_same_bits_wherever_it_starts(core_mod, m, dtype):
+    """Around the lines between the kernels for one row; ldg is the stride of rows that are not there."""
+    from paper_2309_13307_b200 import binding
+    d = (1 << 21) + 5
+    row = core_inputs.gradients(1, d, seed=m, dtype=dtype, device="cuda")[0]
+    store = torch.zeros(d + 16, dtype=row.dtype, device="cuda")
+    ctx = core_mod.Core(7, d, m)
+    P = torch.empty((1, m), dtype=torch.float32, device="cuda")
+    want = ctx.core_project(row[None]).clone()
+    for offset in range(8):
+        store[offset:offset + d] = row
+        for ldg in (d, d + 1, d + 3, d + 6):
+            P.zero_()
+            rc = binding.lib().core_project(ctx._h, store.data_ptr() + offset * store.element_size(),
+                                            binding.CORE_BF16 if dtype == "bf16" else binding.CORE_F32, 1, ldg, P.data_ptr())
+            assert rc == 0 and torch.equal(P, want), (offset, ldg)

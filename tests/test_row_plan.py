@@ -47,3 +47,13 @@ def test_many_rows_have_room_for_their_ranges(rows, dtype):
                 check_plan(p, m, d)
                 warps, table = (28, 65_536 + 12_288) if p["turn"] else (10, 0)
                 assert p["smem"] >= table + 32 * p["tile_q"] + warps * 64 * 16
+
+
+@pytest.mark.parametrize("dtype,size", [(binding.CORE_F32, 4), (binding.CORE_BF16, 2)])
+def test_a_single_row_has_one_plan_wherever_it_starts(dtype, size):
+    """Plan and kernel decide the order of the sums: for one row they follow from its length and the number of vectors alone."""
+    for m in [*range(1, 40), 64, 100, 1024]:
+        for d in (4097, 262_144, 2_097_152, 2_097_155, 25_557_032):
+            plans = [binding.core_debug_row_plan(m, d, ldg=d + pad, dtype=dtype, misaligned=off)
+                     for pad in (0, 1, 2, 8) for off in range(0, 16, size)]
+            assert all(p == plans[0] for p in plans), (m, d)
