@@ -385,6 +385,13 @@ int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligne
                         int64_t out[10]);
 
 /*
+ * Which reconstruction kernel d coordinates and m vectors take, host-only: out[0] = 0 the one for short vectors, 1 the one for long
+ * vectors with few or very many Gaussians per coordinate, 2 the one with the table of angles; out[1] = 1 if the CTAs of the
+ * reconstruction form the message of a round of one machine themselves.
+ */
+int core_debug_reconstruct_plan(int64_t d, int32_t m, int32_t sm_count, int32_t out[2]);
+
+/*
  * How core_round_host cuts the vectors: the number of slabs of the input (output = 0) or of the estimate (output != 0)
  * in *count, and the lengths of the first `room` of them.  Host-only.
  */

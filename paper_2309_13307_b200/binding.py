@@ -71,6 +71,7 @@ _SIGNATURES = {
                                  _c.POINTER(_c.c_int64)], _c.c_int),
     "core_debug_row_plan": ([_c.c_int, _c.c_int32, _c.c_int64, _c.c_uint32, _c.c_int32, _c.c_int64, _c.c_int32,
                              _c.POINTER(_c.c_int64)], _c.c_int),
+    "core_debug_reconstruct_plan": ([_c.c_int64, _c.c_int32, _c.c_int32, _c.POINTER(_c.c_int32)], _c.c_int),
     "core_debug_host_slabs": ([_c.c_int64, _c.c_int32, _c.c_int, _c.c_int32, _c.c_int, _c.POINTER(_c.c_int64), _c.c_int32,
                                _c.POINTER(_c.c_int32)], _c.c_int),
     "core_debug_ls_reads": ([_c.c_int32, _c.c_int32, _c.c_int64, _c.c_int, _c.c_int32, _c.c_uint32,
@@ -154,6 +155,14 @@ def core_debug_row_plan(m: int, d: int, rows: int = 1, ldg: int | None = None, d
         raise CoreError(rc, "core_debug_row_plan")
     keys = ("tile_q", "tj", "tq", "grid_x", "grid_y", "tiles", "smem", "turn", "columns", "compute")
     return dict(zip(keys, (int(v) for v in out)))
+
+
+def core_debug_reconstruct_plan(d: int, m: int, sm_count: int = 148) -> tuple:
+    out = (ctypes.c_int32 * 2)()
+    rc = lib().core_debug_reconstruct_plan(d, m, sm_count, out)
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_reconstruct_plan")
+    return ("short", "wide", "turn")[out[0]], bool(out[1])
 
 
 def core_debug_host_slabs(d: int, n: int = 1, dtype: int = CORE_F32, output: bool = False, sm_count: int = 148) -> list:

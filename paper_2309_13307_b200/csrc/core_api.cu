@@ -908,6 +908,14 @@ int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligne
     return CORE_OK;
 }
 
+int core_debug_reconstruct_plan(int64_t d, int32_t m, int32_t sm_count, int32_t out[2]) {
+    if (!out || d < 1 || m < 1 || sm_count < 1) return CORE_EINVAL;
+    out[0] = (int32_t)reconstruct_kernel_for((d + 3) >> 2, m, sm_count);
+    const RowPlan row = make_row_plan(nullptr, CORE_F32, 1, d, m, d, sm_count);
+    out[1] = reconstruct_joins(row.grid_x, 1, m, d, sm_count) ? 1 : 0;
+    return CORE_OK;
+}
+
 int core_debug_host_slabs(int64_t d, int32_t n, int dtype, int32_t sm_count, int output, int64_t *lengths, int32_t room, int32_t *count) {
     if (!lengths || !count || d < 1 || n < 1 || !valid_dtype(dtype) || sm_count < 1 || room < 0) return CORE_EINVAL;
     const SlabRule rule = output ? output_slabs(d, sm_count) : input_slabs(d, n, elem_size(dtype));

@@ -155,6 +155,8 @@ struct MessageParts {
     int chunks;
     int n;
 };
+enum class RecKernel { kShort, kWide, kTurn };         // for short vectors; for long ones, without and with the table of angles
+RecKernel reconstruct_kernel_for(int64_t nq, int32_t m, int sm_count);     // nq blocks of four coordinates
 bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count);
 cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, int32_t m,
                                int64_t k_begin, int64_t k_end, float *out, int sm_count,

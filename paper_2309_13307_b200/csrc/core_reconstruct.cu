@@ -1,8 +1,8 @@
 // Fused regenerate-and-reconstruct kernel: gtilde[k] = (1/m) sum_j pbar[j] xi_j[k]
 // (Algorithm 1, receiver's step; the equation that follows Algorithm 1).
 //
-// A thread owns a coordinate block of four coordinates and runs over the vectors j,
-// regenerating xi_j for it from the same counters the projection used.  The
+// A thread owns one or two blocks of four coordinates and runs over the vectors j,
+// regenerating xi_j for them from the same counters the projection used.  The
 // part of the Philox evaluation that depends only on the block is computed once per
 // thread; the part that depends only on j is tabulated per CTA in shared memory next
 // to pbar[j], so the loop reads one 16-byte broadcast per j.  Every output coordinate
@@ -15,6 +15,10 @@ namespace core {
 
 namespace {
 
+constexpr int kWideUQ = 2;                        // the kernel for few or very many vectors: coordinate blocks per thread,
+constexpr int kWideQ = kThreads * kWideUQ;        // per CTA step,
+constexpr int kWideJStep = 2;                     // vectors generated together,
+constexpr int kWideCtas = 3;                      // resident CTAs per SM (register-limited)
 constexpr int kJChunk = 2048;                     // vectors tabulated at a time (32 KB)
 constexpr int kTurnWarps = 32;                    // the kernel for long vectors: one CTA per SM
 constexpr int kTurnJStep = 4;                     // vectors generated together
@@ -34,10 +38,10 @@ struct ReconstructArgs {
     ReconstructEpilogue epi;   // base == nullptr: store the estimate itself
 };
 
-// acc += sum over JS consecutive table entries of pbar[j] * xi_j[block], j ascending.
-template <int JS>
-__device__ __forceinline__ void rec_step(const uint4 *entries, const QPart &qp, const RoundKeys &keys, float4 &acc) {
-    uint4 w[JS];
+// acc[u] += sum over JS consecutive table entries of pbar[j] * xi_j[block u], j ascending.
+template <int JS, int UQ>
+__device__ __forceinline__ void rec_step(const uint4 *entries, const QPart (&qp)[UQ], const RoundKeys &keys, float4 (&acc)[UQ]) {
+    uint4 w[JS * UQ];
     float p[JS];
 #pragma unroll
     for (int s = 0; s < JS; ++s) {
@@ -47,20 +51,25 @@ __device__ __forceinline__ void rec_step(const uint4 *entries, const QPart &qp, 
         jp.x0 = e.x;
         jp.x2 = e.y;
         jp.w3 = e.z;
-        w[s] = philox_combine(jp, qp, keys);
+#pragma unroll
+        for (int u = 0; u < UQ; ++u) w[s * UQ + u] = philox_combine(jp, qp[u], keys);
     }
-    BmParts r[JS];
-    box_muller_parts<JS>(w, r);
+    BmParts r[JS * UQ];
+    box_muller_parts<JS * UQ>(w, r);
     // pbar_j xi_j with the message meeting the radius first: ((pbar S) y) sp and (pbar S) cs, four packed
     // instructions per call instead of five, and xi_j itself (pbar = 1) bit for bit what the projection
     // multiplies with.  Accumulator lanes: (x, z) = cosine lanes of pair a, b; (y, w) = sine lanes.
 #pragma unroll
     for (int s = 0; s < JS; ++s) {
-        const float2 ps = __fmul2_rn(make_float2(p[s], p[s]), r[s].s);
-        const float2 psy = __fmul2_rn(ps, r[s].y);
-        const float2 c2 = __ffma2_rn(psy, r[s].sp, make_float2(acc.x, acc.z));
-        const float2 s2 = __ffma2_rn(ps, r[s].cs, make_float2(acc.y, acc.w));
-        acc = make_float4(c2.x, s2.x, c2.y, s2.y);
+#pragma unroll
+        for (int u = 0; u < UQ; ++u) {
+            const BmParts rr = r[s * UQ + u];
+            const float2 ps = __fmul2_rn(make_float2(p[s], p[s]), rr.s);
+            const float2 psy = __fmul2_rn(ps, rr.y);
+            const float2 c2 = __ffma2_rn(psy, rr.sp, make_float2(acc[u].x, acc[u].z));
+            const float2 s2 = __ffma2_rn(ps, rr.cs, make_float2(acc[u].y, acc[u].w));
+            acc[u] = make_float4(c2.x, s2.x, c2.y, s2.y);
+        }
     }
 }
 
@@ -245,7 +254,65 @@ reconstruct_kernel(const __grid_constant__ ReconstructArgs a) {
     }
 }
 
-// Short vectors: the kernel above would leave most of its warps without a unit (d = 8192 is 64 of them),
+// Long vectors where the table of angles does not pay: few vectors, whose Gaussians cost less than the stores and the table, or more
+// vectors than fit beside it.  512 blocks per CTA and step, two per thread, three CTAs per SM that walk over the vector; where the
+// vectors are more than kJChunk their table is made anew for every chunk.
+__global__ void __launch_bounds__(kThreads, kWideCtas)
+reconstruct_wide_kernel(const __grid_constant__ ReconstructArgs a) {
+    grid_trigger();
+    grid_wait();
+    __shared__ uint4 table[kJChunk];              // {JPart.x0, JPart.x2, JPart.w3, bits of pbar[j]}
+    const int tid = threadIdx.x;
+    const uint64_t q_begin = (uint64_t)a.k_begin >> 2;
+    const uint64_t q_end = ((uint64_t)a.k_end + 3) >> 2;
+    const uint64_t groups = (q_end - q_begin + kWideQ - 1) / kWideQ;
+    const float inv_m = 1.0f / (float)a.m;
+
+    bool have_table = false;
+    uint32_t table_qhi = 0;
+
+    for (uint64_t grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+        // q_begin is a multiple of kWideQ (launch_reconstruct checks), so a group never
+        // straddles a multiple of 2^32 and all its blocks share the high counter word.
+        const uint64_t gq0 = q_begin + grp * kWideQ;
+        const uint32_t grp_qhi = (uint32_t)(gq0 >> 32);
+
+        float4 acc[kWideUQ];
+        QPart qp[kWideUQ];
+        uint64_t qv[kWideUQ];
+#pragma unroll
+        for (int u = 0; u < kWideUQ; ++u) {
+            qv[u] = gq0 + (uint64_t)(tid + u * kThreads);
+            qp[u] = philox_qpart((uint32_t)qv[u], a.t, a.keys);
+            acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+
+        for (int j0 = 0; j0 < a.m; j0 += kJChunk) {
+            const int jn = min(kJChunk, a.m - j0);
+            if (!have_table || table_qhi != grp_qhi || a.m > kJChunk) {
+                __syncthreads();                  // everyone is done with the previous table
+                for (int jj = tid; jj < jn; jj += kThreads) {
+                    const JPart jp = philox_jpart((uint32_t)(j0 + jj), grp_qhi, a.keys);
+                    table[jj] = make_uint4(jp.x0, jp.x2, jp.w3, __float_as_uint(__ldcg(a.pbar + j0 + jj)));
+                }
+                __syncthreads();
+                have_table = true;
+                table_qhi = grp_qhi;
+            }
+            int jj = 0;
+            for (; jj + kWideJStep <= jn; jj += kWideJStep) rec_step<kWideJStep, kWideUQ>(table + jj, qp, a.keys, acc);
+            for (; jj < jn; ++jj) rec_step<1, kWideUQ>(table + jj, qp, a.keys, acc);
+        }
+
+#pragma unroll
+        for (int u = 0; u < kWideUQ; ++u) {
+            if (qv[u] >= q_end) continue;
+            emit_block(a, qv[u], q_begin, make_float4(acc[u].x * inv_m, acc[u].y * inv_m, acc[u].z * inv_m, acc[u].w * inv_m));
+        }
+    }
+}
+
+// Short vectors: the kernels above would leave most of their warps without work (d = 8192 is 64 units),
 // so here the SLICES warp groups of a CTA share out the vectors of 256 / SLICES blocks; the partial sums
 // of a block meet in shared memory and are added in ascending order of the vector ranges.  Few vectors
 // get few slices (a slice wants at least four vectors to generate together); where even eight slices leave SMs
@@ -280,8 +347,8 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
     const uint64_t q0 = q_begin + (uint64_t)(blockIdx.x / ranks) * QB;     // multiple of 32: one high counter word per CTA
     const uint32_t q_hi = (uint32_t)(q0 >> 32);
     const uint64_t q = q0 + (uint64_t)ql;
-    const QPart qp = philox_qpart((uint32_t)q, a.t, a.keys);
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    const QPart qp[1] = {philox_qpart((uint32_t)q, a.t, a.keys)};
+    float4 acc[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
     const int mine = ((a.m + (int)ranks - 1) / (int)ranks + 3) & ~3;       // vectors of this CTA
     const int m_begin = min((int)rank * mine, a.m), m_end = min(m_begin + mine, a.m);
     for (int j0 = m_begin; j0 < m_end; j0 += kJChunk) {
@@ -314,11 +381,11 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
         const int per = (jn + SLICES - 1) / SLICES;                         // vectors per slice
         const int j_begin = min(slice * per, jn), j_end = min(j_begin + per, jn);
         int jj = j_begin;
-        for (; jj + 4 <= j_end; jj += 4) rec_step<4>(table + jj, qp, a.keys, acc);
-        for (; jj < j_end; ++jj) rec_step<1>(table + jj, qp, a.keys, acc);
+        for (; jj + 4 <= j_end; jj += 4) rec_step<4, 1>(table + jj, qp, a.keys, acc);
+        for (; jj < j_end; ++jj) rec_step<1, 1>(table + jj, qp, a.keys, acc);
     }
     if (m_begin >= m_end) grid_wait();             // a CTA without vectors
-    part[slice][ql] = acc;
+    part[slice][ql] = acc[0];
     __syncthreads();
     float4 s = part[0][ql];
     if (slice == 0) {
@@ -389,17 +456,24 @@ unsigned grid_for(int64_t items, int threads, int cap) {
 
 }  // namespace
 
-// The kernel for long vectors wants five units per SM (six in one SM and five in another are 13 % apart; at four the kernel
-// below, with its clusters, is ahead) and work for the microsecond or two that its table of angles takes: us, the one
-// below -> this one, d = 1e5, m = 64: 9.1 -> 9.8, m = 256: 26.3 -> 25.5; d = 1e6, m = 8: 10.3 -> 11.5, m = 32: 31.0 -> 29.4;
-// d = 3e6, m = 8: 25.0 -> 24.2; d = 4e4, m = 1024: 45.6 -> 47.1.
-static bool long_vector(int64_t nq, int32_t m, int sm_count) {
-    return m <= kTurnVectors && nq >= 160 * (int64_t)sm_count && nq >= ((int64_t)1 << 22) / m;
+// The kernel with the table of angles wants five units per SM (six in one SM and five in another are 13 % apart; at four the one for
+// short vectors, with its clusters, is ahead) and work for the microsecond or two that its table takes: us, the one for short
+// vectors -> this one, d = 1e5, m = 64: 9.1 -> 9.8, m = 256: 26.3 -> 25.5; d = 1e6, m = 8: 10.3 -> 11.5, m = 32: 31.0 -> 29.4; d = 3e6,
+// m = 8: 25.0 -> 24.2; d = 4e4, m = 1024: 45.6 -> 47.1.  With few vectors it takes as much more work to be ahead of the wide
+// kernel (m = 6, d = 3.6e6: 21.9 -> 23.1, 9.8e6: 1 % ahead), with up to three it never is (m = 1, d = 1e8: 157.8 -> 168.3; m = 2: 233 -> 244;
+// m = 3, d = 2e7: 64.9 -> 67.1).  Other vectors of eight wide steps per SM or more take the wide kernel (the one for short
+// vectors there: m = 1, d = 1e7: 17.4 -> 33.2; m = 4, d = 3e6: 14.7 -> 17.9).
+RecKernel reconstruct_kernel_for(int64_t nq, int32_t m, int sm_count) {
+    const int64_t work = (int64_t)(m < 8 ? 3 : 1) << 22;
+    if (m > 3 && m <= kTurnVectors && nq >= 160 * (int64_t)sm_count && nq >= work / m) return RecKernel::kTurn;
+    return (nq + kWideQ - 1) / kWideQ >= 8 * (int64_t)sm_count ? RecKernel::kWide : RecKernel::kShort;
 }
 // Every CTA forms the whole message: worth it while that is at most eight loads per thread (with 32, d = 8192 and m = 64, the
-// launch it saves was the cheaper one: 100.7 against 105.9 us a step).
+// launch it saves was the cheaper one: 100.7 against 105.9 us a step) and the CTAs are those of a short vector (m = 1, d = 1.6e7: 15625
+// of them form it 15625 times: a round of one machine 121 -> 524).
 bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count) {
-    return m <= kJoinVectors && (int64_t)n * m <= kJoinEntries && (int64_t)chunks * n * m <= 2048 && !long_vector((d + 3) >> 2, m, sm_count);
+    return m <= kJoinVectors && (int64_t)n * m <= kJoinEntries && (int64_t)chunks * n * m <= 2048 &&
+           reconstruct_kernel_for((d + 3) >> 2, m, sm_count) == RecKernel::kShort;
 }
 
 cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, int32_t m,
@@ -425,7 +499,8 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, i
     a.keys = keys;
     const int64_t nq = ((k_end + 3) >> 2) - (k_begin >> 2);
     if (parts) a.parts = *parts;
-    if (!long_vector(nq, m, sm_count)) {
+    const RecKernel kernel = reconstruct_kernel_for(nq, m, sm_count);
+    if (kernel == RecKernel::kShort) {
         // more slices = fewer blocks per CTA = more CTAs: as many as it takes to go round evenly (four are resident per
         // SM), while a slice keeps at least four vectors, or sixteen where it is only for the last wave's sake
         int slices = 1, ranks = 1;
@@ -452,6 +527,10 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, i
             case 2: return go(reconstruct_small_kernel<2>);
             default: return go(reconstruct_small_kernel<1>);
         }
+    }
+    if (kernel == RecKernel::kWide) {
+        const int64_t steps = (nq + kWideQ - 1) / kWideQ, ctas = (int64_t)sm_count * kWideCtas;
+        return launch_chained(true, reconstruct_wide_kernel, dim3((unsigned)(steps < ctas ? steps : ctas)), dim3(kThreads), 0, stream, a);
     }
     const size_t smem = kTurnBytes + kTurnShares + sizeof(uint4) * (size_t)m;
     return launch_chained(true, reconstruct_kernel, dim3((unsigned)sm_count), dim3(kTurnWarps * 32), smem, stream, a);

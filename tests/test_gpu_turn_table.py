@@ -52,6 +52,25 @@ def test_long_reconstructions(core_mod, d, m):
         assert rel_l2(gt[k0:k1], oracle.reconstruct_slice(5, 2, pbar.astype(np.float64), k0, k1)) <= REC_TOL
 
 
+@pytest.mark.parametrize("d,m,kernel", [(2_422_789, 1, "wide"), (2_422_789, 5, "wide"), (2_424_833, 2, "wide"), (2_422_784, 3, "short"),
+                                        (5_000_003, 3, "wide"), (9_786_709, 6, "turn"), (2_424_833, 8_193, "wide")])
+def test_long_reconstructions_without_the_table(core_mod, d, m, kernel):
+    from paper_2309_13307_b200 import binding
+    assert binding.core_debug_reconstruct_plan(d, m)[0] == kernel
+    test_long_reconstructions(core_mod, d, m)
+
+
+@pytest.mark.parametrize("n,d,m", [(1, 4_000_003, 1), (3, 4_000_003, 2), (2, 2_500_001, 4), (1, 300_001, 1), (2, 1_000_003, 2)])
+def test_rounds_of_few_vectors_equal_their_parts(core_mod, n, d, m):
+    G = core_inputs.gradients(n, d, seed=m, device="cuda")
+    ctx = core_mod.Core(5, d, m)
+    pbar, gt = ctx.core_round(G)
+    ctx.core_set_round(0)
+    want = ctx.core_aggregate(ctx.core_project(G))
+    assert float((pbar - want).abs().max()) <= P_TOL * float(G.norm(dim=1).mean())
+    assert torch.equal(ctx.core_reconstruct(pbar), gt)
+
+
 def test_reconstructions_do_not_depend_on_what_ran_before(core_mod):
     """Warps that share a unit meet in shared memory: the same bits on every launch."""
     d, m = 151_600, 333
