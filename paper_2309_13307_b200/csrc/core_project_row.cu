@@ -33,7 +33,6 @@
 #include <cuda_bf16.h>
 
 #include <climits>
-#include <type_traits>
 
 namespace core {
 
@@ -271,8 +270,6 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         for (int v = 0; v < kRowJT; ++v) jp[v] = philox_jpart((uint32_t)(jbase + jl + v * a.tj), q_hi, a.keys);
     };
     if (tile_begin < tile_end) fill_table(tile_begin, tile0, tid, kRowThreads);
-    // in short launches while the kernel before this one ends; in long ones the registers are wanted for staging
-    if constexpr (!TURN) make_jp((uint32_t)(first_q() >> 32));
     grid_wait();
 
     // the first tile is staged by all warps, nobody having anything else to do yet; a short tile with many rows (the
@@ -326,42 +323,31 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         outer[v] = 0.f;
         if (TURN && tid < kRowCompute) totals[v * kRowCompute + tid] = 0.f;
     }
-    // Few and short variables are carried around the loop: the registers are what limits the warps of an SM.
-    const int my_tiles = (int)(tile_end - tile_begin);
-    const int group2 = kGroups > 1 ? warp / (kRowCompute / 32 / kGroups) * 2 : 0;
-    const int last_blocks = my_tiles > 0 ? blocks_of(tile_end - 1) : 0;
-    // the block, counted from this CTA's first, at which the high counter word changes (once in 2^32 blocks)
-    const uint64_t to_change = 0x100000000ull - (first_q() & 0xFFFFFFFFull);
-    int change = to_change < (uint64_t)INT_MAX ? (int)to_change : INT_MAX;
-    if constexpr (TURN) make_jp((uint32_t)(first_q() >> 32));
-    for (int i = 0; i < my_tiles; ++i) {
-        const int st = TOGETHER ? 0 : i & 1;
-        const int blocks = i == my_tiles - 1 ? last_blocks : a.tile_q;
-        if (i >= 1) {
-            if constexpr (TOGETHER) {
-                __syncthreads();                             // everyone is done with the tile
-                row_stage_any<GT>(2, a, 4 * (tile_begin + i) * a.tile_q, blocks, warp, kRowWarps, 0, a.rows, lane, tile0);
-                fill_table(tile_begin + i, tile0, tid, kRowThreads);
-                __syncthreads();
-            } else {
-                bar_sync(kFull + group2 + st, kHandOver);
-            }
-        }
-        const float4 *const cur = tile0 + 2 * st * a.tile_q;
-        std::conditional_t<TURN, float, float2> acc[kRowJT];
-#pragma unroll
-        for (int v = 0; v < kRowJT; ++v) acc[v] = {};
-        if (active) {
-            const float4 *entry = cur + 2 * ql;
-            for (int upto = min(blocks, change - i * a.tile_q);;) {
-                for (const float4 *const stop = cur + 2 * upto; entry < stop; entry += 2 * a.tq) {
-                    const float4 g = entry[0], e = entry[1];
-                    QPart qp;
-                    qp.hi_b = __float_as_uint(e.x);
-                    qp.lo_b = __float_as_uint(e.y);
-                    qp.w3 = __float_as_uint(e.z);
-                    const float2 gc = make_float2(g.x, g.y), gs = make_float2(g.z, g.w);
-                    if constexpr (TURN) {
+    if constexpr (TURN) {
+        // Few and short variables are carried around the loop: the registers are what limits the warps of an SM.
+        const int my_tiles = (int)(tile_end - tile_begin);
+        const int group2 = warp / (kRowCompute / 32 / kGroups) * 2;
+        const int last_blocks = my_tiles > 0 ? blocks_of(tile_end - 1) : 0;
+        // the block, counted from this CTA's first, at which the high counter word changes (once in 2^32 blocks)
+        const uint64_t to_change = 0x100000000ull - (first_q() & 0xFFFFFFFFull);
+        int change = to_change < (uint64_t)INT_MAX ? (int)to_change : INT_MAX;
+        make_jp((uint32_t)(first_q() >> 32));
+        for (int i = 0; i < my_tiles; ++i) {
+            const int st = i & 1;
+            const int blocks = i == my_tiles - 1 ? last_blocks : a.tile_q;
+            if (i >= 1) bar_sync(kFull + group2 + st, kHandOver);
+            const float4 *const cur = tile0 + 2 * st * a.tile_q;
+            float acc[kRowJT] = {};
+            if (active) {
+                const float4 *entry = cur + 2 * ql;
+                for (int upto = min(blocks, change - i * a.tile_q);;) {
+                    for (const float4 *const stop = cur + 2 * upto; entry < stop; entry += 2 * a.tq) {
+                        const float4 g = entry[0], e = entry[1];
+                        QPart qp;
+                        qp.hi_b = __float_as_uint(e.x);
+                        qp.lo_b = __float_as_uint(e.y);
+                        qp.w3 = __float_as_uint(e.z);
+                        const float2 gc = make_float2(g.x, g.y), gs = make_float2(g.z, g.w);
                         uint4 w[kRowJT];
                         float2 l[kRowJT];
 #pragma unroll
@@ -373,34 +359,81 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                             const float2 t = __ffma2_rn(r.n, gs, __fmul2_rn(r.c, gc));
                             acc[v] = fmaf(r.s.x, t.x, fmaf(r.s.y, t.y, acc[v]));
                         }
-                    } else {
+                    }
+                    if (upto == blocks) break;
+                    upto = blocks;
+                    change = INT_MAX;
+                    make_jp((uint32_t)(first_q() >> 32) + 1);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < kRowJT; ++v)
+                if (active) totals[v * kRowCompute + tid] += acc[v];
+            if (i + 2 < my_tiles) bar_arrive(kEmpty + group2 + st, kHandOver);
+        }
+    } else {
+        // The loop above, with the vectors' half formed before the first tile, cost bf16 rows staged by all warps up to 6 %: registers were
+        // spilled (us, one row, d = 1.4e6: m = 2: 14.5 -> 15.5; shifted, m = 4: 17.3 -> 18.0; this loop: 14.5, 17.1).
+        uint32_t jp_q_hi = 0;
+        bool have_jp = false;
+        for (int64_t tile = tile_begin; tile < tile_end; ++tile) {
+            const int i = (int)(tile - tile_begin), st = TOGETHER ? 0 : i & 1;
+            if (i >= 1) {
+                if constexpr (TOGETHER) {
+                    __syncthreads();                         // everyone is done with the tile
+                    row_stage_any<GT>(2, a, 4 * tile * a.tile_q, blocks_of(tile), warp, kRowWarps, 0, a.rows, lane, tile0);
+                    fill_table(tile, tile0, tid, kRowThreads);
+                    __syncthreads();
+                } else {
+                    bar_sync(kFull + st, kHandOver);
+                }
+            }
+            const float4 *cur = tile0 + 2 * st * a.tile_q;
+            const int blocks = blocks_of(tile);
+            const uint64_t q0 = a.q_base + (uint64_t)tile * a.tile_q;
+            // blocks of this tile that share the high counter word of the first one (all of them but once in 2^32)
+            const uint64_t left = 0x100000000ull - (q0 & 0xFFFFFFFFull);
+            int upto = left < (uint64_t)blocks ? (int)left : blocks;
+            uint32_t q_hi = (uint32_t)(q0 >> 32);
+            float2 acc[kRowJT];
+#pragma unroll
+            for (int v = 0; v < kRowJT; ++v) acc[v] = make_float2(0.f, 0.f);
+            int qq = ql;
+            if (active) {
+                for (;;) {
+                    if (!have_jp || q_hi != jp_q_hi) {
+                        make_jp(q_hi);
+                        jp_q_hi = q_hi;
+                        have_jp = true;
+                    }
+                    const float4 *entry = cur + 2 * qq;
+                    for (; qq < upto; qq += a.tq, entry += 2 * a.tq) {
+                        const float4 g = entry[0], e = entry[1];
+                        QPart qp;
+                        qp.hi_b = __float_as_uint(e.x);
+                        qp.lo_b = __float_as_uint(e.y);
+                        qp.w3 = __float_as_uint(e.z);
                         uint4 w[kRowJT];
-                        BmParts r[kRowJT];
 #pragma unroll
                         for (int v = 0; v < kRowJT; ++v) w[v] = philox_combine(jp[v], qp, a.keys);
+                        BmParts r[kRowJT];
                         box_muller_parts<kRowJT>(w, r);
+                        const float2 gc = make_float2(g.x, g.y), gs = make_float2(g.z, g.w);
 #pragma unroll
                         for (int v = 0; v < kRowJT; ++v) {
                             const float2 c = __fmul2_rn(__fmul2_rn(r[v].y, r[v].sp), gc);
                             acc[v] = __ffma2_rn(r[v].s, __ffma2_rn(r[v].cs, gs, c), acc[v]);
                         }
                     }
+                    if (upto == blocks) break;
+                    upto = blocks;
+                    ++q_hi;
                 }
-                if (upto == blocks) break;
-                upto = blocks;
-                change = INT_MAX;
-                make_jp((uint32_t)(first_q() >> 32) + 1);
             }
-        }
 #pragma unroll
-        for (int v = 0; v < kRowJT; ++v) {
-            if constexpr (TURN) {
-                if (active) totals[v * kRowCompute + tid] += acc[v];
-            } else {
-                outer[v] += acc[v].x + acc[v].y;
-            }
+            for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
+            if (!TOGETHER && tile + 2 < tile_end) bar_arrive(kEmpty + st, kHandOver);
         }
-        if (!TOGETHER && i + 2 < my_tiles) bar_arrive(kEmpty + group2 + st, kHandOver);
     }
 
     // The next kernel is let in only now: its CTAs, waiting beside this kernel's, would be in the way of the generating warps
