@@ -488,12 +488,14 @@ static bool row_together(int32_t rows, bool aligned, int32_t m) { return (int64_
 // generation (one in seven instead of one in five): lines through measured shapes (us, without -> with; aligned rows, d = 1e7: n = 5,
 // m = 32: 537 -> 522 the round; n = 32, m = 100: 1649 -> 1584; but n = 4, m = 16: 300 -> 330, n = 8, m = 32: 539 -> 549;
 // shifted, d = 1e7: n = 7, m = 64: 1073 -> 1063; n = 5, m = 100 at d = 1e6: 178 -> 171; but n = 3, m = 32: 579 -> 603,
-// n = 16, m = 128: 2147 -> 2190).  By size (n = 1): d = 3e5, m = 64: 23.3 -> 21.8; d = 5e4, m = 400: 23.0 -> 22.8.
+// n = 16, m = 128: 2147 -> 2190).  By size (n = 1): d = 3e5, m = 64: 23.3 -> 21.8; d = 5e4, m = 400: 23.0 -> 22.8.  Few blocks for
+// many vectors share out badly over one CTA per SM, so more than 512 vectors need three times the work: at 2^24 Gaussians m = 768: 20.0 -> 22.3,
+// 4096: 20.1 -> 22.7, 8192: 20.4 -> 22.3; at 2.7 times as many -0.4, -2.4, -1.3 %.
 // The message of a single row must not depend on where the row starts, so there the line asks for the number of vectors alone, and lies
 // where aligned and shifted rows both gain (d = 1e7, aligned / shifted: m = 24: 216 -> 198 / 226 -> 205; but m = 13, d = 1e8: 1387 -> 1302 /
 // 1548 -> 1707; m = 20, d = 3e6: 60 -> 60 / 62 -> 66).
 static bool row_turn(int32_t rows, bool aligned, int32_t m, int64_t d) {
-    if (d < ((int64_t)1 << 24) / m) return false;
+    if (d < ((int64_t)(m > 512 ? 3 : 1) << 24) / m) return false;
     if (rows == 1) return m > 20;
     return aligned ? 11 * (int64_t)rows + 40 < 4 * (int64_t)m : 8 * (int64_t)rows + 10 < m;
 }

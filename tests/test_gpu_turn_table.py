@@ -82,7 +82,8 @@ def test_reconstructions_do_not_depend_on_what_ran_before(core_mod):
 
 
 @pytest.mark.parametrize("n,d,m,dtype,offset,pad", [
-    (1, 16_385, 1024, "f32", 0, 0), (1, 16_400, 1030, "bf16", 0, 8), (1, 5_600, 3073, "f32", 3, 0), (1, 100_003, 170, "bf16", 5, 0),
+    (1, 16_385, 1024, "f32", 0, 0), (1, 16_400, 1030, "bf16", 0, 8), (1, 5_600, 3073, "f32", 3, 0),
+    (1, 49_153, 1024, "f32", 0, 0), (1, 48_900, 1030, "bf16", 0, 8), (1, 16_385, 3073, "f32", 3, 0), (1, 100_003, 170, "bf16", 5, 0),
     (1, 1_200_001, 14, "f32", 0, 0), (3, 600_001, 61, "f32", 0, 3), (4, 262_147, 130, "bf16", 1, 6), (20, 335_546, 101, "f32", 0, 2),
 ])
 def test_projections(core_mod, n, d, m, dtype, offset, pad):

@@ -57,3 +57,11 @@ def test_a_single_row_has_one_plan_wherever_it_starts(dtype, size):
             plans = [binding.core_debug_row_plan(m, d, ldg=d + pad, dtype=dtype, misaligned=off)
                      for pad in (0, 1, 2, 8) for off in range(0, 16, size)]
             assert all(p == plans[0] for p in plans), (m, d)
+
+
+def test_short_rows_of_many_vectors_keep_the_polynomials():
+    """More than 512 vectors take the table of angles from 3 * 2^24 Gaussians on, fewer from 2^24."""
+    for m, least in ((512, 1 << 24), (513, 3 << 24), (768, 3 << 24), (1024, 3 << 24), (4096, 3 << 24), (16_384, 3 << 24)):
+        for rows in (1, 2):
+            assert not binding.core_debug_row_plan(m, least // m - 1, rows=rows)["turn"]
+            assert binding.core_debug_row_plan(m, (least // m + 3) // 4 * 4, rows=rows)["turn"]
