@@ -41,7 +41,7 @@ constexpr uint32_t kPassRingBytes = 128u * 1024u;       // bytes in flight per S
 // per lane leave the registers, and rows of up to 24 KB the shared memory, for it (gradients, us: 16 x 2048 rows of
 // 2049 columns: 125 with one, 84 with two, 66 with four; 8 x 1500 x 5500: 56 with two, 46 with four); the 512-thread
 // kernel of 16 warps per row has registers for two up to 24 columns, and gains by two up to 28, as far as the shared memory has
-// room for two slots of them (14064 columns), although some registers are then spilled (8 x 64 rows of 100000: 80 with one, 70 with two; 16 x 512
+// room for two slots of them (14064 columns) and the rows are many enough (make_ls_pass), although some registers are then spilled (8 x 64 rows of 100000: 80 with one, 70 with two; 16 x 512
 // of 14000: 89, 80).
 constexpr int pass_batch(int warps_per_row, int columns) {
     return warps_per_row == 1 ? (columns <= 2 ? 16 : 32 / columns) : warps_per_row == 16 ? (columns > 28 ? 1 : 2) : columns <= 24 ? 4 : 2;
@@ -601,7 +601,14 @@ LsPass make_ls_pass(int32_t n, int64_t rows, int64_t d, bool machines_apart, int
     while (p.columns < per_lane) p.columns *= 2;
     if (p.group_warps > 1) p.columns = per_lane > 20 ? (per_lane + 3) / 4 * 4 : per_lane > 16 || p.group_warps == kPassMaxWarps ? 20 : per_lane > 12 ? 16 : 12;
     const uint32_t smem = 220u * 1024u;
-    if (p.columns == 28 && (p.group_warps < kPassMaxWarps || 4 * (p.slice * 4 + 56) > (int)smem)) p.columns = 32;      // no room for two slots of two rows
+    if (p.columns == 28) {
+        // Two rows at a time want room for two slots of two rows, and rows enough per unit (before that the ring's start, in chunks of two
+        // rows, counts more than the chain).  us, one row at a time -> two, by rows per unit: one CTA per row (13300 columns), 4: 21.0 ->
+        // 23.7, 16: 5 % slower, 24: equal, 40: 4 % faster; clusters of two (26476), 4: 26.7 -> 28.6, 8 to 11: 1 to 4 % faster, 16: 2 % slower,
+        // 24: 3 % faster; of four and eight, 2: 1 to 2 % slower, 3: 4 % faster, 8: 8 to 11 %.
+        const int64_t least = p.cluster == 1 ? 24 : p.cluster == 2 ? 8 : 3;
+        if (p.group_warps < kPassMaxWarps || 4 * (p.slice * 4 + 56) > (int)smem || (int64_t)n * rows * p.cluster < least * sm_count) p.columns = 32;
+    }
     p.warps = p.group_warps == 1 || p.columns == 12 || p.group_warps == 16 ? 16 : 8;
     const int groups = p.warps / p.group_warps;
     const uint32_t row_bytes = (uint32_t)p.slice * 4;

@@ -84,7 +84,9 @@ def test_rows_shorter_than_a_copy_unit(core_mod, n, rows, d, offset):
 
 @pytest.mark.parametrize("n,rows,d,offset", [
     (2, 75, 10240, 0), (1, 40, 10241, 1), (2, 150, 12288, 0), (3, 50, 12289, 1), (1, 160, 13824, 0), (2, 30, 14064, 2), (2, 75, 14065, 3),   # a CTA
-    (2, 40, 20480, 0), (1, 37, 20481, 1), (2, 37, 28126, 0), (1, 30, 28133, 3), (1, 20, 100003, 0)])                                  # clusters
+    (2, 40, 20480, 0), (1, 37, 20481, 1), (2, 37, 28126, 0), (1, 30, 28133, 3), (1, 20, 100003, 0),                                   # clusters
+    (2, 1776, 12289, 1), (1, 3551, 14064, 0), (3, 197, 25505, 3), (1, 592, 28126, 0), (1, 120, 56001, 1), (1, 57, 110003, 0)])      # 28 columns: rows enough
 def test_columns_per_lane_of_long_rows(core_mod, n, rows, d, offset):
-    """20, 24, 28 and 32 columns per lane, two rows at a time or one, up to the last row length of each."""
+    """20, 24, 28 and 32 columns per lane, two rows at a time or one, up to the last row length of each and on both sides of the number of
+    rows from which 28 columns are taken."""
     test_gradients_loss_and_step(core_mod, n, rows, d, offset)
