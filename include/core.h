@@ -129,10 +129,10 @@ int core_device_status(int32_t *status_out);
  * message may differ in the last bits from the same row's among others: one row and
  * several take different kernels.)
  * Machines are processed in groups: up to 64 per pass where the tensor-memory
- * kernel applies (9 or more machines, m >= 96; more than 32 only when m lets a CTA
- * hold 256 vectors, about m >= 256), otherwise up to 16.  The
- * tensor-core kernels form their products with every operand split into a tf32
- * head and tail (same error bar, same reproducibility).  May grow the
+ * kernel applies (9 or more machines, m > 64 for passes of up to 16 and m >= 96 for
+ * longer ones; more than 32 only when m lets a CTA hold 256 vectors, about m >= 256),
+ * otherwise up to 16.  That kernel forms its products with every operand split
+ * into a tf32 head and tail (same error bar, same reproducibility).  May grow the
  * workspace.
  */
 int core_project(core_ctx *ctx, const void *G_dev, int dtype, int32_t n, int64_t ldg, float *P_dev);
@@ -316,8 +316,8 @@ int core_ls_gradients(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G_o
 /* ---- failure paths, made on the host or bounded on the device (no counterpart in the paper) ---- */
 
 /*
- * Which projection kernel later calls use: -1 the library's choice by shape (default), 0 or 1 the scalar
- * kernel, 2 the tensor-memory (tcgen05) kernel for every group of machines it can take (up to 64).  Process-wide; for measuring where one kernel
+ * Which projection kernel later calls use: -1 the library's choice by shape (default), 0 the scalar
+ * kernel (1, once a kernel of its own, means the same), 2 the tensor-memory (tcgen05) kernel for every group of machines it can take (up to 64).  Process-wide; for measuring where one kernel
  * overtakes the other and for testing each on shapes the default would not give it.
  */
 int core_debug_force_project_kernel(int kind);
@@ -358,7 +358,7 @@ int core_debug_wait_clock(const uint64_t *readings_ns, int32_t count, uint64_t l
 
 /* words_dev[4*(q-q0) + l] = word l of block q of vector j, q0 <= q < q0+nq, current t. */
 int core_debug_philox(core_ctx *ctx, uint32_t j, uint64_t q0, int64_t nq, uint32_t *words_dev);
-/* z_dev[4*(q-q0) + l] = xi_j[4q + l]. */
+/* z_dev[4*(q-q0) + l] = xi_j[4q + l], by the polynomials (kernels that take angles from a table are within 2.4e-6 of them). */
 int core_debug_gaussians(core_ctx *ctx, uint32_t j, uint64_t q0, int64_t nq, float *z_dev);
 /* Box-Muller alone: z_dev[4b..4b+3] from the caller's words_dev[4b..4b+3], b < nb. */
 int core_debug_box_muller(core_ctx *ctx, const uint32_t *words_dev, int64_t nb, float *z_dev);

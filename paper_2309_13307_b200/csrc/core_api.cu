@@ -445,10 +445,10 @@ static SlabRule input_slabs(int64_t d, int32_t n, size_t es) {
     // at least 256 KB per machine and copy
     return {std::min(most, slab_limit(d, std::max((int64_t)4 << 20, (int64_t)n << 18), es * (size_t)n)), most, INT64_MAX, 1};
 }
-// Every slab is one launch of the reconstruction.  Its kernel for long vectors shares any length out evenly; long slabs are
-// whole multiples of 96 units of 32 blocks per SM all the same, four of those multiples on 148 SMs, so that SMs have the same
-// number of units, three per warp.  (Twice as long: longer steps up to them where the copies are the slower
-// side: n = 1, d = 3e7, m = 64: 4.80 -> 4.90 ms.)
+// Every slab is one launch of the reconstruction.  Long slabs are whole multiples of 48 units of 32 blocks per SM, at most four
+// of them on 148 SMs: with the table of angles every SM has the same number of units then (six per warp in the longest slabs), and
+// 48 units are also one wave of the kernel for few or very many vectors.  (Longest slabs of eight multiples: longer steps up to
+// them where the copies are the slower side: n = 1, d = 3e7, m = 64: 4.80 -> 4.90 ms.)
 static SlabRule output_slabs(int64_t d, int sm_count) {
     const int64_t most = slab_limit(d, (int64_t)16 << 20, sizeof(float));
     return {std::min(most, slab_limit(d, (int64_t)1 << 20, sizeof(float))), most,

@@ -430,7 +430,8 @@ __global__ void debug_philox_kernel(const __grid_constant__ DebugArgs a, uint4 *
     }
 }
 
-// Goes through the split evaluation the round kernels use, so that path is what is checked.
+// Goes through the split evaluation of Philox, which all round kernels use, and the polynomials of those without the table of angles.
+// (The Gaussians of those with it are read back by messages and gradients that are unit vectors.)
 __global__ void debug_gaussians_kernel(const __grid_constant__ DebugArgs a, float4 *z) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < a.nq; r += stride) {

@@ -7,9 +7,13 @@
 //   counter = (q lo, q hi, j, t)   q = coordinate block k >> 2, j = vector, t = round
 //   u(w)    = ((w >> 9) + 1/2) 2^-23
 //   pair    = sqrt(-2 ln u(w_even)) * (cos, sin)(2 pi u(w_odd))
-// One counter yields xi_j[4q .. 4q+3].  Nothing here touches memory: both the
-// projection and the reconstruction kernel call these functions and so see
-// identical vectors.
+// One counter yields xi_j[4q .. 4q+3].  The words are the same in every kernel.
+// From them there are two ways to the angle: polynomials, in registers alone
+// (the projections of several machines, short reconstructions and rows, those of
+// few or very many vectors), and a table in a CTA's shared memory (last section;
+// long reconstructions, long single rows).  Each is within 1.2e-6 of Box-Muller,
+// so a projection by one and a reconstruction by the other see vectors that
+// differ by 2.4e-6 at most.
 #pragma once
 
 #include <cstdint>

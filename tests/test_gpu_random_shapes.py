@@ -1,5 +1,5 @@
 """Seeded random shapes against the oracle (through the C ABI): machine counts on both sides of every
-kernel choice (scalar, warp-level, tensor-memory with 128 or 256 vectors per CTA and 16, 32 or 64 machines
+kernel choice (scalar, tensor-memory with 128 or 256 vectors per CTA and 16, 32 or 64 machines
 per pass), vector counts around the CTA-row sizes, ragged lengths, unaligned rows and padded leading
 dimensions, both gradient types.  Same bars as the other round tests."""
 import random

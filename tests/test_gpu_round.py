@@ -101,7 +101,7 @@ def test_medium_sizes(core_mod, n, m, d, dtype, dist):
     check_round(core_mod, G, m, seed=5, t=1)
 
 
-@pytest.mark.parametrize("n,d,m", [(3, 5003, 7), (10, 3001, 70), (13, 3001, 256)])   # scalar, warp-level and tcgen05 projection
+@pytest.mark.parametrize("n,d,m", [(3, 5003, 7), (10, 3001, 70), (13, 3001, 256)])   # scalar and (two shapes) tcgen05 projection
 def test_unaligned_rows_and_leading_dimension(core_mod, n, d, m):
     for dtype in ("f32", "bf16"):
         # ld > d with an odd stride, and a base pointer that is not 16-byte aligned
@@ -130,7 +130,7 @@ def test_device_status_word(core_mod):
 
 @pytest.mark.parametrize("n,m,dtype", [
     (2, 8, "f32"), (4, 40, "bf16"), (8, 64, "f32"),       # scalar projection
-    (10, 70, "f32"), (12, 72, "bf16"),                    # warp-level tensor-core projection
+    (10, 70, "f32"), (12, 72, "bf16"),                    # tcgen05 projection, CTA rows half full
     (16, 256, "bf16"), (9, 128, "f32"),                   # tcgen05 projection
     (32, 128, "f32"), (27, 256, "bf16"),                  # tcgen05 projection, 32 machines per pass
     (64, 256, "bf16"), (40, 512, "f32"),                  # tcgen05 projection, 64 machines per pass
@@ -223,7 +223,7 @@ def test_host_round_many_slabs(core_mod, m):
 @pytest.mark.parametrize("kind,n,m,dtype", [(2, 5, 128, "f32"), (2, 8, 256, "bf16"), (2, 3, 40, "f32"), (2, 20, 33, "bf16"),
                                           (0, 16, 256, "bf16"), (0, 12, 128, "f32"), (1, 16, 256, "f32")])
 def test_each_projection_kernel_on_shapes_the_default_would_not_give_it(core_mod, kind, n, m, dtype):
-    """The tensor-memory kernel with few machines and few vectors, the scalar and the warp-level kernels on
+    """The tensor-memory kernel with few machines and few vectors, the scalar kernel (kinds 0 and 1) on
     shapes that normally go to the tensor-memory kernel: all must meet the same bars."""
     from paper_2309_13307_b200 import binding
     G = core_inputs.gradients(n, 50_021, seed=21, dtype=dtype, device="cuda")

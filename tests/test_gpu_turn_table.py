@@ -39,6 +39,27 @@ def test_gaussians(core_mod, d, m, j):
     assert np.abs(got - want).max() <= XI_TOL
 
 
+@pytest.mark.parametrize("n,d,m,dtype,offset", [(1, 800_003, 21, "f32", 0), (1, 200_001, 100, "bf16", 3), (1, 30_000, 2049, "f32", 1),
+                                                (2, 600_001, 61, "bf16", 0), (4, 600_001, 61, "f32", 1)])
+def test_unit_vectors_read_the_projections_gaussians_back(core_mod, n, d, m, dtype, offset):
+    """The message of e_k is xi_j[k], element by element: every other term of the sum is an exact zero."""
+    from paper_2309_13307_b200 import binding
+    size = 2 if dtype == "bf16" else 4
+    G = torch.zeros((n, d + offset), dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device="cuda")[:, offset:]
+    plan = binding.core_debug_row_plan(m, d, rows=n, ldg=d + offset, dtype=binding.CORE_BF16 if dtype == "bf16" else binding.CORE_F32,
+                                       misaligned=offset * size % 16)
+    assert plan["turn"]
+    tile = 4 * plan["tile_q"]
+    ctx = core_mod.Core(6, d, m)
+    for k in sorted({0, 5, tile - 1, tile, d // 2, (plan["tiles"] - 1) * tile - 2, (plan["tiles"] - 1) * tile, d - 1}):
+        G[:, k] = 1
+        ctx.core_set_round(3)
+        got = (ctx.core_project(G)[0] if n == 1 else ctx.core_round(G)[0]).cpu().numpy().astype(np.float64)
+        G[:, k] = 0
+        want = np.array([oracle.xi_range(6, 3, j, k, k + 1)[0] for j in range(m)])
+        assert np.abs(got - want).max() <= XI_TOL, k
+
+
 @pytest.mark.parametrize("d,m", [
     (94_717, 178), (94_720, 1025), (94_721, 2049), (151_552, 111), (151_553, 112), (303_100, 64), (1_000_003, 17), (6_000_000, 3),
     (17_000_001, 1), (17_000_001, 2), (100_003, 8192), (100_003, 8195), (700_001, 131),
