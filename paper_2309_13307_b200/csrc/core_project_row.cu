@@ -19,7 +19,7 @@
 // scalar instructions per counter.
 //
 // Three modes.  kRowTurn, wherever there is work for it: angles from the table, one CTA of 24 generating and 4 staging warps
-// per SM, d = 2.5e7, m = 256: 4904 us = 1.31e12 Gaussians/s.  kRowShort: angles from the polynomials, two CTAs of 8 and 2
+// per SM, d = 2.56e7, m = 256: 4944 us = 1.32e12 Gaussians/s.  kRowShort: angles from the polynomials, two CTAs of 8 and 2
 // warps per SM (5325 us there), for short work.  kRowTogether: the same, all warps stage.  In kRowTurn the registers decide:
 // 72 per thread hold the loop only because the sums over tiles live in shared memory and scalar accumulators
 // (packed ones need pairs: 5138 us) and 32-bit counts go around it (64-bit tile numbers: 5095); 20 generating warps of 80 registers:
@@ -39,6 +39,9 @@ namespace core {
 namespace {
 
 constexpr int kRowJT = 4;                        // vectors per generating thread
+// With the table: steps that are added up before they meet the sums in shared memory.  The chain of additions is this long, then as
+// long as a CTA's tiles have such parts; both about a hundred in rows of 2.5e7 (errors grow with the square root of their sum).
+constexpr int kRowSumSteps = 64;
 
 // With the table of angles one CTA fills an SM, without it two do.
 template <bool TURN>
@@ -49,7 +52,8 @@ struct RowCta {
     static constexpr int kGroups = TURN ? 3 : 1;             // of generating warps that take a tile over by themselves
     static constexpr int kWarps = kThreads / 32;
     static constexpr int kPerSm = TURN ? 1 : 2;
-    static constexpr int kTileBlocks = TURN ? 2048 : 1024;   // most blocks of a tile
+    static constexpr int kTileBlocks = TURN ? 2048 : 1024;   // most blocks of a tile,
+    static constexpr int kTileSteps = TURN ? 128 : 64;       // and most steps of a generating thread in one
 };
 
 struct RowArgs {
@@ -337,10 +341,15 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
             const int blocks = i == my_tiles - 1 ? last_blocks : a.tile_q;
             if (i >= 1) bar_sync(kFull + group2 + st, kHandOver);
             const float4 *const cur = tile0 + 2 * st * a.tile_q;
-            float acc[kRowJT] = {};
             if (active) {
                 const float4 *entry = cur + 2 * ql;
-                for (int upto = min(blocks, change - i * a.tile_q);;) {
+                for (int upto = 0; upto < blocks;) {
+                    if (upto == change - i * a.tile_q) {
+                        change = INT_MAX;
+                        make_jp((uint32_t)(first_q() >> 32) + 1);
+                    }
+                    upto = min(min(upto + kRowSumSteps * a.tq, blocks), change - i * a.tile_q);
+                    float acc[kRowJT] = {};
                     for (const float4 *const stop = cur + 2 * upto; entry < stop; entry += 2 * a.tq) {
                         const float4 g = entry[0], e = entry[1];
                         QPart qp;
@@ -360,15 +369,10 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                             acc[v] = fmaf(r.s.x, t.x, fmaf(r.s.y, t.y, acc[v]));
                         }
                     }
-                    if (upto == blocks) break;
-                    upto = blocks;
-                    change = INT_MAX;
-                    make_jp((uint32_t)(first_q() >> 32) + 1);
+#pragma unroll
+                    for (int v = 0; v < kRowJT; ++v) totals[v * kRowCompute + tid] += acc[v];
                 }
             }
-#pragma unroll
-            for (int v = 0; v < kRowJT; ++v)
-                if (active) totals[v * kRowCompute + tid] += acc[v];
             if (i + 2 < my_tiles) bar_arrive(kEmpty + group2 + st, kHandOver);
         }
     } else {
@@ -539,10 +543,14 @@ static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
     const int64_t nq = (d + 3) >> 2;
     int64_t slots = (int64_t)sm_count * per_sm / p.grid_y;             // CTAs across coordinates that are resident together
     if (slots < 1) slots = 1;
-    // blocks per tile: as many steps per tile and generating thread as fit (32, or 1024 blocks: two tiles take 64 KB),
+    // blocks per tile: as many steps per tile and generating thread as fit (1024 blocks without the table, 2048 with it: two tiles
+    // take 64 or 128 KB), at most 64 or 128, beyond which nothing is gained.  At every tile a group's warps wait for its slowest:
+    // us, 32 steps -> this: d = 2.56e7, m = 256: one row 5006 -> 4944, eight rows 5035 -> 4987; 32 rows of 1e7, m = 1000: 7830 -> 7746;
+    // 16 bf16 rows of 3.1e7, m = 1024: 24198 -> 23915; without the table, seven shifted rows of 1e7, m = 64: 595 -> 589,
     // and of the tile counts per CTA from there on the one that leaves the fewest steps to the CTA with most of them
     // (d = 1e6, m = 100: 104 -> 98 us)
-    const int64_t most = 32 * p.tq < room ? 32 * p.tq : room / p.tq * p.tq;
+    const int steps_most = turn ? RowCta<true>::kTileSteps : RowCta<false>::kTileSteps;
+    const int64_t most = steps_most * p.tq < room ? steps_most * p.tq : room / p.tq * p.tq;
     const int64_t least_tiles = (nq + slots * most - 1) / (slots * most);
     int64_t best_steps = -1;
     for (int64_t k = least_tiles; k <= 2 * least_tiles && k < least_tiles + 16; ++k) {
