@@ -1,6 +1,7 @@
 // Machine gradients of the least-squares objective that drives Algorithm 2, for rows too long for the single pass
 // of core_ls_pass.cu: f_i(x) = 1/(2 rows) ||A_i x - b_i||^2, g_i = A_i^T (A_i x - b_i) / rows in two streaming passes
 // over A (both HBM-bound), every sum in a fixed order.  Also the comparison step of Algorithm 3.
+#include "core_finish.cuh"
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -134,9 +135,7 @@ keep_better_kernel(const double *__restrict__ f_parts, int64_t parts, double sca
     grid_wait();
     __shared__ int decision;
     if (threadIdx.x < 32) {
-        double s = 0.0;                         // as in ls_loss_sum_kernel: the same bits
-#pragma unroll 8
-        for (int64_t u = threadIdx.x; u < parts; u += 32) s += __ldcg(f_parts + u);
+        double s = sum_strided(f_parts + threadIdx.x, (int)((parts - threadIdx.x + 31) / 32), 32);      // as in ls_loss_sum_kernel: the same bits
 #pragma unroll
         for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (threadIdx.x == 0) {

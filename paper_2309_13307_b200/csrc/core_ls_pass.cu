@@ -18,6 +18,7 @@
 // n = 50, 11620 x 54: gradients 377 -> 31, loss 212 -> 28; n = 16, 256 x 20000: gradients 133 -> 72; n = 8, 2048 x 8192
 // (537 MB): loss 107 -> 88, gradients 87 -> 92.  Tried: cp.async instead of bulk copies (20 % slower), rings of 96 to
 // 192 KB (equal), evict_normal instead of evict_first (3 to 10 us slower), 8 warps for one-warp rows (25 % slower).
+#include "core_finish.cuh"
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -486,19 +487,14 @@ __global__ void ls_pass_reduce_kernel(const float *__restrict__ part, int64_t ro
     if (k >= d) return;
     const int64_t first = ((i * rows + 1) * units - 1) / total, last = ((i + 1) * rows * units - 1) / total;
     const float *p = part + i * slots_per_machine * ldp + k;
-    float s = 0.f;
-#pragma unroll 8
-    for (int64_t u = first; u <= last; ++u, p += ldp) s += __ldcg(p);
-    G[i * d + k] = s * inv_rows;
+    G[i * d + k] = sum_strided(p, (int)(last - first) + 1, ldp) * inv_rows;
 }
 
 // loss[0] = scale * sum of the units' sums of squares: lane l sums units l, l + 32, ..., then a fixed tree.
 __global__ void ls_loss_sum_kernel(const double *__restrict__ loss_part, int64_t units, double scale, double *loss) {
     grid_trigger();
     grid_wait();
-    double s = 0.0;
-#pragma unroll 8
-    for (int64_t u = threadIdx.x; u < units; u += 32) s += __ldcg(loss_part + u);
+    double s = sum_strided(loss_part + threadIdx.x, (int)((units - threadIdx.x + 31) / 32), 32);
 #pragma unroll
     for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (threadIdx.x == 0) loss[0] = s * scale;
