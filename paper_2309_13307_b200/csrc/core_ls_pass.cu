@@ -229,12 +229,17 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     const int first = lane + 32 * wg;
     // The first rows on their way to L2 while the kernels before this one finish (to L2 only: whoever still writes A writes
     // it there)
-    if (leader && !edge && a.cluster == 1)
+    if (leader && !edge)
         for (int s = 0; s < a.slots; ++s) {
             const int k = grp + s * GROUPS;
             if (k >= chunks) break;
-            const BulkRange r = prefetch_range(src + (int64_t)s * src_step, (uint32_t)min(R, nrows - first_row(k)) * row_bytes);
-            if (r.b1 > r.b0) bulk_prefetch(reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0));
+            const int count = min(R, nrows - first_row(k));
+            const bool sliced = MULTI && a.cluster > 1;
+            for (int i = 0; i < (sliced ? count : 1); ++i) {
+                const BulkRange r = prefetch_range(src + (int64_t)s * src_step + (int64_t)((uint32_t)i * row_bytes),
+                                                   sliced ? (uint32_t)dn * 4 : (uint32_t)count * row_bytes);
+                if (r.b1 > r.b0) bulk_prefetch(reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0));
+            }
         }
     grid_wait();
     if (leader)
