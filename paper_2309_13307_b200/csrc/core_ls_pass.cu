@@ -708,7 +708,9 @@ void ls_pass_reads(const LsPass &p, int64_t d, uintptr_t a_begin, int64_t *befor
             for (int i = 0; i < count; ++i)
                 for (int64_t col = 0; col < d; col += p.slice) {
                     const uintptr_t from = src + (uintptr_t)i * row_bytes + (uintptr_t)col * 4;
-                    copy(from, from + (uintptr_t)std::min<int64_t>(p.slice, d - col) * 4);
+                    const uint32_t bytes = (uint32_t)std::min<int64_t>(p.slice, d - col) * 4;
+                    copy(from, from + bytes);
+                    if (!u.edge) touch(prefetch_range(from, bytes));
                 }
         }
     }
