@@ -29,7 +29,7 @@ __global__ void aggregate_kernel(const float *__restrict__ P, int n, int m, floa
     grid_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m) return;
-    pbar[j] = sum_strided(P + j, n, m) / (float)n;
+    pbar[j] = sum_strided<16>(P + j, n, m) / (float)n;
 }
 
 // Both of the above in one launch for a single group of machines whose messages nobody asks for:

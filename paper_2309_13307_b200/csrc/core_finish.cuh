@@ -11,25 +11,57 @@ namespace core {
 
 constexpr int kFinishSlices = 8;
 
-// p[0] + p[stride] + ... of `count` numbers, in ascending order, eight loads in flight at a time also where fewer are left: a loop
-// unrolled by the compiler fetches its last up to seven one after the other, each a round trip to L2 (us: a round of
-// four machines, d = 4096, m = 16: 8.2 -> 7.1; a decentralised step of 16 machines, d = 20000, m = 64: 86.4 -> 84.0).
-template <typename T>
+// p[0] + p[stride] + ... of `count` numbers, in ascending order, AT (4, 8 or 16) loads in flight at a time, and the last ones, fewer than that,
+// together too: a loop unrolled by the compiler may fetch those one after the other, each a round trip to L2 (us: a round of four
+// machines, d = 4096, m = 16: 8.2 -> 7.1; a decentralised step of 16 machines, d = 20000, m = 64: 86.4 -> 84.0).
+template <int AT, typename T>
 __device__ __forceinline__ T sum_strided(const T *p, int count, int64_t stride) {
     T s = 0;
-    for (int c = 0; c < count; c += 8, p += 8 * stride) {
-        T v[8];
+    for (; count >= AT; count -= AT, p += AT * stride) {
+        T v[AT];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = c + i < count ? __ldcg(p + i * stride) : (T)0;
+        for (int i = 0; i < AT; ++i) v[i] = __ldcg(p + i * stride);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s += v[i];
+        for (int i = 0; i < AT; ++i) s += v[i];
     }
-    return s;
+    T a[8], b[4], c[2], d = 0;
+    if (AT > 8 && count & 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a[i] = __ldcg(p + i * stride);
+        p += 8 * stride;
+    }
+    if (AT > 4 && count & 4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) b[i] = __ldcg(p + i * stride);
+        p += 4 * stride;
+    }
+    if (count & 2) {
+        c[0] = __ldcg(p);
+        c[1] = __ldcg(p + stride);
+        p += 2 * stride;
+    }
+    if (count & 1) d = __ldcg(p);
+    if (AT > 8 && count & 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s += a[i];
+    }
+    if (AT > 4 && count & 4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s += b[i];
+    }
+    if (count & 2) {
+        s += c[0];
+        s += c[1];
+    }
+    return count & 1 ? s + d : s;
 }
 
+// (Fewer at a time in kernels that want their registers for something else: the gossip of 17 to 32 machines spilled with sixteen: 1.2 us
+// a step.)
+template <int AT = 16>
 __device__ __forceinline__ float finish_slice(const float *partial, int chunks, int64_t total, int64_t idx, int slice) {
     const int begin = chunks * slice / kFinishSlices, end = chunks * (slice + 1) / kFinishSlices;
-    return sum_strided(partial + (int64_t)begin * total + idx, end - begin, total);
+    return sum_strided<AT>(partial + (int64_t)begin * total + idx, end - begin, total);
 }
 
 // The slices of an entry, `stride` floats apart.

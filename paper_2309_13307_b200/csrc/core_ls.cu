@@ -135,7 +135,7 @@ keep_better_kernel(const double *__restrict__ f_parts, int64_t parts, double sca
     grid_wait();
     __shared__ int decision;
     if (threadIdx.x < 32) {
-        double s = sum_strided(f_parts + threadIdx.x, (int)((parts - threadIdx.x + 31) / 32), 32);      // as in ls_loss_sum_kernel: the same bits
+        double s = sum_strided<8>(f_parts + threadIdx.x, (int)((parts - threadIdx.x + 31) / 32), 32);      // as in ls_loss_sum_kernel: the same bits
 #pragma unroll
         for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (threadIdx.x == 0) {

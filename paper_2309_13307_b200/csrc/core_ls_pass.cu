@@ -229,18 +229,20 @@ ls_pass_kernel(const __grid_constant__ PassArgs a) {
     const int first = lane + 32 * wg;
     // The first rows on their way to L2 while the kernels before this one finish (to L2 only: whoever still writes A writes
     // it there)
-    if (leader && !edge)
+    if (leader && !edge && a.cluster == 1)
         for (int s = 0; s < a.slots; ++s) {
             const int k = grp + s * GROUPS;
             if (k >= chunks) break;
-            const int count = min(R, nrows - first_row(k));
-            const bool sliced = MULTI && a.cluster > 1;
-            for (int i = 0; i < (sliced ? count : 1); ++i) {
-                const BulkRange r = prefetch_range(src + (int64_t)s * src_step + (int64_t)((uint32_t)i * row_bytes),
-                                                   sliced ? (uint32_t)dn * 4 : (uint32_t)count * row_bytes);
-                if (r.b1 > r.b0) bulk_prefetch(reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0));
-            }
+            const BulkRange r = prefetch_range(src + (int64_t)s * src_step, (uint32_t)min(R, nrows - first_row(k)) * row_bytes);
+            if (r.b1 > r.b0) bulk_prefetch(reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0));
         }
+    if constexpr (W == 16)                              // (the only ones in clusters, a slice of each row)
+        if (leader && !edge && a.cluster > 1)
+            for (int k = 0; k < min(a.slots, chunks); ++k)
+                for (int i = 0; i < min(R, nrows - first_row(k)); ++i) {
+                    const BulkRange r = prefetch_range(src + (int64_t)k * src_step + (int64_t)((uint32_t)i * row_bytes), (uint32_t)dn * 4);
+                    if (r.b1 > r.b0) bulk_prefetch(reinterpret_cast<const void *>(r.b0), (uint32_t)(r.b1 - r.b0));
+                }
     grid_wait();
     if (leader)
         for (int s = 0; s < a.slots; ++s)
@@ -492,14 +494,14 @@ __global__ void ls_pass_reduce_kernel(const float *__restrict__ part, int64_t ro
     if (k >= d) return;
     const int64_t first = ((i * rows + 1) * units - 1) / total, last = ((i + 1) * rows * units - 1) / total;
     const float *p = part + i * slots_per_machine * ldp + k;
-    G[i * d + k] = sum_strided(p, (int)(last - first) + 1, ldp) * inv_rows;
+    G[i * d + k] = sum_strided<16>(p, (int)(last - first) + 1, ldp) * inv_rows;
 }
 
 // loss[0] = scale * sum of the units' sums of squares: lane l sums units l, l + 32, ..., then a fixed tree.
 __global__ void ls_loss_sum_kernel(const double *__restrict__ loss_part, int64_t units, double scale, double *loss) {
     grid_trigger();
     grid_wait();
-    double s = sum_strided(loss_part + threadIdx.x, (int)((units - threadIdx.x + 31) / 32), 32);
+    double s = sum_strided<8>(loss_part + threadIdx.x, (int)((units - threadIdx.x + 31) / 32), 32);
 #pragma unroll
     for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (threadIdx.x == 0) loss[0] = s * scale;

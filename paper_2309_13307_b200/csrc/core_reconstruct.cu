@@ -327,7 +327,7 @@ __device__ __forceinline__ void store_cluster(const void *smem, uint32_t rank, f
 }
 
 template <int SLICES>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
     grid_trigger();
     constexpr int QB = kThreads / SLICES;          // blocks per CTA
@@ -364,7 +364,7 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
             float *const slices = reinterpret_cast<float *>(table + kJoinVectors);
             for (int e = tid; e < entries * kFinishSlices; e += kThreads) {
                 const int entry = e % entries, i = entry / jn, j = entry % jn;
-                slices[e] = finish_slice(a.parts.partial, a.parts.chunks, (int64_t)n * a.m, (int64_t)i * a.m + j0 + j, e / entries);
+                slices[e] = finish_slice<4>(a.parts.partial, a.parts.chunks, (int64_t)n * a.m, (int64_t)i * a.m + j0 + j, e / entries);
             }
             __syncthreads();
             for (int jj = tid; jj < jn; jj += kThreads) {

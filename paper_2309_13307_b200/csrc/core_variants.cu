@@ -82,7 +82,7 @@ gossip_step_kernel(const float *W, const float *partial, int chunks, const float
         const int entries = n * kGossipCols;
         for (int e = tid; e < entries * kFinishSlices; e += blockDim.x) {
             const int entry = e % entries, slice = e / entries, jj = j0 + entry % kGossipCols;
-            slices[e] = jj < m ? finish_slice(partial, chunks, (int64_t)n * m, (int64_t)(entry / kGossipCols) * m + jj, slice) : 0.f;
+            slices[e] = jj < m ? finish_slice<NR >= 32 ? 4 : 8>(partial, chunks, (int64_t)n * m, (int64_t)(entry / kGossipCols) * m + jj, slice) : 0.f;
         }
         __syncthreads();
         if (tid < entries) buffers[0][col][i] = finish_join(slices + tid, entries);
