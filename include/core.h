@@ -17,7 +17,8 @@
  *   normal  Box-Muller on (w0,w1) and (w2,w3): r = sqrt(-2 ln u(w_even)),
  *           theta = 2 pi u(w_odd); xi_j[4q..4q+3] = (r_a cos th_a, r_a sin th_a,
  *           r_b cos th_b, r_b sin th_b).
- * The vectors are never stored: every kernel regenerates what it needs.
+ * The vectors are never stored in device memory: every kernel regenerates what it needs (a short round, which is one kernel, keeps
+ * them in shared memory between its projection and its reconstruction).
  *
  * Conventions for every entry point
  *   - Pointers named *_dev are DEVICE pointers owned by the caller; *_host are
@@ -127,7 +128,7 @@ int core_device_status(int32_t *status_out);
  * order: results are bitwise reproducible for a given (n, m, d, dtype), wherever the rows start
  * and whatever ldg is.  (A row's
  * message may differ in the last bits from the same row's among others: one row and
- * several take different kernels.)
+ * several take different kernels, and a short one, of at most 49152 = m times the blocks of four coordinates and 4096 vectors, a third.)
  * Machines are processed in groups: up to 64 per pass where the tensor-memory
  * kernel applies (9 or more machines, m > 64 for passes of up to 16 and m >= 96 for
  * longer ones; more than 32 only when m lets a CTA hold 256 vectors, about m >= 256),
@@ -367,7 +368,7 @@ int core_debug_box_muller(core_ctx *ctx, const uint32_t *words_dev, int64_t nb, 
  * Launch geometry the projection of separate messages would use for the first pass over n machines (at most
  * 64 per pass), m vectors and d coordinates on a device with sm_count SMs.  Host-only: touches no device.  n = 1
  * gives the plan of the scalar kernel, which a single row takes only where core_debug_force_project_kernel asks for
- * it: one row, and the combined row of a round, go through a kernel of their own.
+ * it: one row, and the combined row of a round, go through kernels of their own.
  * out[0..9] = machines per pass (rounded up to a power of two; 16, 32 or 64 for the tensor-memory kernel), vectors per thread,
  * coordinate blocks per thread step, blocks per shared-memory tile, threads across
  * vectors, threads across blocks, CTAs across coordinates, CTAs across vectors,
@@ -379,13 +380,14 @@ int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t 
  * Launch geometry of the kernel that projects one row, or the sum of `rows` rows, which start `misaligned` bytes beyond a multiple
  * of 16 and `ldg` elements apart.  Host-only.  out[0..9] = blocks per shared-memory tile, threads across vectors (four vectors
  * each), threads across blocks, CTAs across coordinates, CTAs across vectors, tiles of d, dynamic shared memory bytes, 1 if the angles
- * come from a table (0: polynomials), CTAs across coordinates that the workspace has room for, generating threads per CTA.
+ * come from a table (0: polynomials), CTAs across coordinates that the workspace has room for, generating threads per CTA.  (Short vectors
+ * whose round is one launch do without.)
  */
 int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligned, int32_t m, int64_t d, int32_t sm_count,
                         int64_t out[10]);
 
 /*
- * Which reconstruction kernel d coordinates and m vectors take, host-only: out[0] = 0 the one for short vectors, 1 the one for long
+ * Which reconstruction kernel d coordinates and m vectors take, host-only: out[0] = 0 one of the two for short vectors, 1 the one for long
  * vectors with few or very many Gaussians per coordinate, 2 the one with the table of angles; out[1] = 1 if the CTAs of the
  * reconstruction form the message of a round of one machine themselves.
  */

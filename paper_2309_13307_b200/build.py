@@ -11,9 +11,10 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libcore_b200.so")
-SOURCES = ["core_api.cu", "core_project.cu", "core_project_row.cu", "core_project_tc.cu", "core_finish.cu", "core_reconstruct.cu", "core_ls.cu", "core_ls_pass.cu",
+SOURCES = ["core_api.cu", "core_project.cu", "core_project_row.cu", "core_project_tc.cu", "core_finish.cu", "core_reconstruct.cu", "core_short.cu", "core_ls.cu", "core_ls_pass.cu",
            "core_static.cu", "core_pipes.cu", "core_variants.cu"]
 HEADERS = [os.path.join(CSRC, "core_rng.cuh"), os.path.join(CSRC, "core_internal.h"), os.path.join(CSRC, "core_sync.cuh"), os.path.join(CSRC, "core_finish.cuh"),
+           os.path.join(CSRC, "core_emit.cuh"),
            os.path.join(INCLUDE, "core.h")]
 
 

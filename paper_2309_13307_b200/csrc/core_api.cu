@@ -143,6 +143,11 @@ bool combine_first(const core_ctx *ctx, int32_t n) {
     return n > 1 && !project_kernel_forced() && ctx->d >= (kCombineFirst + ctx->m - 1) / ctx->m;
 }
 
+// A short vector's round of n machines goes through one kernel, and so does the projection of one (unless a test asks for one of the others).
+ShortPlan short_plan(const core_ctx *ctx, int32_t n) {
+    return project_kernel_forced() ? ShortPlan{} : make_short_plan(n, 1, ctx->m, ctx->d, ctx->sm_count);
+}
+
 size_t row_partial_bytes(const core_ctx *ctx, int64_t d) {
     return round_up((size_t)row_plan_columns(ctx->m, d, ctx->sm_count) * ctx->m * sizeof(float), 256);
 }
@@ -182,6 +187,24 @@ int project_into(core_ctx *ctx, const void *G, int dtype, int32_t n, int64_t ldg
         CORE_CUDA(ctx, launch_finish_project(partial, plan.grid_x, ng, ctx->m, P + (size_t)i0 * ctx->m, accumulate,
                                              stream));
     }
+    return CORE_OK;
+}
+
+// The messages of n machines' whole vectors.
+int project_all(core_ctx *ctx, const void *G, int dtype, int32_t n, int64_t ldg, float *partial, float *P) {
+    const ShortPlan plan = n == 1 ? short_plan(ctx, 1) : ShortPlan{};
+    if (plan.ctas == 0) return project_into(ctx, G, dtype, n, ldg, ctx->d, 0, partial, P, false, ctx->stream);
+    CORE_CUDA(ctx, launch_short_round(plan, ctx->keys, ctx->t, G, dtype, 1, n, ldg, 1.0f, ctx->d, ctx->m, P, nullptr, nullptr, nullptr, ctx->stream));
+    return CORE_OK;
+}
+
+// The estimate of the whole vector, or the update made from it.
+int reconstruct_all(core_ctx *ctx, float *pbar, float *out, const ReconstructEpilogue *epilogue, const MessageParts *parts = nullptr) {
+    const ShortPlan plan = make_short_plan(1, 1, ctx->m, ctx->d, ctx->sm_count);
+    if (plan.ctas > 0)
+        CORE_CUDA(ctx, launch_short_reconstruct(plan, ctx->keys, ctx->t, pbar, ctx->d, ctx->m, out, ctx->sm_count, epilogue, parts, ctx->stream));
+    else
+        CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream, epilogue, parts));
     return CORE_OK;
 }
 
@@ -298,8 +321,7 @@ int core_project(core_ctx *ctx, const void *G_dev, int dtype, int32_t n, int64_t
     if (int rc = check_ctx(ctx)) return rc;
     if (!G_dev || !P_dev || n < 1 || ldg < ctx->d || !valid_dtype(dtype)) return CORE_EINVAL;
     if (int rc = ensure_workspace(ctx, partial_bytes(ctx, n, ctx->d, dtype))) return rc;
-    return project_into(ctx, G_dev, dtype, n, ldg, ctx->d, 0, static_cast<float *>(ctx->ws), P_dev, false,
-                        ctx->stream);
+    return project_all(ctx, G_dev, dtype, n, ldg, static_cast<float *>(ctx->ws), P_dev);
 }
 
 int core_reserve_workspace(core_ctx *ctx, int32_t n, int dtype) {
@@ -321,9 +343,7 @@ int core_aggregate(core_ctx *ctx, const float *P_dev, int32_t n, float *pbar_dev
 int core_reconstruct(core_ctx *ctx, const float *pbar_dev, float *gtilde_dev) {
     if (int rc = check_ctx(ctx)) return rc;
     if (!pbar_dev || !gtilde_dev) return CORE_EINVAL;
-    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, const_cast<float *>(pbar_dev), ctx->m, 0, ctx->d, gtilde_dev, ctx->sm_count,
-                                      ctx->stream));
-    return CORE_OK;
+    return reconstruct_all(ctx, const_cast<float *>(pbar_dev), gtilde_dev, nullptr);
 }
 
 // A step chosen on the device from the combined messages, between aggregation and reconstruction
@@ -347,14 +367,14 @@ static int finish_round(core_ctx *ctx, const void *G, int dtype, int32_t rows, i
                         float *pbar_dev, float *out, const ReconstructEpilogue *epilogue, const StepRule *rule) {
     const RowPlan plan = make_row_plan(G, dtype, rows, ldg, ctx->m, ctx->d, ctx->sm_count);
     CORE_CUDA(ctx, launch_project_row(plan, ctx->keys, ctx->t, G, dtype, rows, ldg, scale, ctx->d, ctx->m, 0, partial, ctx->stream));
-    const MessageParts parts{partial, plan.grid_x, 1};
-    const bool join = !rule && reconstruct_joins(plan.grid_x, 1, ctx->m, ctx->d, ctx->sm_count);
-    if (!join) {
+    if (!rule && reconstruct_joins(plan.grid_x, 1, ctx->m, ctx->d, ctx->sm_count)) {
+        const MessageParts parts{partial, plan.grid_x, 1};
+        if (int rc = reconstruct_all(ctx, pbar_dev, out, epilogue, &parts)) return rc;
+    } else {
         CORE_CUDA(ctx, launch_finish_project(partial, plan.grid_x, 1, ctx->m, pbar_dev, false, ctx->stream));
         if (int rc = apply_step_rule(ctx, rule, pbar_dev)) return rc;
+        if (int rc = reconstruct_all(ctx, pbar_dev, out, epilogue)) return rc;
     }
-    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar_dev, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream, epilogue,
-                                      join ? &parts : nullptr));
     ctx->t += 1;
     return CORE_OK;
 }
@@ -368,6 +388,13 @@ static int round_with_epilogue(core_ctx *ctx, const void *G_dev, int dtype, int3
     if (int rc = ensure_workspace(ctx, pb + Pb)) return rc;
     float *partial = static_cast<float *>(ctx->ws);
     float *P = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + pb);
+    const ShortPlan in_one = short_plan(ctx, n);
+    if (in_one.ctas > 0 && !rule) {
+        CORE_CUDA(ctx, launch_short_round(in_one, ctx->keys, ctx->t, G_dev, dtype, 1, n, ldg, 1.0f, ctx->d, ctx->m, nullptr, pbar_dev, out, epilogue,
+                                          ctx->stream));
+        ctx->t += 1;
+        return CORE_OK;
+    }
     if (single_row(n) || combine_first(ctx, n))
         return finish_round(ctx, G_dev, dtype, n, ldg, 1.0f / (float)n, partial, pbar_dev, out, epilogue, rule);
     if (project_group(n, ctx->m) == n) {
@@ -377,19 +404,17 @@ static int round_with_epilogue(core_ctx *ctx, const void *G_dev, int dtype, int3
                                       ctx->stream));
         if (!rule && reconstruct_joins(plan.grid_x, n, ctx->m, ctx->d, ctx->sm_count)) {
             const MessageParts parts{partial, plan.grid_x, n};
-            CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar_dev, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream,
-                                              epilogue, &parts));
+            if (int rc = reconstruct_all(ctx, pbar_dev, out, epilogue, &parts)) return rc;
             ctx->t += 1;
             return CORE_OK;
         }
         CORE_CUDA(ctx, launch_finish_aggregate(partial, plan.grid_x, n, ctx->m, pbar_dev, ctx->stream));
     } else {
-        if (int rc = project_into(ctx, G_dev, dtype, n, ldg, ctx->d, 0, partial, P, false, ctx->stream)) return rc;
+        if (int rc = project_all(ctx, G_dev, dtype, n, ldg, partial, P)) return rc;
         CORE_CUDA(ctx, launch_aggregate(P, n, ctx->m, pbar_dev, ctx->stream));
     }
     if (int rc = apply_step_rule(ctx, rule, pbar_dev)) return rc;
-    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, pbar_dev, ctx->m, 0, ctx->d, out, ctx->sm_count, ctx->stream,
-                                      epilogue));
+    if (int rc = reconstruct_all(ctx, pbar_dev, out, epilogue)) return rc;
     ctx->t += 1;
     return CORE_OK;
 }
@@ -688,6 +713,13 @@ static int ls_round(core_ctx *ctx, core_ls *ls, const LsPoint &at, float *out, c
         ld = ls->d;
         scale = 1.0f / (float)ls->n;
     }
+    const ShortPlan plan = make_short_plan(1, count, ctx->m, ctx->d, ctx->sm_count);
+    if (plan.ctas > 0 && !rule) {
+        CORE_CUDA(ctx, launch_short_round(plan, ctx->keys, ctx->t, rows, CORE_F32, count, 1, ld, scale, ctx->d, ctx->m, nullptr, ctx->pbar, out, epilogue,
+                                          ctx->stream));
+        ctx->t += 1;
+        return CORE_OK;
+    }
     if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
     return finish_round(ctx, rows, CORE_F32, count, ld, scale, static_cast<float *>(ctx->ws), ctx->pbar, out, epilogue, rule);
 }
@@ -787,7 +819,7 @@ int core_decentralized_step(core_ctx *ctx, core_ls *ls, const float *W_dev, int3
         CORE_CUDA(ctx, launch_gossip_step(W_dev, partial, plan.grid_x, nullptr, n, ctx->m, rounds, P_next, reader, spread_dev, ctx->stream));
         P = P_next;
     } else {
-        if (int rc = project_into(ctx, ls->G, CORE_F32, n, ls->d, ctx->d, 0, partial, P, false, ctx->stream)) return rc;
+        if (int rc = project_all(ctx, ls->G, CORE_F32, n, ls->d, partial, P)) return rc;
         if (one_launch) {
             CORE_CUDA(ctx, launch_gossip_step(W_dev, nullptr, 0, P, n, ctx->m, rounds, P_next, reader, spread_dev, ctx->stream));
             P = P_next;
@@ -799,8 +831,7 @@ int core_decentralized_step(core_ctx *ctx, core_ls *ls, const float *W_dev, int3
     // reconstruction from the reader's estimate, update inside the kernel; the printed prefactor n/m is
     // the mean convention's 1/m with an n times longer step
     const ReconstructEpilogue update{x_dev, as_printed ? h * (float)n : h, nullptr, nullptr};
-    CORE_CUDA(ctx, launch_reconstruct(ctx->keys, ctx->t, P + (size_t)reader * ctx->m, ctx->m, 0, ctx->d, x_dev,
-                                      ctx->sm_count, ctx->stream, &update));
+    if (int rc = reconstruct_all(ctx, P + (size_t)reader * ctx->m, x_dev, &update)) return rc;
     ctx->t += 1;
     return CORE_OK;
 }

@@ -163,6 +163,26 @@ cudaError_t launch_reconstruct(const RoundKeys &keys, uint32_t t, float *pbar, i
                                cudaStream_t stream, const ReconstructEpilogue *epilogue = nullptr,
                                const MessageParts *parts = nullptr);
 
+// The whole round of a short vector in one launch of one cluster (core_short.cu): `machines` messages of a row each (the very numbers
+// of the separate kernels), or one message of the sum of `rows` rows times scale.  pbar receives the combined message.
+struct ShortPlan {
+    int ctas;         // of the cluster; 0: the kernel does not apply
+    int per;          // blocks per CTA
+    int stride;       // of the Gaussians' rows in shared memory, in blocks
+    int lanes;        // threads that share a vector's projection
+    int slices;       // ranges of the vectors in the reconstruction
+    int columns, tile, tq, uq;       // several messages: columns, blocks and lanes of the separate kernel's tiles
+    size_t smem;
+};
+ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int sm_count);
+// The reconstruction alone, with the same bits (per and ctas of the plan do not matter).
+cudaError_t launch_short_reconstruct(const ShortPlan &plan, const RoundKeys &keys, uint32_t t, float *pbar, int64_t d, int32_t m, float *out,
+                                     int sm_count, const ReconstructEpilogue *epilogue, const MessageParts *parts, cudaStream_t stream);
+// With P not null (one message) it is written there and nothing is reconstructed.
+cudaError_t launch_short_round(const ShortPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype, int32_t rows,
+                               int32_t machines, int64_t ldg, float scale, int64_t d, int32_t m, float *P, float *pbar, float *out,
+                               const ReconstructEpilogue *epilogue, cudaStream_t stream);
+
 cudaError_t launch_debug_philox(const RoundKeys &keys, uint32_t t, uint32_t j, uint64_t q0, int64_t nq,
                                 uint32_t *words, cudaStream_t stream);
 cudaError_t launch_debug_gaussians(const RoundKeys &keys, uint32_t t, uint32_t j, uint64_t q0, int64_t nq,

@@ -102,13 +102,9 @@ __host__ __device__ inline BulkRange prefetch_range(uintptr_t from, uint32_t byt
     return {from & ~(uintptr_t)15, (from & ~(uintptr_t)15) + (bytes & ~15u)};
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // v to `addr` of CTA `rank` of the cluster; its 4 bytes are counted on the barrier at `bar` there.
 __device__ __forceinline__ void send_remote(uint32_t addr, uint32_t bar, uint32_t rank, float v) {

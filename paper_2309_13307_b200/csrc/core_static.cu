@@ -95,6 +95,17 @@ int core_project_static(uint64_t seed, uint32_t t, int64_t d, int32_t m, const v
         if (cuda_error_out) *cuda_error_out = (int)e;
         return CORE_ECUDA;
     }
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    const RoundKeys keys = expand_keys(seed);
+    const ShortPlan short_plan = n > 1 || project_kernel_forced() ? ShortPlan{} : make_short_plan(1, 1, m, d, sm_count);     // as core_project does
+    if (short_plan.ctas > 0) {
+        e = launch_short_round(short_plan, keys, t, G_dev, dtype, 1, n, ldg, 1.0f, d, m, P_dev, nullptr, nullptr, nullptr, stream);
+        if (e != cudaSuccess) {
+            if (cuda_error_out) *cuda_error_out = (int)e;
+            return CORE_ECUDA;
+        }
+        return CORE_OK;
+    }
     const bool single = n == 1 && !project_kernel_forced();           // as core_project does
     ProjectPlan plan = make_project_plan(n, m, d, dtype, sm_count);
     RowPlan row_plan = make_row_plan(G_dev, dtype, 1, ldg, m, d, sm_count);
@@ -105,8 +116,6 @@ int core_project_static(uint64_t seed, uint32_t t, int64_t d, int32_t m, const v
     int &columns = single ? row_plan.grid_x : plan.grid_x;
     if ((size_t)columns > max_columns) columns = (int)max_columns;
 
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const RoundKeys keys = expand_keys(seed);
     // every (column, machine, vector) entry below grid_x * n * m is overwritten by the kernel
     // before the second kernel reads it: nothing in the array has to start at zero
     e = single ? launch_project_row(row_plan, keys, t, G_dev, dtype, 1, ldg, 1.0f, d, m, 0, scratch, stream)

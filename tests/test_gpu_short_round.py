@@ -1,0 +1,116 @@
+"""Short vectors, whose round is one launch: a cluster keeps the Gaussians between projection and reconstruction.  At the sizes where it can
+go wrong: CTAs without blocks, every cluster size, several machines' messages (the very numbers of the separate kernels), ragged
+and unaligned rows, both sides of the lines to the separate kernels, replays from a graph, steps side by side.  Also rows whose
+projection adds up its sums in clusters."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+import core_inputs
+import oracle
+from helpers import P_TOL, REC_TOL, rel_l2, row_norms
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def core_mod():
+    import paper_2309_13307_b200 as core_mod
+    core_mod.lib()
+    return core_mod
+
+
+@pytest.mark.parametrize("n,d,m,dtype,offset,pad", [
+    (1, 1, 1, "f32", 0, 0), (1, 3, 4096, "bf16", 1, 0), (2, 4, 4097, "f32", 0, 0), (3, 33, 65, "f32", 1, 2), (4, 130, 16, "bf16", 0, 2),
+    (5, 515, 33, "f32", 3, 0), (16, 257, 31, "bf16", 1, 0), (16, 1001, 40, "f32", 0, 3), (17, 300, 20, "f32", 0, 0), (1, 36, 300, "f32", 0, 0),
+    (1, 7001, 37, "f32", 0, 0), (1, 65_533, 4, "bf16", 1, 0), (1, 65_537, 4, "f32", 0, 0), (4, 49_152, 4, "f32", 0, 0), (4, 49_157, 4, "f32", 0, 0),
+    (2, 29, 3000, "f32", 0, 0), (8, 1500, 20, "bf16", 0, 0), (7, 260, 100, "f32", 0, 0), (6, 5000, 9, "f32", 0, 1), (2, 24_000, 6, "bf16", 0, 0),
+])
+def test_round_equals_its_parts_and_the_oracle(core_mod, n, d, m, dtype, offset, pad):
+    from paper_2309_13307_b200 import binding
+    G = core_inputs.gradients(n, d + offset, seed=d + m, dist="scaled_normal", dtype=dtype, device="cuda", ld=d + offset + pad)[:, offset:]
+    Gh = core_inputs.to_oracle_array(G)
+    ctx = core_mod.Core(5, d, m)
+    ctx.core_set_round(2)
+    P = ctx.core_project(G)
+    pbar = ctx.core_aggregate(P)
+    gt = ctx.core_reconstruct(pbar)
+    Po, pbaro, gto = oracle.core_round(5, 2, m, Gh)
+    assert (np.abs(P.cpu().numpy() - Po) <= P_TOL * row_norms(Gh)[:, None]).all()
+    assert rel_l2(gt.cpu().numpy(), gto) <= REC_TOL
+    pbar2, gt2 = ctx.core_round(G)
+    assert torch.equal(pbar2, pbar) and torch.equal(gt2, gt)
+    store = torch.full((d + 1,), 7.0, device="cuda")            # an estimate that does not start on 16 bytes
+    ctx.core_set_round(2)
+    assert torch.equal(ctx.core_reconstruct(pbar, store[1:]), gt) and store[0].item() == 7.0
+    if n <= 16:
+        P3 = torch.empty_like(P)
+        binding.core_project_static(5, 2, m, G, P3)
+        assert torch.equal(P3, P)
+
+
+STEPS = [(1, 5, 3, 8), (3, 40, 54, 16), (2, 7, 130, 9), (20, 11, 784, 64), (2, 150, 1201, 33), (3, 60, 1700, 100),   # one cluster
+         (2, 30, 9000, 65), (1, 149, 4099, 256), (4, 20, 20_003, 20), (2, 9, 32_768, 256), (3, 70, 9578, 18)]          # separate kernels
+
+
+@pytest.mark.parametrize("n,rows,d,m", STEPS)
+def test_steps(core_mod, n, rows, d, m):
+    problem = core_inputs.least_squares(n=n, rows=rows, d=d, seed=n + d, decay=0.5, device="cuda")
+    Ah, bh = problem.A.cpu().numpy(), problem.b.cpu().numpy()
+    ctx, ls = core_mod.Core(4, d, m), core_mod.LeastSquares(problem.A, problem.b)
+    for offset in (0, 1):                                          # iterates that start on 16 bytes, and others
+        x = core_inputs.gradients(1, d + offset, seed=1, device="cuda")[0][offset:]
+        x_prev = core_inputs.gradients(1, d + offset, seed=2, device="cuda")[0][offset:]
+        xo, xpo = x.cpu().numpy().astype(np.float64), x_prev.cpu().numpy().astype(np.float64)
+        ctx.core_set_round(3)
+        for t in (3, 4):
+            ctx.core_agd_step(ls, 0.4, 0.7, x, x_prev)
+            xo, xpo = oracle.agd_step(4, t, m, Ah, bh, 0.4, 0.7, xo, xpo)
+        assert rel_l2(x.cpu().numpy(), xo) <= 1e-5 and rel_l2(x_prev.cpu().numpy(), xpo) <= 1e-5
+    assert core_mod.core_device_status() == 0
+
+
+@pytest.mark.parametrize("n,rows,d,m", [(20, 11, 784, 64), (2, 30, 9000, 65)])
+def test_steps_replayed_from_a_graph_and_side_by_side(core_mod, n, rows, d, m):
+    problem = core_inputs.least_squares(n=n, rows=rows, d=d, seed=7, decay=0.5, device="cuda")
+    start = core_inputs.gradients(1, d, seed=1, device="cuda")[0].contiguous()
+
+    def steps(stream, count, x):
+        ctx, ls = core_mod.Core(4, d, m, stream=stream), core_mod.LeastSquares(problem.A, problem.b)
+        for _ in range(count):
+            ctx.core_gd_step(ls, 0.3, x)
+        stream.synchronize()
+        return ctx, ls
+
+    want = start.clone()
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx, ls = steps(stream, 6, want)
+    # three steps of one graph, replayed with t set back: the same rounds twice
+    x = start.clone()
+    once = start.clone()
+    steps(stream, 3, once)
+    ctx.core_set_round(0)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        for _ in range(3):
+            ctx.core_gd_step(ls, 0.3, x)
+    x.copy_(start)
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(x, once)
+    del graph
+    # three threads, a context and a stream each
+    got = [start.clone() for _ in range(3)]
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=steps, args=(torch.cuda.Stream(), 6, g)) for g in got]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert all(torch.equal(g, want) for g in got)
+    assert core_mod.core_device_status() == 0
