@@ -114,3 +114,22 @@ def test_steps_replayed_from_a_graph_and_side_by_side(core_mod, n, rows, d, m):
     torch.cuda.synchronize()
     assert all(torch.equal(g, want) for g in got)
     assert core_mod.core_device_status() == 0
+
+
+@pytest.mark.parametrize("d,m,dtype,offset", [(8192, 64, "f32", 0), (30_000, 64, "bf16", 0), (9001, 260, "f32", 1), (70_001, 33, "bf16", 3),
+                                              (4097, 130, "f32", 0), (12_001, 100, "f32", 2), (50_000, 24, "f32", 0)])
+def test_rows_whose_sums_meet_in_clusters(core_mod, d, m, dtype, offset):
+    """Two to eight CTAs per column of partial sums, also with CTAs that have no tile and several CTAs across the vectors."""
+    from paper_2309_13307_b200 import binding
+    sm_count = torch.cuda.get_device_properties(0).multi_processor_count
+    plan = binding.core_debug_row_plan(m, d, dtype=binding.CORE_BF16 if dtype == "bf16" else binding.CORE_F32, sm_count=sm_count)
+    assert 2 * plan["grid_x"] <= plan["tiles"] + 1 and not plan["turn"]
+    G = core_inputs.gradients(1, d + offset, seed=d + m, dtype=dtype, device="cuda")[:, offset:]
+    Gh = core_inputs.to_oracle_array(G)
+    ctx = core_mod.Core(6, d, m)
+    ctx.core_set_round(1)
+    P = ctx.core_project(G)
+    assert np.abs(P.cpu().numpy() - oracle.project(6, 1, m, Gh)).max() <= P_TOL * row_norms(Gh)[0]
+    gt = ctx.core_reconstruct(P[0].contiguous())
+    pbar2, gt2 = ctx.core_round(G)
+    assert torch.equal(pbar2, P[0]) and torch.equal(gt2, gt)
