@@ -31,6 +31,8 @@
 #include "core_internal.h"
 #include "core_sync.cuh"
 
+#include <algorithm>
+
 #include <cuda_bf16.h>
 
 #include <climits>
@@ -526,7 +528,10 @@ constexpr size_t kSharedPerCta = 227 * 1024, kSharedPerSm = 228 * 1024;
 static_assert(row_shared<true>(RowCta<true>::kTileBlocks, RowCta<true>::kCompute) <= kSharedPerCta, "the longest tile fits a CTA");
 static_assert(RowCta<false>::kPerSm * (row_shared<false>(RowCta<false>::kTileBlocks, RowCta<false>::kCompute) + 1024) <= kSharedPerSm, "and an SM");
 
-static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
+// More than half a byte to stage per multiply of a Gaussian.
+static bool row_heavy(int dtype, int32_t rows, int32_t m) { return 2 * (int64_t)rows * (dtype == 1 ? 2 : 4) > m; }
+
+static RowPlan plan_rows(bool turn, bool heavy, int32_t m, int64_t d, int sm_count) {
     RowPlan p{};
     p.turn = turn;
     const int compute = turn ? RowCta<true>::kCompute : RowCta<false>::kCompute;
@@ -556,7 +561,10 @@ static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
     // CTA with most of them (d = 1e6, m = 100: 104 -> 98 us).  At every tile a group's warps wait for its slowest: us, at most 32
     // steps -> this: d = 2.56e7, m = 256: one row 5006 -> 4944, eight rows 5035 -> 4987; 32 rows of 1e7, m = 1000: 7830 -> 7746; 16 bf16 rows of
     // 3.1e7, m = 1024: 24198 -> 23915; without the table, seven shifted rows of 1e7, m = 64: 595 -> 589; more steps gained nothing more.
-    const int steps_most = turn ? RowCta<true>::kTileSteps : RowCta<false>::kTileSteps;
+    // Many rows with the table (row_heavy): 32, since nothing is generated before a CTA's first tile is there.  us, 32 -> 128 steps:
+    // 64 rows of 4e6, m = 200: 1260 -> 1273; but 40 of 5e6, m = 357: 2770 -> 2762;
+    // 64 of 2e6, m = 1000: 3025 -> 3001; 24 bf16 rows of 1e7, m = 100: 1543 -> 1534.
+    const int steps_most = turn ? heavy ? 32 : RowCta<true>::kTileSteps : RowCta<false>::kTileSteps;
     const int64_t most = steps_most * p.tq < room ? steps_most * p.tq : room / p.tq * p.tq;
     const int64_t least_tiles = (nq + slots * most - 1) / (slots * most);
     int64_t best_steps = -1;
@@ -580,12 +588,13 @@ static RowPlan plan_rows(bool turn, int32_t m, int64_t d, int sm_count) {
 
 RowPlan make_row_plan(const void *G, int dtype, int32_t rows, int64_t ldg, int32_t m, int64_t d, int sm_count) {
     const bool aligned = row_period(dtype, ldg) == 1 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
-    return plan_rows(row_turn(rows, aligned, m, d), m, d, sm_count);
+    return plan_rows(row_turn(rows, aligned, m, d), row_heavy(dtype, rows, m), m, d, sm_count);
 }
 
 int row_plan_columns(int32_t m, int64_t d, int sm_count) {
-    const int with = plan_rows(true, m, d, sm_count).grid_x, without = plan_rows(false, m, d, sm_count).grid_x;
-    return with > without ? with : without;
+    const int with = plan_rows(true, false, m, d, sm_count).grid_x, heavy = plan_rows(true, true, m, d, sm_count).grid_x;
+    const int without = plan_rows(false, false, m, d, sm_count).grid_x;
+    return std::max({with, heavy, without});
 }
 
 cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint32_t t, const void *G, int dtype, int32_t rows,

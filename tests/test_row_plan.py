@@ -65,3 +65,16 @@ def test_short_rows_of_many_vectors_keep_the_polynomials():
         for rows in (1, 2):
             assert not binding.core_debug_row_plan(m, least // m - 1, rows=rows)["turn"]
             assert binding.core_debug_row_plan(m, (least // m + 3) // 4 * 4, rows=rows)["turn"]
+
+
+@pytest.mark.parametrize("dtype,size", [(binding.CORE_F32, 4), (binding.CORE_BF16, 2)])
+def test_many_rows_with_the_table_have_short_tiles(dtype, size):
+    """Beyond half a byte to stage per vector: 32 steps per tile and generating thread, and room for the columns there too."""
+    for m in (100, 200, 357, 1000):
+        for d in (262_144, 1_000_000, 4_000_000, 20_000_000):
+            for rows in (m // (2 * size), m // (2 * size) + 1, m // 3 - 1):
+                plan = binding.core_debug_row_plan(m, d, rows=rows, dtype=dtype)
+                if plan["turn"]:
+                    heavy = 2 * size * rows > m
+                    assert plan["tile_q"] <= (32 if heavy else 128) * plan["tq"], (m, d, rows)
+                    assert plan["grid_x"] <= plan["columns"] and plan["tiles"] * plan["tile_q"] * 4 >= d
