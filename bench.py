@@ -59,7 +59,7 @@ def planning_bound(sm_max_mhz: float, fmas_per_pair: int) -> float:
     return SM_COUNT * ISSUE_LANES_PER_CLK_SM * sm_max_mhz * 1e6 / (PLANNING_INSTR_PER_GAUSSIAN + fmas_per_pair)
 
 
-ROUND_KERNEL_SOURCES = ("core_internal.h", "core_project.cu", "core_reconstruct.cu", "core_rng.cuh")
+ROUND_KERNEL_SOURCES = ("core_emit.cuh", "core_internal.h", "core_project.cu", "core_reconstruct.cu", "core_rng.cuh")
 
 
 def csrc_digest() -> str:
