@@ -379,9 +379,9 @@ int core_debug_project_plan(int32_t n, int32_t m, int64_t d, int dtype, int32_t 
 /*
  * Launch geometry of the kernel that projects one row, or the sum of `rows` rows, which start `misaligned` bytes beyond a multiple
  * of 16 and `ldg` elements apart.  Host-only.  out[0..9] = blocks per shared-memory tile, threads across vectors (four vectors
- * each), threads across blocks, columns of partial sums across coordinates (a CTA each or, of short rows, a cluster), CTAs across
- * vectors, tiles of d, dynamic shared memory bytes (without a cluster's inbox), 1 if the angles come from a table (0: polynomials), columns
- * that the workspace has room for, generating threads per CTA.  (Short vectors whose round is one launch do without.)
+ * each), threads across blocks, CTAs across coordinates, CTAs across vectors, tiles of d, dynamic shared memory bytes, 1 if the angles
+ * come from a table (0: polynomials), CTAs across coordinates that the workspace has room for, generating threads per CTA.  (Short vectors
+ * whose round is one launch do without.)
  */
 int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligned, int32_t m, int64_t d, int32_t sm_count,
                         int64_t out[10]);

@@ -7,15 +7,9 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#include "core_sync.cuh"
-
 namespace core {
 
 constexpr int kFinishSlices = 8;
-// What a reconstruction that finishes the message takes (every CTA of it does): vectors, messages' entries, partial sums.
-constexpr int kJoinVectors = 512;
-constexpr int kJoinEntries = 768;
-constexpr int kJoinLoads = 2048;
 
 // p[0] + p[stride] + ... of `count` numbers, in ascending order, AT (4, 8 or 16) loads in flight at a time, and the last ones, fewer than that,
 // together too: a loop unrolled by the compiler may fetch those one after the other, each a round trip to L2 (us: a round of four
@@ -76,36 +70,6 @@ __device__ __forceinline__ float finish_join(const float *slices, int stride) {
 #pragma unroll
     for (int r = 1; r < kFinishSlices; ++r) s += slices[r * stride];
     return s;
-}
-
-// A projection's last sums, sum(idx) for idx < count: store(idx, sum), or, in a cluster of `ranks` CTAs (cluster_arrive() at their
-// start), their sums over the CTAs in ascending order, by the first one, into whose `inbox` the others write.  Short vectors: fewer
-// columns of partial sums, which the reconstruction can then finish itself.
-template <typename Sum, typename Store>
-__device__ __forceinline__ void column_sums(float *inbox, int ranks, int count, int tid, int threads, Sum &&sum, Store &&store) {
-    if (ranks <= 1) {
-        for (int idx = tid; idx < count; idx += threads) store(idx, sum(idx));
-        return;
-    }
-    const uint32_t rank = cluster_rank();
-    cluster_wait();                                          // the first CTA has started
-    for (int idx = tid; idx < count; idx += threads) store_remote(inbox + rank * count + idx, 0, sum(idx));
-    cluster_arrive();
-    cluster_wait();
-    if (rank > 0) return;
-    for (int idx = tid; idx < count; idx += threads) {
-        float s = inbox[idx];
-        for (int r = 1; r < ranks; ++r) s += inbox[r * count + idx];
-        store(idx, s);
-    }
-}
-// CTAs per column of a projection of one row by `columns` CTAs for every vector: as many as it takes for the reconstruction to finish the
-// message itself, if up to eight do.
-inline int column_ctas(int64_t columns, int32_t m) {
-    if (m > kJoinVectors) return 1;
-    for (int cluster = 1; cluster <= 8; cluster *= 2)
-        if ((columns + cluster - 1) / cluster * m <= kJoinLoads) return cluster;
-    return 1;
 }
 
 }  // namespace core

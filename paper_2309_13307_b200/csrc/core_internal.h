@@ -40,13 +40,6 @@ cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 blo
     const ChainedLaunch launch(chain, grid, block, smem, stream);
     return cudaLaunchKernelEx(&launch.cfg, kernel, static_cast<P>(args)...);
 }
-// ... in clusters.
-template <typename Args>
-cudaError_t launch_clusters(bool chain, void (*kernel)(Args), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, const Args &args) {
-    if (cudaError_t e = allow_shared(reinterpret_cast<const void *>(kernel), smem)) return e;
-    const ChainedLaunch launch(chain, grid, block, smem, stream, cluster);
-    return cudaLaunchKernelEx(&launch.cfg, kernel, args);
-}
 // CTAs of a chained kernel go wherever there is room first.  If they do not fill the chip, that packs them on few SMs (n = 7,
 // d = 3210, m = 940: 45 -> 64 us), so kernels that generate are chained only where they do fill it (`capacity` CTAs are
 // resident together), or where the whole work, d * m Gaussians, takes less than the 2 us or so that are at stake.
@@ -113,8 +106,7 @@ struct RowPlan {
     int tile_q;       // coordinate blocks (of 4) per shared-memory tile
     int tj;           // threads across vectors (four vectors each)
     int tq;           // threads across coordinate blocks
-    int grid_x;       // columns of partial sums across coordinates, a CTA each or
-    int cluster;      // a cluster of that many
+    int grid_x;       // CTAs across coordinates
     int grid_y;       // CTAs across vectors
     int compute;      // generating threads of a CTA
     int64_t tiles;

@@ -27,7 +27,6 @@
 // The generating warps take tiles over in three groups of eight, each with barriers of its own: with one barrier for all, every warp
 // waited for the slowest one at each tile (us, one group -> three: d = 2.5e7, m = 256: 4958 -> 4904; d = 1e6, m = 100:
 // 88.7 -> 87.9; eight rows, d = 1e7, the whole round: 3838 -> 3805).
-#include "core_finish.cuh"
 #include "core_internal.h"
 #include "core_sync.cuh"
 
@@ -74,8 +73,6 @@ struct RowArgs {
     int tile_q;      // coordinate blocks per tile
     int tj;          // threads across vectors
     int tq;          // threads across blocks: tj * tq generating threads at most
-    int cluster;     // CTAs whose sums become one column
-    uint32_t inbox;  // where the first of them gets the others', bytes from the start of its shared memory
     uint32_t t;
     RoundKeys keys;
 };
@@ -240,7 +237,7 @@ __device__ __forceinline__ void row_stage_any(int stride, const RowArgs &a, int6
 
 enum RowMode { kRowShort, kRowTogether, kRowTurn };
 
-template <typename GT, RowMode MODE, bool CLUSTER = false>
+template <typename GT, RowMode MODE>
 __global__ void __launch_bounds__(RowCta<MODE == kRowTurn>::kThreads, RowCta<MODE == kRowTurn>::kPerSm)
 project_row_kernel(const __grid_constant__ RowArgs a) {
     constexpr bool TOGETHER = MODE == kRowTogether, TURN = MODE == kRowTurn;
@@ -270,7 +267,6 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
         }
     };
 
-    if constexpr (CLUSTER) cluster_arrive();                 // this CTA has started
     if constexpr (TURN) fill_turn_table<kRowWarps>(reinterpret_cast<float2 *>(smem_raw), warp, lane);
     const int ql = tid / a.tj, jl = tid - ql * a.tj, jbase = blockIdx.y * a.tj * kRowJT;
     auto first_q = [&] { return a.q_base + (uint64_t)tile_begin * a.tile_q; };
@@ -473,15 +469,11 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
             lanes = ranges;
         }
     }
-    column_sums(reinterpret_cast<float *>(smem_raw + a.inbox), CLUSTER ? a.cluster : 1, plane, tid, kRowCompute,
-                [&](int idx) {
-                    float s = 0.f;
-                    for (int l = 0; l < lanes; ++l) s += red[l * plane + idx];
-                    return TURN ? kTurnScale * s : s;
-                },
-                [&](int idx, float s) {
-                    if (jbase + idx < a.m) a.partial[(int64_t)(CLUSTER ? blockIdx.x / a.cluster : blockIdx.x) * a.m + jbase + idx] = s;
-                });
+    for (int idx = tid; idx < plane; idx += kRowCompute) {
+        float s = 0.f;
+        for (int l = 0; l < lanes; ++l) s += red[l * plane + idx];
+        if (jbase + idx < a.m) a.partial[(int64_t)blockIdx.x * a.m + jbase + idx] = TURN ? kTurnScale * s : s;
+    }
 }
 
 }  // namespace
@@ -577,12 +569,8 @@ static RowPlan plan_rows(bool turn, bool heavy, int32_t m, int64_t d, int sm_cou
     }
     p.tiles = (nq + p.tile_q - 1) / p.tile_q;
     p.grid_x = (int)(slots < p.tiles ? slots : p.tiles);
-    // Short rows: clusters, so that fewer columns are left, where all of them are resident together (up to seven eighths of the places: not
-    // every one can be part of a cluster).  us, the round of one machine: d = 8192, m = 64: 9.3 -> 8.2; d = 30000: 14.3 -> 11.3.
-    p.cluster = !turn && slots >= p.tiles && 8 * (int64_t)p.grid_x * p.grid_y <= 7 * (int64_t)sm_count * per_sm ? column_ctas(p.grid_x, m) : 1;
     p.chain = chain_pays((int64_t)p.grid_x * p.grid_y, (int64_t)sm_count * per_sm, d, m);
     p.smem = turn ? row_shared<true>(p.tile_q, p.tj * p.tq) : row_shared<false>(p.tile_q, p.tj * p.tq);
-    p.grid_x = (p.grid_x + p.cluster - 1) / p.cluster;
     return p;
 }
 
@@ -615,21 +603,14 @@ cudaError_t launch_project_row(const RowPlan &plan, const RoundKeys &keys, uint3
     a.tile_q = plan.tile_q;
     a.tj = plan.tj;
     a.tq = plan.tq;
-    a.cluster = plan.cluster;
-    a.inbox = (uint32_t)plan.smem;
     a.t = t;
     a.keys = keys;
-    const dim3 grid(plan.grid_x * plan.cluster, plan.grid_y);
-    const size_t inbox = plan.cluster > 1 ? (size_t)plan.cluster * kRowJT * plan.tj * sizeof(float) : 0;
-    auto go = [&](auto kernel) {
-        return launch_clusters(plan.chain, kernel, grid, dim3(plan.turn ? RowCta<true>::kThreads : RowCta<false>::kThreads), plan.smem + inbox, stream,
-                               plan.cluster, a);
-    };
+    const dim3 grid(plan.grid_x, plan.grid_y);
+    auto go = [&](auto kernel) { return launch_chained(plan.chain, kernel, grid, dim3(plan.turn ? RowCta<true>::kThreads : RowCta<false>::kThreads), plan.smem, stream, a); };
     const bool together = row_together(rows, a.aligned, m);
     auto pick = [&](auto element) {
         using GT = decltype(element);
         if (plan.turn) return go(project_row_kernel<GT, kRowTurn>);
-        if (plan.cluster > 1) return together ? go(project_row_kernel<GT, kRowTogether, true>) : go(project_row_kernel<GT, kRowShort, true>);
         return together ? go(project_row_kernel<GT, kRowTogether>) : go(project_row_kernel<GT, kRowShort>);
     };
     return dtype == 1 ? pick(__nv_bfloat16{}) : pick(float{});

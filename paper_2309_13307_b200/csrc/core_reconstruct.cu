@@ -275,8 +275,8 @@ reconstruct_wide_kernel(const __grid_constant__ ReconstructArgs a) {
 // of a block meet in shared memory and are added in ascending order of the vector ranges.  Few vectors
 // get few slices (a slice wants at least four vectors to generate together); where even eight slices leave SMs
 // idle and vectors are many, a cluster of up to eight CTAs shares them out as well, and the first one adds up.
-// Of the message that is formed here, the slices take the place of the table that its vectors leave.
-static_assert(kJoinEntries * kFinishSlices * 4 <= (kJChunk - kJoinVectors) * 16, "room for the slices");
+constexpr int kJoinVectors = 512;                  // most vectors whose message is formed here: the rest of the
+constexpr int kJoinEntries = (kJChunk - kJoinVectors) * 16 / 4 / kFinishSlices;     // table takes the slices of n * m entries
 
 __device__ __forceinline__ void store_cluster(const void *smem, uint32_t rank, float4 v) {
     uint32_t remote;
@@ -431,7 +431,7 @@ RecKernel reconstruct_kernel_for(int64_t nq, int32_t m, int sm_count) {
 // launch it saves was the cheaper one: 100.7 against 105.9 us a step) and the CTAs are those of a short vector (m = 1, d = 1.6e7: 15625
 // of them form it 15625 times: a round of one machine 121 -> 524).
 bool reconstruct_joins(int chunks, int32_t n, int32_t m, int64_t d, int sm_count) {
-    return m <= kJoinVectors && (int64_t)n * m <= kJoinEntries && (int64_t)chunks * n * m <= kJoinLoads &&
+    return m <= kJoinVectors && (int64_t)n * m <= kJoinEntries && (int64_t)chunks * n * m <= 2048 &&
            reconstruct_kernel_for((d + 3) >> 2, m, sm_count) == RecKernel::kShort;
 }
 

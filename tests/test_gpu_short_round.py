@@ -1,7 +1,7 @@
 """Short vectors, whose round is one launch: a cluster keeps the Gaussians between projection and reconstruction.  At the sizes where it can
 go wrong: CTAs without blocks, every cluster size, several machines' messages (the very numbers of the separate kernels), ragged
-and unaligned rows, both sides of the lines to the separate kernels, replays from a graph, steps side by side.  Also rows whose
-projection adds up its sums in clusters."""
+and unaligned rows, both sides of the lines to the separate kernels, replays from a graph, steps side by side.  Also rows a little too
+long for that."""
 import threading
 
 import numpy as np
@@ -118,12 +118,12 @@ def test_steps_replayed_from_a_graph_and_side_by_side(core_mod, n, rows, d, m):
 
 @pytest.mark.parametrize("d,m,dtype,offset", [(8192, 64, "f32", 0), (30_000, 64, "bf16", 0), (9001, 260, "f32", 1), (70_001, 33, "bf16", 3),
                                               (4097, 130, "f32", 0), (12_001, 100, "f32", 2), (50_000, 24, "f32", 0)])
-def test_rows_whose_sums_meet_in_clusters(core_mod, d, m, dtype, offset):
-    """Two to eight CTAs per column of partial sums, also with CTAs that have no tile and several CTAs across the vectors."""
+def test_short_rows_of_many_ctas(core_mod, d, m, dtype, offset):
+    """Rows a little too long for one launch: a column of partial sums per CTA, all CTAs resident together."""
     from paper_2309_13307_b200 import binding
     sm_count = torch.cuda.get_device_properties(0).multi_processor_count
     plan = binding.core_debug_row_plan(m, d, dtype=binding.CORE_BF16 if dtype == "bf16" else binding.CORE_F32, sm_count=sm_count)
-    assert 2 * plan["grid_x"] <= plan["tiles"] + 1 and not plan["turn"]
+    assert plan["grid_x"] == plan["tiles"] and not plan["turn"]
     G = core_inputs.gradients(1, d + offset, seed=d + m, dtype=dtype, device="cuda")[:, offset:]
     Gh = core_inputs.to_oracle_array(G)
     ctx = core_mod.Core(6, d, m)
