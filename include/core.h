@@ -349,6 +349,12 @@ int core_debug_wait_timeout(uint32_t limit_us, int32_t code, uint32_t observed_h
 int core_debug_ls_hold_back(core_ls *ls, int32_t chunk);
 
 /*
+ * The round that ends a least-squares step, on rows of the caller's: pbar[j] = <scale * (row 0 + ... + row rows-1), xi_j> and the
+ * estimate made from it; rows are `ldg` floats apart.  Advances t.
+ */
+int core_debug_combined_round(core_ctx *ctx, const float *rows_dev, int32_t rows, int64_t ldg, float scale, float *pbar_dev, float *gtilde_dev);
+
+/*
  * Host-only replay of the clock of those waits: with the device timer read as readings_ns[0..count-1], the index of
  * the reading at which a wait of limit_ns gives up, or -1.  What lies between two readings counts 1 ms at most (the
  * timer runs on while the GPU works for somebody else).

@@ -56,6 +56,7 @@ _SIGNATURES = {
     "core_debug_force_project_kernel": ([_c.c_int], _c.c_int),
     "core_debug_wait_timeout": ([_c.c_uint32, _c.c_int32, _c.POINTER(_c.c_uint32)], _c.c_int),
     "core_debug_ls_hold_back": ([_c.c_void_p, _c.c_int32], _c.c_int),
+    "core_debug_combined_round": ([_c.c_void_p, _c.c_void_p, _c.c_int32, _c.c_int64, _c.c_float, _c.c_void_p, _c.c_void_p], _c.c_int),
     "core_debug_wait_clock": ([_c.POINTER(_c.c_uint64), _c.c_int32, _c.c_uint64, _c.POINTER(_c.c_int32)], _c.c_int),
     "core_ls_gradients": ([_c.c_void_p, _c.c_void_p, _c.c_void_p, _c.c_void_p], _c.c_int),
     "core_debug_philox": ([_c.c_void_p, _c.c_uint32, _c.c_uint64, _c.c_int64, _c.c_void_p], _c.c_int),
@@ -432,6 +433,15 @@ class Core:
         words = torch.empty((nq, 4), dtype=torch.int32, device="cuda")
         self._check(lib().core_debug_philox(self._h, j, q0, nq, words.data_ptr()), "core_debug_philox")
         return words
+
+    def core_debug_combined_round(self, rows_dev: torch.Tensor, scale: float):
+        ptr, code, n, ld = _rows(rows_dev)
+        if not rows_dev.is_cuda or code != CORE_F32 or rows_dev.shape[1] != self.d:
+            raise ValueError("rows must be a float32 CUDA tensor of shape [rows, d]")
+        pbar = torch.empty(self.m, dtype=torch.float32, device=rows_dev.device)
+        gtilde = torch.empty(self.d, dtype=torch.float32, device=rows_dev.device)
+        self._check(lib().core_debug_combined_round(self._h, ptr, n, ld, scale, pbar.data_ptr(), gtilde.data_ptr()), "core_debug_combined_round")
+        return pbar, gtilde
 
     def core_debug_gaussians(self, j: int, q0: int, nq: int) -> torch.Tensor:
         z = torch.empty((nq, 4), dtype=torch.float32, device="cuda")

@@ -691,6 +691,20 @@ static int ls_loss_into(core_ctx *ctx, core_ls *ls, const float *x, double *loss
     return CORE_OK;
 }
 
+// The round of one combined gradient, scale times the sum of `count` rows, of a context's whole vector.
+static int combined_round(core_ctx *ctx, const float *rows, int32_t count, int64_t ld, float scale, float *pbar, float *out,
+                          const ReconstructEpilogue *epilogue, const StepRule *rule) {
+    const ShortPlan plan = make_short_plan(1, count, ctx->m, ctx->d, ctx->sm_count);
+    if (plan.ctas > 0 && !rule) {
+        CORE_CUDA(ctx, launch_short_round(plan, ctx->keys, ctx->t, rows, CORE_F32, count, 1, ld, scale, ctx->d, ctx->m, nullptr, pbar, out, epilogue,
+                                          ctx->stream));
+        ctx->t += 1;
+        return CORE_OK;
+    }
+    if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
+    return finish_round(ctx, rows, CORE_F32, count, ld, scale, static_cast<float *>(ctx->ws), pbar, out, epilogue, rule);
+}
+
 // The round of a step at the point `at`: only the mean message is wanted, so the gradient is one row.  The
 // projection adds the units' partial gradients while it stages its tiles; the machine gradients are never written.
 static int ls_round(core_ctx *ctx, core_ls *ls, const LsPoint &at, float *out, const ReconstructEpilogue *epilogue,
@@ -713,15 +727,7 @@ static int ls_round(core_ctx *ctx, core_ls *ls, const LsPoint &at, float *out, c
         ld = ls->d;
         scale = 1.0f / (float)ls->n;
     }
-    const ShortPlan plan = make_short_plan(1, count, ctx->m, ctx->d, ctx->sm_count);
-    if (plan.ctas > 0 && !rule) {
-        CORE_CUDA(ctx, launch_short_round(plan, ctx->keys, ctx->t, rows, CORE_F32, count, 1, ld, scale, ctx->d, ctx->m, nullptr, ctx->pbar, out, epilogue,
-                                          ctx->stream));
-        ctx->t += 1;
-        return CORE_OK;
-    }
-    if (int rc = ensure_workspace(ctx, row_partial_bytes(ctx, ctx->d))) return rc;
-    return finish_round(ctx, rows, CORE_F32, count, ld, scale, static_cast<float *>(ctx->ws), ctx->pbar, out, epilogue, rule);
+    return combined_round(ctx, rows, count, ld, scale, ctx->pbar, out, epilogue, rule);
 }
 
 int core_ls_gradients(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G_out_dev) {
@@ -886,6 +892,12 @@ int core_debug_ls_hold_back(core_ls *ls, int32_t chunk) {
     if (!ls || chunk < -1) return CORE_EINVAL;
     ls->step_pass.hold_back = ls->machine_pass.hold_back = chunk < 0 ? INT32_MAX : chunk;
     return CORE_OK;
+}
+
+int core_debug_combined_round(core_ctx *ctx, const float *rows_dev, int32_t rows, int64_t ldg, float scale, float *pbar_dev, float *gtilde_dev) {
+    if (int rc = check_ctx(ctx)) return rc;
+    if (!rows_dev || rows < 1 || ldg < ctx->d || !pbar_dev || !gtilde_dev) return CORE_EINVAL;
+    return combined_round(ctx, rows_dev, rows, ldg, scale, pbar_dev, gtilde_dev, nullptr, nullptr);
 }
 
 int core_debug_wait_clock(const uint64_t *readings_ns, int32_t count, uint64_t limit_ns, int32_t *given_up_at) {

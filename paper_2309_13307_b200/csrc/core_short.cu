@@ -252,7 +252,8 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int i = (e + u * kShortThreads) / mine, q = (e + u * kShortThreads) % mine;
-                if (i < machines) g[i * per + q] = v[u];
+                const float scale = APART ? 1.f : a.scale;
+                if (i < machines) g[i * per + q] = make_float4(v[u].x * scale, v[u].y * scale, v[u].z * scale, v[u].w * scale);
             }
         }
     }
