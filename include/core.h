@@ -393,6 +393,15 @@ int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligne
                         int64_t out[10]);
 
 /*
+ * Launch geometry of the kernels for short vectors.  Host-only.  The round in one launch, of `machines` messages of a row each or, for one
+ * machine, of the sum of `rows` rows: out[0..5] = CTAs of its cluster, blocks of four coordinates per CTA, columns of partial sums, threads
+ * that share a vector's message, ranges of the vectors in the reconstruction, dynamic shared memory bytes; all 0 where separate kernels
+ * make the round.  The reconstruction alone: out[6..8] = CTAs, blocks per CTA, threads per CTA (0: core_debug_reconstruct_plan tells
+ * which kernel makes it).
+ */
+int core_debug_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int32_t sm_count, int64_t out[9]);
+
+/*
  * Which reconstruction kernel d coordinates and m vectors take, host-only: out[0] = 0 one of the two for short vectors, 1 the one for long
  * vectors with few or very many Gaussians per coordinate, 2 the one with the table of angles; out[1] = 1 if the CTAs of the
  * reconstruction form the message of a round of one machine themselves.

@@ -72,6 +72,7 @@ _SIGNATURES = {
                                  _c.POINTER(_c.c_int64)], _c.c_int),
     "core_debug_row_plan": ([_c.c_int, _c.c_int32, _c.c_int64, _c.c_uint32, _c.c_int32, _c.c_int64, _c.c_int32,
                              _c.POINTER(_c.c_int64)], _c.c_int),
+    "core_debug_short_plan": ([_c.c_int32, _c.c_int32, _c.c_int32, _c.c_int64, _c.c_int32, _c.POINTER(_c.c_int64)], _c.c_int),
     "core_debug_reconstruct_plan": ([_c.c_int64, _c.c_int32, _c.c_int32, _c.POINTER(_c.c_int32)], _c.c_int),
     "core_debug_host_slabs": ([_c.c_int64, _c.c_int32, _c.c_int, _c.c_int32, _c.c_int, _c.POINTER(_c.c_int64), _c.c_int32,
                                _c.POINTER(_c.c_int32)], _c.c_int),
@@ -155,6 +156,15 @@ def core_debug_row_plan(m: int, d: int, rows: int = 1, ldg: int | None = None, d
     if rc != CORE_OK:
         raise CoreError(rc, "core_debug_row_plan")
     keys = ("tile_q", "tj", "tq", "grid_x", "grid_y", "tiles", "smem", "turn", "columns", "compute")
+    return dict(zip(keys, (int(v) for v in out)))
+
+
+def core_debug_short_plan(m: int, d: int, machines: int = 1, rows: int = 1, sm_count: int = 148) -> dict:
+    out = (ctypes.c_int64 * 9)()
+    rc = lib().core_debug_short_plan(machines, rows, m, d, sm_count, out)
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_short_plan")
+    keys = ("ctas", "per", "columns", "lanes", "slices", "smem", "alone_ctas", "alone_per", "alone_threads")
     return dict(zip(keys, (int(v) for v in out)))
 
 

@@ -18,6 +18,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 namespace core {
@@ -414,6 +415,17 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
     return p;
 }
 
+// At most a CTA per SM, and four warps each: a step's next kernel wants the other SMs early (17 machines, d = 313, m = 9: a warp
+// on ten SMs made a step of 26.7 us one of 27.8).  A thread per block and range, and threads for the table of the vectors.
+ShortGrid make_short_grid(const ShortPlan &plan, int32_t m, int64_t d, int sm_count) {
+    const int nq = (int)((d + 3) >> 2), most = kShortThreads / plan.slices, least = 128 / plan.slices;
+    ShortGrid g;
+    g.per = std::clamp((nq + sm_count - 1) / sm_count, least, most);
+    g.threads = (std::max(g.per * plan.slices, std::min(m / 4, 256)) + 31) / 32 * 32;
+    g.ctas = (nq + g.per - 1) / g.per;
+    return g;
+}
+
 static ShortArgs short_args(const ShortPlan &plan, const RoundKeys &keys, uint32_t t, int64_t d, int32_t m, float *pbar, float *out,
                             const ReconstructEpilogue *epilogue) {
     ShortArgs a{};
@@ -464,18 +476,11 @@ cudaError_t launch_short_round(const ShortPlan &plan, const RoundKeys &keys, uin
 cudaError_t launch_short_reconstruct(const ShortPlan &plan, const RoundKeys &keys, uint32_t t, float *pbar, int64_t d, int32_t m, float *out,
                                      int sm_count, const ReconstructEpilogue *epilogue, const MessageParts *parts, cudaStream_t stream) {
     ShortArgs a = short_args(plan, keys, t, d, m, pbar, out, epilogue);
-    // at most a CTA per SM, and four warps each: a step's next kernel wants the other SMs early (17 machines, d = 313, m = 9: a warp
-    // on ten SMs made a step of 26.7 us one of 27.8)
-    const int nq = (int)((d + 3) >> 2), most = kShortThreads / plan.slices, least = 128 / plan.slices;
-    a.per = (nq + sm_count - 1) / sm_count;
-    a.per = a.per < least ? least : a.per > most ? most : a.per;
-    // ... and threads for the table
-    int threads = a.per * plan.slices;
-    if (threads < m / 4) threads = m / 4 < 256 ? m / 4 : 256;
-    threads = (threads + 31) / 32 * 32;
+    const ShortGrid grid = make_short_grid(plan, m, d, sm_count);
+    a.per = grid.per;
     const MessageParts join = parts ? *parts : MessageParts{};
-    const size_t smem = ((size_t)m + threads) * 16 + (parts ? (size_t)kFinishSlices * parts->n * m * 4 : 0);
-    return launch_chained(true, short_reconstruct_kernel, dim3((unsigned)((nq + a.per - 1) / a.per)), dim3(threads), smem, stream, a, join);
+    const size_t smem = ((size_t)m + grid.threads) * 16 + (parts ? (size_t)kFinishSlices * parts->n * m * 4 : 0);
+    return launch_chained(true, short_reconstruct_kernel, dim3((unsigned)grid.ctas), dim3(grid.threads), smem, stream, a, join);
 }
 
 }  // namespace core
