@@ -954,7 +954,7 @@ int core_debug_row_plan(int dtype, int32_t rows, int64_t ldg, uint32_t misaligne
 int core_debug_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int32_t sm_count, int64_t out[9]) {
     if (!out || machines < 1 || rows < 1 || m < 1 || d < 1 || sm_count < 1) return CORE_EINVAL;
     const ShortPlan p = make_short_plan(machines, rows, m, d, sm_count), alone = make_short_plan(1, 1, m, d, sm_count);
-    const ShortGrid g = alone.ctas > 0 ? make_short_grid(alone, m, d, sm_count) : ShortGrid{};
+    const ShortGrid g = alone.ctas > 0 ? make_short_grid(alone, m, d, sm_count, nullptr) : ShortGrid{};
     const int64_t v[9] = {p.ctas, p.per, p.columns, p.lanes, p.slices, (int64_t)p.smem, g.ctas, g.per, g.threads};
     for (int i = 0; i < 9; ++i) out[i] = p.ctas > 0 || i > 5 ? v[i] : 0;
     return CORE_OK;

@@ -179,7 +179,7 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
 struct ShortGrid {
     int per, threads, ctas;
 };
-ShortGrid make_short_grid(const ShortPlan &plan, int32_t m, int64_t d, int sm_count);
+ShortGrid make_short_grid(const ShortPlan &plan, int32_t m, int64_t d, int sm_count, const MessageParts *parts);
 cudaError_t launch_short_reconstruct(const ShortPlan &plan, const RoundKeys &keys, uint32_t t, float *pbar, int64_t d, int32_t m, float *out,
                                      int sm_count, const ReconstructEpilogue *epilogue, const MessageParts *parts, cudaStream_t stream);
 // With P not null (one message) it is written there and nothing is reconstructed.

@@ -98,12 +98,16 @@ short_reconstruct_kernel(const __grid_constant__ ShortArgs a, const MessageParts
     grid_wait();
     if (parts.partial) {
         const int entries = parts.n * a.m;
-        for (int e = tid; e < entries * kFinishSlices; e += threads)
-            sums[e] = finish_slice(parts.partial, parts.chunks, entries, e % entries, e / entries);
+        const bool few = parts.chunks <= kFinishSlices;                       // a column per slice at most: the same sums without them
+        if (few)
+            for (int e = tid; e < entries; e += threads) sums[e] = sum_strided<8>(parts.partial + e, parts.chunks, entries);
+        else
+            for (int e = tid; e < entries * kFinishSlices; e += threads)
+                sums[e] = finish_slice<8>(parts.partial, parts.chunks, entries, e % entries, e / entries);
         __syncthreads();
         for (int j = tid; j < a.m; j += threads) {
             float sum = 0.f;
-            for (int i = 0; i < parts.n; ++i) sum += finish_join(sums + i * a.m + j, entries);
+            for (int i = 0; i < parts.n; ++i) sum += few ? sums[i * a.m + j] : finish_join(sums + i * a.m + j, entries);
             sum /= (float)parts.n;
             table[j].w = __float_as_uint(sum);
             if (blockIdx.x == 0) a.pbar[j] = sum;
@@ -417,11 +421,15 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
 
 // At most a CTA per SM, and four warps each: a step's next kernel wants the other SMs early (17 machines, d = 313, m = 9: a warp
 // on ten SMs made a step of 26.7 us one of 27.8).  A thread per block and range, and threads for the table of the vectors.
-ShortGrid make_short_grid(const ShortPlan &plan, int32_t m, int64_t d, int sm_count) {
-    const int nq = (int)((d + 3) >> 2), most = kShortThreads / plan.slices, least = 128 / plan.slices;
+// With parts every CTA finishes the whole message: half as many CTAs, of eight warps, and a thread per sum, as far as 512 go, since a
+// thread's sums wait for L2 one after the other (us, rounds of three machines, m = 200, d = 219: 17.0 -> 6.9; five, m = 100, d = 141:
+// 15.2 -> 6.4; accelerated steps by separate kernels, with the 128 threads and twice as many CTAs: 40 rows, d = 16000, m = 8: 14.4 instead of 15.8).
+ShortGrid make_short_grid(const ShortPlan &plan, int32_t m, int64_t d, int sm_count, const MessageParts *parts) {
+    const int nq = (int)((d + 3) >> 2), most = kShortThreads / plan.slices, least = (parts ? 256 : 128) / plan.slices;
+    const int sums = parts ? parts->n * m * (parts->chunks > kFinishSlices ? kFinishSlices : 1) : 0;
     ShortGrid g;
     g.per = std::clamp((nq + sm_count - 1) / sm_count, least, most);
-    g.threads = (std::max(g.per * plan.slices, std::min(m / 4, 256)) + 31) / 32 * 32;
+    g.threads = (std::max({g.per * plan.slices, std::min(m / 4, 256), std::min(sums, kShortThreads)}) + 31) / 32 * 32;
     g.ctas = (nq + g.per - 1) / g.per;
     return g;
 }
@@ -476,7 +484,7 @@ cudaError_t launch_short_round(const ShortPlan &plan, const RoundKeys &keys, uin
 cudaError_t launch_short_reconstruct(const ShortPlan &plan, const RoundKeys &keys, uint32_t t, float *pbar, int64_t d, int32_t m, float *out,
                                      int sm_count, const ReconstructEpilogue *epilogue, const MessageParts *parts, cudaStream_t stream) {
     ShortArgs a = short_args(plan, keys, t, d, m, pbar, out, epilogue);
-    const ShortGrid grid = make_short_grid(plan, m, d, sm_count);
+    const ShortGrid grid = make_short_grid(plan, m, d, sm_count, parts);
     a.per = grid.per;
     const MessageParts join = parts ? *parts : MessageParts{};
     const size_t smem = ((size_t)m + grid.threads) * 16 + (parts ? (size_t)kFinishSlices * parts->n * m * 4 : 0);
