@@ -81,6 +81,31 @@ __device__ __forceinline__ void add_block(float4 &s, float4 v) { s = make_float4
 // Blocks of a reconstruction in which the vectors are cut into ranges added up in ascending order, whichever kernel does it.
 __device__ __forceinline__ int slice_end(int m, int slice, int slices) { return m * (slice + 1) / slices; }
 
+// The sum of a block's ranges, places[r * stride] for r < ranges (a power of two), in the first `blocks` threads, each a block's.  More than
+// eight ranges, up to 64: eight at a time by as many threads first, so that none adds up more than eight in a row.
+__device__ __forceinline__ float4 join_ranges(float4 *places, int stride, int ranges, int blocks, int tid) {
+    if (ranges > 8) {
+        const int group = tid / stride, q = tid - group * stride;
+        if (8 * group < ranges && q < blocks) {
+            float4 *const first = places + 8 * group * stride + q;
+            float4 v[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) v[r] = first[r * stride];
+#pragma unroll
+            for (int r = 1; r < 8; ++r) add_block(v[0], v[r]);
+            *first = v[0];
+        }
+        __syncthreads();
+        stride *= 8;
+        ranges /= 8;
+    }
+    if (tid >= blocks) return make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 s = places[tid];
+#pragma unroll 8
+    for (int r = 1; r < ranges; ++r) add_block(s, places[r * stride + tid]);
+    return s;
+}
+
 // The reconstruction alone: the same values and sums, on as many CTAs as there are blocks for, without a cluster.  With parts it
 // finishes the message itself, as launch_finish_aggregate does.
 __global__ void __launch_bounds__(kShortThreads)
@@ -91,6 +116,8 @@ short_reconstruct_kernel(const __grid_constant__ ShortArgs a, const MessageParts
     float4 *const scratch = reinterpret_cast<float4 *>(table + a.m);          // [thread]
     float *const sums = reinterpret_cast<float *>(scratch + blockDim.x);      // [slice of the columns][machine][vector]
     const int tid = threadIdx.x, threads = blockDim.x, nq = (int)((a.d + 3) >> 2), q0 = (int)blockIdx.x * a.per, mine = min(a.per, nq - q0);
+    const int slice = tid / a.per, q = tid - slice * a.per;
+    const QPart qp = philox_qpart((uint32_t)(q0 + q), a.t, a.keys);
     for (int j = tid; j < a.m; j += threads) {
         const JPart jp = philox_jpart((uint32_t)j, 0u, a.keys);
         table[j] = make_uint4(jp.x0, jp.x2, jp.w3, 0u);
@@ -113,13 +140,18 @@ short_reconstruct_kernel(const __grid_constant__ ShortArgs a, const MessageParts
             if (blockIdx.x == 0) a.pbar[j] = sum;
         }
     } else {
-        for (int j = tid; j < a.m; j += threads) table[j].w = __float_as_uint(__ldcg(a.pbar + j));
+        for (int j = tid; j < a.m; j += 4 * threads) {                        // four loads in flight
+            float p[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p[i] = j + i * threads < a.m ? __ldcg(a.pbar + j + i * threads) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (j + i * threads < a.m) table[j + i * threads].w = __float_as_uint(p[i]);
+        }
     }
     __syncthreads();
-    const int q = tid % a.per, slice = tid / a.per;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (q < mine && slice < a.slices) {
-        const QPart qp = philox_qpart((uint32_t)(q0 + q), a.t, a.keys);
         int j = slice_end(a.m, slice - 1, a.slices);
         const int end = slice_end(a.m, slice, a.slices);
         auto add = [&](auto count) {
@@ -149,9 +181,8 @@ short_reconstruct_kernel(const __grid_constant__ ShortArgs a, const MessageParts
     }
     scratch[tid] = s;
     __syncthreads();
+    s = join_ranges(scratch, a.per, a.slices, mine, tid);
     if (tid < mine) {
-#pragma unroll 8
-        for (int r = 1; r < a.slices; ++r) add_block(s, scratch[r * a.per + tid]);
         const float inv_m = 1.0f / (float)a.m;
         emit_block(a, (uint64_t)(q0 + tid), 0, make_float4(s.x * inv_m, s.y * inv_m, s.z * inv_m, s.w * inv_m));
     }
@@ -366,9 +397,8 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
             scratch[tid] = s;
         }
         __syncthreads();
+        s = join_ranges(scratch, pass, slices, here, tid);
         if (tid < here) {
-#pragma unroll 8
-            for (int r = 1; r < slices; ++r) add_block(s, scratch[r * pass + q]);
             const float inv_m = 1.0f / (float)m;
             emit_block(a, (uint64_t)(q0 + qb + q), 0, make_float4(s.x * inv_m, s.y * inv_m, s.z * inv_m, s.w * inv_m));
         }
@@ -409,7 +439,7 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
     p.lanes = 1;
     while (p.lanes < 32 && 2 * p.lanes * m <= kShortThreads && p.lanes < p.per) p.lanes *= 2;
     p.slices = 1;
-    while (p.slices < kShortSlices && 4 * p.slices < m) p.slices *= 2;
+    while (p.slices < kShortSlices && 6 * p.slices <= m) p.slices *= 2;      // three vectors and more in each
     // per CTA: the Gaussians, its part of the rows, a 16-byte place per thread, the vectors' half of Philox; the shares of the messages, the
     // combined message, the columns' slices
     const size_t entries = (size_t)machines * m;
@@ -429,7 +459,7 @@ ShortGrid make_short_grid(const ShortPlan &plan, int32_t m, int64_t d, int sm_co
     const int sums = parts ? parts->n * m * (parts->chunks > kFinishSlices ? kFinishSlices : 1) : 0;
     ShortGrid g;
     g.per = std::clamp((nq + sm_count - 1) / sm_count, least, most);
-    g.threads = (std::max({g.per * plan.slices, std::min(m / 4, 256), std::min(sums, kShortThreads)}) + 31) / 32 * 32;
+    g.threads = (std::max({g.per * plan.slices, std::min(m / 2, kShortThreads), std::min(sums, kShortThreads)}) + 31) / 32 * 32;
     g.ctas = (nq + g.per - 1) / g.per;
     return g;
 }
