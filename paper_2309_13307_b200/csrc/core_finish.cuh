@@ -6,24 +6,33 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <type_traits>
 
 namespace core {
 
 constexpr int kFinishSlices = 8;
 
-// p[0] + p[stride] + ... of `count` numbers, in ascending order, AT (4, 8 or 16) loads in flight at a time, and the last ones, fewer than that,
-// together too: a loop unrolled by the compiler may fetch those one after the other, each a round trip to L2 (us: a round of four
-// machines, d = 4096, m = 16: 8.2 -> 7.1; a decentralised step of 16 machines, d = 20000, m = 64: 86.4 -> 84.0).
-template <int AT, typename T>
+// p[0] + p[stride] + ... of `count` numbers, in ascending order, FIRST and then AT (4, 8 or 16) loads in flight at a time, and the last ones, fewer
+// than that, together too: a loop unrolled by the compiler may fetch those one after the other, each a round trip to L2 (us: a decentralised
+// step of 16 machines, d = 20000, m = 64: 86.4 -> 84.0).
+template <int AT, int FIRST = AT, typename T>
 __device__ __forceinline__ T sum_strided(const T *p, int count, int64_t stride) {
     T s = 0;
-    for (; count >= AT; count -= AT, p += AT * stride) {
-        T v[AT];
+    auto batch = [&](auto size) {
+        constexpr int N = decltype(size)::value;
+        T v[N];
 #pragma unroll
-        for (int i = 0; i < AT; ++i) v[i] = __ldcg(p + i * stride);
+        for (int i = 0; i < N; ++i) v[i] = __ldcg(p + i * stride);
 #pragma unroll
-        for (int i = 0; i < AT; ++i) s += v[i];
+        for (int i = 0; i < N; ++i) s += v[i];
+        count -= N;
+        p += N * stride;
+    };
+    if constexpr (FIRST > AT) {
+#pragma unroll 1
+        while (count >= FIRST) batch(std::integral_constant<int, FIRST>{});
     }
+    while (count >= AT) batch(std::integral_constant<int, AT>{});
     T a[8], b[4], c[2], d = 0;
     if (AT > 8 && count & 8) {
 #pragma unroll
@@ -58,10 +67,10 @@ __device__ __forceinline__ T sum_strided(const T *p, int count, int64_t stride) 
 
 // (Fewer at a time in kernels that want their registers for something else: the gossip of 17 to 32 machines spilled with sixteen: 1.2 us
 // a step.)
-template <int AT = 16>
+template <int AT = 16, int FIRST = AT>
 __device__ __forceinline__ float finish_slice(const float *partial, int chunks, int64_t total, int64_t idx, int slice) {
     const int begin = chunks * slice / kFinishSlices, end = chunks * (slice + 1) / kFinishSlices;
-    return sum_strided<AT>(partial + (int64_t)begin * total + idx, end - begin, total);
+    return sum_strided<AT, FIRST>(partial + (int64_t)begin * total + idx, end - begin, total);
 }
 
 // The slices of an entry, `stride` floats apart.

@@ -322,7 +322,8 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
             float *const slices = reinterpret_cast<float *>(table + kJoinVectors);
             for (int e = tid; e < entries * kFinishSlices; e += kThreads) {
                 const int entry = e % entries, i = entry / jn, j = entry % jn;
-                slices[e] = finish_slice<4>(a.parts.partial, a.parts.chunks, (int64_t)n * a.m, (int64_t)i * a.m + j0 + j, e / entries);
+                // (eight in flight while there are; sixteen, or eight for the last ones too, would spill)
+                slices[e] = finish_slice<4, 8>(a.parts.partial, a.parts.chunks, (int64_t)n * a.m, (int64_t)i * a.m + j0 + j, e / entries);
             }
             __syncthreads();
             for (int jj = tid; jj < jn; jj += kThreads) {
