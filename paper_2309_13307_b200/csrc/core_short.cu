@@ -29,6 +29,7 @@ constexpr int kShortThreads = 512;
 constexpr int kShortCluster = 8;                  // most CTAs
 constexpr int kShortVectors = 4096;               // most vectors
 constexpr int kShortMachines = 8;                 // most messages kept apart
+constexpr int kShortLaneBlocks = 16;              // blocks of a lane from which a vector gets more than one warp
 constexpr int kShortSlices = 64;                  // most ranges of the vectors (reconstruction) a block's sum is cut into
 
 struct ShortArgs {
@@ -43,7 +44,7 @@ struct ShortArgs {
     int m;
     int per;                   // blocks per CTA
     int stride;                // of the Gaussians' rows (one per vector) in shared memory, in blocks
-    int lanes;                 // threads that share a vector's projection: a power of two
+    int lanes;                 // threads that share a vector's projection: a power of two, whole warps from 32 on
     int columns;               // of several messages: the separate kernel's tiles, whose sums are formed as it forms them:
     int tile;                  // blocks of one,
     int tq, uq;                // lanes that share it out, blocks of a lane's step
@@ -332,20 +333,35 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
             for (uint32_t r = 0; r < ranks; ++r) store_remote(inbox + (column0 + column) * entries + e, r, sum);
         }
     } else {
-        for (int j0 = 0; j0 < m; j0 += kShortThreads / a.lanes) {
-            const int sub = tid & (a.lanes - 1), j = j0 + tid / a.lanes;
-            float p = 0.f;
+        const auto dot = [&](int j, int sub) {
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);                       // four sums: a chain is as long as a lane has blocks
             if (j < m)
                 for (int q = sub; q < mine; q += a.lanes) {
                     const float4 v = z[j * a.stride + q], b = g[q];
-                    p = fmaf(b.x, v.x, p);
-                    p = fmaf(b.y, v.y, p);
-                    p = fmaf(b.z, v.z, p);
-                    p = fmaf(b.w, v.w, p);
+                    s = make_float4(fmaf(b.x, v.x, s.x), fmaf(b.y, v.y, s.y), fmaf(b.z, v.z, s.z), fmaf(b.w, v.w, s.w));
                 }
-            for (int o = a.lanes / 2; o > 0; o /= 2) p += __shfl_xor_sync(0xffffffffu, p, o);
-            if (j < m)
-                for (uint32_t r = sub; r < ranks; r += a.lanes) store_remote(inbox + rank * m + j, r, p);
+            return (s.x + s.y) + (s.z + s.w);
+        };
+        if (a.lanes <= 32) {
+            for (int j0 = 0; j0 < m; j0 += kShortThreads / a.lanes) {
+                const int sub = tid & (a.lanes - 1), j = j0 + tid / a.lanes;
+                float p = dot(j, sub);
+                for (int o = a.lanes / 2; o > 0; o /= 2) p += __shfl_xor_sync(0xffffffffu, p, o);
+                if (j < m)
+                    for (uint32_t r = sub; r < ranks; r += a.lanes) store_remote(inbox + rank * m + j, r, p);
+            }
+        } else {                                                              // several warps per vector: all vectors are here at once
+            const int sub = tid & (a.lanes - 1), j = tid / a.lanes, warps = a.lanes / 32;
+            float p = dot(j, sub);
+            for (int o = 16; o > 0; o /= 2) p += __shfl_xor_sync(0xffffffffu, p, o);
+            float *const part = reinterpret_cast<float *>(scratch);
+            if (tid % 32 == 0) part[tid / 32] = p;
+            __syncthreads();
+            if (j < m && sub < (int)ranks) {
+                p = part[j * warps];
+                for (int w = 1; w < warps; ++w) p += part[j * warps + w];
+                store_remote(inbox + rank * m + j, sub, p);
+            }
         }
     }
     cluster_arrive();
@@ -414,7 +430,10 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
 // m = 256: 7.1 -> 17.2 by one CTA) keep the separate kernels, as do more partial gradients than that many per CTA, which take longer
 // to add up on eight SMs than on all (148 of d = 9578: the step 18 -> 37; 148 of 3513: 33.7 -> 32.3).
 constexpr int kShortCounters[3] = {48 << 10, 24 << 10, 8 << 10};
+// Few vectors leave a thread more blocks than vectors, one after the other: up to 2560 blocks per CTA (m = 1: d = 192 670: 11.8 -> 12.6, d = 88 472:
+// 8.0 -> 7.6).
 constexpr int kShortRowBlocks = 16 << 10;
+constexpr int kShortBlocks = 2560;
 ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int sm_count) {
     ShortPlan p{};
     const int64_t nq = (d + 3) >> 2;
@@ -437,7 +456,9 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
     p.per = (int)((units + ctas - 1) / ctas) * p.tile;
     p.stride = p.per | 1;
     p.lanes = 1;
-    while (p.lanes < 32 && 2 * p.lanes * m <= kShortThreads && p.lanes < p.per) p.lanes *= 2;
+    // up to a warp per vector, several warps where that leaves a lane more than sixteen blocks in a row (m = 3, d = 64 000: 63, and the error of the
+    // message, rms, 3.3e-7 of the gradient's norm, where the separate kernels' is 3.0e-7 and this 1.7e-7)
+    while ((p.lanes < 32 ? p.lanes : kShortLaneBlocks * p.lanes) < p.per && 2 * p.lanes * m <= kShortThreads) p.lanes *= 2;
     p.slices = 1;
     while (p.slices < kShortSlices && 6 * p.slices <= m) p.slices *= 2;      // three vectors and more in each
     // per CTA: the Gaussians, its part of the rows, a 16-byte place per thread, the vectors' half of Philox; the shares of the messages, the
@@ -445,7 +466,7 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
     const size_t entries = (size_t)machines * m;
     p.smem = ((size_t)m * p.stride + (size_t)machines * p.per + kShortThreads + m) * 16 +
              ((apart ? p.columns + kFinishSlices : ctas) * entries + m) * 4;
-    if (p.smem <= 200 * 1024 && (int64_t)rows * p.per <= kShortRowBlocks) p.ctas = ctas;
+    if (p.smem <= 200 * 1024 && (int64_t)rows * p.per <= kShortRowBlocks && p.per <= kShortBlocks) p.ctas = ctas;
     return p;
 }
 
