@@ -368,19 +368,31 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
     cluster_wait();
     if constexpr (APART) {
         // the columns as the finishing kernels add them up, then the mean over the machines
-        for (int e = tid; e < entries * kFinishSlices; e += kShortThreads) {
-            const int entry = e % entries, slice = e / entries, end = a.columns * (slice + 1) / kFinishSlices;
-            float s = 0.f;
+        // (up to eight columns, one per slice: the columns themselves)
+        if (a.columns > kFinishSlices) {
+            for (int e = tid; e < entries * kFinishSlices; e += kShortThreads) {
+                const int entry = e % entries, slice = e / entries, end = a.columns * (slice + 1) / kFinishSlices;
+                float s = 0.f;
 #pragma unroll 4
-            for (int c = a.columns * slice / kFinishSlices; c < end; ++c) s += inbox[c * entries + entry];
-            sums[e] = s;
+                for (int c = a.columns * slice / kFinishSlices; c < end; ++c) s += inbox[c * entries + entry];
+                sums[e] = s;
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
     for (int j = tid; j < m; j += kShortThreads) {
         float sum = 0.f;
         if constexpr (APART) {
-            for (int i = 0; i < machines; ++i) sum += finish_join(sums + i * m + j, entries);
+            for (int i = 0; i < machines; ++i) {
+                if (a.columns > kFinishSlices) {
+                    sum += finish_join(sums + i * m + j, entries);
+                } else {
+                    float s = 0.f;
+#pragma unroll 4
+                    for (int c = 0; c < a.columns; ++c) s += inbox[c * entries + i * m + j];
+                    sum += s;
+                }
+            }
             sum /= (float)machines;
         } else {
 #pragma unroll 8
@@ -432,6 +444,11 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
 constexpr int kShortCounters[3] = {48 << 10, 24 << 10, 8 << 10};
 // Few vectors leave a thread more blocks than vectors, one after the other: up to 2560 blocks per CTA (m = 1: d = 192 670: 11.8 -> 12.6, d = 88 472:
 // 8.0 -> 7.6).
+// Several messages of few vectors: the columns of a warp's threads lie in the same banks, and few threads have a column. So
+// only columns of the small tiles, fewer than 4096 blocks of all machines per CTA, and no more than 13 312 sums of a vector and a machine's block (us: two
+// machines, m = 1, d = 44 234: 7.0 -> 13.2; eight, m = 1, d = 32 111: 8.3 -> 16.6; eight, m = 2, d = 16 054: 7.5 -> 9.9; four, m = 37, d = 2599:
+// 7.5 -> 7.6; but three, m = 3, d = 14 744: 7.8 -> 5.8).
+constexpr int kShortApartBlocks = 4096, kShortApartSums = 13 << 10;
 constexpr int kShortRowBlocks = 16 << 10;
 constexpr int kShortBlocks = 2560;
 ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int sm_count) {
@@ -454,6 +471,7 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
     while (ctas < kShortCluster && nq * m > (int64_t)256 * ctas && ctas < units) ctas *= 2;
     p.columns = (int)units;
     p.per = (int)((units + ctas - 1) / ctas) * p.tile;
+    if (apart && (p.tile > 32 || (int64_t)machines * p.per >= kShortApartBlocks || (int64_t)machines * p.per * m > kShortApartSums)) return p;
     p.stride = p.per | 1;
     p.lanes = 1;
     // up to a warp per vector, several warps where that leaves a lane more than sixteen blocks in a row (m = 3, d = 64 000: 63, and the error of the
