@@ -439,8 +439,7 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
 // Where the one launch applies.  Most counters (m times the blocks) for one message, two to four, five to eight; us, a round by separate
 // kernels -> by one: one machine, m = 64, 9600 counters: 6.8 -> 3.4, m = 8, 48000: 6.7 -> 5.4, m = 16, 65536: 6.0 -> 6.3; four machines, m = 24,
 // 12000: 6.5 -> 5.0, m = 24, 36000: 7.9 -> 8.3; eight machines, m = 8, 4000: 5.9 -> 4.4.  Few columns for many vectors (four machines, d = 54,
-// m = 256: 7.1 -> 17.2 by one CTA) keep the separate kernels, as do more partial gradients than that many per CTA, which take longer
-// to add up on eight SMs than on all (148 of d = 9578: the step 18 -> 37; 148 of 3513: 33.7 -> 32.3).
+// m = 256: 7.1 -> 17.2 by one CTA) keep the separate kernels.
 constexpr int kShortCounters[3] = {48 << 10, 24 << 10, 8 << 10};
 // Few vectors leave a thread more blocks than vectors, one after the other: up to 2560 blocks per CTA (m = 1: d = 192 670: 11.8 -> 12.6, d = 88 472:
 // 8.0 -> 7.6).
@@ -449,7 +448,11 @@ constexpr int kShortCounters[3] = {48 << 10, 24 << 10, 8 << 10};
 // machines, m = 1, d = 44 234: 7.0 -> 13.2; eight, m = 1, d = 32 111: 8.3 -> 16.6; eight, m = 2, d = 16 054: 7.5 -> 9.9; four, m = 37, d = 2599:
 // 7.5 -> 7.6; but three, m = 3, d = 14 744: 7.8 -> 5.8).
 constexpr int kShortApartBlocks = 4096, kShortApartSums = 13 << 10;
-constexpr int kShortRowBlocks = 16 << 10;
+// Partial gradients take longer to add up on eight SMs than on all, the more the longer a CTA's part is, and what follows is in
+// series with it: per block of a CTA two units for a row, four for a vector and forty. us, steps by separate kernels -> by one:
+// 148 rows, d = 2561, m = 65: 16.0 -> 18.9 (48 276 units); 26 rows, d = 18 174, m = 2: 15.7 -> 17.6 (56 800); 80 rows, d = 5000, m = 24: 11.9 -> 12.9
+// (46 472); but 8 rows, d = 16 000, m = 8: 13.9 -> 12.9 (44 000); 148 rows, d = 3500, m = 8: 16.2 -> 12.3 (40 480).
+constexpr int kShortRowUnits = 44000;
 constexpr int kShortBlocks = 2560;
 ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int sm_count) {
     ShortPlan p{};
@@ -484,7 +487,8 @@ ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
     const size_t entries = (size_t)machines * m;
     p.smem = ((size_t)m * p.stride + (size_t)machines * p.per + kShortThreads + m) * 16 +
              ((apart ? p.columns + kFinishSlices : ctas) * entries + m) * 4;
-    if (p.smem <= 200 * 1024 && (int64_t)rows * p.per <= kShortRowBlocks && p.per <= kShortBlocks) p.ctas = ctas;
+    if (rows > 1 && (2 * (int64_t)rows + 4 * m + 40) * p.per > kShortRowUnits) return p;
+    if (p.smem <= 200 * 1024 && p.per <= kShortBlocks) p.ctas = ctas;
     return p;
 }
 
