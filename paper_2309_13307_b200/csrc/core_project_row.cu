@@ -41,9 +41,10 @@ namespace core {
 namespace {
 
 constexpr int kRowJT = 4;                        // vectors per generating thread
-// With the table: steps that are added up before they meet the sums in shared memory.  The chain of additions is this long, then as
-// long as a CTA's tiles have such parts; both about a hundred in rows of 2.5e7 (errors grow with the square root of their sum).
-constexpr int kRowSumSteps = 64;
+// Steps that are added up before they meet the sum of all: the longest chain of additions but that one, which has as many links as a CTA's
+// tiles have such parts.  A message's rounding error grows with the square root of such a chain: 64 steps made that of rows whose CTAs
+// have one long tile a quarter larger (d = 1 000 003, m = 100: rms 1.76e-7 of the row's norm -> 2.31e-7).
+constexpr int kRowSumSteps = 32;
 
 // With the table of angles one CTA fills an SM, without it two do.
 template <bool TURN>
