@@ -398,21 +398,26 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
             const float4 *cur = tile0 + 2 * st * a.tile_q;
             const int blocks = blocks_of(tile);
             const uint64_t q0 = a.q_base + (uint64_t)tile * a.tile_q;
-            // blocks of this tile that share the high counter word of the first one (all of them but once in 2^32)
-            const uint64_t left = 0x100000000ull - (q0 & 0xFFFFFFFFull);
-            int upto = left < (uint64_t)blocks ? (int)left : blocks;
+            // the block of this tile at which the high counter word changes (once in 2^32 blocks)
+            const uint64_t to_change = 0x100000000ull - (q0 & 0xFFFFFFFFull);
+            int change = to_change < (uint64_t)blocks ? (int)to_change : INT_MAX;
             uint32_t q_hi = (uint32_t)(q0 >> 32);
-            float2 acc[kRowJT];
-#pragma unroll
-            for (int v = 0; v < kRowJT; ++v) acc[v] = make_float2(0.f, 0.f);
             int qq = ql;
             if (active) {
-                for (;;) {
+                for (int upto = 0; upto < blocks;) {
+                    if (upto == change) {
+                        ++q_hi;
+                        change = INT_MAX;
+                    }
                     if (!have_jp || q_hi != jp_q_hi) {
                         make_jp(q_hi);
                         jp_q_hi = q_hi;
                         have_jp = true;
                     }
+                    upto = min(min(upto + kRowSumSteps * a.tq, blocks), change);
+                    float2 acc[kRowJT];
+#pragma unroll
+                    for (int v = 0; v < kRowJT; ++v) acc[v] = make_float2(0.f, 0.f);
                     const float4 *entry = cur + 2 * qq;
                     for (; qq < upto; qq += a.tq, entry += 2 * a.tq) {
                         const float4 g = entry[0], e = entry[1];
@@ -432,13 +437,10 @@ project_row_kernel(const __grid_constant__ RowArgs a) {
                             acc[v] = __ffma2_rn(r[v].s, __ffma2_rn(r[v].cs, gs, c), acc[v]);
                         }
                     }
-                    if (upto == blocks) break;
-                    upto = blocks;
-                    ++q_hi;
+#pragma unroll
+                    for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
                 }
             }
-#pragma unroll
-            for (int v = 0; v < kRowJT; ++v) outer[v] += acc[v].x + acc[v].y;
             if (!TOGETHER && tile + 2 < tile_end) bar_arrive(kEmpty + st, kHandOver);
         }
     }
