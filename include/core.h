@@ -323,6 +323,10 @@ int core_ls_gradients(core_ctx *ctx, core_ls *ls, const float *x_dev, float *G_o
  */
 int core_debug_force_project_kernel(int kind);
 
+/* Whether later calls take the kernels for short vectors (on != 0, the default) or leave them out.  Process-wide, for tests of the others at
+ * small sizes. */
+int core_debug_short_kernels(int on);
+
 /*
  * The next `count` device allocations of this library fail as if the device were out of memory
  * (count = 0 switches this off).  Lets a test see CORE_ENOMEM from core_init, core_project,

@@ -54,6 +54,7 @@ _SIGNATURES = {
     "core_reserve_workspace": ([_c.c_void_p, _c.c_int32, _c.c_int], _c.c_int),
     "core_debug_fail_allocations": ([_c.c_int], _c.c_int),
     "core_debug_force_project_kernel": ([_c.c_int], _c.c_int),
+    "core_debug_short_kernels": ([_c.c_int], _c.c_int),
     "core_debug_wait_timeout": ([_c.c_uint32, _c.c_int32, _c.POINTER(_c.c_uint32)], _c.c_int),
     "core_debug_ls_hold_back": ([_c.c_void_p, _c.c_int32], _c.c_int),
     "core_debug_combined_round": ([_c.c_void_p, _c.c_void_p, _c.c_int32, _c.c_int64, _c.c_float, _c.c_void_p, _c.c_void_p], _c.c_int),
@@ -223,6 +224,12 @@ def core_debug_force_project_kernel(kind: int) -> None:
     rc = lib().core_debug_force_project_kernel(int(kind))
     if rc != CORE_OK:
         raise CoreError(rc, "core_debug_force_project_kernel")
+
+
+def core_debug_short_kernels(on: bool) -> None:
+    rc = lib().core_debug_short_kernels(int(on))
+    if rc != CORE_OK:
+        raise CoreError(rc, "core_debug_short_kernels")
 
 
 def core_debug_fail_allocations(count: int) -> None:

@@ -145,7 +145,7 @@ bool combine_first(const core_ctx *ctx, int32_t n) {
 
 // A short vector's round of n machines goes through one kernel, and so does the projection of one (unless a test asks for one of the others).
 ShortPlan short_plan(const core_ctx *ctx, int32_t n) {
-    return project_kernel_forced() ? ShortPlan{} : make_short_plan(n, 1, ctx->m, ctx->d, ctx->sm_count);
+    return project_kernel_forced() || short_kernels_off() ? ShortPlan{} : make_short_plan(n, 1, ctx->m, ctx->d, ctx->sm_count);
 }
 
 size_t row_partial_bytes(const core_ctx *ctx, int64_t d) {
@@ -200,7 +200,7 @@ int project_all(core_ctx *ctx, const void *G, int dtype, int32_t n, int64_t ldg,
 
 // The estimate of the whole vector, or the update made from it.
 int reconstruct_all(core_ctx *ctx, float *pbar, float *out, const ReconstructEpilogue *epilogue, const MessageParts *parts = nullptr) {
-    const ShortPlan plan = make_short_plan(1, 1, ctx->m, ctx->d, ctx->sm_count);
+    const ShortPlan plan = short_kernels_off() ? ShortPlan{} : make_short_plan(1, 1, ctx->m, ctx->d, ctx->sm_count);
     if (plan.ctas > 0)
         CORE_CUDA(ctx, launch_short_reconstruct(plan, ctx->keys, ctx->t, pbar, ctx->d, ctx->m, out, ctx->sm_count, epilogue, parts, ctx->stream));
     else
@@ -694,7 +694,7 @@ static int ls_loss_into(core_ctx *ctx, core_ls *ls, const float *x, double *loss
 // The round of one combined gradient, scale times the sum of `count` rows, of a context's whole vector.
 static int combined_round(core_ctx *ctx, const float *rows, int32_t count, int64_t ld, float scale, float *pbar, float *out,
                           const ReconstructEpilogue *epilogue, const StepRule *rule) {
-    const ShortPlan plan = make_short_plan(1, count, ctx->m, ctx->d, ctx->sm_count);
+    const ShortPlan plan = short_kernels_off() ? ShortPlan{} : make_short_plan(1, count, ctx->m, ctx->d, ctx->sm_count);
     if (plan.ctas > 0 && !rule) {
         CORE_CUDA(ctx, launch_short_round(plan, ctx->keys, ctx->t, rows, CORE_F32, count, 1, ld, scale, ctx->d, ctx->m, nullptr, pbar, out, epilogue,
                                           ctx->stream));
@@ -861,6 +861,11 @@ int core_ls_loss_host(core_ctx *ctx, core_ls *ls, const float *x_dev, double *lo
 int core_debug_force_project_kernel(int kind) {
     if (kind < -1 || kind > 2) return CORE_EINVAL;
     project_force_kernel(kind);
+    return CORE_OK;
+}
+
+int core_debug_short_kernels(int on) {
+    short_kernels_set(on != 0);
     return CORE_OK;
 }
 

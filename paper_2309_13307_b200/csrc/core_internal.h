@@ -174,6 +174,9 @@ struct ShortPlan {
     int columns, tile, tq, uq;       // several messages: columns, blocks and lanes of the separate kernel's tiles
     size_t smem;
 };
+// Test hook: none of these kernels.
+void short_kernels_set(bool on);
+bool short_kernels_off();
 ShortPlan make_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, int sm_count);
 // The reconstruction alone, with the same bits (per and ctas of the plan do not matter): `per` blocks and `threads` threads per CTA.
 struct ShortGrid {

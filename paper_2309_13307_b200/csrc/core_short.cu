@@ -436,6 +436,12 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
 
 }  // namespace
 
+namespace {
+bool g_off = false;
+}
+void short_kernels_set(bool on) { g_off = !on; }
+bool short_kernels_off() { return g_off; }
+
 // Where the one launch applies.  Most counters (m times the blocks) for one message, two to four, five to eight; us, a round by separate
 // kernels -> by one: one machine, m = 64, 9600 counters: 6.8 -> 3.4, m = 8, 48000: 6.7 -> 5.4, m = 16, 65536: 6.0 -> 6.3; four machines, m = 24,
 // 12000: 6.5 -> 5.0, m = 24, 36000: 7.9 -> 8.3; eight machines, m = 8, 4000: 5.9 -> 4.4.  Few columns for many vectors (four machines, d = 54,

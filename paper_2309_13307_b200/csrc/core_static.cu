@@ -97,7 +97,7 @@ int core_project_static(uint64_t seed, uint32_t t, int64_t d, int32_t m, const v
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const RoundKeys keys = expand_keys(seed);
-    const ShortPlan short_plan = n > 1 || project_kernel_forced() ? ShortPlan{} : make_short_plan(1, 1, m, d, sm_count);     // as core_project does
+    const ShortPlan short_plan = n > 1 || project_kernel_forced() || short_kernels_off() ? ShortPlan{} : make_short_plan(1, 1, m, d, sm_count);     // as core_project does
     if (short_plan.ctas > 0) {
         e = launch_short_round(short_plan, keys, t, G_dev, dtype, 1, n, ldg, 1.0f, d, m, P_dev, nullptr, nullptr, nullptr, stream);
         if (e != cudaSuccess) {

@@ -1,7 +1,7 @@
 """Short vectors, whose round is one launch: a cluster keeps the Gaussians between projection and reconstruction.  At the sizes where it can
 go wrong: CTAs without blocks, every cluster size, several machines' messages (the very numbers of the separate kernels), ragged
-and unaligned rows, both sides of the lines to the separate kernels, replays from a graph, steps side by side.  Also rows a little too
-long for that."""
+and unaligned rows, both sides of the lines to the separate kernels (which case takes which is asserted in test_short_plan.py), replays from
+a graph, steps side by side.  Also rows a little too long for that, and the separate kernels at the sizes of the short ones."""
 import threading
 
 import numpy as np
@@ -10,7 +10,9 @@ import torch
 
 import core_inputs
 import oracle
+import test_gpu_round_paths as round_paths
 from helpers import P_TOL, REC_TOL, rel_l2, row_norms
+from test_short_plan import ROUTES, ROW_ROUTES
 
 pytestmark = pytest.mark.gpu
 
@@ -51,6 +53,74 @@ def test_round_equals_its_parts_and_the_oracle(core_mod, n, d, m, dtype, offset,
         assert torch.equal(P3, P)
 
 
+@pytest.fixture
+def without_short_kernels(core_mod):
+    from paper_2309_13307_b200 import binding
+    binding.core_debug_short_kernels(False)
+    yield
+    binding.core_debug_short_kernels(True)
+
+
+@pytest.mark.parametrize("n,d,m,dtype,offset,pad,ctas", ROUTES)
+def test_routes(core_mod, n, d, m, dtype, offset, pad, ctas):
+    from paper_2309_13307_b200 import binding
+    test_round_equals_its_parts_and_the_oracle(core_mod, n, d, m, dtype, offset, pad)
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("routes of another device")
+    G = core_inputs.gradients(n, d + offset, seed=1, dtype=dtype, device="cuda", ld=d + offset + pad)[:, offset:]
+    ctx = core_mod.Core(5, d, m)
+    pbar, gt = ctx.core_round(G)
+    binding.core_debug_short_kernels(False)
+    try:
+        ctx.core_set_round(0)
+        want, want_gt = ctx.core_round(G)
+    finally:
+        binding.core_debug_short_kernels(True)
+    # messages kept apart are the same numbers by either; a single one is added up in another order, and so is the estimate
+    if n > 1:
+        assert torch.equal(pbar, want)
+    assert float((pbar - want).abs().max()) <= P_TOL * float(G.float().norm(dim=1).mean())
+    assert rel_l2(gt.cpu().numpy(), want_gt.cpu().numpy()) <= REC_TOL
+
+
+@pytest.mark.parametrize("rows,d,m,ctas", ROW_ROUTES)
+def test_sums_of_rows(core_mod, rows, d, m, ctas):
+    G = core_inputs.gradients(rows, d, seed=d + m, device="cuda", ld=(d + 3) // 4 * 4)
+    ctx = core_mod.Core(3, d, m)
+    pbar, gt = ctx.core_debug_combined_round(G, 0.5)
+    row = np.ascontiguousarray((0.5 * G.cpu().numpy().astype(np.float64).sum(axis=0, keepdims=True)).astype(np.float32))
+    assert np.abs(pbar.cpu().numpy() - oracle.project(3, 0, m, row)[0]).max() <= P_TOL * row_norms(row)[0]
+    assert rel_l2(gt.cpu().numpy(), oracle.reconstruct(3, 0, pbar.cpu().numpy().astype(np.float64), d)) <= REC_TOL
+
+
+SINGLE_ROWS = round_paths.test_single_machine_projection.pytestmark[0].args[1]
+RECONSTRUCTIONS = round_paths.test_short_reconstructions.pytestmark[0].args[1]
+
+
+@pytest.mark.parametrize("d,m,dtype,offset", [*SINGLE_ROWS, *((d, m, t, o) for d in (1, 3, 5, 17) for m, t, o in ((4097, "f32", 1), (2, "bf16", 1), (9, "f32", 2),
+                                                                                                               (21, "bf16", 6), (5000, "f32", 3)))])
+def test_single_rows_without_the_short_kernels(core_mod, without_short_kernels, d, m, dtype, offset):
+    round_paths.test_single_machine_projection(core_mod, d, m, dtype, offset)
+
+
+@pytest.mark.parametrize("d,m", RECONSTRUCTIONS)
+def test_reconstructions_without_the_short_kernels(core_mod, without_short_kernels, d, m):
+    round_paths.test_short_reconstructions(core_mod, d, m)
+
+
+@pytest.mark.parametrize("m,d", [(64, 2900), (3, 64_000), (400, 262_144), (100, 1_000_003)])
+def test_rounding_errors_of_a_message(core_mod, m, d):
+    """A chain of k additions of terms alike has an rms error of 2^-24 sqrt(k / 6) of the row's norm; with k <= 32 (24 in one launch) and the
+    Gaussians' own errors (7.5e-8 each) and the later sums, 1.3e-7 together, that is 1.9e-7.  Chains of 64 would be 2.3e-7."""
+    errors = []
+    for seed in range(max(1, 400 // m)):
+        G = core_inputs.gradients(1, d, seed=seed, device="cuda")
+        Gh = core_inputs.to_oracle_array(G)
+        got = core_mod.Core(100 + seed, d, m).core_project(G).cpu().numpy().astype(np.float64)
+        errors.append((got - oracle.project(100 + seed, 0, m, Gh)) / row_norms(Gh)[0])
+    assert np.sqrt(np.mean(np.square(errors))) <= 2.1e-7
+
+
 STEPS = [(1, 5, 3, 8), (3, 40, 54, 16), (2, 7, 130, 9), (20, 11, 784, 64), (2, 150, 1201, 33), (3, 60, 1700, 100),   # one cluster
          (2, 30, 9000, 65), (1, 149, 4099, 256), (4, 20, 20_003, 20), (2, 9, 32_768, 256), (3, 70, 9578, 18)]          # separate kernels
 
@@ -88,7 +158,7 @@ def test_steps_replayed_from_a_graph_and_side_by_side(core_mod, n, rows, d, m):
     stream = torch.cuda.Stream()
     torch.cuda.synchronize()
     ctx, ls = steps(stream, 6, want)
-    # three steps of one graph, replayed with t set back: the same rounds twice
+    # three steps of one graph, replayed twice from the same start: the same rounds, with nothing left over from the first
     x = start.clone()
     once = start.clone()
     steps(stream, 3, once)
@@ -97,11 +167,12 @@ def test_steps_replayed_from_a_graph_and_side_by_side(core_mod, n, rows, d, m):
     with torch.cuda.graph(graph, stream=stream):
         for _ in range(3):
             ctx.core_gd_step(ls, 0.3, x)
-    x.copy_(start)
-    torch.cuda.synchronize()
-    graph.replay()
-    torch.cuda.synchronize()
-    assert torch.equal(x, once)
+    for _ in range(2):
+        x.copy_(start)
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(x, once)
     del graph
     # three threads, a context and a stream each
     got = [start.clone() for _ in range(3)]
