@@ -122,13 +122,15 @@ int core_device_status(int32_t *status_out);
  *           Rows may have any alignment.  Several rows whose byte addresses and
  *           stride are multiples of 16 are copied asynchronously, others element by
  *           element, with the same result; a single row is read 16 bytes at a time
- *           wherever it starts.
+ *           wherever it starts (a short one a block of four coordinates at a time, where
+ *           its address is a multiple of a block's bytes and ldg of 4).
  *   P_dev   n*m floats, row-major.
  * fp32 multiply-add with two-level fp32 accumulation and a fixed reduction
  * order: results are bitwise reproducible for a given (n, m, d, dtype), wherever the rows start
  * and whatever ldg is.  (A row's
  * message may differ in the last bits from the same row's among others: one row and
- * several take different kernels, and a short one, of at most 49152 = m times the blocks of four coordinates and 4096 vectors, a third.)
+ * several take different kernels, and a short one a third: at most 4096 vectors, m times the blocks of four coordinates at most 49152, and
+ * less where that many do not fit a CTA's shared memory or a CTA gets more than 2560 blocks; core_debug_short_plan tells.)
  * Machines are processed in groups: up to 64 per pass where the tensor-memory
  * kernel applies (9 or more machines, m > 64 for passes of up to 16 and m >= 96 for
  * longer ones; more than 32 only when m lets a CTA hold 256 vectors, about m >= 256),
@@ -408,7 +410,7 @@ int core_debug_short_plan(int32_t machines, int32_t rows, int32_t m, int64_t d, 
 /*
  * Which reconstruction kernel d coordinates and m vectors take, host-only: out[0] = 0 one of the two for short vectors, 1 the one for long
  * vectors with few or very many Gaussians per coordinate, 2 the one with the table of angles; out[1] = 1 if the CTAs of the
- * reconstruction form the message of a round of one machine themselves.
+ * reconstruction form the message of a round of one machine themselves, where that round is not one launch (core_debug_short_plan).
  */
 int core_debug_reconstruct_plan(int64_t d, int32_t m, int32_t sm_count, int32_t out[2]);
 

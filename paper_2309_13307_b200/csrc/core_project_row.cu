@@ -20,7 +20,7 @@
 //
 // Three modes.  kRowTurn, wherever there is work for it: angles from the table, one CTA of 24 generating and 4 staging warps
 // per SM, d = 2.56e7, m = 256: 4944 us = 1.32e12 Gaussians/s.  kRowShort: angles from the polynomials, two CTAs of 8 and 2
-// warps per SM (5325 us there), for short work.  kRowTogether: the same, all warps stage.  In kRowTurn the registers decide:
+// warps per SM (d = 2.5e7: 5325 us, with the table 4904), for short work.  kRowTogether: the same, all warps stage.  In kRowTurn the registers decide:
 // 72 per thread hold the loop only because the sums over tiles live in shared memory and scalar accumulators
 // (packed ones need pairs: 5138 us) and 32-bit counts go around it (64-bit tile numbers: 5095); 20 generating warps of 80 registers:
 // 5169, 28 of 64: 5144, two counters at a time: 5379.
@@ -558,7 +558,8 @@ static RowPlan plan_rows(bool turn, bool heavy, int32_t m, int64_t d, int sm_cou
     // 3.1e7, m = 1024: 24198 -> 23915; without the table, seven shifted rows of 1e7, m = 64: 595 -> 589; more steps gained nothing more.
     // Many rows with the table (row_heavy): 32, since nothing is generated before a CTA's first tile is there.  us, 32 -> 128 steps:
     // 64 rows of 4e6, m = 200: 1260 -> 1273; but 40 of 5e6, m = 357: 2770 -> 2762;
-    // 64 of 2e6, m = 1000: 3025 -> 3001; 24 bf16 rows of 1e7, m = 100: 1543 -> 1534.
+    // 64 of 2e6, m = 1000: 3025 -> 3001; 24 bf16 rows of 1e7, m = 100: 1543 -> 1534.  Not without the table, where all warps stage: 64 shifted rows
+    // of 4e6, m = 200, with 32 steps instead of 64: 1409 -> 1522.
     const int steps_most = turn ? heavy ? 32 : RowCta<true>::kTileSteps : RowCta<false>::kTileSteps;
     const int64_t most = steps_most * p.tq < room ? steps_most * p.tq : room / p.tq * p.tq;
     const int64_t least_tiles = (nq + slots * most - 1) / (slots * most);

@@ -296,9 +296,9 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
     const int tid = threadIdx.x, ql = tid % QB, slice = tid / QB;
     uint32_t rank = 0, ranks = 1;
     if constexpr (RANKS > 1) {
-        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        rank = cluster_rank();
         asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(ranks));
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA has started
+        cluster_arrive();                          // this CTA has started
     }
     const uint64_t q_begin = (uint64_t)a.k_begin >> 2;
     const uint64_t q_end = ((uint64_t)a.k_end + 3) >> 2;
@@ -355,10 +355,11 @@ reconstruct_small_kernel(const __grid_constant__ ReconstructArgs a) {
         }
     }
     if constexpr (RANKS > 1) {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");       // the first CTA has started
+        cluster_wait();                            // the first CTA has started
         if (ranks > 1) {
             if (slice == 0 && rank > 0) store_cluster(&inbox[rank][ql], 0, s);
-            asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            cluster_arrive();
+            cluster_wait();
             if (rank > 0) return;
             if (slice == 0)
                 for (int r = 1; r < (int)ranks; ++r) {
