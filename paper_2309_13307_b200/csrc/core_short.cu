@@ -30,6 +30,7 @@ constexpr int kShortCluster = 8;                  // most CTAs
 constexpr int kShortVectors = 4096;               // most vectors
 constexpr int kShortMachines = 8;                 // most messages kept apart
 constexpr int kShortLaneBlocks = 16;              // blocks of a lane from which a vector gets more than one warp
+constexpr int kShortChainBlocks = 4;              // most blocks of a lane that are added up in one chain
 constexpr int kShortSlices = 64;                  // most ranges of the vectors (reconstruction) a block's sum is cut into
 
 struct ShortArgs {
@@ -333,8 +334,23 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
             for (uint32_t r = 0; r < ranks; ++r) store_remote(inbox + (column0 + column) * entries + e, r, sum);
         }
     } else {
+        // Up to four blocks of a lane in one chain of up to 16 additions, more in four sums, whose chains are as long as the lane has blocks
+        // (rms error of a message, of the gradient's norm, m = 64, d = 2900, twelve blocks: one chain 1.8e-7, four sums 1.5e-7).
+        const bool chain = per <= kShortChainBlocks * a.lanes;
         const auto dot = [&](int j, int sub) {
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);                       // four sums: a chain is as long as a lane has blocks
+            if (chain) {
+                float p = 0.f;
+                if (j < m)
+                    for (int q = sub; q < mine; q += a.lanes) {
+                        const float4 v = z[j * a.stride + q], b = g[q];
+                        p = fmaf(b.x, v.x, p);
+                        p = fmaf(b.y, v.y, p);
+                        p = fmaf(b.z, v.z, p);
+                        p = fmaf(b.w, v.w, p);
+                    }
+                return p;
+            }
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
             if (j < m)
                 for (int q = sub; q < mine; q += a.lanes) {
                     const float4 v = z[j * a.stride + q], b = g[q];

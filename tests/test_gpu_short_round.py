@@ -121,6 +121,41 @@ def test_rounding_errors_of_a_message(core_mod, m, d):
     assert np.sqrt(np.mean(np.square(errors))) <= 2.1e-7
 
 
+@pytest.mark.parametrize("d,m", [(54, 16), (7, 3), (784, 64), (1000, 64), (1030, 64), (2900, 64)])
+def test_order_of_a_single_message(core_mod, d, m):
+    """The very numbers: up to four blocks of a lane in one chain, more in four sums; lanes in pairs, CTAs in ascending order."""
+    from paper_2309_13307_b200 import binding
+    plan = binding.core_debug_short_plan(m, d)
+    per, lanes, blocks = plan["per"], plan["lanes"], (d + 3) // 4
+    G = core_inputs.gradients(1, d, seed=m, device="cuda")
+    ctx = core_mod.Core(8, d, m)
+    got = ctx.core_project(G)[0].cpu().numpy()
+    g = np.zeros(4 * blocks, np.float32)
+    g[:d] = G[0].cpu().numpy()
+    g = g.reshape(blocks, 4)
+    z = np.stack([ctx.core_debug_gaussians(j, 0, blocks).cpu().numpy() for j in range(m)])
+
+    def fma(a, b, c):                                              # the product is exact in 64 bits
+        return (np.float64(a) * b.astype(np.float64) + c).astype(np.float32)
+
+    want = np.zeros(m, np.float32)
+    for first in range(0, blocks, per):
+        end = min(first + per, blocks)
+        parts = np.zeros((lanes, m), np.float32)
+        for lane in range(lanes):
+            s = np.zeros((4, m), np.float32)
+            chain = 0 if per <= 4 * lanes else None
+            for q in range(first + lane, end, lanes):
+                for c in range(4):
+                    to = c if chain is None else chain
+                    s[to] = fma(g[q, c], z[:, q, c], s[to])
+            parts[lane] = s[0] if chain == 0 else (s[0] + s[1]) + (s[2] + s[3])
+        while len(parts) > 1:
+            parts = parts[:len(parts) // 2] + parts[len(parts) // 2:]
+        want = want + parts[0]
+    assert np.array_equal(got, want)
+
+
 STEPS = [(1, 5, 3, 8), (3, 40, 54, 16), (2, 7, 130, 9), (20, 11, 784, 64), (2, 150, 1201, 33), (3, 60, 1700, 100),   # one cluster
          (2, 30, 9000, 65), (1, 149, 4099, 256), (4, 20, 20_003, 20), (2, 9, 32_768, 256), (3, 70, 9578, 18)]          # separate kernels
 
