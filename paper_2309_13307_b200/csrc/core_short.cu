@@ -383,32 +383,21 @@ short_round_kernel(const __grid_constant__ ShortArgs a) {
     cluster_arrive();
     cluster_wait();
     if constexpr (APART) {
-        // the columns as the finishing kernels add them up, then the mean over the machines
-        // (up to eight columns, one per slice: the columns themselves)
-        if (a.columns > kFinishSlices) {
-            for (int e = tid; e < entries * kFinishSlices; e += kShortThreads) {
-                const int entry = e % entries, slice = e / entries, end = a.columns * (slice + 1) / kFinishSlices;
-                float s = 0.f;
+        // the columns as the finishing kernels add them up, then the mean over the machines (up to eight columns, a slice each at most, in the
+        // same way: a second way in the kernel cost all rounds more, four machines, d = 4096, m = 16: 5.17 -> 5.27 us, d = 700: 4.17 -> 4.34)
+        for (int e = tid; e < entries * kFinishSlices; e += kShortThreads) {
+            const int entry = e % entries, slice = e / entries, end = a.columns * (slice + 1) / kFinishSlices;
+            float s = 0.f;
 #pragma unroll 4
-                for (int c = a.columns * slice / kFinishSlices; c < end; ++c) s += inbox[c * entries + entry];
-                sums[e] = s;
-            }
-            __syncthreads();
+            for (int c = a.columns * slice / kFinishSlices; c < end; ++c) s += inbox[c * entries + entry];
+            sums[e] = s;
         }
+        __syncthreads();
     }
     for (int j = tid; j < m; j += kShortThreads) {
         float sum = 0.f;
         if constexpr (APART) {
-            for (int i = 0; i < machines; ++i) {
-                if (a.columns > kFinishSlices) {
-                    sum += finish_join(sums + i * m + j, entries);
-                } else {
-                    float s = 0.f;
-#pragma unroll 4
-                    for (int c = 0; c < a.columns; ++c) s += inbox[c * entries + i * m + j];
-                    sum += s;
-                }
-            }
+            for (int i = 0; i < machines; ++i) sum += finish_join(sums + i * m + j, entries);
             sum /= (float)machines;
         } else {
 #pragma unroll 8
